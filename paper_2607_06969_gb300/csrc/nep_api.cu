@@ -26,6 +26,7 @@ struct nep_model {
     int tune_angular[nep::kSizeBins];   // angular kernel variant per size class, -1 = default
     int tune_radial[nep::kSizeBins];    // radial kernel block size per size class, 0 = default
     int tune_finish[nep::kSizeBins];    // finish kernel block size per size class, 0 = default
+    bool pinned[nep::kSizeBins];        // the caller chose launch parameters of the one-thread-per-atom kernels
 };
 
 namespace {
@@ -231,6 +232,20 @@ int angular_variant(const nep_model* m, const nep_system* s) {
 }
 int radial_block(const nep_model* m, const nep_system* s) { return m->tune_radial[size_bin(s)]; }
 int finish_block(const nep_model* m, const nep_system* s) { return m->tune_finish[size_bin(s)]; }
+// Lanes per atom of an evaluation: 0 for the one-thread-per-atom kernels.
+// A call whose launch choices the caller pinned (nep_set_variant,
+// nep_set_launch) runs those kernels.  The lines lie where the two forms
+// measured equal (one evaluation in a graph, rock salt at 0.033 atoms per A^3):
+//   32 against 8 lanes: 3,686 atoms 48.5 / 46.3 us (38-30-1), 57 / 56 (52-64-1)
+//   8 lanes against one thread: 19,757 atoms 97 / 123 us (38-30-1), 112 / 140
+//   (42-50-1), 147 / 154 (52-64-1); 35,374 atoms 144 / 124, 167 / 142, 221 / 157
+//   the same with the FP16 network: 100 / 135 and 152 / 193; 146 / 138, 226 / 199
+int group_lanes(const nep_model* m, const nep_system* s) {
+    if (m->pinned[size_bin(s)] || !m->ks->group_fits(m->hp.n_hidden)) return 0;
+    const bool wide = m->hp.n_hidden * m->lay.D > 2500;
+    const int most = (wide ? 20000 : 26000) + (m->hp.precision ? 6000 : 0);
+    return s->n_atoms <= 3000 ? 32 : (s->n_atoms <= most ? 8 : 0);
+}
 bool block_choice(int b) {
     for (int c : nep::kBlockChoices)
         if (b == c) return true;
@@ -437,10 +452,16 @@ nep_status efv_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, floa
     auto mark = [&](int k) -> cudaError_t {
         return nt ? cudaEventRecordWithFlags(m->timing[k], st, rec_flags) : cudaSuccess;
     };
+    const int G = N > 0 ? group_lanes(m, s) : 0;
     NEP_CUDA(mark(0), "timing event");
-    if (N > 0) NEP_CUDA(m->ks->radial(a, st, radial_block(m, s)), "radial kernel");
-    NEP_CUDA(mark(1), "timing event");
-    if (N > 0) NEP_CUDA(m->ks->angular(a, st, vd), "angular kernel");
+    if (G) {
+        NEP_CUDA(mark(1), "timing event");       // the radial sums are part of the next kernel
+        NEP_CUDA(m->ks->group_atom(a, st, G), "atom kernel");
+    } else {
+        if (N > 0) NEP_CUDA(m->ks->radial(a, st, radial_block(m, s)), "radial kernel");
+        NEP_CUDA(mark(1), "timing event");
+        if (N > 0) NEP_CUDA(m->ks->angular(a, st, vd), "angular kernel");
+    }
     NEP_CUDA(mark(2), "timing event");
     nep::FinishArgs f;
     f.atom_off = s->atom_off;
@@ -449,7 +470,8 @@ nep_status efv_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, floa
     f.force = force;
     f.e_out = e_atom;
     f.n_owned = n_owned < 0 ? N : n_owned;
-    NEP_CUDA(m->ks->finish(a, f, w.max_chunks, st, finish_block(m, s)), "finish kernel");
+    if (G) NEP_CUDA(m->ks->group_finish(a, f, w.max_chunks, st, G), "finish kernel");
+    else NEP_CUDA(m->ks->finish(a, f, w.max_chunks, st, finish_block(m, s)), "finish kernel");
     NEP_CUDA(mark(3), "timing event");
     NEP_CUDA(nep::launch_final_reduce(B, at<int>(work, w.chunk_start), at<double>(work, w.partial), e_tot,
                                       virial, st),
@@ -623,9 +645,11 @@ nep_status nep_create(const nep_hparams* hp, const float* params_host, size_t n_
         m->tune_angular[b] = -1;
         m->tune_radial[b] = 0;
         m->tune_finish[b] = 0;
+        m->pinned[b] = false;
     }
     cudaError_t e = ks ? ks->init(hp->n_hidden) : cudaSuccess;
     if (e == cudaSuccess && ks) e = ks->train_init(hp->n_hidden);
+    if (e == cudaSuccess && ks) e = ks->group_init(hp->n_hidden);
     if (e != cudaSuccess) {
         delete m;
         return cuda_fail(e, "kernel attributes");
@@ -1148,7 +1172,10 @@ nep_status nep_set_variant(nep_model* m, int size_class, int variant) {
     if (variant < -1 || variant >= nep::kVariants)
         return fail(NEP_ERR_ARG, "variant must be -1 or 0..%d", nep::kVariants - 1);
     for (int b = 0; b < nep::kSizeBins; ++b)
-        if (size_class < 0 || b == size_class) m->tune_angular[b] = variant;
+        if (size_class < 0 || b == size_class) {
+            m->tune_angular[b] = variant;
+            m->pinned[b] = variant >= 0;
+        }
     return NEP_OK;
 }
 
@@ -1165,6 +1192,7 @@ nep_status nep_set_launch(nep_model* m, int size_class, int variant, int radial_
             m->tune_angular[b] = variant;
             m->tune_radial[b] = radial_block;
             m->tune_finish[b] = finish_block;
+            m->pinned[b] = variant >= 0 || radial_block || finish_block;
         }
     return NEP_OK;
 }

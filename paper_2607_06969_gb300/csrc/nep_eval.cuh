@@ -1190,7 +1190,11 @@ cudaError_t init_t(int H) {
                                    &launch_finish_t<Cfg<NR, NA, KR, KA, H4, T>>,                 \
                                    &train_init_t<Cfg<NR, NA, KR, KA, H4, T>>,                    \
                                    &train_t<Cfg<NR, NA, KR, KA, H4, T>>,                         \
-                                   &grad_chunks_t<Cfg<NR, NA, KR, KA, H4, T>>};
+                                   &grad_chunks_t<Cfg<NR, NA, KR, KA, H4, T>>,                   \
+                                   &group_fits_t<Cfg<NR, NA, KR, KA, H4, T>>,                    \
+                                   &group_init_t<Cfg<NR, NA, KR, KA, H4, T>>,                    \
+                                   &launch_group_t<Cfg<NR, NA, KR, KA, H4, T>>,                  \
+                                   &launch_group_finish_t<Cfg<NR, NA, KR, KA, H4, T>>};
 #endif
 
 }  // namespace nep

@@ -132,6 +132,11 @@ struct KernelSet {
     cudaError_t (*train_init)(int H);
     cudaError_t (*train)(const TrainArgs&, cudaStream_t);   // tangent ... gradient
     int (*grad_chunks)(int N);
+    // a group of G lanes per atom (nep_group.cuh), G = 8 or 32
+    bool (*group_fits)(int H);
+    cudaError_t (*group_init)(int H);
+    cudaError_t (*group_atom)(const EvalArgs&, cudaStream_t, int G);
+    cudaError_t (*group_finish)(const EvalArgs&, const FinishArgs&, int max_chunks, cudaStream_t, int G);
 };
 
 const KernelSet* find_kernel_set(int n_rad, int n_ang, int k_rad, int k_ang, int has_4body,

@@ -24,6 +24,7 @@
 //             in fixed order.
 #pragma once
 #include "nep_eval.cuh"
+#include "nep_group.cuh"
 #include "nep_mlp_tc.cuh"
 
 namespace nep {

@@ -22,6 +22,7 @@ def nb():
 
 def setup(nb, h, counts, tag, skin=0.0, cap=128, cap_ang=64, seed=5, precision=0):
     s = I.packing_batch(counts, tag=tag)
+    s.box[np.diff(s.atom_off) == 0] = 20.0          # an empty configuration still has a box
     model = nb.Model(h, I.init_params(h, seed=seed).astype(np.float32), precision=precision)
     dsys = nb.DeviceSystem.from_inputs(s)
     nl = nb.NeighborList(s.n_atoms, cap, cap_ang)
@@ -68,3 +69,73 @@ def test_fp64_gradient_chunk_edges(nb, counts):
         at = (t + 1) * (h.n_hidden * h.dim + 2 * h.n_hidden + 1) - 1
         want = a_e[s.cfg_of_atom()][s.types == t].sum()
         assert abs(whole[at] - want) <= 1e-10 * s.n_atoms
+
+
+MODELS = dict(small=I.HYPER_SMALL, table2=I.HYPER_TABLE2, large=I.HYPER_LARGE,
+              tiny=I.Hyper(n_rad=3, n_ang=2, k_rad=4, k_ang=3, n_hidden=5, rc_rad=5.0, rc_ang=4.0))
+
+
+def both_forms(nb, model, dsys, nl, ws):
+    """(default choice, one thread per atom) of one evaluation, as arrays."""
+    got = [t.cpu().numpy().copy() for t in nb.energy_forces_virial(model, dsys, nl, ws)]
+    nb.set_variant(model, 0)
+    want = [t.cpu().numpy().copy() for t in nb.energy_forces_virial(model, dsys, nl, ws)]
+    nb.set_variant(model, -1)
+    again = [t.cpu().numpy().copy() for t in nb.energy_forces_virial(model, dsys, nl, ws)]
+    for x, y in zip(got, again):
+        assert np.array_equal(x, y)
+    return got, want
+
+
+def assert_close(got, want, n, tol=1.0):
+    """FP32 sums of some tens of terms of order 0.1 to 1 in another order:
+    1e-6 eV in E_i, 1e-5 eV/A in the forces, and per atom in the totals."""
+    assert np.abs(got[0] - want[0]).max() <= tol * 1e-6
+    assert np.abs(got[1] - want[1]).max() <= tol * 1e-5
+    assert np.all(np.abs(got[2] - want[2]) <= tol * 1e-6 * np.maximum(n, 1))
+    assert np.all(np.abs(got[3] - want[3]).max(1) <= tol * 1e-5 * np.maximum(n, 1))
+
+
+@pytest.mark.parametrize("hname", list(MODELS))
+@pytest.mark.parametrize("counts,skin", [([1], 0.0), ([3], 0.0), ([2, 0, 33], 0.5), ([24, 127, 130], 1.0),
+                                         ([1500, 1499], 0.0), ([1500, 1501], 0.0), ([3700, 17, 300], 1.0)])
+def test_lane_groups_agree_with_one_thread_per_atom(nb, hname, counts, skin):
+    """A group of lanes per atom (32 up to 3,000 atoms, then 8): fewer atoms
+    than one block holds, remainders of a block, an empty configuration, both
+    sides of the line between the two group sizes, boxes shorter than the
+    cutoff (images) and with a skin."""
+    h = MODELS[hname]
+    s, model, dsys, nl, ws = setup(nb, h, counts, 62, skin=skin, cap=160, cap_ang=80)
+    assert_close(*both_forms(nb, model, dsys, nl, ws), np.diff(s.atom_off))
+
+
+def test_lane_groups_many_angular_pairs(nb):
+    """More angular pairs per atom than the group's slot list holds (96)."""
+    s = I.packing_batch([500, 40], density=0.25, dmin=1.1, tag=63)
+    h = I.HYPER_SMALL
+    model = nb.Model(h, I.init_params(h, seed=5).astype(np.float32))
+    dsys = nb.DeviceSystem.from_inputs(s)
+    nl = nb.NeighborList(s.n_atoms, 640, 256)
+    ws = nb.Workspace(model, s.n_atoms, s.n_cfg, 640, 256)
+    nb.neighbors(model, dsys, nl, 0.0, ws)
+    assert nb.check_list(nl) == nb.NEP_OK, nb.last_error()
+    assert int(nl.cnt_ang.max()) > 96
+    got, want = both_forms(nb, model, dsys, nl, ws)
+    # six to seven times the pairs of the normal density, and sums as much larger
+    scale = max(1.0, float(np.abs(want[1]).max()))
+    assert_close(got, want, np.diff(s.atom_off), tol=10.0 * scale)
+
+
+@pytest.mark.parametrize("precision", [1, 2])
+@pytest.mark.parametrize("hname", ["small", "table2", "large"])
+def test_lane_groups_16bit_network(nb, hname, precision):
+    """The 16-bit network of the group form rounds q, W0 and g as the tensor-
+    core kernel does: the two differ only where FP32 sums in another order put
+    an operand on the other side of a rounding step (2^-11 or 2^-8 of it, one
+    operand in about a thousand), far below the 16-bit error itself."""
+    h = MODELS[hname]
+    s, model, dsys, nl, ws = setup(nb, h, [130, 77], 64, precision=precision)
+    got, want = both_forms(nb, model, dsys, nl, ws)
+    step = 2.0 ** -11 if precision == 1 else 2.0 ** -8
+    assert np.abs(got[0] - want[0]).max() <= 0.5 * step
+    assert np.sqrt(np.mean((got[1] - want[1]) ** 2)) <= 0.1 * step
