@@ -71,6 +71,7 @@ struct WsLayout {
     size_t amask;
     size_t gen_p, gen_R, gen_w;   // generic FP32 path: dE/dq (radial), dE/dS, per-atom virial
     size_t plan, cell_of, rank, cell_cnt, cell_start, cell_atoms, cell_pos, scan_tmp, shell, row_start, slot_row;
+    size_t ticket;                // reduction tickets [B]: the cell counts' place, idle during an evaluation
     size_t total;
     int max_chunks, cmax;
 };
@@ -116,6 +117,7 @@ WsLayout ws_layout(const nep_model* m, int N, int B, int cap, int cap_ang) {
     w.cell_of = take(4 * n);
     w.rank = take(4 * n);
     w.cell_cnt = take(4 * ((size_t)w.cmax + 1));
+    w.ticket = w.cell_cnt;        // cmax >= 27 B
     w.cell_start = take(4 * ((size_t)w.cmax + 1));
     w.cell_atoms = take(4 * n);
     w.cell_pos = take(16 * n);
@@ -435,10 +437,10 @@ nep_status efv_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, floa
                     float* force, double* e_tot, double* virial, void* work, const WsLayout& w,
                     cudaStream_t st, int n_owned = -1) {
     const int N = s->n_atoms, B = s->n_cfg;
-    NEP_CUDA(nep::launch_pack(s->pos, s->type, s->atom_off, N, B, m->hp.n_types, at<float4>(work, w.pos4),
-                              at<int>(work, w.cfg), nl->status, st),
+    NEP_CUDA(nep::launch_pack_plan(s->pos, s->type, s->atom_off, N, B, m->hp.n_types, at<float4>(work, w.pos4),
+                                   at<int>(work, w.cfg), nl->status, at<int>(work, w.chunk_start),
+                                   at<int>(work, w.ticket), st),
              "pack");
-    NEP_CUDA(nep::launch_chunk_plan(s->atom_off, B, at<int>(work, w.chunk_start), st), "chunk plan");
     if (!m->ks) return efv_generic(m, s, nl, e_atom, force, e_tot, virial, work, w, st, n_owned);
     const nep::EvalArgs a = make_args(m, s, nl, work, w);
     const int vd = angular_variant(m, s);
@@ -470,12 +472,12 @@ nep_status efv_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, floa
     f.force = force;
     f.e_out = e_atom;
     f.n_owned = n_owned < 0 ? N : n_owned;
+    f.ticket = at<int>(work, w.ticket);
+    f.e_tot = e_tot;
+    f.virial = virial;
     if (G) NEP_CUDA(m->ks->group_finish(a, f, w.max_chunks, st, G), "finish kernel");
     else NEP_CUDA(m->ks->finish(a, f, w.max_chunks, st, finish_block(m, s)), "finish kernel");
     NEP_CUDA(mark(3), "timing event");
-    NEP_CUDA(nep::launch_final_reduce(B, at<int>(work, w.chunk_start), at<double>(work, w.partial), e_tot,
-                                      virial, st),
-             "final reduce");
     return NEP_OK;
 }
 
@@ -485,10 +487,10 @@ nep_status train_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, co
                       double* loss, void* work, const TrainLayout& tl, cudaStream_t st) {
     const int N = s->n_atoms, B = s->n_cfg;
     const WsLayout& w = tl.w;
-    NEP_CUDA(nep::launch_pack(s->pos, s->type, s->atom_off, N, B, m->hp.n_types, at<float4>(work, w.pos4),
-                              at<int>(work, w.cfg), nl->status, st),
+    NEP_CUDA(nep::launch_pack_plan(s->pos, s->type, s->atom_off, N, B, m->hp.n_types, at<float4>(work, w.pos4),
+                                   at<int>(work, w.cfg), nl->status, at<int>(work, w.chunk_start),
+                                   at<int>(work, w.ticket), st),
              "pack");
-    NEP_CUDA(nep::launch_chunk_plan(s->atom_off, B, at<int>(work, w.chunk_start), st), "chunk plan");
     nep::EvalArgs a = make_args(m, s, nl, work, w);
     a.q16_kind = 0;
     a.S = at<float>(work, w.S);
@@ -509,10 +511,10 @@ nep_status train_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, co
         f.force = at<float>(work, tl.force);
         f.e_out = nullptr;
         f.n_owned = N;
+        f.ticket = at<int>(work, w.ticket);
+        f.e_tot = at<double>(work, tl.etot);
+        f.virial = at<double>(work, tl.vir);
         NEP_CUDA(m->ks->finish(a, f, w.max_chunks, st, 0), "finish kernel");
-        NEP_CUDA(nep::launch_final_reduce(B, at<int>(work, w.chunk_start), at<double>(work, w.partial),
-                                          at<double>(work, tl.etot), at<double>(work, tl.vir), st),
-                 "final reduce");
         NEP_CUDA(nep::launch_loss(N, B, s->atom_off, at<int>(work, w.chunk_start), w.max_chunks,
                                   at<float>(work, tl.force), f_lbl, at<double>(work, tl.etot),
                                   at<double>(work, tl.vir), e_lbl, v_lbl, w_host, loss_mode,
@@ -1209,11 +1211,11 @@ nep_status nep_autotune(nep_model* m, const nep_system* sys, const nep_nlist* nl
     if ((s = check_work(m, sys, nl, work, work_bytes, &w)) != NEP_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
     const int N = sys->n_atoms;
-    NEP_CUDA(nep::launch_pack(sys->pos, sys->type, sys->atom_off, N, sys->n_cfg, m->hp.n_types,
-                              at<float4>(work, w.pos4), at<int>(work, w.cfg), nl->status, st),
+    NEP_CUDA(nep::launch_pack_plan(sys->pos, sys->type, sys->atom_off, N, sys->n_cfg, m->hp.n_types,
+                                   at<float4>(work, w.pos4), at<int>(work, w.cfg), nl->status,
+                                   at<int>(work, w.chunk_start), at<int>(work, w.ticket), st),
              "pack");
     const nep::EvalArgs a = make_args(m, sys, nl, work, w);
-    NEP_CUDA(nep::launch_chunk_plan(sys->atom_off, sys->n_cfg, at<int>(work, w.chunk_start), st), "chunk plan");
     cudaEvent_t e0, e1;
     NEP_CUDA(cudaEventCreate(&e0), "event");
     NEP_CUDA(cudaEventCreate(&e1), "event");
@@ -1239,6 +1241,8 @@ nep_status nep_autotune(nep_model* m, const nep_system* sys, const nep_nlist* nl
     f.force = at<float>(work, w.fpart);   // scratch target: the tuner's forces are not kept
     f.e_out = nullptr;
     f.n_owned = N;
+    f.ticket = at<int>(work, w.ticket);
+    f.e_tot = f.virial = nullptr;
     int vd = nep::kDefaultAngularVariant, rb = 0, fb = 0;
     cudaError_t err = cudaSuccess;
     if (N > 0) {

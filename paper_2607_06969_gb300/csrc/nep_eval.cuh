@@ -1153,7 +1153,7 @@ cudaError_t launch_finish_t(const EvalArgs& a, const FinishArgs& f, int max_chun
         else
             launch_finish_b<C, kFinishThreads>(a, f, st);
     }
-    return launch_chunk_reduce(a, f, max_chunks, st);
+    return launch_totals(a, f, max_chunks, st);
 }
 
 // resident CTAs per SM of one angular variant; a variant that parks S in

@@ -629,7 +629,7 @@ template <class C>
 cudaError_t launch_group_finish_t(const EvalArgs& a, const FinishArgs& f, int max_chunks, cudaStream_t st, int G) {
     if (G == 32) launch_group_finish_g<C, 32>(a, f, st);
     else launch_group_finish_g<C, 8>(a, f, st);
-    return launch_chunk_reduce(a, f, max_chunks, st);
+    return launch_totals(a, f, max_chunks, st);
 }
 #endif
 

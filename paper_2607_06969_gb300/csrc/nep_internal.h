@@ -97,6 +97,9 @@ struct FinishArgs {
     const int* atom_off;           // [B+1]
     const int* chunk_start;        // [B+1] reduction chunks per configuration
     double* partial;               // [chunks][10] FP64 E and virial per chunk
+    int* ticket;                   // [B] chunks summed so far
+    double* e_tot;                 // [B] or null
+    double* virial;                // [B][9] or null
     float* force;                  // [3][N]
     float* e_out;                  // [N] or null
     int n_owned;                   // atoms [0, n_owned) enter the E and virial sums
@@ -145,9 +148,12 @@ const KernelSet* find_kernel_set(int n_rad, int n_ang, int k_rad, int k_ang, int
 // runtime kernels (nep_runtime.cu)
 cudaError_t launch_pack(const float* pos, const int* type, const int* atom_off, int N, int B,
                         int T, float4* pos4, int* cfg, int* status, cudaStream_t st);
+// the same with the reduction chunks planned and the reduction tickets cleared
+cudaError_t launch_pack_plan(const float* pos, const int* type, const int* atom_off, int N, int B, int T,
+                             float4* pos4, int* cfg, int* status, int* chunk_start, int* ticket, cudaStream_t st);
 cudaError_t launch_chunk_plan(const int* atom_off, int B, int* chunk_start, cudaStream_t st);
-// FP64 sums of E_i and the per-atom virials per reduction chunk
-cudaError_t launch_chunk_reduce(const EvalArgs& a, const FinishArgs& f, int max_chunks, cudaStream_t st);
+// FP64 sums of E_i and the per-atom virials per configuration
+cudaError_t launch_totals(const EvalArgs& a, const FinishArgs& f, int max_chunks, cudaStream_t st);
 cudaError_t launch_final_reduce(int B, const int* chunk_start, const double* partial,
                                 double* e_tot, double* virial, cudaStream_t st);
 

@@ -25,24 +25,9 @@ __device__ __forceinline__ int find_segment(const int* off, int B, int x) {
 }
 
 // ------------------------------------------------------------------ packing
-__global__ void k_pack(const float* __restrict__ pos, const int* __restrict__ type,
-                       const int* __restrict__ atom_off, int N, int B, int T, float4* pos4,
-                       int* cfg, int* status) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    int t = type[i];
-    if (t < 0 || t >= T) {
-        set_flag(status, 3);
-        t = 0;
-    }
-    const float x = pos[i], y = pos[N + i], z = pos[2 * N + i];
-    if (!(isfinite(x) && isfinite(y) && isfinite(z))) set_flag(status, 3);
-    pos4[i] = make_float4(x, y, z, __int_as_float(t));
-    cfg[i] = find_segment(atom_off, B, i);
-}
-
-// exclusive scan of per-configuration chunk counts (one CTA)
-__global__ void k_chunk_plan(const int* __restrict__ atom_off, int B, int* chunk_start) {
+// Exclusive scan of the configurations' chunk counts by one CTA (any multiple
+// of 32 threads up to 1,024), and the reduction tickets cleared.
+__device__ void chunk_plan_block(const int* __restrict__ atom_off, int B, int* chunk_start, int* ticket) {
     __shared__ int carry;
     __shared__ int warp_sums[32];
     if (threadIdx.x == 0) carry = 0;
@@ -53,6 +38,7 @@ __global__ void k_chunk_plan(const int* __restrict__ atom_off, int B, int* chunk
         if (b < B) {
             const int n = atom_off[b + 1] - atom_off[b];
             v = (n + kChunk - 1) / kChunk;
+            if (ticket) ticket[b] = 0;
         }
         // block inclusive scan
         const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -81,6 +67,33 @@ __global__ void k_chunk_plan(const int* __restrict__ atom_off, int B, int* chunk
     if (threadIdx.x == 0) chunk_start[B] = carry;
 }
 
+__global__ void __launch_bounds__(1024) k_chunk_plan(const int* __restrict__ atom_off, int B, int* chunk_start,
+                                                     int* ticket) {
+    chunk_plan_block(atom_off, B, chunk_start, ticket);
+}
+
+// positions, species and configuration of each atom in the kernels' layout;
+// with chunk_start, one more block plans the reduction chunks meanwhile
+__global__ void __launch_bounds__(256) k_pack(const float* __restrict__ pos, const int* __restrict__ type,
+                                              const int* __restrict__ atom_off, int N, int B, int T, float4* pos4,
+                                              int* cfg, int* status, int* chunk_start, int* ticket) {
+    if (chunk_start && blockIdx.x == gridDim.x - 1) {
+        chunk_plan_block(atom_off, B, chunk_start, ticket);
+        return;
+    }
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N) return;
+    int t = type[i];
+    if (t < 0 || t >= T) {
+        set_flag(status, 3);
+        t = 0;
+    }
+    const float x = pos[i], y = pos[N + i], z = pos[2 * N + i];
+    if (!(isfinite(x) && isfinite(y) && isfinite(z))) set_flag(status, 3);
+    pos4[i] = make_float4(x, y, z, __int_as_float(t));
+    cfg[i] = find_segment(atom_off, B, i);
+}
+
 constexpr int kRedThreads = 256;
 
 // (hi, lo) += x without rounding loss: Knuth's two-sum, in FP32.  The pair
@@ -95,47 +108,75 @@ __device__ __forceinline__ void two_sum_add(float& hi, float& lo, float x) {
     lo = __fadd_rn(lo, err);
 }
 
-// one CTA per reduction chunk (atoms of one configuration): sums of the
-// energies and per-atom virials, each thread over a fixed atom subset in
-// two-sum pairs, a fixed warp tree of pairs, then FP64 across the warps
-__global__ void __launch_bounds__(kRedThreads) k_chunk_reduce(const EvalArgs a, FinishArgs f) {
+// E and virial of every configuration, one CTA per reduction chunk (atoms of
+// one configuration) and one warp per component (E and the nine of V): each
+// lane sums a fixed subset of the chunk's atoms in two-sum pairs, a fixed warp
+// tree joins them, and the CTA that finishes a configuration's last chunk sums
+// the chunks' FP64 partials in a fixed order (lanes take chunks l, l + 32, ...;
+// a fixed tree).  Which CTA does that varies, what it computes does not.
+// With a warp per component no sum crosses warps; the former two kernels (all
+// ten components in every thread, then one CTA per configuration) took 4.4 +
+// 5.8 us at 194 atoms and 21.9 + 8.8 us at 900,000.
+constexpr int kTotalsThreads = 320;
+__global__ void __launch_bounds__(kTotalsThreads) k_totals(const EvalArgs a, FinishArgs f) {
     const int k = blockIdx.x;
     const int B = a.B, N = a.N;
     const int total = f.chunk_start[B];
-    if (k >= total) return;
+    const int lane = threadIdx.x & 31, c = threadIdx.x >> 5;
+    if (k >= total) {
+        // the blocks past the last chunk (at least one per empty configuration)
+        // write the zeros of configurations without atoms
+        for (int b = k - total; b < B; b += gridDim.x - total)
+            if (f.chunk_start[b] == f.chunk_start[b + 1] && lane == 0) {
+                if (c == 0) {
+                    if (f.e_tot) f.e_tot[b] = 0.0;
+                } else if (f.virial) {
+                    f.virial[(size_t)b * 9 + c - 1] = 0.0;
+                }
+            }
+        return;
+    }
     const int b = find_segment(f.chunk_start, B, k);
-    const int a0 = f.atom_off[b] + (k - f.chunk_start[b]) * kChunk;
+    const int k0 = f.chunk_start[b], nk = f.chunk_start[b + 1] - k0;
+    const int a0 = f.atom_off[b] + (k - k0) * kChunk;
     const int a1 = min(min(f.atom_off[b + 1], a0 + kChunk), f.n_owned);
-    float hi[10], lo[10];
-#pragma unroll
-    for (int c = 0; c < 10; ++c) hi[c] = lo[c] = 0.0f;
-    for (int i = a0 + threadIdx.x; i < a1; i += kRedThreads) {
-        two_sum_add(hi[0], lo[0], a.e_atom[i]);
-#pragma unroll
-        for (int c = 0; c < 9; ++c) two_sum_add(hi[1 + c], lo[1 + c], a.wat[(size_t)c * N + i]);
+    const float* src = c == 0 ? a.e_atom : a.wat + (size_t)(c - 1) * N;
+    float h = 0.0f, l = 0.0f;
+#pragma unroll 4
+    for (int i = a0 + lane; i < a1; i += 32) two_sum_add(h, l, src[i]);
+    for (int o = 16; o > 0; o >>= 1) {
+        const float oh = __shfl_down_sync(0xffffffffu, h, o);
+        const float ol = __shfl_down_sync(0xffffffffu, l, o);
+        two_sum_add(h, l, oh);
+        l = __fadd_rn(l, ol);
     }
-    __shared__ double red[10][kRedThreads / 32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int c = 0; c < 10; ++c) {
-        float h = hi[c], l = lo[c];
-        for (int o = 16; o > 0; o >>= 1) {
-            const float oh = __shfl_down_sync(0xffffffffu, h, o);
-            const float ol = __shfl_down_sync(0xffffffffu, l, o);
-            two_sum_add(h, l, oh);
-            l = __fadd_rn(l, ol);
+    double v = (double)h + (double)l;
+    if (nk > 1) {
+        if (lane == 0) {
+            f.partial[(size_t)k * 10 + c] = v;
+            __threadfence();
         }
-        if (lane == 0) red[c][w] = (double)h + (double)l;
+        __shared__ int last;
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(f.ticket + b, 1) == nk - 1;
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        if (threadIdx.x == 0) f.ticket[b] = 0;   // ready for another reduction over the same plan
+        v = 0.0;
+        for (int q = lane; q < nk; q += 32) v += __ldcg(f.partial + (size_t)(k0 + q) * 10 + c);
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     }
-    __syncthreads();
-    if (threadIdx.x < 10) {
-        double v = 0.0;
-        for (int q = 0; q < kRedThreads / 32; ++q) v += red[threadIdx.x][q];
-        f.partial[(size_t)k * 10 + threadIdx.x] = v;
+    if (lane == 0) {
+        if (c == 0) {
+            if (f.e_tot) f.e_tot[b] = v;
+        } else if (f.virial) {
+            f.virial[(size_t)b * 9 + c - 1] = v;
+        }
     }
 }
 
-// one block per configuration: threads take chunk partials k = t, t+256, ...
+// FP64 path: one block per configuration: threads take chunk partials k = t, t+256, ...
 // and a fixed tree (warp shuffles, then the 8 warp sums in order) combines
 // them, so the sum order never changes
 __global__ void __launch_bounds__(kRedThreads) k_final_reduce(int B, const int* __restrict__ chunk_start,
@@ -763,17 +804,35 @@ inline int blocks(int n, int t) { return (n + t - 1) / t; }
 // ------------------------------------------------------------ launchers
 cudaError_t launch_pack(const float* pos, const int* type, const int* atom_off, int N, int B,
                         int T, float4* pos4, int* cfg, int* status, cudaStream_t st) {
-    if (N > 0) k_pack<<<blocks(N, 256), 256, 0, st>>>(pos, type, atom_off, N, B, T, pos4, cfg, status);
+    if (N > 0)
+        k_pack<<<blocks(N, 256), 256, 0, st>>>(pos, type, atom_off, N, B, T, pos4, cfg, status, nullptr, nullptr);
+    return cudaGetLastError();
+}
+
+// the plan rides in the packing launch (1.9 us less) unless its scan by one
+// block of 256 threads would outlast it
+cudaError_t launch_pack_plan(const float* pos, const int* type, const int* atom_off, int N, int B, int T,
+                             float4* pos4, int* cfg, int* status, int* chunk_start, int* ticket, cudaStream_t st) {
+    const bool fused = B <= 2048;
+    if (fused) {
+        k_pack<<<blocks(N, 256) + 1, 256, 0, st>>>(pos, type, atom_off, N, B, T, pos4, cfg, status, chunk_start,
+                                                   ticket);
+    } else {
+        if (N > 0)
+            k_pack<<<blocks(N, 256), 256, 0, st>>>(pos, type, atom_off, N, B, T, pos4, cfg, status, nullptr,
+                                                   nullptr);
+        k_chunk_plan<<<1, 1024, 0, st>>>(atom_off, B, chunk_start, ticket);
+    }
     return cudaGetLastError();
 }
 
 cudaError_t launch_chunk_plan(const int* atom_off, int B, int* chunk_start, cudaStream_t st) {
-    k_chunk_plan<<<1, 1024, 0, st>>>(atom_off, B, chunk_start);
+    k_chunk_plan<<<1, 1024, 0, st>>>(atom_off, B, chunk_start, nullptr);
     return cudaGetLastError();
 }
 
-cudaError_t launch_chunk_reduce(const EvalArgs& a, const FinishArgs& f, int max_chunks, cudaStream_t st) {
-    if (max_chunks > 0) k_chunk_reduce<<<max_chunks, kRedThreads, 0, st>>>(a, f);
+cudaError_t launch_totals(const EvalArgs& a, const FinishArgs& f, int max_chunks, cudaStream_t st) {
+    if (max_chunks > 0) k_totals<<<max_chunks, kTotalsThreads, 0, st>>>(a, f);
     return cudaGetLastError();
 }
 
