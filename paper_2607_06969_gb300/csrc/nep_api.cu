@@ -568,10 +568,6 @@ nep_status neighbors_impl(nep_model* m, const nep_system* s, float skin, nep_nli
                     "a box edge is shorter than 2*(rc+skin)+0.01; the list needs a shift array");
     nl->skin = skin;
     nl->min_image = mi ? 1 : 0;
-    NEP_CUDA(cudaMemsetAsync(nl->status, 0, 4 * sizeof(int), st), "clear status");
-    NEP_CUDA(nep::launch_pack(s->pos, s->type, s->atom_off, N, B, m->hp.n_types, at<float4>(work, w.pos4),
-                              at<int>(work, w.cfg), nl->status, st),
-             "pack");
     nep::NbrWork nw;
     nw.plan = at<nep::CellPlan>(work, w.plan);
     nw.cell_of = at<int>(work, w.cell_of);
@@ -587,8 +583,11 @@ nep_status neighbors_impl(nep_model* m, const nep_system* s, float skin, nep_nli
     nw.cmax = w.cmax;
     nep_nlist copy = *nl;
     if (mi) copy.shift = nullptr;
-    NEP_CUDA(nep::launch_neighbors(s->pos, at<float4>(work, w.pos4), s->atom_off, s->box, at<int>(work, w.cfg), N, B, rc_list,
-                                   rc_list_ang, m->hp.rc_rad, mi ? 1 : 0, &copy, nw, st),
+    float min_edge = s->box_host[0];
+    for (int x = 1; x < 3 * B; ++x) min_edge = s->box_host[x] < min_edge ? s->box_host[x] : min_edge;
+    NEP_CUDA(nep::launch_neighbors(s->pos, s->type, m->hp.n_types, at<float4>(work, w.pos4), s->atom_off, s->box,
+                                   at<int>(work, w.cfg), N, B, rc_list, rc_list_ang, m->hp.rc_rad, min_edge, &copy,
+                                   nw, st),
              "neighbour build");
     return NEP_OK;
 }
@@ -1023,10 +1022,7 @@ nep_status nep_md_step(nep_model* m, const nep_system* sys, nep_nlist* nl, float
     float* pos = const_cast<float*>(sys->pos);
     NEP_CUDA(nep::launch_kick(vel, force, sys->type, inv_m, N, 0.5f * dt, pos, dt, st), "kick/drift");
     if (rebuild) {
-        NEP_CUDA(nep::launch_pack(sys->pos, sys->type, sys->atom_off, N, sys->n_cfg, m->hp.n_types,
-                                  at<float4>(work, w.pos4), at<int>(work, w.cfg), nl->status, st),
-                 "pack");
-        NEP_CUDA(nep::launch_wrap(pos, at<int>(work, w.cfg), sys->box, N, st), "wrap");
+        NEP_CUDA(nep::launch_wrap_segments(pos, sys->atom_off, sys->n_cfg, sys->box, N, st), "wrap");
         if ((s = neighbors_impl(m, sys, skin, nl, work, w, st)) != NEP_OK) return s;
     } else if (!nl->min_image && !nl->shift) {
         return fail(NEP_ERR_STATE, "list was not built");

@@ -172,9 +172,11 @@ struct NbrWork {
     int cmax;
 };
 size_t nbr_cell_capacity(int N, int B);
-cudaError_t launch_neighbors(const float* pos, const float4* pos4, const int* atom_off, const float* box,
-                             const int* cfg, int N, int B, float rc_list, float rc_list_ang, float rc_phys,
-                             int min_image, nep_nlist* nl, const NbrWork& w, cudaStream_t st);
+// clears nl->status, packs the atoms and builds the list and its reverse index;
+// min_edge: the shortest box edge
+cudaError_t launch_neighbors(const float* pos, const int* type, int T, float4* pos4, const int* atom_off,
+                             const float* box, int* cfg, int N, int B, float rc_list, float rc_list_ang,
+                             float rc_phys, float min_edge, nep_nlist* nl, const NbrWork& w, cudaStream_t st);
 
 // FP64 evaluation and training gradient (nep_fp64.cu): runtime
 // hyper-parameters, every quantity in double.  Bounds of the per-thread
@@ -272,7 +274,6 @@ cudaError_t fp32_peak(cudaStream_t st, double* tflops);
 cudaError_t wait_selftest(cudaStream_t st, int* outcome);
 cudaError_t launch_kick(float* vel, const float* force, const int* type, const float* inv_mass,
                         int N, float half_dt, float* pos, float dt, cudaStream_t st);
-cudaError_t launch_wrap(float* pos, const int* cfg, const float* box, int N, cudaStream_t st);
 cudaError_t launch_wrap_segments(float* pos, const int* atom_off, int B, const float* box, int N, cudaStream_t st);
 cudaError_t launch_loss(int N, int B, const int* atom_off, const int* chunk_start, int max_chunks,
                         const float* force, const float* f_lbl, const double* e_tot,

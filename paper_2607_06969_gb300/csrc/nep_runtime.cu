@@ -233,10 +233,9 @@ constexpr int kCellDiv = 3;
 constexpr int kMaxRows = (2 * kCellDiv + 1) * (2 * kCellDiv + 1);
 static_assert(kMaxRows < kRowStride, "row starts must fit one atom's stride");
 
-__global__ void k_cell_plan(const float* __restrict__ box, const int* __restrict__ atom_off, int B,
-                            float rc, CellPlan* plan, int* status) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
+// plan of one configuration; base holds its cell count until the prefix is taken
+__device__ CellPlan cell_plan_of(const float* __restrict__ box, const int* __restrict__ atom_off, int b, float rc,
+                                 int* status) {
     const int nb = atom_off[b + 1] - atom_off[b];
     float L[3] = {box[3 * b], box[3 * b + 1], box[3 * b + 2]};
     int nc[3];
@@ -262,9 +261,15 @@ __global__ void k_cell_plan(const float* __restrict__ box, const int* __restrict
         p.half[d] = (int)ceilf((rc + kCellMargin) / cs);
         if (p.half[d] < 1) p.half[d] = 1;
     }
-    p.base = nc[0] * nc[1] * nc[2];   // count here, prefix in k_plan_scan
+    p.base = nc[0] * nc[1] * nc[2];
     p.pad = 0;
-    plan[b] = p;
+    return p;
+}
+
+__global__ void k_cell_plan(const float* __restrict__ box, const int* __restrict__ atom_off, int B,
+                            float rc, CellPlan* plan, int* status) {
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (b < B) plan[b] = cell_plan_of(box, atom_off, b, rc, status);
 }
 
 __global__ void k_plan_scan(CellPlan* plan, int B) {
@@ -405,6 +410,91 @@ __device__ __forceinline__ int floor_div(int a, int b) {
     int q = a / b;
     if ((a % b != 0) && ((a < 0) != (b < 0))) --q;
     return q;
+}
+
+// The whole binning of a small system in one CTA: status cleared, atoms packed
+// (as k_pack), the configurations' cell plans and their prefix, atoms counted
+// into cells in shared memory, the cells' scan, and the positions in cell
+// order, atoms of a cell by index.  One launch in place of twelve of about 2
+// us each: at 58 atoms those were half of the list build's time.
+constexpr int kCellsSmallN = 4096, kCellsSmallB = 256;
+__global__ void __launch_bounds__(1024) k_cells_small(
+    const float* __restrict__ pos, const int* __restrict__ type, const int* __restrict__ atom_off,
+    const float* __restrict__ box, int N, int B, int T, float rc, float4* pos4, int* cfg, int* status,
+    CellPlan* plan, int* cell_of, int* cell_start, float4* cell_pos) {
+    extern __shared__ int cnt[];                    // [cells], then the cells' ends
+    __shared__ int in_cell[kCellsSmallN];           // atoms in cell order, any order within a cell
+    __shared__ int ws[32];
+    const int tid = threadIdx.x;
+    if (tid < 4) status[tid] = 0;
+    __syncthreads();
+    CellPlan p;
+    p.base = 0;
+    if (tid < B) p = cell_plan_of(box, atom_off, tid, rc, status);
+    int ncell;
+    const int base = block_excl_scan_1024(p.base, ws, &ncell);
+    if (tid < B) {
+        p.base = base;
+        plan[tid] = p;
+    }
+    for (int c = tid; c < ncell; c += 1024) cnt[c] = 0;
+    __syncthreads();
+    constexpr int kPer = kCellsSmallN / 1024;
+    int id[kPer];
+    float4 q[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        const int i = tid + u * 1024;
+        id[u] = -1;
+        if (i >= N) continue;
+        int t = type[i];
+        if (t < 0 || t >= T) {
+            set_flag(status, 3);
+            t = 0;
+        }
+        const float x = pos[i], y = pos[N + i], z = pos[2 * N + i];
+        const int b = find_segment(atom_off, B, i);
+        const float L[3] = {box[3 * b], box[3 * b + 1], box[3 * b + 2]};
+        if (!(x >= 0.0f && x < L[0] && y >= 0.0f && y < L[1] && z >= 0.0f && z < L[2]))
+            set_flag(status, 3);                    // NaN and infinities fail the test too
+        pos4[i] = make_float4(x, y, z, __int_as_float(t));
+        cfg[i] = b;
+        const CellPlan pb = plan[b];
+        int c[3];
+        cell_coords(pb, x, y, z, L, c);
+        id[u] = pb.base + (c[0] * pb.nc[1] + c[1]) * pb.nc[2] + c[2];
+        q[u] = make_float4(x, y, z, __int_as_float(i));
+        cell_of[i] = id[u];
+        atomicAdd(cnt + id[u], 1);
+    }
+    __syncthreads();
+    // exclusive scan of the counts, each thread a contiguous run of cells
+    const int per = (ncell + 1023) / 1024, c0 = min(tid * per, ncell), c1 = min(c0 + per, ncell);
+    int sum = 0;
+    for (int c = c0; c < c1; ++c) sum += cnt[c];
+    int total;
+    int run = block_excl_scan_1024(sum, ws, &total);
+    for (int c = c0; c < c1; ++c) {
+        const int v = cnt[c];
+        cnt[c] = run;
+        cell_start[c] = run;
+        run += v;
+    }
+    if (tid == 0) cell_start[ncell] = N;
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kPer; ++u)
+        if (id[u] >= 0) in_cell[atomicAdd(cnt + id[u], 1)] = tid + u * 1024;
+    __syncthreads();
+    // cnt[c] is now the end of cell c
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        if (id[u] < 0) continue;
+        const int i = tid + u * 1024, s0 = id[u] > 0 ? cnt[id[u] - 1] : 0, s1 = cnt[id[u]];
+        int rank = 0;
+        for (int s = s0; s < s1; ++s) rank += in_cell[s] < i ? 1 : 0;
+        cell_pos[s0 + rank] = q[u];
+    }
 }
 
 // One pass over the stencil.  The list is written in three groups:
@@ -583,48 +673,254 @@ __global__ void __launch_bounds__(128) k_build(const float4* __restrict__ pos4,
     nl.cnt_ang[i] = n_ang;
 }
 
+// The same list from a warp per atom, for systems too small to hide one
+// thread's serial walk (82 to 124 us up to 10,000 atoms).  The stencil rows'
+// candidate ranges go to shared memory in visit order; lanes then take
+// consecutive candidates, each finding its range by bisection.  The first pass
+// over the candidates counts the three groups, the second writes every entry
+// to its final slot, so the list is that of k_build entry for entry.  A range
+// holds cells of one z image; a row has at most 2 half_z / nc_z + 2.
+constexpr int kBuildWarps = 4;
+constexpr int kBuildSegs = 128;      // candidate ranges held at once
+constexpr int kBuildRows = 64;       // stencil rows per round, two per lane
+constexpr int kBuildWarpN = 40000;   // largest system: the whole list build, thread / warp per atom (the
+                                     // reverse search alike): 7,200 atoms 150 / 56 us, 46,522 251 / 220
+                                     // (packings, images), 57,600 203 / 238 (rock salt)
+constexpr float kBuildMinEdge = 16.0f;   // shortest box edge: the list cutoff over this (at most 34 ranges per row)
+__global__ void __launch_bounds__(32 * kBuildWarps) k_build_warp(
+    const float4* __restrict__ pos4, const int* __restrict__ cfg, const float* __restrict__ box,
+    const CellPlan* __restrict__ plan, const int* __restrict__ cell_of, const int* __restrict__ cell_start,
+    const float4* __restrict__ cell_pos, int N, float rc2_rad, float rc2_ang, float rc2_phys,
+    unsigned char* __restrict__ row_start, unsigned char* __restrict__ slot_row, nep_nlist nl) {
+    __shared__ int s_q0[kBuildWarps][kBuildSegs], s_cum[kBuildWarps][kBuildSegs + 1];
+    __shared__ int s_img[kBuildWarps][kBuildSegs];
+    __shared__ unsigned short s_row[kBuildWarps][kBuildSegs];
+    __shared__ int s_rowcnt[kBuildWarps][kMaxRows + 1];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i = blockIdx.x * kBuildWarps + w;
+    if (i >= N) return;
+    int *q0s = s_q0[w], *cum = s_cum[w], *img = s_img[w], *rowcnt = s_rowcnt[w];
+    unsigned short* rowof = s_row[w];
+    const int b = cfg[i];
+    const CellPlan p = plan[b];
+    const float L[3] = {box[3 * b], box[3 * b + 1], box[3 * b + 2]};
+    const float4 pi = pos4[i];
+    int c = cell_of[i] - p.base;
+    const int cz = c % p.nc[2];
+    c /= p.nc[2];
+    const int cy = c % p.nc[1];
+    const int cx = c / p.nc[1];
+    const int wy_rows = 2 * p.half[1] + 1, rows = (2 * p.half[0] + 1) * wy_rows;
+    const bool track = rows <= kMaxRows && nl.cap_ang < 256;
+    if (track)
+        for (int r = lane; r <= rows; r += 32) rowcnt[r] = 0;
+    const float cs[3] = {L[0] / (float)p.nc[0], L[1] / (float)p.nc[1], L[2] / (float)p.nc[2]};
+    const float rl = sqrtf(rc2_rad) + kPruneMargin;
+    const float rl2 = rl * rl;
+    const int maxseg = 2 * p.half[2] / p.nc[2] + 2;
+    const int per_round = max(1, min(kBuildRows, kBuildSegs / maxseg));
+    const unsigned below = (1u << lane) - 1u;
+    int n_ang = 0, n_in = 0, n_out = 0;       // of the whole atom after the first pass
+    bool over = false;
+    int nseg = 0, ncand = 0;
+    for (int pass = 0; pass < 2; ++pass) {
+        int ra = 0, ri = 0, ro = 0;           // entries of each group so far
+        for (int row0 = 0; row0 < rows; row0 += per_round) {
+            if (pass == 0 || rows > per_round) {      // one round keeps its ranges
+                // this lane's rows row0 + 2 lane, + 1: z cells lo..hi of each
+                int lo[2], hi[2], rc[2], sxy[2], mine = 0;
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int row = row0 + 2 * lane + u;
+                    lo[u] = 0;
+                    hi[u] = -1;
+                    rc[u] = sxy[u] = 0;
+                    if (2 * lane + u >= per_round || row >= rows) continue;
+                    const int ox = row / wy_rows - p.half[0], oy = row % wy_rows - p.half[1];
+                    const int ux = cx + ox, sx = floor_div(ux, p.nc[0]), wx = ux - sx * p.nc[0];
+                    const float gx =
+                        fmaxf(fmaxf((float)ux * cs[0] - pi.x, pi.x - (float)(ux + 1) * cs[0]), 0.0f);
+                    const int uy = cy + oy, sy = floor_div(uy, p.nc[1]), wy = uy - sy * p.nc[1];
+                    const float gy =
+                        fmaxf(fmaxf((float)uy * cs[1] - pi.y, pi.y - (float)(uy + 1) * cs[1]), 0.0f);
+                    const float rem = rl2 - gx * gx - gy * gy;
+                    if (rem <= 0.0f) continue;
+                    const float hz = sqrtf(rem);
+                    lo[u] = max(cz - p.half[2], (int)floorf((pi.z - hz) / cs[2]));
+                    hi[u] = min(cz + p.half[2], (int)floorf((pi.z + hz) / cs[2]));
+                    rc[u] = p.base + (wx * p.nc[1] + wy) * p.nc[2];
+                    sxy[u] = pack_shift(sx, sy, 0);
+                    if (lo[u] <= hi[u]) mine += floor_div(hi[u], p.nc[2]) - floor_div(lo[u], p.nc[2]) + 1;
+                }
+                int at = mine;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, at, o);
+                    if (lane >= o) at += y;
+                }
+                nseg = __shfl_sync(0xffffffffu, at, 31);
+                at -= mine;
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    while (lo[u] <= hi[u]) {
+                        const int sz = floor_div(lo[u], p.nc[2]);
+                        const int seg_hi = min(hi[u], (sz + 1) * p.nc[2] - 1);
+                        const int z0 = lo[u] - sz * p.nc[2], z1 = seg_hi - sz * p.nc[2];
+                        lo[u] = seg_hi + 1;
+                        const int q0 = cell_start[rc[u] + z0];
+                        q0s[at] = q0;
+                        cum[at] = cell_start[rc[u] + z1 + 1] - q0;
+                        img[at] = sxy[u] | ((sz & 0xff) << 16);
+                        rowof[at] = (unsigned short)(row0 + 2 * lane + u);
+                        ++at;
+                    }
+                }
+                __syncwarp();
+                // candidates before each range
+                ncand = 0;
+                for (int s0 = 0; s0 < nseg; s0 += 32) {
+                    const int v = s0 + lane < nseg ? cum[s0 + lane] : 0;
+                    int x = v;
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int y = __shfl_up_sync(0xffffffffu, x, o);
+                        if (lane >= o) x += y;
+                    }
+                    if (s0 + lane < nseg) cum[s0 + lane] = ncand + x - v;
+                    ncand += __shfl_sync(0xffffffffu, x, 31);
+                }
+                __syncwarp();
+            }
+            for (int t0 = 0; t0 < ncand; t0 += 32) {
+                const int t = t0 + lane;
+                int kind = 0, j = 0, sh = 0, row = 0;   // 1 angular, 2 inside, 3 shell
+                if (t < ncand) {
+                    int s = 0, e = nseg;              // cum[s] <= t < cum[e]; empty ranges resolve to the last
+                    while (e - s > 1) {
+                        const int mid = (s + e) >> 1;
+                        if (cum[mid] <= t) s = mid;
+                        else e = mid;
+                    }
+                    const float4 pj = cell_pos[q0s[s] + (t - cum[s])];
+                    j = f2i(pj.w);
+                    sh = img[s];
+                    row = rowof[s];
+                    int sx, sy, sz;
+                    unpack_shift(sh, sx, sy, sz);
+                    const float dx = add_rn(sub_rn(pj.x, pi.x), mul_rn((float)sx, L[0]));
+                    const float dy = add_rn(sub_rn(pj.y, pi.y), mul_rn((float)sy, L[1]));
+                    const float dz = add_rn(sub_rn(pj.z, pi.z), mul_rn((float)sz, L[2]));
+                    const float d2 = dist2(dx, dy, dz);
+                    if (d2 < rc2_rad && !(j == i && sh == 0)) kind = d2 < rc2_ang ? 1 : (d2 < rc2_phys ? 2 : 3);
+                }
+                const unsigned ma = __ballot_sync(0xffffffffu, kind == 1);
+                const unsigned mi = __ballot_sync(0xffffffffu, kind == 2);
+                const unsigned mo = __ballot_sync(0xffffffffu, kind == 3);
+                if (pass == 0) {
+                    if (track && kind == 1) atomicAdd(rowcnt + row, 1);
+                } else if (kind) {
+                    const int slot = kind == 1   ? ra + __popc(ma & below)
+                                     : kind == 2 ? n_ang + ri + __popc(mi & below)
+                                                 : n_ang + n_in + ro + __popc(mo & below);
+                    // an overflowing list keeps the part of its angular prefix that fits
+                    if (!over || (kind == 1 && slot < min(nl.cap, nl.cap_ang))) {
+                        const size_t to = (size_t)slot * N + i;
+                        nl.nbr[to] = j;
+                        if (nl.shift) nl.shift[to] = sh;
+                        if (kind == 1 && track) slot_row[to] = (unsigned char)row;
+                    }
+                }
+                ra += __popc(ma);
+                ri += __popc(mi);
+                ro += __popc(mo);
+            }
+            __syncwarp();
+        }
+        if (pass == 0) {
+            n_ang = ra;
+            n_in = ri;
+            n_out = ro;
+            over = n_ang + n_in + n_out > nl.cap || n_ang > nl.cap_ang;
+        }
+    }
+    if (track) {
+        // where each row's angular entries start
+        unsigned char* rs = row_start + (size_t)i * kRowStride;
+        int before = 0;
+        for (int r0 = 0; r0 <= rows; r0 += 32) {
+            const int r = r0 + lane, v = r < rows ? rowcnt[r] : 0;
+            int x = v;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            if (r <= rows) rs[r] = (unsigned char)min(before + x - v, 255);
+            before += __shfl_sync(0xffffffffu, x, 31);
+        }
+    }
+    if (lane == 0) {
+        const int total = n_ang + n_in + n_out;
+        if (over) {
+            set_flag(nl.status, 0);
+            atomicMax(nl.status + 1, total);
+            atomicMax(nl.status + 2, n_ang);
+        }
+        const int kept = min(n_ang, min(nl.cap, nl.cap_ang));
+        nl.cnt[i] = over ? kept : total;
+        nl.cnt_ang[i] = over ? kept : n_ang;
+    }
+}
+
 // rev[s][i] = slot of i (with the opposite image) in the angular prefix of
 // j = nbr[s][i].  j visits i in the mirrored stencil row, rows - 1 - row,
 // so only that row's stretch of j's prefix is searched; stencils too large
 // for the row table fall back to scanning j's whole prefix.
-__global__ void k_rev(int N, const int* __restrict__ cfg, const CellPlan* __restrict__ plan,
-                      const unsigned char* __restrict__ row_start, const unsigned char* __restrict__ slot_row,
-                      nep_nlist nl) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void rev_slot(int N, int i, int s, int rows, bool track,
+                                         const unsigned char* __restrict__ row_start,
+                                         const unsigned char* __restrict__ slot_row, const nep_nlist& nl) {
+    const int j = nl.nbr[(size_t)s * N + i];
+    int want = 0;
+    if (nl.shift) {
+        int a, b, c;
+        unpack_shift(nl.shift[(size_t)s * N + i], a, b, c);
+        want = pack_shift(-a, -b, -c);
+    }
+    const int nj = nl.cnt_ang[j];
+    int t0 = 0, t1 = nj;
+    if (track) {
+        const int mr = rows - 1 - (int)slot_row[(size_t)s * N + i];
+        const unsigned char* rj = row_start + (size_t)j * kRowStride;
+        t0 = rj[mr];
+        t1 = min((int)rj[mr + 1], nj);
+    }
+    int found = -1;
+    for (int t = t0; t < t1; ++t) {
+        if (nl.nbr[(size_t)t * N + j] == i && (!nl.shift || nl.shift[(size_t)t * N + j] == want)) {
+            found = t;
+            break;
+        }
+    }
+    if (found < 0) {
+        set_flag(nl.status, 0);
+        found = 0;
+    }
+    nl.rev[(size_t)s * N + i] = found;
+}
+
+// G = 1: one thread per atom; G = 32: a warp per atom, a lane per slot.  The
+// warps lose the coalescing of the slot-major list, but up to kRevWarpN atoms
+// the shorter walk is worth more (the list build of 57,600 atoms 214 -> 203
+// us, of 112,500 atoms 259 -> 262).
+constexpr int kRevWarpN = 80000;
+template <int G>
+__global__ void __launch_bounds__(128) k_rev(int N, const int* __restrict__ cfg, const CellPlan* __restrict__ plan,
+                                             const unsigned char* __restrict__ row_start,
+                                             const unsigned char* __restrict__ slot_row, nep_nlist nl) {
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) / G;
     if (i >= N) return;
     const int na = nl.cnt_ang[i];
     const CellPlan p = plan[cfg[i]];
     const int rows = (2 * p.half[0] + 1) * (2 * p.half[1] + 1);
     const bool track = rows <= kMaxRows && nl.cap_ang < 256;
-    for (int s = 0; s < na; ++s) {
-        const int j = nl.nbr[(size_t)s * N + i];
-        int want = 0;
-        if (nl.shift) {
-            int a, b, c;
-            unpack_shift(nl.shift[(size_t)s * N + i], a, b, c);
-            want = pack_shift(-a, -b, -c);
-        }
-        const int nj = nl.cnt_ang[j];
-        int t0 = 0, t1 = nj;
-        if (track) {
-            const int mr = rows - 1 - (int)slot_row[(size_t)s * N + i];
-            const unsigned char* rj = row_start + (size_t)j * kRowStride;
-            t0 = rj[mr];
-            t1 = min((int)rj[mr + 1], nj);
-        }
-        int found = -1;
-        for (int t = t0; t < t1; ++t) {
-            if (nl.nbr[(size_t)t * N + j] == i && (!nl.shift || nl.shift[(size_t)t * N + j] == want)) {
-                found = t;
-                break;
-            }
-        }
-        if (found < 0) {
-            set_flag(nl.status, 0);
-            found = 0;
-        }
-        nl.rev[(size_t)s * N + i] = found;
-    }
+    for (int s = threadIdx.x % G; s < na; s += G) rev_slot(N, i, s, rows, track, row_start, slot_row, nl);
 }
 
 // ------------------------------------------------------------ optimiser
@@ -686,14 +982,7 @@ __device__ __forceinline__ float wrap_coord(float x, float L) {
     if (!(x < L)) x = 0.0f;
     return x;
 }
-__global__ void k_wrap(float* pos, const int* __restrict__ cfg, const float* __restrict__ box,
-                       int N) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const int b = cfg[i];
-    for (int d = 0; d < 3; ++d) pos[(size_t)d * N + i] = wrap_coord(pos[(size_t)d * N + i], box[3 * b + d]);
-}
-// the same, with each atom's configuration found from the CSR offsets
+// each atom's configuration is found from the CSR offsets
 __global__ void k_wrap_seg(float* pos, const int* __restrict__ atom_off, int B, const float* __restrict__ box,
                            int N) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -844,30 +1133,48 @@ cudaError_t launch_final_reduce(int B, const int* chunk_start, const double* par
 
 size_t nbr_cell_capacity(int N, int B) { return 2 * (size_t)N + 27 * (size_t)B; }
 
-cudaError_t launch_neighbors(const float* pos, const float4* pos4, const int* atom_off, const float* box,
-                             const int* cfg, int N, int B, float rc_list, float rc_list_ang, float rc_phys,
-                             int min_image, nep_nlist* nl, const NbrWork& w, cudaStream_t st) {
+cudaError_t launch_neighbors(const float* pos, const int* type, int T, float4* pos4, const int* atom_off,
+                             const float* box, int* cfg, int N, int B, float rc_list, float rc_list_ang,
+                             float rc_phys, float min_edge, nep_nlist* nl, const NbrWork& w, cudaStream_t st) {
     cudaError_t e;
-    (void)min_image;
-    if (N == 0) return cudaSuccess;
     const int cmax = w.cmax;
-    k_cell_plan<<<blocks(B, 128), 128, 0, st>>>(box, atom_off, B, rc_list, w.plan, nl->status);
-    k_plan_scan<<<1, 32, 0, st>>>(w.plan, B);
-    if ((e = cudaMemsetAsync(w.cell_cnt, 0, sizeof(int) * (size_t)(cmax + 1), st)) != cudaSuccess)
-        return e;
-    k_bin<<<blocks(N, 256), 256, 0, st>>>(pos, cfg, box, w.plan, N, w.cell_of, w.rank, w.cell_cnt,
-                                          nl->status);
-    const int n = cmax + 1;
-    const int ntiles = blocks(n, kScanTile);
-    k_scan_tiles<<<ntiles, 1024, 0, st>>>(w.cell_cnt, n, w.cell_start, w.scan_tmp);
-    k_scan_sums<<<1, 1024, 0, st>>>(w.scan_tmp, ntiles, w.scan_tmp + ntiles);
-    k_scan_add<<<blocks(n, 256), 256, 0, st>>>(w.cell_start, n, w.scan_tmp);
-    k_fill<<<blocks(N, 256), 256, 0, st>>>(w.cell_of, w.rank, w.cell_start, N, w.cell_atoms);
-    k_sort_cells<<<blocks(cmax, 128), 128, 0, st>>>(w.cell_start, cmax, w.cell_atoms, pos4, w.cell_pos);
+    if (N > 0 && N <= kCellsSmallN && B <= kCellsSmallB) {
+        const int smem = (int)sizeof(int) * (cmax + 1);
+        // 60 KB at most, which needs the attribute
+        if (smem > 30 * 1024 &&
+            (e = cudaFuncSetAttribute(k_cells_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)sizeof(int) * (2 * kCellsSmallN + 27 * kCellsSmallB + 1))))
+            return e;
+        k_cells_small<<<1, 1024, smem, st>>>(pos, type, atom_off, box, N, B, T, rc_list, pos4, cfg, nl->status,
+                                             w.plan, w.cell_of, w.cell_start, w.cell_pos);
+    } else {
+        if ((e = cudaMemsetAsync(nl->status, 0, 4 * sizeof(int), st))) return e;
+        if (N == 0) return cudaSuccess;
+        if ((e = launch_pack(pos, type, atom_off, N, B, T, pos4, cfg, nl->status, st))) return e;
+        k_cell_plan<<<blocks(B, 128), 128, 0, st>>>(box, atom_off, B, rc_list, w.plan, nl->status);
+        k_plan_scan<<<1, 32, 0, st>>>(w.plan, B);
+        if ((e = cudaMemsetAsync(w.cell_cnt, 0, sizeof(int) * (size_t)(cmax + 1), st)) != cudaSuccess) return e;
+        k_bin<<<blocks(N, 256), 256, 0, st>>>(pos, cfg, box, w.plan, N, w.cell_of, w.rank, w.cell_cnt, nl->status);
+        const int n = cmax + 1;
+        const int ntiles = blocks(n, kScanTile);
+        k_scan_tiles<<<ntiles, 1024, 0, st>>>(w.cell_cnt, n, w.cell_start, w.scan_tmp);
+        k_scan_sums<<<1, 1024, 0, st>>>(w.scan_tmp, ntiles, w.scan_tmp + ntiles);
+        k_scan_add<<<blocks(n, 256), 256, 0, st>>>(w.cell_start, n, w.scan_tmp);
+        k_fill<<<blocks(N, 256), 256, 0, st>>>(w.cell_of, w.rank, w.cell_start, N, w.cell_atoms);
+        k_sort_cells<<<blocks(cmax, 128), 128, 0, st>>>(w.cell_start, cmax, w.cell_atoms, pos4, w.cell_pos);
+    }
     const float rr = rc_list * rc_list, ra = rc_list_ang * rc_list_ang, rp = rc_phys * rc_phys;
-    k_build<<<blocks(N, 128), 128, 0, st>>>(pos4, cfg, box, w.plan, w.cell_of, w.cell_start,
-                                            w.cell_pos, N, rr, ra, rp, w.shell, w.row_start, w.slot_row, *nl);
-    k_rev<<<blocks(N, 128), 128, 0, st>>>(N, cfg, w.plan, w.row_start, w.slot_row, *nl);
+    if (N <= kBuildWarpN && min_edge * kBuildMinEdge >= rc_list)
+        k_build_warp<<<blocks(N, kBuildWarps), 32 * kBuildWarps, 0, st>>>(pos4, cfg, box, w.plan, w.cell_of,
+                                                                          w.cell_start, w.cell_pos, N, rr, ra, rp,
+                                                                          w.row_start, w.slot_row, *nl);
+    else
+        k_build<<<blocks(N, 128), 128, 0, st>>>(pos4, cfg, box, w.plan, w.cell_of, w.cell_start,
+                                                w.cell_pos, N, rr, ra, rp, w.shell, w.row_start, w.slot_row, *nl);
+    if (N <= kRevWarpN)
+        k_rev<32><<<blocks(N, 4), 128, 0, st>>>(N, cfg, w.plan, w.row_start, w.slot_row, *nl);
+    else
+        k_rev<1><<<blocks(N, 128), 128, 0, st>>>(N, cfg, w.plan, w.row_start, w.slot_row, *nl);
     return cudaGetLastError();
 }
 
@@ -931,11 +1238,6 @@ cudaError_t launch_pack_adjoint(int N, int B, const float* lam, const double* a_
                                 float4* lam4, float* aE, float* mu, cudaStream_t st) {
     const int n = N > B ? N : B;
     if (n > 0) k_pack_adjoint<<<blocks(n, 256), 256, 0, st>>>(N, B, lam, a_e, mu_in, lam4, aE, mu);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_wrap(float* pos, const int* cfg, const float* box, int N, cudaStream_t st) {
-    if (N > 0) k_wrap<<<blocks(N, 256), 256, 0, st>>>(pos, cfg, box, N);
     return cudaGetLastError();
 }
 

@@ -139,3 +139,41 @@ def test_lane_groups_16bit_network(nb, hname, precision):
     step = 2.0 ** -11 if precision == 1 else 2.0 ** -8
     assert np.abs(got[0] - want[0]).max() <= 0.5 * step
     assert np.sqrt(np.mean((got[1] - want[1]) ** 2)) <= 0.1 * step
+
+
+@pytest.mark.parametrize("n,L,skin,copies", [(3, 5.0, 1.0, 30000), (58, 0.0, 0.0, 1500), (700, 0.0, 1.0, 120),
+                                             (4100, 0.0, 0.5, 22)])
+def test_list_build_small_and_large_forms_agree(nb, n, L, skin, copies):
+    """A configuration listed alone (binned by one CTA up to 4,096 atoms, a
+    warp per atom in the build and the reverse search) gets, entry for entry,
+    the list of each of its copies in a batch large enough for one thread per
+    atom: a few atoms in a box shorter than the cutoff (stencils too large for
+    the row table), boxes with images and without."""
+    h = I.HYPER_SMALL
+    s = I.packing_batch([n], tag=65, dmin=1.5 if L else 2.4, density=n / L ** 3 if L else 0.0325)
+    model = nb.Model(h, I.init_params(h).astype(np.float32))
+    cap, cap_ang = 160, 80
+
+    def build(copies):
+        batch = I.System(pos=np.tile(s.pos, (copies, 1)), types=np.tile(s.types, copies),
+                         box=np.repeat(s.box, copies, 0), atom_off=n * np.arange(copies + 1))
+        dsys = nb.DeviceSystem.from_inputs(batch)
+        nl = nb.NeighborList(batch.n_atoms, cap, cap_ang)
+        ws = nb.Workspace(model, batch.n_atoms, copies, cap, cap_ang)
+        nb.neighbors(model, dsys, nl, skin, ws)
+        assert nb.check_list(nl) == nb.NEP_OK, nb.last_error()
+        get = lambda t: t.cpu().numpy().reshape(-1, batch.n_atoms)   # noqa: E731
+        return [get(t) for t in (nl.cnt, nl.cnt_ang, nl.nbr, nl.rev, nl.shift)], nl.c.min_image
+
+    one, mi = build(1)
+    many, mi2 = build(copies)
+    assert mi == mi2
+    for c in (0, copies - 1):
+        cols = slice(c * n, (c + 1) * n)
+        assert np.array_equal(one[0], many[0][:, cols]) and np.array_equal(one[1], many[1][:, cols])
+        used = np.arange(cap)[:, None] < one[0]
+        ang = np.arange(cap_ang)[:, None] < one[1]
+        assert np.array_equal(one[2][used], many[2][:, cols][used] - c * n)
+        assert np.array_equal(one[3][ang], many[3][:, cols][ang])
+        if not mi:
+            assert np.array_equal(one[4][used], many[4][:, cols][used])
