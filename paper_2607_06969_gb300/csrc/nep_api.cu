@@ -248,6 +248,27 @@ int group_lanes(const nep_model* m, const nep_system* s) {
     const int most = (wide ? 20000 : 26000) + (m->hp.precision ? 6000 : 0);
     return s->n_atoms <= 3000 ? 32 : (s->n_atoms <= most ? 8 : 0);
 }
+// Lanes per atom of the training operator's two parts, the forward of a loss
+// gradient and the per-atom backward; 0 for the one-thread-per-atom kernels,
+// which work together (their forward leaves records for their backward).
+// Measured with the reduction, uneven packings, graph (the group kernels,
+// forward 8 / backward 32 lanes, against one thread per atom):
+//   loss gradient: 10,204 atoms 177 / 253 us (38-30-1), 217 / 348 (42-50-1),
+//   289 / 398 (52-64-1); 20,405 atoms 292 / 329, 360 / 431, 496 / 501;
+//   31,888 atoms 440 / 386, 502 / 497, 722 / 599
+//   adjoint product (no forward): 20,405 atoms 201 / 289, 254 / 389, 348 / 459;
+//   31,888 atoms 317 / 342, 382 / 453, 567 / 554
+// The backward takes 32 lanes at every size: with 8 its 16 atoms per CTA need
+// more shared memory and spill (20,405 atoms 232 / 201 us).
+struct TrainLanes {
+    int forward, backward;
+};
+TrainLanes train_lanes(const nep_model* m, const nep_system* s, bool loss) {
+    const int most = loss ? 22000 : 32000;
+    if (s->n_atoms == 0 || m->pinned[size_bin(s)] || !m->ks->group_train_fits(m->hp.n_hidden) || s->n_atoms > most)
+        return {0, 0};
+    return {s->n_atoms <= 3000 ? 32 : 8, 32};
+}
 bool block_choice(int b) {
     for (int c : nep::kBlockChoices)
         if (b == c) return true;
@@ -493,15 +514,20 @@ nep_status train_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, co
              "pack");
     nep::EvalArgs a = make_args(m, s, nl, work, w);
     a.q16_kind = 0;
-    a.S = at<float>(work, w.S);
-    a.compr = at<float4>(work, tl.compr);
-    a.cnt_compr = at<int>(work, tl.cnt_compr);
-    a.q_out = at<float>(work, tl.q);
-    a.p_out = at<float>(work, tl.p);
-    a.fb_out = a.fb;
-    const int vd = angular_variant(m, s);
-    if (N > 0) NEP_CUDA(m->ks->radial(a, st, 0), "radial kernel");
-    if (N > 0) NEP_CUDA(m->ks->angular(a, st, vd), "angular kernel");
+    const TrainLanes lanes = train_lanes(m, s, e_lbl != nullptr);
+    const int G = lanes.forward;
+    if (!G) {
+        // the training variants of the forward kernels leave their records for the backward
+        a.S = at<float>(work, w.S);
+        a.compr = at<float4>(work, tl.compr);
+        a.cnt_compr = at<int>(work, tl.cnt_compr);
+        a.q_out = at<float>(work, tl.q);
+        a.p_out = at<float>(work, tl.p);
+        if (N > 0) NEP_CUDA(m->ks->radial(a, st, 0), "radial kernel");
+        if (N > 0) NEP_CUDA(m->ks->angular(a, st, angular_variant(m, s)), "angular kernel");
+    } else if (e_lbl) {
+        NEP_CUDA(m->ks->group_atom(a, st, G), "atom kernel");
+    }
     if (e_lbl) {
         // forward forces, energies and virials, then the loss and its adjoints
         nep::FinishArgs f;
@@ -514,7 +540,8 @@ nep_status train_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, co
         f.ticket = at<int>(work, w.ticket);
         f.e_tot = at<double>(work, tl.etot);
         f.virial = at<double>(work, tl.vir);
-        NEP_CUDA(m->ks->finish(a, f, w.max_chunks, st, 0), "finish kernel");
+        if (G) NEP_CUDA(m->ks->group_finish(a, f, w.max_chunks, st, G), "finish kernel");
+        else NEP_CUDA(m->ks->finish(a, f, w.max_chunks, st, 0), "finish kernel");
         NEP_CUDA(nep::launch_loss(N, B, s->atom_off, at<int>(work, w.chunk_start), w.max_chunks,
                                   at<float>(work, tl.force), f_lbl, at<double>(work, tl.etot),
                                   at<double>(work, tl.vir), e_lbl, v_lbl, w_host, loss_mode,
@@ -527,6 +554,9 @@ nep_status train_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, co
                                           at<float>(work, tl.aE), at<float>(work, tl.mu), st),
                  "adjoints");
     }
+    a.q_out = at<float>(work, tl.q);
+    a.p_out = at<float>(work, tl.p);
+    a.fb_out = a.fb;
     nep::TrainArgs t;
     t.e = a;
     t.lam4 = at<float4>(work, tl.lam4);
@@ -541,7 +571,7 @@ nep_status train_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, co
     t.bins = at<float>(work, tl.bins);
     t.gpart = at<float>(work, tl.gpart);
     t.grad = grad;
-    NEP_CUDA(m->ks->train(t, st), "gradient kernels");
+    NEP_CUDA(m->ks->train(t, st, lanes.backward), "gradient kernels");
     return NEP_OK;
 }
 

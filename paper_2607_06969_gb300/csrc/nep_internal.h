@@ -133,10 +133,11 @@ struct KernelSet {
     cudaError_t (*angular)(const EvalArgs&, cudaStream_t, int variant);   // FP32 or tensor-core network
     cudaError_t (*finish)(const EvalArgs&, const FinishArgs&, int max_chunks, cudaStream_t, int block);
     cudaError_t (*train_init)(int H);
-    cudaError_t (*train)(const TrainArgs&, cudaStream_t);   // tangent ... gradient
+    cudaError_t (*train)(const TrainArgs&, cudaStream_t, int G);   // tangent ... gradient; G as for the groups below, 0 without
     int (*grad_chunks)(int N);
     // a group of G lanes per atom (nep_group.cuh), G = 8 or 32
     bool (*group_fits)(int H);
+    bool (*group_train_fits)(int H);
     cudaError_t (*group_init)(int H);
     cudaError_t (*group_atom)(const EvalArgs&, cudaStream_t, int G);
     cudaError_t (*group_finish)(const EvalArgs&, const FinishArgs&, int max_chunks, cudaStream_t, int G);

@@ -24,7 +24,6 @@
 //             in fixed order.
 #pragma once
 #include "nep_eval.cuh"
-#include "nep_group.cuh"
 #include "nep_mlp_tc.cuh"
 
 namespace nep {
@@ -46,6 +45,10 @@ NEP_HD void adjoint_frame(const TrainArgs& t, int i, float4& li, float* mu) {
 #pragma unroll
     for (int k = 0; k < 9; ++k) mu[k] = t.mu[9 * b + k];
 }
+
+}  // namespace nep
+#include "nep_group_train.cuh"
+namespace nep {
 
 // Pair records of a compacted list read ahead: the record two pairs ahead
 // and the neighbour's adjoint one pair ahead, so that the two dependent
@@ -794,6 +797,8 @@ cudaError_t train_init_t(int H) {
     const int smem = (int)smem_bytes_of<C>(H);
     cudaError_t e;
     if ((e = mlp_tc_init_t<C>(H))) return e;
+    if ((e = cudaFuncSetAttribute(kg_grad<C, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynSmem)))
+        return e;
     if ((e = cudaFuncSetAttribute(k_tangent<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
     return cudaFuncSetAttribute(k_grad_partial<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)grad_stage_bytes<C>(H));
@@ -802,13 +807,21 @@ cudaError_t train_init_t(int H) {
 template <class C>
 int grad_chunks_t(int N) { return grad_chunks_of(N); }
 
+// whether a model of H hidden units fits the group kernels' shared memory
 template <class C>
-cudaError_t train_t(const TrainArgs& t, cudaStream_t st) {
+bool group_train_fits_t(int H) {
+    return group_fits_t<C>(H) && GroupGradSmem<C, 32>::bytes(H) <= kMaxDynSmem;
+}
+
+// G: lanes per atom of the per-atom backward (32), 0 for one thread per atom
+template <class C>
+cudaError_t train_t(const TrainArgs& t, cudaStream_t st, int G) {
     const int N = t.e.N;
     const size_t smem = smem_bytes_of<C>(t.e.H);
     if (N > 0) {
         const int grid = (N + kBlock - 1) / kBlock;
-        k_tangent<C><<<grid, kBlock, smem, st>>>(t);
+        if (G) launch_group_grad_g<C, 32>(t, st);
+        else k_tangent<C><<<grid, kBlock, smem, st>>>(t);
         k_grad_partial<C><<<grad_chunks_t<C>(N), kGradThreads, grad_stage_bytes<C>(t.e.H), st>>>(t);
     }
     const ParamLayout L = param_layout(C::T, C::NR, C::NA, C::KR, C::KA, C::H4, t.e.H);
