@@ -266,31 +266,192 @@ NEP_HD float clm(int lm) {
 }
 NEP_HD int lm_l(int lm) { return lm < 3 ? 1 : (lm < 8 ? 2 : (lm < 15 ? 3 : 4)); }
 
-// Real solid harmonics P_lm(u) of a unit vector (homogeneous polynomials of
-// degree l evaluated on the unit sphere), order as in clm().
-NEP_HD void harmonics(float x, float y, float z, float* Y) {
-    float xx = x * x, yy = y * y, zz = z * z, xy = x * y, xz = x * z, yz = y * z;
-    Y[0] = y; Y[1] = z; Y[2] = x;
-    Y[3] = xy; Y[4] = yz; Y[5] = 3.0f * zz - 1.0f; Y[6] = xz; Y[7] = xx - yy;
-    float a5 = 5.0f * zz - 1.0f;
-    Y[8] = y * (3.0f * xx - yy);
-    Y[9] = xy * z;
-    Y[10] = y * a5;
-    Y[11] = z * (5.0f * zz - 3.0f);
-    Y[12] = x * a5;
-    Y[13] = z * (xx - yy);
-    Y[14] = x * (xx - 3.0f * yy);
-    float b7 = 7.0f * zz - 1.0f, c7 = 7.0f * zz - 3.0f;
-    Y[15] = xy * (xx - yy);
-    Y[16] = yz * (3.0f * xx - yy);
-    Y[17] = xy * b7;
-    Y[18] = yz * c7;
-    Y[19] = (35.0f * zz - 30.0f) * zz + 3.0f;
-    Y[20] = xz * c7;
-    Y[21] = (xx - yy) * b7;
-    Y[22] = xz * (xx - 3.0f * yy);
-    Y[23] = xx * (xx - 3.0f * yy) - yy * (3.0f * xx - yy);
+// Real harmonics P_lm(u) of a unit vector u = (x, y, z), l = 1..4, order as in
+// clm().  Each is a polynomial in z times the real or imaginary part c_k, s_k
+// of a power of x + iy (s_2 and s_4 without their factors 2 and 4):
+//   l = 1: y, z, x
+//   l = 2: s2, y z, 3z^2-1, x z, c2
+//   l = 3: s3, s2 z, y q1, p3, x q1, z c2, c3
+//   l = 4: s4, z s3, s2 q2, y q3, p4, x q3, c2 q2, z c3, c4
+// so sums over m of a_m P_m and of its gradient collect the coefficients of
+// each c_k, s_k first: per pair the angular force takes about 95 operations
+// for both sums where evaluating every P_m and its three derivatives took 230.
+template <class R>
+struct Harm {
+    R x, y, z, c2, s2, c3, s3, c4, s4;
+    R zz, q1, q2, q3, p2, p3, p4;    // 5zz-1, 7zz-1, z(7zz-3), 3zz-1, z(5zz-3), (35zz-30)zz+3
+};
+template <class R>
+NEP_HD Harm<R> harm_of(R x, R y, R z) {
+    Harm<R> h;
+    const R xx = x * x, yy = y * y, zz = z * z;
+    const R e1 = R(3.0) * xx - yy, e2 = xx - R(3.0) * yy;
+    h.x = x; h.y = y; h.z = z; h.zz = zz;
+    h.s2 = x * y;
+    h.c2 = xx - yy;
+    h.c3 = x * e2;
+    h.s3 = y * e1;
+    h.c4 = xx * e2 - yy * e1;
+    h.s4 = h.s2 * h.c2;
+    h.q1 = R(5.0) * zz - R(1.0);
+    h.q2 = R(7.0) * zz - R(1.0);
+    h.q3 = z * (R(7.0) * zz - R(3.0));
+    h.p2 = R(3.0) * zz - R(1.0);
+    h.p3 = z * (R(5.0) * zz - R(3.0));
+    h.p4 = (R(35.0) * zz - R(30.0)) * zz + R(3.0);
+    return h;
 }
+// P_m(u); with m a compile-time constant the switch folds away
+template <class R>
+NEP_HD R harm_value(int m, const Harm<R>& h) {
+    switch (m) {
+        case 0: return h.y;
+        case 1: return h.z;
+        case 2: return h.x;
+        case 3: return h.s2;
+        case 4: return h.y * h.z;
+        case 5: return h.p2;
+        case 6: return h.x * h.z;
+        case 7: return h.c2;
+        case 8: return h.s3;
+        case 9: return h.s2 * h.z;
+        case 10: return h.y * h.q1;
+        case 11: return h.p3;
+        case 12: return h.x * h.q1;
+        case 13: return h.z * h.c2;
+        case 14: return h.c3;
+        case 15: return h.s4;
+        case 16: return h.z * h.s3;
+        case 17: return h.s2 * h.q2;
+        case 18: return h.y * h.q3;
+        case 19: return h.p4;
+        case 20: return h.x * h.q3;
+        case 21: return h.c2 * h.q2;
+        case 22: return h.z * h.c3;
+        default: return h.c4;
+    }
+}
+
+// The derivative of every term along a tangent du of the unit sphere
+template <class R>
+struct HarmD {
+    R x, y, z, c2, s2, c3, s3, c4, s4, q1, q2, q3, p2, p3, p4;
+};
+template <class R>
+NEP_HD HarmD<R> harm_along(const Harm<R>& h, R dx, R dy, R dz) {
+    HarmD<R> d;
+    const R zd = h.z * dz, c23 = R(3.0) * h.c2, s26 = R(6.0) * h.s2;
+    d.x = dx; d.y = dy; d.z = dz;
+    d.c2 = R(2.0) * (h.x * dx - h.y * dy);
+    d.s2 = h.x * dy + h.y * dx;
+    d.c3 = c23 * dx - s26 * dy;
+    d.s3 = s26 * dx + c23 * dy;
+    d.c4 = R(4.0) * (h.c3 * dx - h.s3 * dy);
+    d.s4 = h.s3 * dx + h.c3 * dy;
+    d.q1 = R(10.0) * zd;
+    d.q2 = R(14.0) * zd;
+    d.q3 = (R(21.0) * h.zz - R(3.0)) * dz;
+    d.p2 = R(6.0) * zd;
+    d.p3 = (R(15.0) * h.zz - R(3.0)) * dz;
+    d.p4 = (R(140.0) * h.zz - R(60.0)) * zd;
+    return d;
+}
+// along the change of u = r_ij / r when r_ij changes by dr (udr = u . dr)
+template <class R>
+NEP_HD HarmD<R> unit_tangent(const Harm<R>& h, R drx, R dry, R drz, R udr, R ir) {
+    return harm_along(h, (drx - h.x * udr) * ir, (dry - h.y * udr) * ir, (drz - h.z * udr) * ir);
+}
+template <class R>
+NEP_HD R harm_dvalue(int m, const Harm<R>& h, const HarmD<R>& d) {
+    switch (m) {
+        case 0: return d.y;
+        case 1: return d.z;
+        case 2: return d.x;
+        case 3: return d.s2;
+        case 4: return h.y * d.z + d.y * h.z;
+        case 5: return d.p2;
+        case 6: return h.x * d.z + d.x * h.z;
+        case 7: return d.c2;
+        case 8: return d.s3;
+        case 9: return h.s2 * d.z + d.s2 * h.z;
+        case 10: return h.y * d.q1 + d.y * h.q1;
+        case 11: return d.p3;
+        case 12: return h.x * d.q1 + d.x * h.q1;
+        case 13: return h.z * d.c2 + d.z * h.c2;
+        case 14: return d.c3;
+        case 15: return d.s4;
+        case 16: return h.z * d.s3 + d.z * h.s3;
+        case 17: return h.s2 * d.q2 + d.s2 * h.q2;
+        case 18: return h.y * d.q3 + d.y * h.q3;
+        case 19: return d.p4;
+        case 20: return h.x * d.q3 + d.x * h.q3;
+        case 21: return h.c2 * d.q2 + d.c2 * h.q2;
+        case 22: return h.z * d.c3 + d.z * h.c3;
+        default: return d.c4;
+    }
+}
+
+// sum_m a_m grad P_m(u) and sum_m b_m P_m(u): add() takes m = 0..23 in
+// ascending order, each once.  The gradient is that of the polynomials above,
+// whose part along u has no meaning: force() takes it out.
+template <class R>
+struct HarmSums {
+    R C1, S1, C2, S2, C3, S3, C4, S4;                   // coefficients of c_k, s_k (c_1 = x, s_1 = y)
+    R D0, D1, E1, D2, E2, D3, E3;                       // their derivatives by z
+    R v0, v1, w1, v2, w2, v3, w3, v4, w4;               // the same coefficients from b
+    R z6, z10, z14, t3, t4, t5;
+    NEP_HD explicit HarmSums(const Harm<R>& h) {
+        z6 = R(6.0) * h.z;
+        z10 = R(10.0) * h.z;
+        z14 = R(14.0) * h.z;
+        t3 = R(15.0) * h.zz - R(3.0);
+        t4 = R(21.0) * h.zz - R(3.0);
+        t5 = (R(140.0) * h.zz - R(60.0)) * h.z;
+    }
+    NEP_HD void add(int m, const Harm<R>& h, R a, R b) {
+        switch (m) {
+            case 0: S1 = a; w1 = b; break;
+            case 1: D0 = a; v0 = b * h.z; break;
+            case 2: C1 = a; v1 = b; break;
+            case 3: S2 = a; w2 = b; break;
+            case 4: S1 += a * h.z; E1 = a; w1 += b * h.z; break;
+            case 5: D0 += a * z6; v0 += b * h.p2; break;
+            case 6: C1 += a * h.z; D1 = a; v1 += b * h.z; break;
+            case 7: C2 = a; v2 = b; break;
+            case 8: S3 = a; w3 = b; break;
+            case 9: S2 += a * h.z; E2 = a; w2 += b * h.z; break;
+            case 10: S1 += a * h.q1; E1 += a * z10; w1 += b * h.q1; break;
+            case 11: D0 += a * t3; v0 += b * h.p3; break;
+            case 12: C1 += a * h.q1; D1 += a * z10; v1 += b * h.q1; break;
+            case 13: C2 += a * h.z; D2 = a; v2 += b * h.z; break;
+            case 14: C3 = a; v3 = b; break;
+            case 15: S4 = a; w4 = b; break;
+            case 16: S3 += a * h.z; E3 = a; w3 += b * h.z; break;
+            case 17: S2 += a * h.q2; E2 += a * z14; w2 += b * h.q2; break;
+            case 18: S1 += a * h.q3; E1 += a * t4; w1 += b * h.q3; break;
+            case 19: D0 += a * t5; v0 += b * h.p4; break;
+            case 20: C1 += a * h.q3; D1 += a * t4; v1 += b * h.q3; break;
+            case 21: C2 += a * h.q2; D2 += a * z14; v2 += b * h.q2; break;
+            case 22: C3 += a * h.z; D3 = a; v3 += b * h.z; break;
+            default: C4 = a; v4 = b; break;
+        }
+    }
+    // f = u sum_m b_m P_m + (1/r) (1 - u u^T) sum_m a_m grad P_m
+    NEP_HD void force(const Harm<R>& h, R ir, R& fx, R& fy, R& fz) const {
+        const R x2 = R(2.0) * h.x, y2 = R(2.0) * h.y, c23 = R(3.0) * h.c2, s26 = R(6.0) * h.s2;
+        const R c34 = R(4.0) * h.c3, s34 = R(4.0) * h.s3;
+        const R Gx = C1 + x2 * C2 + h.y * S2 + c23 * C3 + s26 * S3 + c34 * C4 + h.s3 * S4;
+        const R Gy = S1 - y2 * C2 + h.x * S2 - s26 * C3 + c23 * S3 - s34 * C4 + h.c3 * S4;
+        const R Gz = D0 + D1 * h.x + E1 * h.y + D2 * h.c2 + E2 * h.s2 + D3 * h.c3 + E3 * h.s3;
+        const R val = v0 + v1 * h.x + w1 * h.y + v2 * h.c2 + w2 * h.s2 + v3 * h.c3 + w3 * h.s3 + v4 * h.c4 +
+                      w4 * h.s4;
+        const R ug = h.x * Gx + h.y * Gy + h.z * Gz;
+        const R rad = val - ir * ug;
+        fx = h.x * rad + Gx * ir;
+        fy = h.y * rad + Gy * ir;
+        fz = h.z * rad + Gz * ir;
+    }
+};
 
 // Component m of the real solid harmonics: value P_m(u) on the unit sphere
 // and the gradient of the homogeneous polynomial at u.  With m a
@@ -338,41 +499,6 @@ NEP_HD void harm_m(int m, const HarmTermsT<R>& t, R& Y, R& gx, R& gy, R& gz) {
         case 22: Y = xz * (xx - R(3.0) * yy); gx = R(3.0) * z * (xx - yy); gy = -R(6.0) * xy * z; gz = x * (xx - R(3.0) * yy); break;
         default: Y = xx * (xx - R(3.0) * yy) - yy * (R(3.0) * xx - yy); gx = R(4.0) * x * (xx - R(3.0) * yy); gy = -R(4.0) * y * (R(3.0) * xx - yy); gz = R(0.0); break;
     }
-}
-
-// g = sum_lm a_lm grad P_lm(u) (gradient of the homogeneous polynomials).
-NEP_HD void harmonics_grad_contract(float x, float y, float z, const float* a, float& gx,
-                                    float& gy, float& gz) {
-    float xx = x * x, yy = y * y, zz = z * z, xy = x * y, xz = x * z, yz = y * z;
-    float xyz = xy * z;
-    // l = 1
-    gx = a[2];
-    gy = a[0];
-    gz = a[1];
-    // l = 2
-    gx += a[3] * y - 2.0f * a[5] * x + a[6] * z + 2.0f * a[7] * x;
-    gy += a[3] * x + a[4] * z - 2.0f * a[5] * y - 2.0f * a[7] * y;
-    gz += a[4] * y + 4.0f * a[5] * z + a[6] * x;
-    // l = 3
-    float d3 = 3.0f * (xx - yy);
-    gx += a[8] * 6.0f * xy + a[9] * yz - a[10] * 2.0f * xy - a[11] * 6.0f * xz
-          + a[12] * (4.0f * zz - 3.0f * xx - yy) + a[13] * 2.0f * xz + a[14] * d3;
-    gy += a[8] * d3 + a[9] * xz + a[10] * (4.0f * zz - xx - 3.0f * yy) - a[11] * 6.0f * yz
-          - a[12] * 2.0f * xy - a[13] * 2.0f * yz - a[14] * 6.0f * xy;
-    gz += a[9] * xy + a[10] * 8.0f * yz + a[11] * (6.0f * zz - 3.0f * xx - 3.0f * yy)
-          + a[12] * 8.0f * xz + a[13] * (xx - yy);
-    // l = 4
-    float e1 = 3.0f * xx - yy, e2 = xx - 3.0f * yy, e3 = xx + yy - 4.0f * zz;
-    gx += a[15] * y * e1 + a[16] * 6.0f * xyz - a[17] * y * (3.0f * xx + yy - 6.0f * zz)
-          - a[18] * 6.0f * xyz + a[19] * 12.0f * x * e3 - a[20] * z * (9.0f * xx + 3.0f * yy - 4.0f * zz)
-          - a[21] * 4.0f * x * (xx - 3.0f * zz) + a[22] * 3.0f * z * (xx - yy) + a[23] * 4.0f * x * e2;
-    gy += a[15] * x * e2 + a[16] * 3.0f * z * (xx - yy) - a[17] * x * (xx + 3.0f * yy - 6.0f * zz)
-          - a[18] * z * (3.0f * xx + 9.0f * yy - 4.0f * zz) + a[19] * 12.0f * y * e3
-          - a[20] * 6.0f * xyz + a[21] * 4.0f * y * (yy - 3.0f * zz) - a[22] * 6.0f * xyz
-          - a[23] * 4.0f * y * e1;
-    gz += a[16] * y * e1 + a[17] * 12.0f * xyz - a[18] * 3.0f * y * e3
-          - a[19] * 16.0f * z * (3.0f * xx + 3.0f * yy - 2.0f * zz) - a[20] * 3.0f * x * e3
-          + a[21] * 12.0f * z * (xx - yy) + a[22] * x * e2;
 }
 
 // 4-body term from the l = 2 block s[0..4] = (xy, yz, 2zz-xx-yy, xz, xx-yy)

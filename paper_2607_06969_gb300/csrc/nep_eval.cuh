@@ -363,17 +363,14 @@ NEP_HD void angular_S(const EvalArgs& a, const float* sm, const SmemLayout& sl, 
         basis<KA>(r, irA, f);
         float g[NA];
         contract_pairs<NA, KA>(sm + sl.cA2 + (ti * T + tj) * C::SA, f, g);
-        const HarmTerms ht = harm_terms(e.x * ir, e.y * ir, e.z * ir);
+        const Harm<float> ht = harm_of(e.x * ir, e.y * ir, e.z * ir);
         // S[n][m] += g_n Y_m, two m at a time (paired FMAs)
         float2 gb[NA];
 #pragma unroll
         for (int n = 0; n < NA; ++n) gb[n] = make_float2(g[n], g[n]);
 #pragma unroll
         for (int m = 0; m < kLM; m += 2) {
-            float Y0, Y1, gx, gy, gz;
-            harm_m(m, ht, Y0, gx, gy, gz);
-            harm_m(m + 1, ht, Y1, gx, gy, gz);
-            const float2 y2 = make_float2(Y0, Y1);
+            const float2 y2 = make_float2(harm_value(m, ht), harm_value(m + 1, ht));
 #pragma unroll
             for (int n = 0; n < NA; ++n) {
                 const float2 s2 = ffma2(gb[n], y2, make_float2(S[n][m], S[n][m + 1]));
@@ -432,12 +429,9 @@ NEP_HD void make_Sb(float (&Sb)[C::NA][kLM], GetS S, GetP pl) {
     }
 }
 
-// angular pair forces: f_ij = u sum_m (b_m - l a_m / r) Y_m + (1/r) sum_m a_m grad P_m(u),
+// angular pair forces: f_ij = u sum_m b_m Y_m + (1/r) (1 - u u^T) sum_m a_m grad P_m(u),
 // a_m = sum_n Sb[n][m] g_n, b_m = sum_n Sb[n][m] g'_n; owner sums and reverse-slot scatter
-// SPLIT: sum (b_m - l a_m / r) Y_m and a_m grad P_m as even and odd partial
-// sums over m, one paired FMA per pair of m (measured faster in the
-// tensor-core kernel, slower in the FP32 one)
-template <class C, bool SPLIT = false>
+template <class C>
 NEP_HD void angular_force(const EvalArgs& a, const float* sm, const SmemLayout& sl, int ti, int i,
                           const float (&Sb)[C::NA][kLM], float& Fx, float& Fy, float& Fz, float* W) {
     constexpr int NA = C::NA, KA = C::KA, T = C::T;
@@ -461,9 +455,8 @@ NEP_HD void angular_force(const EvalArgs& a, const float* sm, const SmemLayout& 
             contract_pairs<NA, KA>(c2, f, g);
             contract_pairs<NA, KA>(c2, fp, gp);
         }
-        const HarmTerms ht = harm_terms(e.x * ir, e.y * ir, e.z * ir);
-        float rad = 0.0f, Gx = 0.0f, Gy = 0.0f, Gz = 0.0f;
-        float2 rad2 = make_float2(0.0f, 0.0f), gx2 = rad2, gy2 = rad2, gz2 = rad2;
+        const Harm<float> ht = harm_of(e.x * ir, e.y * ir, e.z * ir);
+        HarmSums<float> hs(ht);
         // a_m and b_m two m at a time (paired FMAs, each chain in n order)
         float2 gb[NA], gpb[NA];
 #pragma unroll
@@ -480,38 +473,11 @@ NEP_HD void angular_force(const EvalArgs& a, const float* sm, const SmemLayout& 
                 am2 = ffma2(s2, gb[n], am2);
                 bm2 = ffma2(s2, gpb[n], bm2);
             }
-            if constexpr (SPLIT) {
-                float Y0, hx0, hy0, hz0, Y1, hx1, hy1, hz1;
-                harm_m(m0, ht, Y0, hx0, hy0, hz0);
-                harm_m(m0 + 1, ht, Y1, hx1, hy1, hz1);
-                const float2 cl = make_float2(-(float)lm_l(m0) * ir, -(float)lm_l(m0 + 1) * ir);
-                rad2 = ffma2(ffma2(cl, am2, bm2), make_float2(Y0, Y1), rad2);
-                gx2 = ffma2(am2, make_float2(hx0, hx1), gx2);
-                gy2 = ffma2(am2, make_float2(hy0, hy1), gy2);
-                gz2 = ffma2(am2, make_float2(hz0, hz1), gz2);
-            } else {
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int m = m0 + u;
-                    const float am = u ? am2.y : am2.x, bm = u ? bm2.y : bm2.x;
-                    float Y, hx, hy, hz;
-                    harm_m(m, ht, Y, hx, hy, hz);
-                    rad = fmaf(fmaf(-(float)lm_l(m) * ir, am, bm), Y, rad);
-                    Gx = fmaf(am, hx, Gx);
-                    Gy = fmaf(am, hy, Gy);
-                    Gz = fmaf(am, hz, Gz);
-                }
-            }
+            hs.add(m0, ht, am2.x, bm2.x);
+            hs.add(m0 + 1, ht, am2.y, bm2.y);
         }
-        if constexpr (SPLIT) {
-            rad = rad2.x + rad2.y;
-            Gx = gx2.x + gx2.y;
-            Gy = gy2.x + gy2.y;
-            Gz = gz2.x + gz2.y;
-        }
-        const float fx = fmaf(ht.x, rad, Gx * ir);
-        const float fy = fmaf(ht.y, rad, Gy * ir);
-        const float fz = fmaf(ht.z, rad, Gz * ir);
+        float fx, fy, fz;
+        hs.force(ht, ir, fx, fy, fz);
         Fx += fx; Fy += fy; Fz += fz;
         W[0] -= fx * e.x; W[1] -= fx * e.y; W[2] -= fx * e.z;
         W[3] -= fy * e.x; W[4] -= fy * e.y; W[5] -= fy * e.z;

@@ -243,13 +243,9 @@ __device__ int group_sums(const EvalArgs& a, const float* sm, float* gb, float* 
             contract_pairs<NA, KA>(sm + M::cA2() + (fr.ti * T + p.tj) * C::SA, f, g);
 #pragma unroll
             for (int n = 0; n < M::NAp; ++n) gb[M::oG + at * M::NAp + n] = n < NA ? g[n] : 0.0f;
-            const HarmTerms ht = harm_terms(p.dx * ir, p.dy * ir, p.dz * ir);
+            const Harm<float> ht = harm_of(p.dx * ir, p.dy * ir, p.dz * ir);
 #pragma unroll
-            for (int mm = 0; mm < kLM; ++mm) {
-                float Y, gx, gy, gz;
-                harm_m(mm, ht, Y, gx, gy, gz);
-                gb[M::oY + mm * M::GS + at] = Y;
-            }
+            for (int mm = 0; mm < kLM; ++mm) gb[M::oY + mm * M::GS + at] = harm_value(mm, ht);
         }
         __syncwarp();
         for (int q = 0; q < np; ++q) {
@@ -450,8 +446,8 @@ __global__ void __launch_bounds__(kGroupThreads, kGroupMinBlocks) kg_atom(const 
                 contract_pairs<NA, KA>(c2, f, g);
                 contract_pairs<NA, KA>(c2, fp, gp);
             }
-            const HarmTerms ht = harm_terms(p.dx * ir, p.dy * ir, p.dz * ir);
-            float rad = 0.0f, Gx = 0.0f, Gy = 0.0f, Gz = 0.0f;
+            const Harm<float> ht = harm_of(p.dx * ir, p.dy * ir, p.dz * ir);
+            HarmSums<float> hs(ht);
 #pragma unroll
             for (int m0 = 0; m0 < kLM; m0 += 4) {
                 float2 am[2] = {}, bm[2] = {};
@@ -465,22 +461,14 @@ __global__ void __launch_bounds__(kGroupThreads, kGroupMinBlocks) kg_atom(const 
                     bm[0] = ffma2(s0, q2, bm[0]);
                     bm[1] = ffma2(s1, q2, bm[1]);
                 }
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int m = m0 + u;
-                    const float av = (u & 1) ? am[u / 2].y : am[u / 2].x, bv = (u & 1) ? bm[u / 2].y : bm[u / 2].x;
-                    float Y, hx, hy, hz;
-                    harm_m(m, ht, Y, hx, hy, hz);
-                    rad = fmaf(fmaf(-(float)lm_l(m) * ir, av, bv), Y, rad);
-                    Gx = fmaf(av, hx, Gx);
-                    Gy = fmaf(av, hy, Gy);
-                    Gz = fmaf(av, hz, Gz);
-                }
+                hs.add(m0, ht, am[0].x, bm[0].x);
+                hs.add(m0 + 1, ht, am[0].y, bm[0].y);
+                hs.add(m0 + 2, ht, am[1].x, bm[1].x);
+                hs.add(m0 + 3, ht, am[1].y, bm[1].y);
                 NEP_SCHED_BARRIER();
             }
-            const float fx = fmaf(ht.x, rad, Gx * ir);
-            const float fy = fmaf(ht.y, rad, Gy * ir);
-            const float fz = fmaf(ht.z, rad, Gz * ir);
+            float fx, fy, fz;
+            hs.force(ht, ir, fx, fy, fz);
             a.fin[addr] = make_float4(fx, fy, fz, 0.0f);
             acc[0] += fx; acc[1] += fy; acc[2] += fz;
             acc[3] -= fx * p.dx; acc[4] -= fx * p.dy; acc[5] -= fx * p.dz;

@@ -175,13 +175,12 @@ __global__ void __launch_bounds__(kGroupThreads, 3) kg_grad(const TrainArgs t) {
                     row[n] = n < NA ? g[n] : 0.0f;
                     row[NAp + n] = n < NA ? gp[n] * p.udr : 0.0f;
                 }
-                const HarmTerms ht = harm_terms(p.dx * p.ir, p.dy * p.ir, p.dz * p.ir);
+                const Harm<float> ht = harm_of(p.dx * p.ir, p.dy * p.ir, p.dz * p.ir);
+                const HarmD<float> hd = unit_tangent(ht, p.drx, p.dry, p.drz, p.udr, p.ir);
 #pragma unroll
                 for (int mm = 0; mm < kLM; ++mm) {
-                    float Y, hx, hy, hz;
-                    harm_m(mm, ht, Y, hx, hy, hz);
-                    dY[mm] = ((hx * p.drx + hy * p.dry + hz * p.drz) - (float)lm_l(mm) * Y * p.udr) * p.ir;
-                    gb[M::oY + mm * GS + at] = Y;
+                    dY[mm] = harm_dvalue(mm, ht, hd);
+                    gb[M::oY + mm * GS + at] = harm_value(mm, ht);
                 }
             }
             // S += g Y, dS += g' (rhat . dr) Y, then dS += g dY
@@ -402,7 +401,8 @@ __global__ void __launch_bounds__(kGroupThreads, 3) kg_grad(const TrainArgs t) {
                     gb[M::oY + k * GS + lane] = f[k];
                     gb[M::oY + (KA + k) * GS + lane] = fp[k];
                 }
-                const HarmTerms ht = harm_terms(p.dx * p.ir, p.dy * p.ir, p.dz * p.ir);
+                const Harm<float> ht = harm_of(p.dx * p.ir, p.dy * p.ir, p.dz * p.ir);
+                const HarmD<float> hd = unit_tangent(ht, p.drx, p.dry, p.drz, p.udr, p.ir);
                 float2 X[NA], Z[NA];
 #pragma unroll
                 for (int n = 0; n < NA; ++n) X[n] = Z[n] = make_float2(0.0f, 0.0f);
@@ -411,9 +411,8 @@ __global__ void __launch_bounds__(kGroupThreads, 3) kg_grad(const TrainArgs t) {
                     float Y[4], dY[4];
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
-                        float hx, hy, hz;
-                        harm_m(m0 + u, ht, Y[u], hx, hy, hz);
-                        dY[u] = ((hx * p.drx + hy * p.dry + hz * p.drz) - (float)lm_l(m0 + u) * Y[u] * p.udr) * p.ir;
+                        Y[u] = harm_value(m0 + u, ht);
+                        dY[u] = harm_dvalue(m0 + u, ht, hd);
                     }
 #pragma unroll
                     for (int n = 0; n < NA; ++n) {

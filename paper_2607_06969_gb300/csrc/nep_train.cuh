@@ -150,7 +150,7 @@ NEP_HD void tangent_atom(const TrainArgs& t, const float* sm, int i) {
         NEP_SCHED_BARRIER();
     }
 
-    // angular: dS_nlm = sum_j [g'_n (rhat.dr) Y_m + g_n (grad P_m . dr - l Y_m rhat.dr)/r]
+    // angular: dS_nlm = sum_j [g'_n (rhat.dr) Y_m + g_n dY_m], dY_m along the change of rhat
     float dS[NA][kLM];
 #pragma unroll
     for (int n = 0; n < NA; ++n)
@@ -166,8 +166,9 @@ NEP_HD void tangent_atom(const TrainArgs& t, const float* sm, int i) {
         pair_tangent(mu, li, lj, e.x, e.y, e.z, drx, dry, drz);
         const float r = sqrt_f(dist2(e.x, e.y, e.z));
         const float ir = rcp_f(r);
-        const HarmTerms ht = harm_terms(e.x * ir, e.y * ir, e.z * ir);
+        const Harm<float> ht = harm_of(e.x * ir, e.y * ir, e.z * ir);
         const float udr = ht.x * drx + ht.y * dry + ht.z * drz;
+        const HarmD<float> hd = unit_tangent(ht, drx, dry, drz, udr, ir);
         float g[NA], gp[NA];
         {
             float f[KA], fp[KA];
@@ -186,15 +187,12 @@ NEP_HD void tangent_atom(const TrainArgs& t, const float* sm, int i) {
             }
         }
 #pragma unroll
-        for (int m = 0; m < kLM; ++m) {
-            float Y, hx, hy, hz;
-            harm_m(m, ht, Y, hx, hy, hz);
-            const float gdr = (hx * drx + hy * dry + hz * drz) * ir;
-            const float yu = Y * udr;
-            const float lr = (float)lm_l(m) * ir;
+        for (int n = 0; n < NA; ++n) gp[n] *= udr;
 #pragma unroll
-            for (int n = 0; n < NA; ++n)
-                dS[n][m] = fmaf(yu, fmaf(-lr, g[n], gp[n]), fmaf(g[n], gdr, dS[n][m]));
+        for (int m = 0; m < kLM; ++m) {
+            const float Y = harm_value(m, ht), dY = harm_dvalue(m, ht, hd);
+#pragma unroll
+            for (int n = 0; n < NA; ++n) dS[n][m] = fmaf(gp[n], Y, fmaf(g[n], dY, dS[n][m]));
         }
     }
 #pragma unroll
@@ -301,14 +299,13 @@ NEP_HD void xzp_atom(const TrainArgs& t, const float* sm, int i) {
     for (int c = 0; c < nc; ++c) {
         const float4 e = a.comp[c * N + i];
         const float ir = rcp_f(sqrt_f(dist2(e.x, e.y, e.z)));
-        const HarmTerms ht = harm_terms(e.x * ir, e.y * ir, e.z * ir);
+        const Harm<float> ht = harm_of(e.x * ir, e.y * ir, e.z * ir);
         float X[NA];
 #pragma unroll
         for (int n = 0; n < NA; ++n) X[n] = 0.0f;
 #pragma unroll
         for (int m = 0; m < kLM; ++m) {
-            float Y, hx, hy, hz;
-            harm_m(m, ht, Y, hx, hy, hz);
+            const float Y = harm_value(m, ht);
 #pragma unroll
             for (int n = 0; n < NA; ++n) X[n] = fmaf(P[n][m], Y, X[n]);
         }
@@ -358,8 +355,9 @@ NEP_HD void xzr_atom(const TrainArgs& t, const float* sm, int i) {
         float drx, dry, drz;
         pair_tangent(mu, li, lj, e.x, e.y, e.z, drx, dry, drz);
         const float ir = rcp_f(sqrt_f(dist2(e.x, e.y, e.z)));
-        const HarmTerms ht = harm_terms(e.x * ir, e.y * ir, e.z * ir);
+        const Harm<float> ht = harm_of(e.x * ir, e.y * ir, e.z * ir);
         const float udr = ht.x * drx + ht.y * dry + ht.z * drz;
+        const HarmD<float> hd = unit_tangent(ht, drx, dry, drz, udr, ir);
         float X[NA], Z[NA];
 #pragma unroll
         for (int n = 0; n < NA; ++n) {
@@ -368,9 +366,7 @@ NEP_HD void xzr_atom(const TrainArgs& t, const float* sm, int i) {
         }
 #pragma unroll
         for (int m = 0; m < kLM; ++m) {
-            float Y, hx, hy, hz;
-            harm_m(m, ht, Y, hx, hy, hz);
-            const float dY = ((hx * drx + hy * dry + hz * drz) - (float)lm_l(m) * Y * udr) * ir;
+            const float Y = harm_value(m, ht), dY = harm_dvalue(m, ht, hd);
 #pragma unroll
             for (int n = 0; n < NA; ++n) {
                 X[n] = fmaf(R[n][m], dY, X[n]);
