@@ -142,11 +142,13 @@ NEP_HD void unpack_shift(int v, int& sx, int& sy, int& sz) {
 }
 
 // Pair vector r_ij = (x_j - x_i) + s * L with the list's image, or with the
-// minimum image when the list carries no shifts.  Same operation order as the
-// neighbour predicate.
+// minimum image when the list carries no shifts.  The image is added by one
+// FMA: for images of 0, +-1 and +-2 boxes the product is exact, so the result is
+// that of the neighbour predicate's separate product and sum; the vector seen
+// from j is the exact negation in any case.
 NEP_HD void pair_vector(float4 pi, float4 pj, float Lx, float Ly, float Lz, float iLx, float iLy,
                         float iLz, int min_image, int packed, float& dx, float& dy, float& dz) {
-    float ux = sub_rn(pj.x, pi.x), uy = sub_rn(pj.y, pi.y), uz = sub_rn(pj.z, pi.z);
+    const float ux = sub_rn(pj.x, pi.x), uy = sub_rn(pj.y, pi.y), uz = sub_rn(pj.z, pi.z);
     float sx, sy, sz;
     if (min_image) {
         sx = -rint_f(ux * iLx);
@@ -157,14 +159,19 @@ NEP_HD void pair_vector(float4 pi, float4 pj, float Lx, float Ly, float Lz, floa
         unpack_shift(packed, a, b, c);
         sx = (float)a; sy = (float)b; sz = (float)c;
     }
-    dx = add_rn(ux, mul_rn(sx, Lx));
-    dy = add_rn(uy, mul_rn(sy, Ly));
-    dz = add_rn(uz, mul_rn(sz, Lz));
+    dx = fmaf(sx, Lx, ux);
+    dy = fmaf(sy, Ly, uy);
+    dz = fmaf(sz, Lz, uz);
 }
 
+// |r|^2 in the neighbour predicate's operation order
 NEP_HD float dist2(float dx, float dy, float dz) {
     return add_rn(add_rn(mul_rn(dx, dx), mul_rn(dy, dy)), mul_rn(dz, dz));
 }
+// |r|^2 in the evaluation, which decides by it in every kernel alike: the same
+// value for r and -r, within an ulp of dist2 (a pair that far from a cutoff
+// contributes about 1e-13)
+NEP_HD float norm2(float dx, float dy, float dz) { return fmaf(dz, dz, fmaf(dy, dy, mul_rn(dx, dx))); }
 
 // cos(pi z) and sin(pi z) for z = r/rc in [0, 1): with w = z - 1/2,
 // cos(pi z) = -sin(pi w) and sin(pi z) = cos(pi w), |pi w| <= pi/2, summed
@@ -195,20 +202,21 @@ NEP_HD void cutoff_trig(float z, float& c, float& s) {
 }
 
 // Q_k(r) = (T_k(x)+1)/2 f_c(r), x = 2(r/rc-1)^2-1, f_c = (1+cos(pi r/rc))/2.
+// One FMA per recurrence step and one per value: (T + 1) w = T w + w.
 template <int K>
 NEP_HD void basis(float r, float inv_rc, float* f) {
     float cz, sz;
     cutoff_trig(r * inv_rc, cz, sz);
-    float fc2 = 0.25f * (1.0f + cz);                       // f_c / 2
-    float t = r * inv_rc - 1.0f;
-    float x = 2.0f * t * t - 1.0f;
+    const float fc2 = fmaf(0.25f, cz, 0.25f);               // f_c / 2
+    const float t = fmaf(r, inv_rc, -1.0f);
+    const float x = fmaf(2.0f * t, t, -1.0f), x2 = 2.0f * x;
     float Tm = 1.0f, Tk = x;
     f[0] = 2.0f * fc2;
-    if (K > 1) f[1] = (x + 1.0f) * fc2;
+    if (K > 1) f[1] = fmaf(x, fc2, fc2);
 #pragma unroll
     for (int k = 2; k < K; ++k) {
-        float Tn = 2.0f * x * Tk - Tm;
-        f[k] = (Tn + 1.0f) * fc2;
+        const float Tn = fmaf(x2, Tk, -Tm);
+        f[k] = fmaf(Tn, fc2, fc2);
         Tm = Tk;
         Tk = Tn;
     }
@@ -219,25 +227,24 @@ template <int K>
 NEP_HD void basis_d(float r, float inv_rc, float* f, float* fp) {
     float sp, cp;
     cutoff_trig(r * inv_rc, cp, sp);
-    float fc2 = 0.25f * (1.0f + cp);
-    float dfc2 = (-0.25f * 3.14159265358979f) * inv_rc * sp;
-    float t = r * inv_rc - 1.0f;
-    float x = 2.0f * t * t - 1.0f;
-    float dxdr = 4.0f * t * inv_rc;
-    float a = dxdr * fc2;
+    const float fc2 = fmaf(0.25f, cp, 0.25f);
+    const float dfc2 = (-0.25f * 3.14159265358979f) * inv_rc * sp;
+    const float t = fmaf(r, inv_rc, -1.0f);
+    const float x = fmaf(2.0f * t, t, -1.0f), x2 = 2.0f * x;
+    const float a = 4.0f * t * inv_rc * fc2;
     float Tm = 1.0f, Tk = x, dTm = 0.0f, dTk = 1.0f;
     f[0] = 2.0f * fc2;
     fp[0] = 2.0f * dfc2;
     if (K > 1) {
-        f[1] = (x + 1.0f) * fc2;
-        fp[1] = a + (x + 1.0f) * dfc2;
+        f[1] = fmaf(x, fc2, fc2);
+        fp[1] = fmaf(x, dfc2, a + dfc2);
     }
 #pragma unroll
     for (int k = 2; k < K; ++k) {
-        float Tn = 2.0f * x * Tk - Tm;
-        float dTn = 2.0f * Tk + 2.0f * x * dTk - dTm;
-        f[k] = (Tn + 1.0f) * fc2;
-        fp[k] = dTn * a + (Tn + 1.0f) * dfc2;
+        const float Tn = fmaf(x2, Tk, -Tm);
+        const float dTn = fmaf(x2, dTk, fmaf(2.0f, Tk, -dTm));
+        f[k] = fmaf(Tn, fc2, fc2);
+        fp[k] = fmaf(dTn, a, fmaf(Tn, dfc2, dfc2));
         Tm = Tk; Tk = Tn; dTm = dTk; dTk = dTn;
     }
 }

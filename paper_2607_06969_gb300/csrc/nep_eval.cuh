@@ -241,7 +241,7 @@ NEP_HD void radial_atom(const EvalArgs& a, int i) {
         ns.advance(a, i, cnt, s);
         float dx, dy, dz;
         pair_vector(fr.pi, pj, fr.Lx, fr.Ly, fr.Lz, fr.iLx, fr.iLy, fr.iLz, MINIMG, sh, dx, dy, dz);
-        const float d2 = dist2(dx, dy, dz);
+        const float d2 = norm2(dx, dy, dz);
         const int tj = f2i(pj.w);
         if (d2 < rcR2) {
             if (COMPR) {
@@ -358,7 +358,7 @@ NEP_HD void angular_S(const EvalArgs& a, const float* sm, const SmemLayout& sl, 
         if (c + 1 < nc) e_nx = a.comp[(c + 1) * N + i];
         const int tj = f2i(e.w) & 3;
         float r, ir;
-        dist_rinv(dist2(e.x, e.y, e.z), r, ir);
+        dist_rinv(norm2(e.x, e.y, e.z), r, ir);
         float f[KA];
         basis<KA>(r, irA, f);
         float g[NA];
@@ -446,7 +446,7 @@ NEP_HD void angular_force(const EvalArgs& a, const float* sm, const SmemLayout& 
         const int tj = bits & 3;
         const int addr = (int)((unsigned)bits >> 2);
         float r, ir;
-        dist_rinv(dist2(e.x, e.y, e.z), r, ir);
+        dist_rinv(norm2(e.x, e.y, e.z), r, ir);
         float g[NA], gp[NA];
         {
             float f[KA], fp[KA];
@@ -785,7 +785,7 @@ NEP_HD void radial_force_atom(const EvalArgs& a, int i, float& Fx, float& Fy, fl
             const float4 e = q_nx;
             if (s + 1 < ncr) q_nx = a.compr[(s + 1) * N + i];
             const int bits = f2i(e.w);
-            pair((int)((unsigned)bits >> 2), bits & 3, e.x, e.y, e.z, dist2(e.x, e.y, e.z));
+            pair((int)((unsigned)bits >> 2), bits & 3, e.x, e.y, e.z, norm2(e.x, e.y, e.z));
         }
         // incoming angular pair forces: the prefix slots inside rc_A (the
         // mask, in batches of four independent loads, ascending) and every
@@ -838,7 +838,7 @@ NEP_HD void radial_force_atom(const EvalArgs& a, int i, float& Fx, float& Fy, fl
             ns.advance(a, i, cnt_ang, s);
             float dx, dy, dz;
             pair_vector(fr.pi, pj, fr.Lx, fr.Ly, fr.Lz, fr.iLx, fr.iLy, fr.iLz, MINIMG, sh, dx, dy, dz);
-            const float d2 = dist2(dx, dy, dz);
+            const float d2 = norm2(dx, dy, dz);
             if (d2 < rcA2) {
                 if (s < 64) {
                     amask |= 1ull << s;
@@ -863,7 +863,7 @@ NEP_HD void radial_force_atom(const EvalArgs& a, int i, float& Fx, float& Fy, fl
             ns.advance(a, i, nr, s);
             float dx, dy, dz;
             pair_vector(fr.pi, pj, fr.Lx, fr.Ly, fr.Lz, fr.iLx, fr.iLy, fr.iLz, MINIMG, sh, dx, dy, dz);
-            const float d2 = dist2(dx, dy, dz);
+            const float d2 = norm2(dx, dy, dz);
             if (d2 < rcR2) pair(j, f2i(pj.w), dx, dy, dz, d2);
         }
     }

@@ -168,7 +168,7 @@ __device__ __forceinline__ GroupPair group_pair(const EvalArgs& a, const AtomFra
     const float4 pj = a.pos4[p.j];
     p.tj = f2i(pj.w);
     pair_vector(fr.pi, pj, fr.Lx, fr.Ly, fr.Lz, fr.iLx, fr.iLy, fr.iLz, a.min_image, sh, p.dx, p.dy, p.dz);
-    p.d2 = dist2(p.dx, p.dy, p.dz);
+    p.d2 = norm2(p.dx, p.dy, p.dz);
     return p;
 }
 
@@ -212,7 +212,7 @@ __device__ int group_sums(const EvalArgs& a, const float* sm, float* gb, float* 
         GroupPair p;
         p.tj = f2i(pj.w);
         pair_vector(fr.pi, pj, fr.Lx, fr.Ly, fr.Lz, fr.iLx, fr.iLy, fr.iLz, a.min_image, sh, p.dx, p.dy, p.dz);
-        p.d2 = act ? dist2(p.dx, p.dy, p.dz) : 1.0f;
+        p.d2 = act ? norm2(p.dx, p.dy, p.dz) : 1.0f;
         float r, ir;
         dist_rinv(p.d2, r, ir);
         if (act && p.d2 < rcR2) {
@@ -520,7 +520,7 @@ __global__ void __launch_bounds__(kGroupThreads) kg_finish(const EvalArgs a, flo
         j1 = s + 2 * G < cnt ? a.nbr[(size_t)(s + 2 * G) * N + i] : i;
         p.tj = f2i(pj.w);
         pair_vector(fr.pi, pj, fr.Lx, fr.Ly, fr.Lz, fr.iLx, fr.iLy, fr.iLz, a.min_image, sh, p.dx, p.dy, p.dz);
-        p.d2 = dist2(p.dx, p.dy, p.dz);
+        p.d2 = norm2(p.dx, p.dy, p.dz);
         if (!(p.d2 < rcR2)) continue;
         float Pj[KR];
         const float* row = a.Pr + ((size_t)p.j * T + fr.ti) * KR;

@@ -54,7 +54,7 @@ __device__ __forceinline__ void tangent_pair(const EvalArgs& a, const AtomFrame&
                                              float4 li, const float* mu, TangentPair& p) {
     p.tj = f2i(pj.w);
     pair_vector(fr.pi, pj, fr.Lx, fr.Ly, fr.Lz, fr.iLx, fr.iLy, fr.iLz, a.min_image, sh, p.dx, p.dy, p.dz);
-    p.d2 = dist2(p.dx, p.dy, p.dz);
+    p.d2 = norm2(p.dx, p.dy, p.dz);
     dist_rinv(p.d2, p.r, p.ir);
     p.drx = -(lj.x - li.x) - (mu[0] * p.dx + mu[1] * p.dy + mu[2] * p.dz);
     p.dry = -(lj.y - li.y) - (mu[3] * p.dx + mu[4] * p.dy + mu[5] * p.dz);

@@ -121,7 +121,7 @@ NEP_HD void tangent_atom(const TrainArgs& t, const float* sm, int i) {
         const int tj = f2i(e.w) & 3;
         float drx, dry, drz;
         pair_tangent(mu, li, lj, e.x, e.y, e.z, drx, dry, drz);
-        const float r = sqrt_f(dist2(e.x, e.y, e.z));
+        const float r = sqrt_f(norm2(e.x, e.y, e.z));
         const float ir = rcp_f(r);
         const float udr = (e.x * drx + e.y * dry + e.z * drz) * ir;
         float f[KR], fp[KR];
@@ -164,7 +164,7 @@ NEP_HD void tangent_atom(const TrainArgs& t, const float* sm, int i) {
         const int tj = f2i(e.w) & 3;
         float drx, dry, drz;
         pair_tangent(mu, li, lj, e.x, e.y, e.z, drx, dry, drz);
-        const float r = sqrt_f(dist2(e.x, e.y, e.z));
+        const float r = sqrt_f(norm2(e.x, e.y, e.z));
         const float ir = rcp_f(r);
         const Harm<float> ht = harm_of(e.x * ir, e.y * ir, e.z * ir);
         const float udr = ht.x * drx + ht.y * dry + ht.z * drz;
@@ -298,7 +298,7 @@ NEP_HD void xzp_atom(const TrainArgs& t, const float* sm, int i) {
     const int nc = a.cnt_comp[i];
     for (int c = 0; c < nc; ++c) {
         const float4 e = a.comp[c * N + i];
-        const float ir = rcp_f(sqrt_f(dist2(e.x, e.y, e.z)));
+        const float ir = rcp_f(sqrt_f(norm2(e.x, e.y, e.z)));
         const Harm<float> ht = harm_of(e.x * ir, e.y * ir, e.z * ir);
         float X[NA];
 #pragma unroll
@@ -354,7 +354,7 @@ NEP_HD void xzr_atom(const TrainArgs& t, const float* sm, int i) {
         as.next(c, e, lj);
         float drx, dry, drz;
         pair_tangent(mu, li, lj, e.x, e.y, e.z, drx, dry, drz);
-        const float ir = rcp_f(sqrt_f(dist2(e.x, e.y, e.z)));
+        const float ir = rcp_f(sqrt_f(norm2(e.x, e.y, e.z)));
         const Harm<float> ht = harm_of(e.x * ir, e.y * ir, e.z * ir);
         const float udr = ht.x * drx + ht.y * dry + ht.z * drz;
         const HarmD<float> hd = unit_tangent(ht, drx, dry, drz, udr, ir);
@@ -400,7 +400,7 @@ NEP_HD void cbins_atom(const TrainArgs& t, const float* sm, int i) {
     for (int c = 0; c < nc; ++c) {
         const float4 e = a.comp[c * N + i];
         const int tj = f2i(e.w) & 3;
-        const float r = sqrt_f(dist2(e.x, e.y, e.z));
+        const float r = sqrt_f(norm2(e.x, e.y, e.z));
         float f[KA], fp[KA];
         basis_d<KA>(r, irA, f, fp);
         float X[NA], Z[NA];
