@@ -454,14 +454,25 @@ nep_status efv_generic(nep_model* m, const nep_system* s, const nep_nlist* nl, f
     return NEP_OK;
 }
 
+// The closing half kick of an MD step, taken over by the evaluation where its
+// last kernel per atom can do it (done is set).
+struct ClosingKick {
+    float* vel;
+    float half_dt;
+    const float* inv_mass;
+    bool done;
+};
+
+// packed: positions, configurations and the chunk plan are in the workspace
 nep_status efv_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, float* e_atom,
                     float* force, double* e_tot, double* virial, void* work, const WsLayout& w,
-                    cudaStream_t st, int n_owned = -1) {
+                    cudaStream_t st, int n_owned = -1, bool packed = false, ClosingKick* kick = nullptr) {
     const int N = s->n_atoms, B = s->n_cfg;
-    NEP_CUDA(nep::launch_pack_plan(s->pos, s->type, s->atom_off, N, B, m->hp.n_types, at<float4>(work, w.pos4),
-                                   at<int>(work, w.cfg), nl->status, at<int>(work, w.chunk_start),
-                                   at<int>(work, w.ticket), st),
-             "pack");
+    if (!packed)
+        NEP_CUDA(nep::launch_pack_plan(s->pos, s->type, s->atom_off, N, B, m->hp.n_types, at<float4>(work, w.pos4),
+                                       at<int>(work, w.cfg), nl->status, at<int>(work, w.chunk_start),
+                                       at<int>(work, w.ticket), st),
+                 "pack");
     if (!m->ks) return efv_generic(m, s, nl, e_atom, force, e_tot, virial, work, w, st, n_owned);
     const nep::EvalArgs a = make_args(m, s, nl, work, w);
     const int vd = angular_variant(m, s);
@@ -496,6 +507,13 @@ nep_status efv_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, floa
     f.ticket = at<int>(work, w.ticket);
     f.e_tot = e_tot;
     f.virial = virial;
+    f.vel = nullptr;
+    if (G && kick) {
+        f.vel = kick->vel;
+        f.half_dt = kick->half_dt;
+        for (int t = 0; t < nep::kMaxTypes; ++t) f.inv_mass[t] = kick->inv_mass[t];
+        kick->done = true;
+    }
     if (G) NEP_CUDA(m->ks->group_finish(a, f, w.max_chunks, st, G), "finish kernel");
     else NEP_CUDA(m->ks->finish(a, f, w.max_chunks, st, finish_block(m, s)), "finish kernel");
     NEP_CUDA(mark(3), "timing event");
@@ -540,6 +558,7 @@ nep_status train_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, co
         f.ticket = at<int>(work, w.ticket);
         f.e_tot = at<double>(work, tl.etot);
         f.virial = at<double>(work, tl.vir);
+        f.vel = nullptr;
         if (G) NEP_CUDA(m->ks->group_finish(a, f, w.max_chunks, st, G), "finish kernel");
         else NEP_CUDA(m->ks->finish(a, f, w.max_chunks, st, 0), "finish kernel");
         NEP_CUDA(nep::launch_loss(N, B, s->atom_off, at<int>(work, w.chunk_start), w.max_chunks,
@@ -1050,15 +1069,22 @@ nep_status nep_md_step(nep_model* m, const nep_system* sys, nep_nlist* nl, float
     cudaStream_t st = (cudaStream_t)stream;
     const int N = sys->n_atoms;
     float* pos = const_cast<float*>(sys->pos);
-    NEP_CUDA(nep::launch_kick(vel, force, sys->type, inv_m, N, 0.5f * dt, pos, dt, st), "kick/drift");
+    if (!rebuild && !nl->min_image && !nl->shift) return fail(NEP_ERR_STATE, "list was not built");
     if (rebuild) {
+        NEP_CUDA(nep::launch_kick(vel, force, sys->type, inv_m, N, 0.5f * dt, pos, dt, st), "kick/drift");
         NEP_CUDA(nep::launch_wrap_segments(pos, sys->atom_off, sys->n_cfg, sys->box, N, st), "wrap");
         if ((s = neighbors_impl(m, sys, skin, nl, work, w, st)) != NEP_OK) return s;
-    } else if (!nl->min_image && !nl->shift) {
-        return fail(NEP_ERR_STATE, "list was not built");
+    } else {
+        NEP_CUDA(nep::launch_kick_pack(vel, force, sys->type, inv_m, N, sys->n_cfg, m->hp.n_types, 0.5f * dt, pos, dt,
+                                       sys->atom_off, at<float4>(work, w.pos4), at<int>(work, w.cfg), nl->status,
+                                       at<int>(work, w.chunk_start), at<int>(work, w.ticket), st),
+                 "kick/drift");
     }
-    if ((s = efv_impl(m, sys, nl, nullptr, force, e_tot, virial, work, w, st)) != NEP_OK) return s;
-    NEP_CUDA(nep::launch_kick(vel, force, sys->type, inv_m, N, 0.5f * dt, nullptr, 0.0f, st), "kick");
+    ClosingKick kick{vel, 0.5f * dt, inv_m, false};
+    if ((s = efv_impl(m, sys, nl, nullptr, force, e_tot, virial, work, w, st, -1, !rebuild, &kick)) != NEP_OK)
+        return s;
+    if (!kick.done)
+        NEP_CUDA(nep::launch_kick(vel, force, sys->type, inv_m, N, 0.5f * dt, nullptr, 0.0f, st), "kick");
     return NEP_OK;
 }
 
@@ -1269,6 +1295,7 @@ nep_status nep_autotune(nep_model* m, const nep_system* sys, const nep_nlist* nl
     f.n_owned = N;
     f.ticket = at<int>(work, w.ticket);
     f.e_tot = f.virial = nullptr;
+    f.vel = nullptr;
     int vd = nep::kDefaultAngularVariant, rb = 0, fb = 0;
     cudaError_t err = cudaSuccess;
     if (N > 0) {

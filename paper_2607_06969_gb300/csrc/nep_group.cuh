@@ -489,9 +489,10 @@ __global__ void __launch_bounds__(kGroupThreads, kGroupMinBlocks) kg_atom(const 
 
 // F_i and the per-atom virial: radial pair forces of both directions from the
 // projected adjoints of both atoms, the owner's angular part, and the incoming
-// angular slots (those whose pair lies inside rc_ang)
+// angular slots (those whose pair lies inside rc_ang); in MD also the closing
+// half kick, which saves small systems its launch
 template <class C, int G>
-__global__ void __launch_bounds__(kGroupThreads) kg_finish(const EvalArgs a, float* force, float* e_out) {
+__global__ void __launch_bounds__(kGroupThreads) kg_finish(const EvalArgs a, const FinishArgs fa) {
     constexpr int KR = C::KR, T = C::T, NG = kGroupThreads / G;
     __shared__ __align__(16) float Pi[NG][round4(T * KR)];
     const int N = a.N, lane = threadIdx.x % G, group = threadIdx.x / G;
@@ -561,10 +562,18 @@ __global__ void __launch_bounds__(kGroupThreads) kg_finish(const EvalArgs a, flo
     for (int k = 0; k < 9; ++k) acc[k] = lanes_sum<G>(acc[k]);
     if (!valid) return;
     if (lane == 0) {
-        force[i] = a.fpart[i] + acc[0];
-        force[N + i] = a.fpart[N + i] + acc[1];
-        force[2 * (size_t)N + i] = a.fpart[2 * (size_t)N + i] + acc[2];
-        if (e_out) e_out[i] = a.e_atom[i];
+        float im = fa.inv_mass[0];
+#pragma unroll
+        for (int t = 1; t < kMaxTypes; ++t) im = fr.ti == t ? fa.inv_mass[t] : im;
+        const float s = fa.half_dt * im;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const size_t at = (size_t)c * N + i;
+            const float F = a.fpart[at] + acc[c];
+            fa.force[at] = F;
+            if (fa.vel) fa.vel[at] = fmaf(s, F, fa.vel[at]);
+        }
+        if (fa.e_out) fa.e_out[i] = a.e_atom[i];
     }
     const float Wsym[9] = {acc[3], acc[6], acc[7], acc[6], acc[4], acc[8], acc[7], acc[8], acc[5]};
 #pragma unroll
@@ -598,7 +607,7 @@ cudaError_t launch_group_g(const EvalArgs& a, cudaStream_t st) {
 template <class C, int G>
 void launch_group_finish_g(const EvalArgs& a, const FinishArgs& f, cudaStream_t st) {
     constexpr int NG = kGroupThreads / G;
-    kg_finish<C, G><<<(a.N + NG - 1) / NG, kGroupThreads, 0, st>>>(a, f.force, f.e_out);
+    kg_finish<C, G><<<(a.N + NG - 1) / NG, kGroupThreads, 0, st>>>(a, f);
 }
 
 template <class C>

@@ -103,6 +103,10 @@ struct FinishArgs {
     float* force;                  // [3][N]
     float* e_out;                  // [N] or null
     int n_owned;                   // atoms [0, n_owned) enter the E and virial sums
+    // MD, group kernels only: the closing half kick v += half_dt F / m (vel null: none)
+    float* vel;                    // [3][N]
+    float half_dt;
+    float inv_mass[kMaxTypes];
 };
 
 // Offsets of the parameter blocks in the flat vector.
@@ -275,6 +279,10 @@ cudaError_t fp32_peak(cudaStream_t st, double* tflops);
 cudaError_t wait_selftest(cudaStream_t st, int* outcome);
 cudaError_t launch_kick(float* vel, const float* force, const int* type, const float* inv_mass,
                         int N, float half_dt, float* pos, float dt, cudaStream_t st);
+// launch_kick with the drift, and launch_pack_plan at the new positions
+cudaError_t launch_kick_pack(float* vel, const float* force, const int* type, const float* inv_mass, int N, int B,
+                             int T, float half_dt, float* pos, float dt, const int* atom_off, float4* pos4, int* cfg,
+                             int* status, int* chunk_start, int* ticket, cudaStream_t st);
 cudaError_t launch_wrap_segments(float* pos, const int* atom_off, int B, const float* box, int N, cudaStream_t st);
 cudaError_t launch_loss(int N, int B, const int* atom_off, const int* chunk_start, int max_chunks,
                         const float* force, const float* f_lbl, const double* e_tot,

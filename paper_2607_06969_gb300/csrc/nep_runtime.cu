@@ -28,6 +28,22 @@ __device__ __forceinline__ int find_segment(const int* off, int B, int x) {
 // Exclusive scan of the configurations' chunk counts by one CTA (any multiple
 // of 32 threads up to 1,024), and the reduction tickets cleared.
 __device__ void chunk_plan_block(const int* __restrict__ atom_off, int B, int* chunk_start, int* ticket) {
+    if (B <= 32) {                       // one warp, no block-wide waits
+        const int b = threadIdx.x;
+        if (b >= 32) return;
+        int x = b < B ? (atom_off[b + 1] - atom_off[b] + kChunk - 1) / kChunk : 0;
+        const int v = x;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (b >= o) x += y;
+        }
+        if (b < B) {
+            chunk_start[b] = x - v;
+            if (ticket) ticket[b] = 0;
+        }
+        if (b == 31) chunk_start[B] = x;
+        return;
+    }
     __shared__ int carry;
     __shared__ int warp_sums[32];
     if (threadIdx.x == 0) carry = 0;
@@ -72,6 +88,20 @@ __global__ void __launch_bounds__(1024) k_chunk_plan(const int* __restrict__ ato
     chunk_plan_block(atom_off, B, chunk_start, ticket);
 }
 
+__device__ __forceinline__ void pack_atom(const float* pos, const int* __restrict__ type,
+                                          const int* __restrict__ atom_off, int N, int B, int T, int i, float4* pos4,
+                                          int* cfg, int* status) {
+    int t = type[i];
+    if (t < 0 || t >= T) {
+        set_flag(status, 3);
+        t = 0;
+    }
+    const float x = pos[i], y = pos[N + i], z = pos[2 * (size_t)N + i];
+    if (!(isfinite(x) && isfinite(y) && isfinite(z))) set_flag(status, 3);
+    pos4[i] = make_float4(x, y, z, __int_as_float(t));
+    cfg[i] = find_segment(atom_off, B, i);
+}
+
 // positions, species and configuration of each atom in the kernels' layout;
 // with chunk_start, one more block plans the reduction chunks meanwhile
 __global__ void __launch_bounds__(256) k_pack(const float* __restrict__ pos, const int* __restrict__ type,
@@ -82,16 +112,7 @@ __global__ void __launch_bounds__(256) k_pack(const float* __restrict__ pos, con
         return;
     }
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    int t = type[i];
-    if (t < 0 || t >= T) {
-        set_flag(status, 3);
-        t = 0;
-    }
-    const float x = pos[i], y = pos[N + i], z = pos[2 * N + i];
-    if (!(isfinite(x) && isfinite(y) && isfinite(z))) set_flag(status, 3);
-    pos4[i] = make_float4(x, y, z, __int_as_float(t));
-    cfg[i] = find_segment(atom_off, B, i);
+    if (i < N) pack_atom(pos, type, atom_off, N, B, T, i, pos4, cfg, status);
 }
 
 constexpr int kRedThreads = 256;
@@ -961,17 +982,37 @@ struct InvMass {
     float v[kMaxTypes];
 };
 
-__global__ void k_kick(float* __restrict__ vel, const float* __restrict__ force,
-                       const int* __restrict__ type, InvMass im, int N, float half_dt,
-                       float* __restrict__ pos, float dt) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const float s = half_dt * im.v[type[i] & (kMaxTypes - 1)];
+__device__ __forceinline__ void kick_atom(float* __restrict__ vel, const float* __restrict__ force, int type,
+                                          const InvMass& im, int N, int i, float half_dt, float* __restrict__ pos,
+                                          float dt) {
+    const float s = half_dt * im.v[type & (kMaxTypes - 1)];
     for (int d = 0; d < 3; ++d) {
         float v = vel[(size_t)d * N + i] + s * force[(size_t)d * N + i];
         vel[(size_t)d * N + i] = v;
         if (pos) pos[(size_t)d * N + i] += dt * v;
     }
+}
+__global__ void k_kick(float* __restrict__ vel, const float* __restrict__ force,
+                       const int* __restrict__ type, InvMass im, int N, float half_dt,
+                       float* __restrict__ pos, float dt) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < N) kick_atom(vel, force, type[i], im, N, i, half_dt, pos, dt);
+}
+// the opening half kick and the drift, then the atom packed at its new
+// position (as k_pack, whose launch and pass over the positions this saves)
+__global__ void __launch_bounds__(256) k_kick_pack(float* __restrict__ vel, const float* __restrict__ force,
+                                                   const int* __restrict__ type, InvMass im, int N, float half_dt,
+                                                   float* __restrict__ pos, float dt,
+                                                   const int* __restrict__ atom_off, int B, int T, float4* pos4,
+                                                   int* cfg, int* status, int* chunk_start, int* ticket) {
+    if (chunk_start && blockIdx.x == gridDim.x - 1) {
+        chunk_plan_block(atom_off, B, chunk_start, ticket);
+        return;
+    }
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N) return;
+    kick_atom(vel, force, type[i], im, N, i, half_dt, pos, dt);
+    pack_atom(pos, type, atom_off, N, B, T, i, pos4, cfg, status);
 }
 
 // x wrapped into [0, L)
@@ -1100,9 +1141,10 @@ cudaError_t launch_pack(const float* pos, const int* type, const int* atom_off, 
 
 // the plan rides in the packing launch (1.9 us less) unless its scan by one
 // block of 256 threads would outlast it
+constexpr int kPlanFusedB = 2048;
 cudaError_t launch_pack_plan(const float* pos, const int* type, const int* atom_off, int N, int B, int T,
                              float4* pos4, int* cfg, int* status, int* chunk_start, int* ticket, cudaStream_t st) {
-    const bool fused = B <= 2048;
+    const bool fused = B <= kPlanFusedB;
     if (fused) {
         k_pack<<<blocks(N, 256) + 1, 256, 0, st>>>(pos, type, atom_off, N, B, T, pos4, cfg, status, chunk_start,
                                                    ticket);
@@ -1218,6 +1260,20 @@ cudaError_t launch_kick(float* vel, const float* force, const int* type, const f
     InvMass im;
     for (int t = 0; t < kMaxTypes; ++t) im.v[t] = inv_mass[t];
     if (N > 0) k_kick<<<blocks(N, 256), 256, 0, st>>>(vel, force, type, im, N, half_dt, pos, dt);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_kick_pack(float* vel, const float* force, const int* type, const float* inv_mass, int N, int B,
+                             int T, float half_dt, float* pos, float dt, const int* atom_off, float4* pos4, int* cfg,
+                             int* status, int* chunk_start, int* ticket, cudaStream_t st) {
+    InvMass im;
+    for (int t = 0; t < kMaxTypes; ++t) im.v[t] = inv_mass[t];
+    const bool fused = B <= kPlanFusedB;
+    if (N > 0 || fused)
+        k_kick_pack<<<blocks(N, 256) + (fused ? 1 : 0), 256, 0, st>>>(vel, force, type, im, N, half_dt, pos, dt,
+                                                                      atom_off, B, T, pos4, cfg, status,
+                                                                      fused ? chunk_start : nullptr, ticket);
+    if (!fused) k_chunk_plan<<<1, 1024, 0, st>>>(atom_off, B, chunk_start, ticket);
     return cudaGetLastError();
 }
 
