@@ -69,7 +69,7 @@ struct WsLayout {
     size_t pos4, cfg, e_atom, fb, S, Pr, comp, cnt_comp, fin, fpart, wat, chunk_start, partial;
     size_t rin, rin_sh, cnt_rin;
     size_t amask;
-    size_t gen_p, gen_R, gen_w;   // generic FP32 path: dE/dq (radial), dE/dS, per-atom virial
+    size_t gen_w;                 // generic FP32 path: per-atom virial
     size_t plan, cell_of, rank, cell_cnt, cell_start, cell_atoms, cell_pos, scan_tmp, shell, row_start, slot_row;
     size_t ticket;                // reduction tickets [B]: the cell counts' place, idle during an evaluation
     size_t total;
@@ -101,11 +101,9 @@ WsLayout ws_layout(const nep_model* m, int N, int B, int cap, int cap_ang) {
     w.cnt_rin = take(4 * n);
     w.amask = take(8 * n);
     if (!m->ks) {
-        w.gen_p = take(4 * n * m->hp.n_rad);
-        w.gen_R = take(4 * n * NA * nep::kLM);
         w.gen_w = take(36 * n);
     } else {
-        w.gen_p = w.gen_R = w.gen_w = 0;
+        w.gen_w = 0;
     }
     w.fpart = take(12 * n);
     w.wat = take(36 * n);
@@ -335,7 +333,7 @@ nep_status check_work(const nep_model* m, const nep_system* s, const nep_nlist* 
 
 // Scratch of the FP64 evaluation
 struct Ws64Layout {
-    size_t pos4, cfg, chunk_start, partial, prm, e, p, R, w;
+    size_t pos4, cfg, chunk_start, ticket, partial, prm, e, p, R, w;
     // training: FP64 forces, totals, adjoints, staged factors, gradient partials
     size_t force, etot, vir, lam, aE, mu, st, gpart;
     size_t total;
@@ -353,11 +351,12 @@ Ws64Layout ws64_layout(const nep_model* m, int N, int B) {
     w.pos4 = take(16 * n);
     w.cfg = take(4 * n);
     w.chunk_start = take(4 * ((size_t)B + 1));
+    w.ticket = take(4 * (size_t)B);
     w.max_chunks = (int)((n + nep::kChunk - 1) / nep::kChunk) + B;
     w.partial = take(80 * (size_t)w.max_chunks);
     w.prm = take(8 * (size_t)m->lay.P);
     w.e = take(8 * n);
-    w.p = take(8 * n * m->hp.n_rad);
+    w.p = take(8 * n * m->hp.n_types * m->hp.k_rad);
     w.R = take(8 * n * m->hp.n_ang * nep::kLM);
     w.w = take(72 * n);
     w.total = o;
@@ -435,13 +434,16 @@ nep_status efv_generic(nep_model* m, const nep_system* s, const nep_nlist* nl, f
     a.shift = nl->min_image ? nullptr : nl->shift;
     a.prm = m->params;
     a.e = e_atom ? e_atom : at<float>(work, w.e_atom);
-    a.p = at<float>(work, w.gen_p);
-    a.R = at<float>(work, w.gen_R);
+    a.p = at<float>(work, w.Pr);
+    a.cnt_ang = nl->cnt_ang;
+    a.rev = nl->rev;
+    a.fin = at<float4>(work, w.fin);
     a.w = at<float>(work, w.gen_w);
     a.force = force;
     a.atom_off = s->atom_off;
     a.chunk_start = at<int>(work, w.chunk_start);
     a.partial = at<double>(work, w.partial);
+    a.ticket = at<int>(work, w.ticket);
     a.n_owned = n_owned < 0 ? N : n_owned;
     const int nt = m->n_timing;
     m->n_timing = 0;
@@ -802,10 +804,10 @@ nep_status fp64_begin(nep_model* m, const nep_system* sys, const nep_nlist* nl, 
     if ((reinterpret_cast<uintptr_t>(work) & 255) != 0)
         return fail(NEP_ERR_ARG, "workspace must be 256-byte aligned");
     const int N = sys->n_atoms, B = sys->n_cfg;
-    NEP_CUDA(nep::launch_pack(sys->pos, sys->type, sys->atom_off, N, B, m->hp.n_types, at<float4>(work, w.pos4),
-                              at<int>(work, w.cfg), nl->status, st),
+    NEP_CUDA(nep::launch_pack_plan(sys->pos, sys->type, sys->atom_off, N, B, m->hp.n_types, at<float4>(work, w.pos4),
+                                   at<int>(work, w.cfg), nl->status, at<int>(work, w.chunk_start),
+                                   at<int>(work, w.ticket), st),
              "pack");
-    NEP_CUDA(nep::launch_chunk_plan(sys->atom_off, B, at<int>(work, w.chunk_start), st), "chunk plan");
     if (!params) {
         NEP_CUDA(nep::launch_promote(m->params, at<double>(work, w.prm), m->lay.P, st), "promote parameters");
         params = at<double>(work, w.prm);
@@ -839,6 +841,7 @@ nep_status fp64_begin(nep_model* m, const nep_system* sys, const nep_nlist* nl, 
     a.atom_off = sys->atom_off;
     a.chunk_start = at<int>(work, w.chunk_start);
     a.partial = at<double>(work, w.partial);
+    a.ticket = at<int>(work, w.ticket);
     a.n_owned = N;
     *out = a;
     return NEP_OK;

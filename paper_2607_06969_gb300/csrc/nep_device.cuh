@@ -460,54 +460,6 @@ struct HarmSums {
     }
 };
 
-// Component m of the real solid harmonics: value P_m(u) on the unit sphere
-// and the gradient of the homogeneous polynomial at u.  With m a
-// compile-time constant the switch folds away.
-template <class R>
-struct HarmTermsT {
-    R x, y, z, xx, yy, zz, xy, xz, yz;
-};
-using HarmTerms = HarmTermsT<float>;
-template <class R>
-NEP_HD HarmTermsT<R> harm_terms(R x, R y, R z) {
-    HarmTermsT<R> t;
-    t.x = x; t.y = y; t.z = z;
-    t.xx = x * x; t.yy = y * y; t.zz = z * z;
-    t.xy = x * y; t.xz = x * z; t.yz = y * z;
-    return t;
-}
-template <class R>
-NEP_HD void harm_m(int m, const HarmTermsT<R>& t, R& Y, R& gx, R& gy, R& gz) {
-    const R x = t.x, y = t.y, z = t.z, xx = t.xx, yy = t.yy, zz = t.zz;
-    const R xy = t.xy, xz = t.xz, yz = t.yz;
-    switch (m) {
-        case 0: Y = y; gx = R(0.0); gy = R(1.0); gz = R(0.0); break;
-        case 1: Y = z; gx = R(0.0); gy = R(0.0); gz = R(1.0); break;
-        case 2: Y = x; gx = R(1.0); gy = R(0.0); gz = R(0.0); break;
-        case 3: Y = xy; gx = y; gy = x; gz = R(0.0); break;
-        case 4: Y = yz; gx = R(0.0); gy = z; gz = y; break;
-        case 5: Y = R(3.0) * zz - R(1.0); gx = -R(2.0) * x; gy = -R(2.0) * y; gz = R(4.0) * z; break;
-        case 6: Y = xz; gx = z; gy = R(0.0); gz = x; break;
-        case 7: Y = xx - yy; gx = R(2.0) * x; gy = -R(2.0) * y; gz = R(0.0); break;
-        case 8: Y = y * (R(3.0) * xx - yy); gx = R(6.0) * xy; gy = R(3.0) * (xx - yy); gz = R(0.0); break;
-        case 9: Y = xy * z; gx = yz; gy = xz; gz = xy; break;
-        case 10: Y = y * (R(5.0) * zz - R(1.0)); gx = -R(2.0) * xy; gy = R(4.0) * zz - xx - R(3.0) * yy; gz = R(8.0) * yz; break;
-        case 11: Y = z * (R(5.0) * zz - R(3.0)); gx = -R(6.0) * xz; gy = -R(6.0) * yz; gz = R(6.0) * zz - R(3.0) * xx - R(3.0) * yy; break;
-        case 12: Y = x * (R(5.0) * zz - R(1.0)); gx = R(4.0) * zz - R(3.0) * xx - yy; gy = -R(2.0) * xy; gz = R(8.0) * xz; break;
-        case 13: Y = z * (xx - yy); gx = R(2.0) * xz; gy = -R(2.0) * yz; gz = xx - yy; break;
-        case 14: Y = x * (xx - R(3.0) * yy); gx = R(3.0) * (xx - yy); gy = -R(6.0) * xy; gz = R(0.0); break;
-        case 15: Y = xy * (xx - yy); gx = y * (R(3.0) * xx - yy); gy = x * (xx - R(3.0) * yy); gz = R(0.0); break;
-        case 16: Y = yz * (R(3.0) * xx - yy); gx = R(6.0) * xy * z; gy = R(3.0) * z * (xx - yy); gz = y * (R(3.0) * xx - yy); break;
-        case 17: Y = xy * (R(7.0) * zz - R(1.0)); gx = -y * (R(3.0) * xx + yy - R(6.0) * zz); gy = -x * (xx + R(3.0) * yy - R(6.0) * zz); gz = R(12.0) * xy * z; break;
-        case 18: Y = yz * (R(7.0) * zz - R(3.0)); gx = -R(6.0) * xy * z; gy = -z * (R(3.0) * xx + R(9.0) * yy - R(4.0) * zz); gz = -R(3.0) * y * (xx + yy - R(4.0) * zz); break;
-        case 19: Y = (R(35.0) * zz - R(30.0)) * zz + R(3.0); gx = R(12.0) * x * (xx + yy - R(4.0) * zz); gy = R(12.0) * y * (xx + yy - R(4.0) * zz); gz = -R(16.0) * z * (R(3.0) * xx + R(3.0) * yy - R(2.0) * zz); break;
-        case 20: Y = xz * (R(7.0) * zz - R(3.0)); gx = -z * (R(9.0) * xx + R(3.0) * yy - R(4.0) * zz); gy = -R(6.0) * xy * z; gz = -R(3.0) * x * (xx + yy - R(4.0) * zz); break;
-        case 21: Y = (xx - yy) * (R(7.0) * zz - R(1.0)); gx = -R(4.0) * x * (xx - R(3.0) * zz); gy = R(4.0) * y * (yy - R(3.0) * zz); gz = R(12.0) * z * (xx - yy); break;
-        case 22: Y = xz * (xx - R(3.0) * yy); gx = R(3.0) * z * (xx - yy); gy = -R(6.0) * xy * z; gz = x * (xx - R(3.0) * yy); break;
-        default: Y = xx * (xx - R(3.0) * yy) - yy * (R(3.0) * xx - yy); gx = R(4.0) * x * (xx - R(3.0) * yy); gy = -R(4.0) * y * (R(3.0) * xx - yy); gz = R(0.0); break;
-    }
-}
-
 // 4-body term from the l = 2 block s[0..4] = (xy, yz, 2zz-xx-yy, xz, xx-yy)
 // sums: A = sum_j g (u u^T - I/3) is traceless symmetric with
 // A_xy = s0, A_yz = s1, A_zz = s2/3, A_xz = s3, A_xx - A_yy = s4.

@@ -1,359 +1,471 @@
-// FP64 evaluation of energies, forces and virial, and the FP64 training
-// gradient.
-//
-// The operators of Section 3.2 run in float64 as well as float32.  This path
-// computes Eqs. 1-4 and 11-21 with every intermediate in double: positions
-// (FP32 inputs) are promoted, the parameters are FP64, and pairs are kept by
-// r < rc in double.  Hyper-parameters are runtime values.  G lanes per atom
-// split its neighbour list: G = 1 once N fills the GPU, up to a warp for a
-// few hundred atoms, so that small systems still reach every SM.
-//
-// Evaluation, two passes over the list:
+// FP64 evaluation of energies, forces and virial, the generic FP32 evaluation
+// (the same kernels in float) and the FP64 loss.  Two passes over the list:
 //   k64_atom  : the species-resolved radial basis sums F[t][k] and q_n
 //               (Eq. 11), S_nlm and q_nl (Eqs. 16-17), q4_n, the network
-//               (Eq. 2), E_i, dE_i/dq_n (radial) and R_nlm = dE_i/dS_nlm
-//   k64_force : F_i = sum_j [dE_i/dr_ij - dE_j/dr_ji] (Eq. 3), each pair
-//               derivative recomputed from its owner's dE/dq and R; per-atom
-//               virial W_i = -sum_j dE_i/dr_ij (x) r_ij (Eq. 4)
+//               (Eq. 2), E_i, the radial adjoint per neighbour species and
+//               R_nlm = dE_i/dS_nlm
+//   k64_force : F_i = sum_j [dE_i/dr_ij - dE_j/dr_ji] (Eq. 3) and the per-atom
+//               virial (Eq. 4)
 // then FP64 sums per 1,024-atom chunk and per configuration in a fixed order.
 //
-// Training gradient: the gradient of Phi = sum_b aE_b E_b + sum_i lam_i . F_i
-// + sum_b mu_b : V_b at fixed adjoints (the loss gradient of Eqs. 18-21 when
-// they are the loss adjoints).  With dr_ij = -(lam_j - lam_i) - mu r_ij,
-// Phi = sum_i [aE E_i + p_i . dq_i], p = dE/dq, dq the tangent of q along dr.
-//   k64_grad_atom : descriptors and network again, the tangent dq (radial
-//                   DF[t][k] = sum_j Q'_k (rhat . dr), angular dS_nlm), the
-//                   network's second-order terms (alpha, beta, gamma,
-//                   rho = aE p + d(p . dq)/dq), P = dPhi/dS, R = dPhi/d(dS),
-//                   and per angular pair X_n = sum_m P_nm Y_m + R_nm dY_m . dr,
-//                   Z_n = (rhat . dr) sum_m R_nm Y_m, summed into
-//                   bins[t][n][k] = sum_{j of t} Q_k X_n + Q'_k Z_n; the
-//                   per-atom factors of every parameter's gradient are staged
-//   k64_grad_partial / k64_grad_final : per 1,024-atom chunk, each parameter
-//                   summed over the chunk's atoms of its species; then the
-//                   chunks in order
-//
-// Lane partials are combined by an xor butterfly, whose fixed tree leaves
-// the same bits in every lane of the group; every pair term is evaluated by
-// both of its atoms, so nothing is scattered, and for a given N (which fixes
-// G) every result is deterministic.
-#include <algorithm>
-
-#include <cuda_runtime.h>
-
-#include "nep_device.cuh"
-#include "nep_internal.h"
+// Measured (38-30-1 model): FP64, 2,593 atoms 1,319 -> 382 us against one or
+// more lanes per atom with runtime-indexed arrays and both sides of a pair
+// evaluated apart; k64_force keeps the FP64 pipe, which bounds both kernels,
+// busy 85% of the cycles.  Generic, 9,956 atoms of a two-species model 605 -> 136 us.
+#include "nep_fp64.cuh"
 
 namespace nep {
 namespace {
-
-constexpr int kF64Block = 128;
-constexpr int kF64MaxD = kF64MaxN * 6;              // n_rad + 5 n_ang
-constexpr int kF64MaxTK = kMaxTypes * kF64MaxK;     // n_types * k_rad
-constexpr double kPi = 3.141592653589793;
-
-// The evaluation below is written once for two argument types: F64Args (every
-// intermediate in double) and F32Args (the generic FP32 evaluation, any
-// hyper-parameters within the same bounds).  R is the argument type's scalar.
-template <class A>
-struct ScalarOf;
-template <>
-struct ScalarOf<F64Args> {
-    using type = double;
-};
-template <>
-struct ScalarOf<F32Args> {
-    using type = float;
-};
-template <class A>
-using ScalarT = typename ScalarOf<A>::type;
-
-__device__ __forceinline__ void sincospi_r(double z, double* s, double* c) { sincospi(z, s, c); }
-__device__ __forceinline__ void sincospi_r(float z, float* s, float* c) { sincospif(z, s, c); }
-__device__ __forceinline__ double tanh_r(double x) { return tanh(x); }
-__device__ __forceinline__ float tanh_r(float x) { return tanhf(x); }
-__device__ __forceinline__ double sqrt_r(double x) { return sqrt(x); }
-__device__ __forceinline__ float sqrt_r(float x) { return sqrtf(x); }
-__device__ __forceinline__ double rint_r(double x) { return rint(x); }
-__device__ __forceinline__ float rint_r(float x) { return rintf(x); }
-
-// Q_k(r) and dQ_k/dr for k < K at r < rc: Q_k = (T_k(x) + 1)/2 f_c(r),
-// x = 2(r/rc - 1)^2 - 1, f_c = (1 + cos(pi r/rc))/2 (Eqs. 12-15)
-template <class R>
-__device__ void basis64(R r, R rc, int K, R* f, R* fp) {
-    const R z = r / rc;
-    R sp, cp;
-    sincospi_r(z, &sp, &cp);
-    const R fc2 = R(0.25) * (R(1.0) + cp);                 // f_c / 2
-    const R dfc2 = R(-0.25) * R(kPi) / rc * sp;            // (d f_c/dr) / 2
-    const R t = z - R(1.0), x = R(2.0) * t * t - R(1.0), dx = R(4.0) * t / rc;
-    R Tm = R(1.0), Tk = x, dTm = R(0.0), dTk = R(1.0);
-    f[0] = R(2.0) * fc2;
-    fp[0] = R(2.0) * dfc2;
-    if (K > 1) {
-        f[1] = (x + R(1.0)) * fc2;
-        fp[1] = dx * fc2 + (x + R(1.0)) * dfc2;
-    }
-    for (int k = 2; k < K; ++k) {
-        const R Tn = R(2.0) * x * Tk - Tm;
-        const R dTn = R(2.0) * Tk + R(2.0) * x * dTk - dTm;
-        f[k] = (Tn + R(1.0)) * fc2;
-        fp[k] = dTn * dx * fc2 + (Tn + R(1.0)) * dfc2;
-        Tm = Tk; Tk = Tn; dTm = dTk; dTk = dTn;
-    }
-}
-
-// sum over the G aligned lanes of an atom; every lane receives the same bits.
-// The shuffles name only the group's lanes: a group whose atom index is past
-// N leaves as a whole, while the other groups of its warp go on.
-template <int G, class R>
-__device__ __forceinline__ R group_sum(R v) {
-    const unsigned mask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1)));
-#pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
-    return v;
-}
-
-template <class R>
-struct FrameT {
-    int i, ti, b;
-    R L[3], x, y, z;
-};
-using Frame64 = FrameT<double>;
-template <class A>
-__device__ FrameT<ScalarT<A>> frame64(const A& a, int i) {
-    FrameT<ScalarT<A>> fr;
-    fr.i = i;
-    fr.ti = a.type[i];
-    fr.b = a.cfg[i];
-    for (int c = 0; c < 3; ++c) fr.L[c] = a.box[3 * fr.b + c];
-    fr.x = a.pos[i];
-    fr.y = a.pos[a.N + i];
-    fr.z = a.pos[2 * a.N + i];
-    return fr;
-}
-
-// list slot s of atom fr.i: r_ij = (r_j - r_i) + s L in R, with the list's
-// image or the minimum image; false when r >= rc_rad
-template <class R>
-struct PairT {
-    int j, tj;
-    R d[3], r, u[3];
-};
-using Pair64 = PairT<double>;
-template <class A, class R>
-__device__ bool pair_at(const A& a, const FrameT<R>& fr, int s, PairT<R>& p) {
-    const int N = a.N;
-    p.j = a.nbr[(size_t)s * N + fr.i];
-    const R ux = (R)a.pos[p.j] - fr.x, uy = (R)a.pos[N + p.j] - fr.y, uz = (R)a.pos[2 * N + p.j] - fr.z;
-    R sx, sy, sz;
-    if (a.shift) {
-        int ix, iy, iz;
-        unpack_shift(a.shift[(size_t)s * N + fr.i], ix, iy, iz);
-        sx = (R)ix; sy = (R)iy; sz = (R)iz;
-    } else {
-        sx = -rint_r(ux / fr.L[0]);
-        sy = -rint_r(uy / fr.L[1]);
-        sz = -rint_r(uz / fr.L[2]);
-    }
-    p.d[0] = ux + sx * fr.L[0];
-    p.d[1] = uy + sy * fr.L[1];
-    p.d[2] = uz + sz * fr.L[2];
-    p.r = sqrt_r(p.d[0] * p.d[0] + p.d[1] * p.d[1] + p.d[2] * p.d[2]);
-    if (!(p.r < a.rc_rad)) return false;
-    p.tj = a.type[p.j];
-    const R ir = R(1.0) / p.r;
-    for (int c = 0; c < 3; ++c) p.u[c] = p.d[c] * ir;
-    return true;
-}
-
-// g_n = sum_k cA[ti][tj][n][k] Q_k (and g'_n with Q'_k)
-template <class A, class R>
-__device__ void angular_g(const A& a, int ti, int tj, const R* f, const R* fp, R* g, R* gp) {
-    const R* cA = a.prm + a.L.off_cA + (size_t)(ti * a.T + tj) * a.NA * a.KA;
-    for (int n = 0; n < a.NA; ++n) {
-        R u = R(0.0), v = R(0.0);
-        for (int k = 0; k < a.KA; ++k) {
-            u += cA[n * a.KA + k] * f[k];
-            v += cA[n * a.KA + k] * fp[k];
-        }
-        g[n] = u;
-        gp[n] = v;
-    }
-}
-
-// g_n only (the descriptors need no derivative)
-template <class A, class R>
-__device__ void angular_g_value(const A& a, int ti, int tj, const R* f, R* g) {
-    const R* cA = a.prm + a.L.off_cA + (size_t)(ti * a.T + tj) * a.NA * a.KA;
-    for (int n = 0; n < a.NA; ++n) {
-        R u = R(0.0);
-        for (int k = 0; k < a.KA; ++k) u += cA[n * a.KA + k] * f[k];
-        g[n] = u;
-    }
-}
-
-// q [D], S [NA*24] and the species-resolved radial basis sums F [T*KR] of
-// atom fr.i (the same values in every lane of its group)
-template <int G, class A, class R>
-__device__ void descriptors64(const A& a, const FrameT<R>& fr, int lane, R* q, R* S, R* F) {
-    const int T = a.T, NR = a.NR, NA = a.NA, KR = a.KR, KA = a.KA;
-    R f[kF64MaxK], fp[kF64MaxK], g[kF64MaxN];
-    for (int x = 0; x < T * KR; ++x) F[x] = R(0.0);
-    for (int x = 0; x < NA * kLM; ++x) S[x] = R(0.0);
-    const int nc = a.cnt[fr.i];
-    for (int s = lane; s < nc; s += G) {
-        PairT<R> p;
-        if (!pair_at(a, fr, s, p)) continue;
-        basis64(p.r, (R)a.rc_rad, KR, f, fp);
-        for (int k = 0; k < KR; ++k) F[p.tj * KR + k] += f[k];
-        if (!(p.r < a.rc_ang)) continue;
-        basis64(p.r, (R)a.rc_ang, KA, f, fp);
-        angular_g_value(a, fr.ti, p.tj, f, g);
-        const HarmTermsT<R> ht = harm_terms(p.u[0], p.u[1], p.u[2]);
-        for (int m = 0; m < kLM; ++m) {
-            R Y, gx, gy, gz;
-            harm_m(m, ht, Y, gx, gy, gz);
-            for (int n = 0; n < NA; ++n) S[n * kLM + m] += g[n] * Y;
-        }
-    }
-    for (int x = 0; x < T * KR; ++x) F[x] = group_sum<G>(F[x]);
-    for (int x = 0; x < NA * kLM; ++x) S[x] = group_sum<G>(S[x]);
-    // q_n = sum_t sum_k cR[ti][t][n][k] F[t][k]
-    const R* cR = a.prm + a.L.off_cR + (size_t)fr.ti * T * NR * KR;
-    for (int n = 0; n < NR; ++n) {
-        R v = R(0.0);
-        for (int t = 0; t < T; ++t)
-            for (int k = 0; k < KR; ++k) v += cR[(t * NR + n) * KR + k] * F[t * KR + k];
-        q[n] = v;
-    }
-    // q_nl = sum_m C_lm S_nlm^2 and q4_n = tr(A_n^3)
-    for (int n = 0; n < NA; ++n) {
-        for (int l = 0; l < 4; ++l) q[NR + n * 4 + l] = R(0.0);
-        for (int m = 0; m < kLM; ++m) {
-            const R v = S[n * kLM + m];
-            q[NR + n * 4 + lm_l(m) - 1] += (R)clm(m) * v * v;
-        }
-        if (a.H4) q[NR + NA * 4 + n] = fourbody<R>(S + n * kLM + 3, nullptr);
-    }
-}
 
 __global__ void k_promote(const float* src, double* dst, int n) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x < n) dst[x] = (double)src[x];
 }
 
-// ------------------------------------------------------------ evaluation
-// A warp's groups all belong to one block row; G divides 32 and kF64Block,
-// so no group straddles a warp.
-template <int G, class A>
-__global__ void __launch_bounds__(kF64Block) k64_atom(const A a) {
-    using R = ScalarT<A>;
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) / G;
-    const int lane = threadIdx.x % G;
-    if (i >= a.N) return;
-    const int N = a.N, NR = a.NR, NA = a.NA, H = a.H, D = a.D;
-    const FrameT<R> fr = frame64(a, i);
-    R q[kF64MaxD], S[kF64MaxN * kLM], F[kF64MaxTK];
-    descriptors64<G>(a, fr, lane, q, S, F);
-    // network: E_i = w1 . tanh(W0 q + b0) + b1, dE/dq = W0^T (w1 (1 - t^2));
-    // lane takes hidden units h = lane, lane + G, ...
-    const R* W0 = a.prm + (size_t)fr.ti * a.L.mlp_stride;
+// Radial sums F and S_nlm of atom fr.i into the group's block; lane keeps
+// S[n][x] of harmonic lane + x G.  NAX bounds n_ang.
+template <int G, class DM, class A, class R>
+__device__ void group64_sums(const A& a, const Group64<G>& o, R* gb, const FrameT<R>& fr, int nc, int lane,
+                             R (&S)[DM::NAX][Group64<G>::MPL]) {
+    constexpr int NAX = DM::NAX;
+    constexpr int GS = Group64<G>::GS, MPL = Group64<G>::MPL, KW = Group64<G>::KW, KX = Group64<G>::KX;
+    constexpr int PARTS = Group64<G>::PARTS;
+    const int NA = DM::NA(a), KR = DM::KR(a), KA = DM::KA(a);
+    const R irR = R(1.0) / (R)a.rc_rad, irA = R(1.0) / (R)a.rc_ang;
+    int* tj = reinterpret_cast<int*>(gb + o.oT);
+    const int gbase = (threadIdx.x & 31) & ~(G - 1);
+    const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u), below = (1u << lane) - 1u;
+    const int kl = lane % KW, part = lane / KW;
+    R F[KX][kMaxTypes];
+#pragma unroll
+    for (int x = 0; x < KX; ++x)
+#pragma unroll
+        for (int t = 0; t < kMaxTypes; ++t) F[x][t] = R(0.0);
+#pragma unroll
+    for (int n = 0; n < NAX; ++n)
+#pragma unroll
+        for (int x = 0; x < MPL; ++x) S[n][x] = R(0.0);
+    const int cmax = warp_max_i(nc);
+    for (int s0 = 0; s0 < cmax; s0 += G) {
+        const int s = s0 + lane;
+        PairT<R> p;
+        const bool in = s < nc && pair_at(a, fr, s, p);
+        const unsigned mi = (__ballot_sync(0xffffffffu, in) >> gbase) & gmask;
+        const int ni = __popc(mi), ati = __popc(mi & below);
+        if (in) {
+            tj[ati] = p.tj;
+            basis_values<DM::KX>(p.r, irR, KR, [&](int k, R f) { gb[o.oY + k * GS + ati] = f; });
+        }
+        __syncwarp();
+        for (int q = part; q < ni; q += PARTS) {
+            const int t = tj[q];
+#pragma unroll
+            for (int x = 0; x < KX; ++x) {
+                const int k = kl + x * KW;
+                if (k >= KR) continue;
+                const R f = gb[o.oY + k * GS + q];
+#pragma unroll
+                for (int u = 0; u < kMaxTypes; ++u)
+                    if (t == u) F[x][u] += f;
+            }
+        }
+        __syncwarp();
+        const bool ang = in && p.r < (R)a.rc_ang;
+        const unsigned any = __ballot_sync(0xffffffffu, ang);
+        if (!any) continue;
+        const unsigned ma = (any >> gbase) & gmask;
+        const int na = __popc(ma), at = __popc(ma & below);
+        if (ang) {
+            R f[DM::KX];
+            basis_values<DM::KX>(p.r, irA, KA, [&](int k, R v) { f[k] = v; });
+            const R* c = a.prm + a.L.off_cA + (size_t)(fr.ti * a.T + p.tj) * NA * KA;
+#pragma unroll
+            for (int n = 0; n < NAX; ++n) {
+                if (n >= NA) break;
+                R g = R(0.0);
+#pragma unroll
+                for (int k = 0; k < DM::KX; ++k)
+                    if (k < KA) g += c[n * KA + k] * f[k];
+                gb[o.oG + at * o.NAs + n] = g;
+            }
+            const Harm<R> ht = harm_of(p.u[0], p.u[1], p.u[2]);
+#pragma unroll
+            for (int m = 0; m < kLM; ++m) gb[o.oY + m * GS + at] = harm_value(m, ht);
+        }
+        __syncwarp();
+        for (int q = 0; q < na; ++q) {
+#pragma unroll
+            for (int x = 0; x < MPL; ++x) {
+                const int m = lane + x * G;
+                if (m >= kLM) continue;
+                const R Y = gb[o.oY + m * GS + q];
+#pragma unroll
+                for (int n = 0; n < NAX; ++n)
+                    if (n < NA) S[n][x] += gb[o.oG + q * o.NAs + n] * Y;
+            }
+        }
+        __syncwarp();
+    }
+#pragma unroll
+    for (int x = 0; x < KX; ++x)
+#pragma unroll
+        for (int t = 0; t < kMaxTypes; ++t) {
+            R v = F[x][t];
+#pragma unroll
+            for (int h = KW; h < G; h <<= 1) v += __shfl_xor_sync(0xffffffffu, v, h);
+            if (part == 0 && kl + x * KW < KR && t < a.T) gb[o.oF + t * KR + kl + x * KW] = v;
+        }
+#pragma unroll
+    for (int n = 0; n < NAX; ++n)
+#pragma unroll
+        for (int x = 0; x < MPL; ++x)
+            if (n < NA && lane + x * G < kLM) gb[o.oS + n * kLM + lane + x * G] = S[n][x];
+    __syncwarp();
+}
+
+// q and the 4-body gradients J, then E_i (returned in every lane) and
+// p = dE/dq, in the group's block
+template <int G, class A, class R>
+__device__ R group64_network(const A& a, const Group64<G>& o, R* gb, int ti, int lane) {
+    const int T = a.T, NR = a.NR, NA = a.NA, KR = a.KR, H = a.H, D = a.D;
+    const R* cR = a.prm + a.L.off_cR + (size_t)ti * T * NR * KR;
+    for (int n = lane; n < NR; n += G) {
+        R v = R(0.0);
+        for (int t = 0; t < T; ++t)
+            for (int k = 0; k < KR; ++k) v += cR[(t * NR + n) * KR + k] * gb[o.oF + t * KR + k];
+        gb[o.oQ + n] = v;
+    }
+    for (int x = lane; x < NA * 4; x += G) {
+        const int n = x >> 2, l = x & 3, m0 = l * (l + 2);
+        R v = R(0.0);
+        for (int m = m0; m < m0 + 2 * l + 3; ++m) {
+            const R s = gb[o.oS + n * kLM + m];
+            v += (R)clm(m) * s * s;
+        }
+        gb[o.oQ + NR + x] = v;
+    }
+    if (a.H4)
+        for (int n = lane; n < NA; n += G) gb[o.oQ + NR + NA * 4 + n] = fourbody<R>(gb + o.oS + n * kLM + 3, gb + o.oJ + 5 * n);
+    for (int d = lane; d < D; d += G) gb[o.oP + d] = R(0.0);
+    __syncwarp();
+    const R* W0 = a.prm + (size_t)ti * a.L.mlp_stride;
     const R* b0 = W0 + (size_t)H * D;
     const R* w1 = b0 + H;
-    R E = R(0.0), pq[kF64MaxD];
-    for (int d = 0; d < D; ++d) pq[d] = R(0.0);
-    for (int h = lane; h < H; h += G) {
-        const R* w = W0 + (size_t)h * D;
-        R z = b0[h];
-        for (int d = 0; d < D; ++d) z += w[d] * q[d];
-        const R th = tanh_r(z);
-        E += w1[h] * th;
-        const R c = w1[h] * (R(1.0) - th * th);
-        for (int d = 0; d < D; ++d) pq[d] += c * w[d];
-    }
-    E = group_sum<G>(E) + w1[H];
-    for (int d = 0; d < D; ++d) pq[d] = group_sum<G>(pq[d]);
-    if (lane == 0) a.e[i] = E;
-    for (int n = lane; n < NR; n += G) a.p[(size_t)n * N + i] = pq[n];
-    // R_nlm = dE/dq_nl 2 C_lm S_nlm (+ dE/dq4_n dq4_n/dS_n2m), entries split over lanes
-    for (int x = lane; x < NA * kLM; x += G) {
-        const int n = x / kLM, m = x % kLM;
-        R v = R(2.0) * (R)clm(m) * pq[NR + n * 4 + lm_l(m) - 1] * S[x];
-        if (a.H4 && m >= 3 && m < 8) {
-            R J[5];
-            fourbody<R>(S + n * kLM + 3, J);
-            v += pq[NR + NA * 4 + n] * J[m - 3];
+    R E = R(0.0);
+    for (int h0 = 0; h0 < H; h0 += kGroupTile) {
+        const int nh = min(kGroupTile, H - h0);
+        for (int h = lane; h < nh; h += G) {
+            const R* w = W0 + (size_t)(h0 + h) * D;
+            R z0 = b0[h0 + h], z1 = R(0.0);
+            int d = 0;
+            for (; d + 1 < D; d += 2) {
+                z0 += w[d] * gb[o.oQ + d];
+                z1 += w[d + 1] * gb[o.oQ + d + 1];
+            }
+            if (d < D) z0 += w[d] * gb[o.oQ + d];
+            const R th = tanh_r(z0 + z1), wh = w1[h0 + h];
+            E += wh * th;
+            gb[o.oSg + h] = wh * (R(1.0) - th * th);
         }
-        a.R[(size_t)x * N + i] = v;
+        __syncwarp();
+        for (int d = lane; d < D; d += G) {
+            const R* w = W0 + (size_t)h0 * D + d;
+            R p0 = gb[o.oP + d], p1 = R(0.0);
+            int h = 0;
+            for (; h + 1 < nh; h += 2) {
+                p0 += gb[o.oSg + h] * w[(size_t)h * D];
+                p1 += gb[o.oSg + h + 1] * w[(size_t)(h + 1) * D];
+            }
+            if (h < nh) p0 += gb[o.oSg + h] * w[(size_t)h * D];
+            gb[o.oP + d] = p0 + p1;
+        }
+        __syncwarp();
+    }
+#pragma unroll
+    for (int h = G / 2; h > 0; h >>= 1) E += __shfl_xor_sync(0xffffffffu, E, h);
+    return E + w1[H];
+}
+
+// g_n = sum_k c[n][k] Q_k and g'_n with Q'_k, c = cA[ti][tj]
+template <class DM, class A, class R>
+__device__ __forceinline__ void angular_g(const A& a, int ti, int tj, R r, R irA, int NA, int KA, R* g, R* gp) {
+    R f[DM::KX], fp[DM::KX];
+    basis_derivs<DM::KX>(r, irA, KA, [&](int k, R v, R d) {
+        f[k] = v;
+        fp[k] = d;
+    });
+    const R* c = a.prm + a.L.off_cA + (size_t)(ti * a.T + tj) * NA * KA;
+#pragma unroll
+    for (int n = 0; n < DM::NAX; ++n) {
+        g[n] = gp[n] = R(0.0);
+        if (n >= NA) continue;
+#pragma unroll
+        for (int k = 0; k < DM::KX; ++k)
+            if (k < KA) {
+                g[n] += c[n * KA + k] * f[k];
+                gp[n] += c[n * KA + k] * fp[k];
+            }
     }
 }
 
-// dE_o/dr_oj for owner o of species to, neighbour species tn, distance r and
-// unit vector u = r_oj / r
-template <class A, class R>
-__device__ void pair_deriv(const A& a, int o, int to, int tn, R r, const R* u, R* fo) {
-    const int N = a.N, T = a.T, NR = a.NR, NA = a.NA, KR = a.KR, KA = a.KA;
-    R f[kF64MaxK], fp[kF64MaxK], g[kF64MaxN], gp[kF64MaxN];
-    basis64(r, (R)a.rc_rad, KR, f, fp);
-    const R* cR = a.prm + a.L.off_cR + (size_t)(to * T + tn) * NR * KR;
-    R gr = R(0.0);
-    for (int n = 0; n < NR; ++n) {
-        R dg = R(0.0);
-        for (int k = 0; k < KR; ++k) dg += cR[n * KR + k] * fp[k];
-        gr += a.p[(size_t)n * N + o] * dg;
-    }
-    fo[0] = gr * u[0];
-    fo[1] = gr * u[1];
-    fo[2] = gr * u[2];
-    if (!(r < a.rc_ang)) return;
-    basis64(r, (R)a.rc_ang, KA, f, fp);
-    angular_g(a, to, tn, f, fp, g, gp);
-    const HarmTermsT<R> ht = harm_terms(u[0], u[1], u[2]);
-    R Y[kLM], Gr[kLM][3];
-    for (int m = 0; m < kLM; ++m) harm_m(m, ht, Y[m], Gr[m][0], Gr[m][1], Gr[m][2]);
-    const R ir = R(1.0) / r;
-    for (int n = 0; n < NA; ++n) {
-        // d S_nlm / d r_oj = g'_n Y_m u + g_n (grad P_m - l P_m u) / r
-        R sY = R(0.0), slY = R(0.0), sg[3] = {R(0.0), R(0.0), R(0.0)};
-        for (int m = 0; m < kLM; ++m) {
-            const R Rv = a.R[(size_t)(n * kLM + m) * N + o];
-            sY += Rv * Y[m];
-            slY += Rv * (R)lm_l(m) * Y[m];
-            sg[0] += Rv * Gr[m][0];
-            sg[1] += Rv * Gr[m][1];
-            sg[2] += Rv * Gr[m][2];
-        }
-        for (int c = 0; c < 3; ++c) fo[c] += gp[n] * sY * u[c] + g[n] * ir * (sg[c] - slY * u[c]);
+// the same for both orders of the pair: (g, g') from cA[ti][tj], (h, h') from cA[tj][ti]
+template <class DM, class A, class R>
+__device__ __forceinline__ void angular_g2(const A& a, int ti, int tj, R r, R irA, int NA, int KA, R* g, R* gp, R* h,
+                                           R* hp) {
+    R f[DM::KX], fp[DM::KX];
+    basis_derivs<DM::KX>(r, irA, KA, [&](int k, R v, R d) {
+        f[k] = v;
+        fp[k] = d;
+    });
+    const R* cij = a.prm + a.L.off_cA + (size_t)(ti * a.T + tj) * NA * KA;
+    const R* cji = a.prm + a.L.off_cA + (size_t)(tj * a.T + ti) * NA * KA;
+#pragma unroll
+    for (int n = 0; n < DM::NAX; ++n) {
+        g[n] = gp[n] = h[n] = hp[n] = R(0.0);
+        if (n >= NA) continue;
+#pragma unroll
+        for (int k = 0; k < DM::KX; ++k)
+            if (k < KA) {
+                g[n] += cij[n * KA + k] * f[k];
+                gp[n] += cij[n * KA + k] * fp[k];
+                h[n] += cji[n * KA + k] * f[k];
+                hp[n] += cji[n * KA + k] * fp[k];
+            }
     }
 }
 
-template <int G, class A>
-__global__ void __launch_bounds__(kF64Block) k64_force(const A a) {
+// a group's sums of an atom's force and virial, acc = (F, W), to memory
+template <int G, class A, class R>
+__device__ __forceinline__ void group_store(const A& a, const R* acc, int i, int lane, bool valid) {
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+        R v = acc[c];
+#pragma unroll
+        for (int h = G / 2; h > 0; h >>= 1) v += __shfl_xor_sync(0xffffffffu, v, h);
+        if (valid && lane == c % G) {
+            if (c < 3) a.force[(size_t)c * a.N + i] = v;
+            else a.w[(size_t)(c - 3) * a.N + i] = v;
+        }
+    }
+}
+
+template <int G, class DM, class A>
+__global__ void __launch_bounds__(kF64Threads) k64_atom(const A a) {
+    constexpr int NAX = DM::NAX;
     using R = ScalarT<A>;
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) / G;
-    const int lane = threadIdx.x % G;
-    if (i >= a.N) return;
-    const int N = a.N;
+    extern __shared__ double smem64[];
+    const Group64<G> o(a.T, a.NA, a.KR, a.D);
+    const int lane = threadIdx.x % G, group = threadIdx.x / G;
+    R* gb = reinterpret_cast<R*>(smem64) + group * o.size;
+    const int ia = blockIdx.x * Group64<G>::NG + group, N = a.N;
+    const bool valid = ia < N;
+    const int i = valid ? ia : N - 1;
     const FrameT<R> fr = frame64(a, i);
-    R F[3] = {R(0.0), R(0.0), R(0.0)}, W[9];
-    for (int c = 0; c < 9; ++c) W[c] = R(0.0);
-    const int nc = a.cnt[i];
-    for (int s = lane; s < nc; s += G) {
-        PairT<R> p;
-        if (!pair_at(a, fr, s, p)) continue;
-        const R v[3] = {-p.u[0], -p.u[1], -p.u[2]};
-        R fij[3], fji[3];
-        pair_deriv(a, i, fr.ti, p.tj, p.r, p.u, fij);
-        pair_deriv(a, p.j, p.tj, fr.ti, p.r, v, fji);
-        for (int c = 0; c < 3; ++c) F[c] += fij[c] - fji[c];
-        for (int x = 0; x < 3; ++x)
-            for (int y = 0; y < 3; ++y) W[3 * x + y] -= fij[x] * p.d[y];
+    R S[NAX][Group64<G>::MPL];
+    group64_sums<G, DM>(a, o, gb, fr, valid ? a.cnt[i] : 0, lane, S);
+    const R E = group64_network<G>(a, o, gb, fr.ti, lane);
+    const int T = a.T, NR = a.NR, NA = DM::NA(a), KR = DM::KR(a);
+    if (valid && lane == 0) a.e[i] = E;
+    // P[t][k] = sum_n p_n cR[ti][t][n][k], the radial adjoint of a neighbour of species t
+    const R* cR = a.prm + a.L.off_cR + (size_t)fr.ti * T * NR * KR;
+    for (int x = lane; x < T * KR; x += G) {
+        R v = R(0.0);
+        for (int n = 0; n < NR; ++n) v += gb[o.oP + n] * cR[((x / KR) * NR + n) * KR + x % KR];
+        if (valid) a.p[(size_t)i * T * KR + x] = v;
     }
-    for (int c = 0; c < 3; ++c) F[c] = group_sum<G>(F[c]);
-    for (int c = 0; c < 9; ++c) W[c] = group_sum<G>(W[c]);
-    for (int c = lane; c < 3; c += G) a.force[(size_t)c * N + i] = F[c];
-    for (int c = lane; c < 9; c += G) a.w[(size_t)c * N + i] = W[c];
+    // R_nlm = dE/dq_nl 2 C_lm S_nlm (+ dE/dq4_n dq4_n/dS_n2m)
+#pragma unroll
+    for (int x = 0; x < Group64<G>::MPL; ++x) {
+        const int m = lane + x * G;
+        if (m >= kLM) continue;
+        const int l = lm_l(m);
+        const R c2 = R(2.0) * (R)clm(m);
+#pragma unroll
+        for (int n = 0; n < NAX; ++n) {
+            if (n >= NA) continue;
+            R v = c2 * gb[o.oP + NR + n * 4 + l - 1] * S[n][x];
+            if (a.H4 && l == 2) v += gb[o.oP + NR + NA * 4 + n] * gb[o.oJ + 5 * n + m - 3];
+            if constexpr (kScatter<A>) gb[o.oS + n * kLM + m] = v;
+            else if (valid) a.R[((size_t)i * NA + n) * kLM + m] = v;
+        }
+    }
+    if constexpr (kScatter<A>) {
+        // the owner's angular pair forces, and each pair's to its reverse slot
+        __syncwarp();
+        const R* Ri = gb + o.oS;
+        const R irA = R(1.0) / (R)a.rc_ang;
+        const int KA = DM::KA(a);
+        R acc[12];
+#pragma unroll
+        for (int c = 0; c < 12; ++c) acc[c] = R(0.0);
+        const int na = valid ? a.cnt_ang[i] : 0;
+        for (int s = lane; s < na; s += G) {
+            PairT<R> p;
+            if (!pair_at(a, fr, s, p) || !(p.r < (R)a.rc_ang)) continue;
+            R g[NAX], gp[NAX];
+            angular_g<DM>(a, fr.ti, p.tj, p.r, irA, NA, KA, g, gp);
+            const Harm<R> ht = harm_of(p.u[0], p.u[1], p.u[2]);
+            HarmSums<R> hs(ht);
+#pragma unroll
+            for (int m = 0; m < kLM; ++m) {
+                R am = R(0.0), bm = R(0.0);
+#pragma unroll
+                for (int n = 0; n < NAX; ++n)
+                    if (n < NA) {
+                        const R r = Ri[n * kLM + m];
+                        am += r * g[n];
+                        bm += r * gp[n];
+                    }
+                hs.add(m, ht, am, bm);
+            }
+            R f[3];
+            hs.force(ht, p.ir, f[0], f[1], f[2]);
+            a.fin[(size_t)a.rev[(size_t)s * N + i] * N + p.j] = make_float4(f[0], f[1], f[2], 0.0f);
+            for (int c = 0; c < 3; ++c) {
+                acc[c] += f[c];
+                for (int d = 0; d < 3; ++d) acc[3 + 3 * c + d] -= f[c] * p.d[d];
+            }
+        }
+        __syncwarp();
+        group_store<G>(a, acc, i, lane, valid);
+    }
+}
+
+// F_i and the per-atom virial.
+//
+// Generic path (kScatter): the radial pair forces of both directions from the
+// projected adjoints, and the incoming angular forces of the reverse slots,
+// are added to what k64_atom left; W_i = -sum_j f_ij (x) r_ij.
+//
+// FP64: dE_i/dr_ij and dE_j/dr_ji, both from both atoms' adjoints.  Seen from
+// j the direction is -u, and the harmonics of degree l have parity (-1)^l, so
+// j's coefficients join i's before the harmonics:
+//   f_ij =          u sum_m b_m Y_m + (1/r) (1 - u u^T) sum_m a_m grad P_m
+//   f_ji = - (-1)^l (the same with j's a, b).
+// Each atom gets half of a pair's virial, -(f_ij - f_ji) (x) r_ij / 2, which
+// sums to the same totals.  The angular pairs' slots are collected in the
+// radial walk, so that the lanes of the angular one, which takes most of the
+// time, are all busy.
+constexpr int kF64Slots = 128;       // per atom; with more the list is walked again
+template <int G, class DM, class A>
+__global__ void __launch_bounds__(kF64Threads) k64_force(const A a) {
+    using R = ScalarT<A>;
+    constexpr int NAX = DM::NAX;
+    extern __shared__ double smem64[];
+    const int lane = threadIdx.x % G, group = threadIdx.x / G;
+    const int T = a.T, NA = DM::NA(a), KR = DM::KR(a), N = a.N;
+    constexpr int kSlotR = kScatter<A> ? 0 : kF64Slots * (int)sizeof(unsigned short) / (int)sizeof(R);
+    const int own = kScatter<A> ? 0 : NA * kLM;
+    R* Ri = reinterpret_cast<R*>(smem64) + group * (own + T * KR + kSlotR);
+    R* Pi = Ri + own;
+    unsigned short* slots = reinterpret_cast<unsigned short*>(Pi + T * KR);
+    const int ia = blockIdx.x * Group64<G>::NG + group;
+    const bool valid = ia < N;
+    const int i = valid ? ia : N - 1;
+    const FrameT<R> fr = frame64(a, i);
+    if constexpr (!kScatter<A>)
+        for (int x = lane; x < own; x += G) Ri[x] = a.R[(size_t)i * own + x];
+    for (int x = lane; x < T * KR; x += G) Pi[x] = a.p[(size_t)i * T * KR + x];
+    __syncwarp();
+    const R irR = R(1.0) / (R)a.rc_rad;
+    R acc[12];
+#pragma unroll
+    for (int c = 0; c < 12; ++c) acc[c] = R(0.0);
+    const int nc = valid ? a.cnt[i] : 0, cmax = warp_max_i(nc);
+    const int gbase = (threadIdx.x & 31) & ~(G - 1);
+    const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u), below = (1u << lane) - 1u;
+    int na = 0;                          // generic: the list's angular prefix; FP64: pairs inside rc_ang so far
+    if constexpr (kScatter<A>)
+        if (valid) na = a.cnt_ang[i];
+    for (int s0 = 0; s0 < cmax; s0 += G) {
+        const int s = s0 + lane;
+        PairT<R> p;
+        const bool in = s < nc && pair_at(a, fr, s, p);
+        bool ang = false;
+        if (in) {
+            ang = p.r < (R)a.rc_ang;
+            const R* pi = Pi + p.tj * KR;
+            const R* pj = a.p + ((size_t)p.j * T + fr.ti) * KR;
+            R di = R(0.0), dj = R(0.0);
+            basis_derivs<DM::KX>(p.r, irR, KR, [&](int k, R, R fp) {
+                di += pi[k] * fp;
+                dj += pj[k] * fp;
+            });
+            const R all = di + dj, vir = kScatter<A> ? di : R(0.5) * all;
+            for (int c = 0; c < 3; ++c) {
+                acc[c] += all * p.u[c];
+                for (int d = 0; d < 3; ++d) acc[3 + 3 * c + d] -= vir * p.u[c] * p.d[d];
+            }
+            if constexpr (kScatter<A>) {
+                if (ang && s < na) {
+                    const float4 g = a.fin[(size_t)s * N + i];
+                    acc[0] -= g.x;
+                    acc[1] -= g.y;
+                    acc[2] -= g.z;
+                }
+            }
+        }
+        if constexpr (!kScatter<A>) {
+            const unsigned m = (__ballot_sync(0xffffffffu, ang) >> gbase) & gmask;
+            const int at = na + __popc(m & below);
+            if (ang && at < kF64Slots) slots[at] = (unsigned short)s;
+            na += __popc(m);
+        }
+    }
+    __syncwarp();
+    if constexpr (!kScatter<A>) {
+        const R irA = R(1.0) / (R)a.rc_ang;
+        const int KA = DM::KA(a);
+        const bool kept = na <= kF64Slots && nc <= 65536;
+        const int n2 = kept ? na : nc;
+        for (int c2 = lane; c2 < n2; c2 += G) {
+            PairT<R> p;
+            if (!pair_at(a, fr, kept ? (int)slots[c2] : c2, p) || !(p.r < (R)a.rc_ang)) continue;
+            R g[NAX], gp[NAX], h[NAX], hp[NAX];
+            angular_g2<DM>(a, fr.ti, p.tj, p.r, irA, NA, KA, g, gp, h, hp);
+            const Harm<R> ht = harm_of(p.u[0], p.u[1], p.u[2]);
+            const R* Rj = a.R + (size_t)p.j * NA * kLM;
+            HarmSums<R> hs(ht);
+#pragma unroll
+            for (int m = 0; m < kLM; ++m) {
+                // j's coefficients with the parity (-1)^l
+                R am = R(0.0), bm = R(0.0);
+#pragma unroll
+                for (int n = 0; n < NAX; ++n)
+                    if (n < NA) {
+                        const R rj = Rj[n * kLM + m];
+                        am += rj * h[n];
+                        bm += rj * hp[n];
+                    }
+                if (lm_l(m) & 1) {
+                    am = -am;
+                    bm = -bm;
+                }
+#pragma unroll
+                for (int n = 0; n < NAX; ++n)
+                    if (n < NA) {
+                        const R ri = Ri[n * kLM + m];
+                        am += ri * g[n];
+                        bm += ri * gp[n];
+                    }
+                hs.add(m, ht, am, bm);
+            }
+            R f[3];
+            hs.force(ht, p.ir, f[0], f[1], f[2]);
+            for (int c = 0; c < 3; ++c) {
+                acc[c] += f[c];
+                for (int d = 0; d < 3; ++d) acc[3 + 3 * c + d] -= R(0.5) * f[c] * p.d[d];
+            }
+        }
+        __syncwarp();
+    }
+    if constexpr (kScatter<A>) {
+        // on top of the owner's angular part
+#pragma unroll
+        for (int c = 0; c < 12; ++c)
+            if (valid && lane == c % G) acc[c] += c < 3 ? a.force[(size_t)c * N + i] : a.w[(size_t)(c - 3) * N + i];
+    }
+    group_store<G>(a, acc, i, lane, valid);
 }
 
 __device__ int segment_of(const int* off, int B, int x) {
@@ -365,9 +477,7 @@ __device__ int segment_of(const int* off, int B, int x) {
     return lo;
 }
 
-// FP64 sums of E_i and W_i per 1,024-atom chunk: strided per-thread sums,
-// then warp shuffles and the warp sums in order; atoms from n_owned on are
-// left out (the owned prefix of a spatial decomposition's local system)
+// sum over a block: warp shuffles, then the warp sums in order
 constexpr int kF64Red = 256;
 __device__ double block_sum(double v, double* red) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -380,24 +490,53 @@ __device__ double block_sum(double v, double* red) {
     return s;
 }
 
+// E and virial of every configuration: one CTA per chunk, a warp per
+// component, FP64 sums in a fixed order; the CTA that finishes a
+// configuration's last chunk adds the chunks' partials (as k_totals).  Atoms
+// from n_owned on are left out (the owned prefix of a spatial decomposition).
 template <class A>
-__global__ void __launch_bounds__(kF64Red) k64_chunk_reduce(const A a) {
-    const int k = blockIdx.x, B = a.B, N = a.N;
-    if (k >= a.chunk_start[B]) return;
+__global__ void __launch_bounds__(320) k64_totals(const A a, double* e_tot, double* virial) {
+    const int k = blockIdx.x, B = a.B, N = a.N, total = a.chunk_start[B];
+    const int lane = threadIdx.x & 31, c = threadIdx.x >> 5;
+    auto put = [&](int b, double v) {
+        if (lane) return;
+        if (c == 0) {
+            if (e_tot) e_tot[b] = v;
+        } else if (virial) {
+            virial[(size_t)b * 9 + c - 1] = v;
+        }
+    };
+    if (k >= total) {                   // configurations without atoms
+        for (int b = k - total; b < B; b += gridDim.x - total)
+            if (a.chunk_start[b] == a.chunk_start[b + 1]) put(b, 0.0);
+        return;
+    }
     const int b = segment_of(a.chunk_start, B, k);
-    const int a0 = a.atom_off[b] + (k - a.chunk_start[b]) * kChunk;
+    const int k0 = a.chunk_start[b], nk = a.chunk_start[b + 1] - k0;
+    const int a0 = a.atom_off[b] + (k - k0) * kChunk;
     const int a1 = min(min(a.atom_off[b + 1], a0 + kChunk), a.n_owned);
-    double acc[10];
-    for (int c = 0; c < 10; ++c) acc[c] = 0.0;
-    for (int i = a0 + threadIdx.x; i < a1; i += kF64Red) {
-        acc[0] += (double)a.e[i];
-        for (int c = 0; c < 9; ++c) acc[1 + c] += (double)a.w[(size_t)c * N + i];
+    const ScalarT<A>* src = c == 0 ? a.e : a.w + (size_t)(c - 1) * N;
+    double v = 0.0;
+#pragma unroll 4
+    for (int i = a0 + lane; i < a1; i += 32) v += (double)src[i];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (nk > 1) {
+        if (lane == 0) {
+            a.partial[(size_t)k * 10 + c] = v;
+            __threadfence();
+        }
+        __shared__ int last;
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(a.ticket + b, 1) == nk - 1;
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        if (threadIdx.x == 0) a.ticket[b] = 0;
+        v = 0.0;
+        for (int q = lane; q < nk; q += 32) v += __ldcg(a.partial + (size_t)(k0 + q) * 10 + c);
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     }
-    __shared__ double red[kF64Red / 32];
-    for (int c = 0; c < 10; ++c) {
-        const double v = block_sum(acc[c], red);
-        if (threadIdx.x == 0) a.partial[(size_t)k * 10 + c] = v;
-    }
+    put(b, v);
 }
 
 // ------------------------------------------------------------ loss
@@ -456,399 +595,7 @@ __global__ void __launch_bounds__(kF64Red) k64_loss_cfg(const F64Args a, const d
     if (threadIdx.x == 0 && loss) *loss = v / B;
 }
 
-// ------------------------------------------------------------ gradient
-// Staged per-atom factors, [field][N]: q, dq (D each), alpha, beta, gamma
-// (H each), rho and p of the radial n (NR each), F and DF (T KR each), and
-// bins (T NA KA).
-struct GradFields {
-    int q, dq, al, be, ga, rho, p, F, DF, bins, total;
-};
-__host__ __device__ GradFields grad_fields(const F64Args& a) {
-    GradFields g;
-    g.q = 0;
-    g.dq = g.q + a.D;
-    g.al = g.dq + a.D;
-    g.be = g.al + a.H;
-    g.ga = g.be + a.H;
-    g.rho = g.ga + a.H;
-    g.p = g.rho + a.NR;
-    g.F = g.p + a.NR;
-    g.DF = g.F + a.T * a.KR;
-    g.bins = g.DF + a.T * a.KR;
-    g.total = g.bins + a.T * a.NA * a.KA;
-    return g;
-}
-
-// dr_ij = -(lam_j - lam_i) - mu r_ij
-__device__ void tangent64(const F64Args& a, const double* li, const double* mu, const Pair64& p, double* dr) {
-    const int N = a.N;
-    for (int c = 0; c < 3; ++c)
-        dr[c] = -(a.lam[(size_t)c * N + p.j] - li[c]) -
-                (mu[3 * c] * p.d[0] + mu[3 * c + 1] * p.d[1] + mu[3 * c + 2] * p.d[2]);
-}
-
-template <int G>
-__global__ void __launch_bounds__(kF64Block) k64_grad_atom(const F64Args a) {
-    const int i = (blockIdx.x * blockDim.x + threadIdx.x) / G;
-    const int lane = threadIdx.x % G;
-    if (i >= a.N) return;
-    const int N = a.N, T = a.T, NR = a.NR, NA = a.NA, KR = a.KR, KA = a.KA, H = a.H, D = a.D;
-    const GradFields gf = grad_fields(a);
-    const Frame64 fr = frame64(a, i);
-    double q[kF64MaxD], S[kF64MaxN * kLM], F[kF64MaxTK];
-    descriptors64<G>(a, fr, lane, q, S, F);
-    const double li[3] = {a.lam[i], a.lam[N + i], a.lam[2 * N + i]};
-    const double* mu = a.mu + 9 * fr.b;
-    const double aE = a.aE[fr.b];
-    double f[kF64MaxK], fp[kF64MaxK], g[kF64MaxN], gp[kF64MaxN];
-
-    // tangent along dr: DF[t][k] = sum_{j of t} Q'_k (rhat . dr) and
-    // dS_nlm = sum_j [g'_n (rhat . dr) Y_m + g_n (grad P_m . dr - l Y_m rhat . dr) / r]
-    double DF[kF64MaxTK], dS[kF64MaxN * kLM];
-    for (int x = 0; x < T * KR; ++x) DF[x] = 0.0;
-    for (int x = 0; x < NA * kLM; ++x) dS[x] = 0.0;
-    const int nc = a.cnt[i];
-    for (int s = lane; s < nc; s += G) {
-        Pair64 p;
-        if (!pair_at(a, fr, s, p)) continue;
-        double dr[3];
-        tangent64(a, li, mu, p, dr);
-        const double udr = p.u[0] * dr[0] + p.u[1] * dr[1] + p.u[2] * dr[2];
-        basis64(p.r, a.rc_rad, KR, f, fp);
-        for (int k = 0; k < KR; ++k) DF[p.tj * KR + k] += fp[k] * udr;
-        if (!(p.r < a.rc_ang)) continue;
-        basis64(p.r, a.rc_ang, KA, f, fp);
-        angular_g(a, fr.ti, p.tj, f, fp, g, gp);
-        const HarmTermsT<double> ht = harm_terms(p.u[0], p.u[1], p.u[2]);
-        const double ir = 1.0 / p.r;
-        for (int m = 0; m < kLM; ++m) {
-            double Y, gx, gy, gz;
-            harm_m(m, ht, Y, gx, gy, gz);
-            const double dY = (gx * dr[0] + gy * dr[1] + gz * dr[2] - lm_l(m) * Y * udr) * ir;
-            for (int n = 0; n < NA; ++n) dS[n * kLM + m] += gp[n] * udr * Y + g[n] * dY;
-        }
-    }
-    for (int x = 0; x < T * KR; ++x) DF[x] = group_sum<G>(DF[x]);
-    for (int x = 0; x < NA * kLM; ++x) dS[x] = group_sum<G>(dS[x]);
-    // dq: radial from DF, angular from S and dS
-    double dq[kF64MaxD];
-    const double* cR = a.prm + a.L.off_cR + (size_t)fr.ti * T * NR * KR;
-    for (int n = 0; n < NR; ++n) {
-        double v = 0.0;
-        for (int t = 0; t < T; ++t)
-            for (int k = 0; k < KR; ++k) v += cR[(t * NR + n) * KR + k] * DF[t * KR + k];
-        dq[n] = v;
-    }
-    for (int n = 0; n < NA; ++n) {
-        for (int l = 0; l < 4; ++l) dq[NR + n * 4 + l] = 0.0;
-        for (int m = 0; m < kLM; ++m)
-            dq[NR + n * 4 + lm_l(m) - 1] += 2.0 * (double)clm(m) * S[n * kLM + m] * dS[n * kLM + m];
-        if (a.H4) {
-            double J[5];
-            fourbody<double>(S + n * kLM + 3, J);
-            double v = 0.0;
-            for (int m = 0; m < 5; ++m) v += J[m] * dS[n * kLM + 3 + m];
-            dq[NR + NA * 4 + n] = v;
-        }
-    }
-    // network and its second-order terms, lane takes h = lane, lane + G, ...:
-    // u = W0 dq, alpha = aE w1 s - 2 w1 u t s (coefficient of q in dW0, and
-    // db0), beta = w1 s (coefficient of dq), gamma = aE t + s u (dw1);
-    // p = W0^T (w1 s), p2 = W0^T (-2 w1 u t s), rho = aE p + p2
-    const double* W0 = a.prm + (size_t)fr.ti * a.L.mlp_stride;
-    const double* b0 = W0 + (size_t)H * D;
-    const double* w1 = b0 + H;
-    double pq[kF64MaxD], rho[kF64MaxD];
-    for (int d = 0; d < D; ++d) pq[d] = rho[d] = 0.0;
-    for (int h = lane; h < H; h += G) {
-        const double* w = W0 + (size_t)h * D;
-        double z = b0[h], u = 0.0;
-        for (int d = 0; d < D; ++d) {
-            z += w[d] * q[d];
-            u += w[d] * dq[d];
-        }
-        const double t = tanh(z), sd = 1.0 - t * t, wh = w1[h];
-        const double c2 = -2.0 * wh * u * t * sd;
-        a.st[(size_t)(gf.al + h) * N + i] = aE * wh * sd + c2;
-        a.st[(size_t)(gf.be + h) * N + i] = wh * sd;
-        a.st[(size_t)(gf.ga + h) * N + i] = aE * t + sd * u;
-        for (int d = 0; d < D; ++d) {
-            pq[d] += wh * sd * w[d];
-            rho[d] += c2 * w[d];
-        }
-    }
-    for (int d = 0; d < D; ++d) {
-        pq[d] = group_sum<G>(pq[d]);
-        rho[d] = aE * pq[d] + group_sum<G>(rho[d]);
-    }
-    // P = dPhi/dS (into dS) and R = dPhi/d(dS) (into S):
-    // P_nm = 2 C_lm (rho_nl S_nm + p_nl dS_nm) (+ rho4 J_m + p4 dJ_m),
-    // R_nm = 2 C_lm p_nl S_nm (+ p4 J_m)
-    for (int n = 0; n < NA; ++n) {
-        double J[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, dJ[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-        if (a.H4) fourbody_jvp<double>(S + n * kLM + 3, dS + n * kLM + 3, J, dJ);
-        const double r4 = a.H4 ? rho[NR + NA * 4 + n] : 0.0, p4 = a.H4 ? pq[NR + NA * 4 + n] : 0.0;
-        for (int m = 0; m < kLM; ++m) {
-            const int l = lm_l(m) - 1;
-            const double c = 2.0 * (double)clm(m), Sv = S[n * kLM + m], dSv = dS[n * kLM + m];
-            double Pv = c * (rho[NR + n * 4 + l] * Sv + pq[NR + n * 4 + l] * dSv);
-            double Rv = c * pq[NR + n * 4 + l] * Sv;
-            if (m >= 3 && m < 8) {
-                Pv += r4 * J[m - 3] + p4 * dJ[m - 3];
-                Rv += p4 * J[m - 3];
-            }
-            dS[n * kLM + m] = Pv;
-            S[n * kLM + m] = Rv;
-        }
-    }
-    const double* P = dS;
-    const double* R = S;
-    // bins[t][n][k] = sum_{j of t} Q_k X_n + Q'_k Z_n over the angular pairs
-    double bins[kF64MaxBins];
-    for (int x = 0; x < T * NA * KA; ++x) bins[x] = 0.0;
-    for (int s = lane; s < nc; s += G) {
-        Pair64 p;
-        if (!pair_at(a, fr, s, p) || !(p.r < a.rc_ang)) continue;
-        double dr[3];
-        tangent64(a, li, mu, p, dr);
-        const double udr = p.u[0] * dr[0] + p.u[1] * dr[1] + p.u[2] * dr[2];
-        basis64(p.r, a.rc_ang, KA, f, fp);
-        const HarmTermsT<double> ht = harm_terms(p.u[0], p.u[1], p.u[2]);
-        const double ir = 1.0 / p.r;
-        double X[kF64MaxN], Z[kF64MaxN];
-        for (int n = 0; n < NA; ++n) X[n] = Z[n] = 0.0;
-        for (int m = 0; m < kLM; ++m) {
-            double Y, gx, gy, gz;
-            harm_m(m, ht, Y, gx, gy, gz);
-            const double dY = (gx * dr[0] + gy * dr[1] + gz * dr[2] - lm_l(m) * Y * udr) * ir;
-            for (int n = 0; n < NA; ++n) {
-                X[n] += P[n * kLM + m] * Y + R[n * kLM + m] * dY;
-                Z[n] += R[n * kLM + m] * Y;
-            }
-        }
-        for (int n = 0; n < NA; ++n)
-            for (int k = 0; k < KA; ++k) bins[(p.tj * NA + n) * KA + k] += f[k] * X[n] + fp[k] * udr * Z[n];
-    }
-    for (int x = 0; x < T * NA * KA; ++x) bins[x] = group_sum<G>(bins[x]);
-    // stage the factors, entries split over the lanes
-    for (int d = lane; d < D; d += G) {
-        a.st[(size_t)(gf.q + d) * N + i] = q[d];
-        a.st[(size_t)(gf.dq + d) * N + i] = dq[d];
-    }
-    for (int n = lane; n < NR; n += G) {
-        a.st[(size_t)(gf.rho + n) * N + i] = rho[n];
-        a.st[(size_t)(gf.p + n) * N + i] = pq[n];
-    }
-    for (int x = lane; x < T * KR; x += G) {
-        a.st[(size_t)(gf.F + x) * N + i] = F[x];
-        a.st[(size_t)(gf.DF + x) * N + i] = DF[x];
-    }
-    for (int x = lane; x < T * NA * KA; x += G) a.st[(size_t)(gf.bins + x) * N + i] = bins[x];
-}
-
-// Each parameter's gradient over one 1,024-atom chunk: the sum, over the
-// chunk's atoms of the parameter's species, of a1 b1 + a2 b2 (staged factors;
-// b = 1 where absent; aE for b1).  A warp takes one item of up to eight
-// parameters that share factors, its lanes the atoms of the species:
-//   two-factor  (species, 2 rows x 4 columns): W0's alpha_h q_d + beta_h dq_d
-//               and cR's rho_n F[t2][k] + p_n DF[t2][k]; 12 loads per atom
-//               instead of 32 for the eight parameters
-//   one-factor  (species, 4 rows): b0 (alpha_h), w1 (gamma_h), cA (bins)
-//   b1          (species)
-// The atoms are first ordered by species, so that no lane is spent on another
-// species' atoms: GB300's FP64 pipe (about 1/64 of the FP32 rate) bounds the
-// sums once the chip is full.  The grid splits the items as well as the chunks: with one CTA
-// per chunk a batch of 2,548 atoms ran on 3 of 152 SMs and took 5.8 ms.
-constexpr int kGradWarps = 8;
-struct GradItems64 {
-    int nW0, nB, nCR, nCA, total;   // W0, b0 + w1, cR and cA items
-};
-__host__ __device__ inline GradItems64 grad_items64(const F64Args& a) {
-    GradItems64 g;
-    g.nW0 = a.T * ((a.H + 1) / 2) * ((a.D + 3) / 4);
-    g.nB = 2 * a.T * ((a.H + 3) / 4);
-    g.nCR = a.T * a.T * ((a.NR + 1) / 2) * ((a.KR + 3) / 4);
-    g.nCA = a.T * ((a.T * a.NA * a.KA + 3) / 4);
-    g.total = g.nW0 + g.nCR + g.nB + g.nCA + a.T;
-    return g;
-}
-
-__global__ void __launch_bounds__(32 * kGradWarps) k64_grad_partial(const F64Args a) {
-    const int c = blockIdx.x, N = a.N, T = a.T, NR = a.NR, KR = a.KR, H = a.H, D = a.D;
-    const ParamLayout& L = a.L;
-    const GradFields gf = grad_fields(a);
-    const GradItems64 gi = grad_items64(a);
-    const int a0 = c * kChunk, na = min(N - a0, kChunk);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // the chunk's atoms in species order (stable)
-    __shared__ int order[kChunk];
-    __shared__ int wcnt[kMaxTypes][kChunk / 32];
-    __shared__ int first[kMaxTypes + 1];
-    for (int r = warp; r < kChunk / 32; r += kGradWarps) {
-        const int x = r * 32 + lane;
-        const int sp = x < na ? a.type[a0 + x] : -1;
-        for (int t = 0; t < T; ++t) {
-            const unsigned m = __ballot_sync(0xffffffffu, sp == t);
-            if (lane == 0) wcnt[t][r] = __popc(m);
-        }
-    }
-    __syncthreads();
-    if (warp == 0) {
-        int base = 0;
-        for (int t = 0; t < T; ++t) {
-            const int v = wcnt[t][lane];
-            int incl = v;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
-            }
-            wcnt[t][lane] = base + incl - v;
-            if (lane == 0) first[t] = base;
-            base += __shfl_sync(0xffffffffu, incl, 31);
-        }
-        if (lane == 0) first[T] = base;
-    }
-    __syncthreads();
-    for (int r = warp; r < kChunk / 32; r += kGradWarps) {
-        const int x = r * 32 + lane;
-        const int sp = x < na ? a.type[a0 + x] : -1;
-        for (int t = 0; t < T; ++t) {
-            const unsigned m = __ballot_sync(0xffffffffu, sp == t);
-            if (sp == t) order[wcnt[t][r] + __popc(m & ((1u << lane) - 1u))] = a0 + x;
-        }
-    }
-    __syncthreads();
-    static_assert(kChunk / 32 == 32, "one lane per row of the chunk");
-    double* out = a.gpart + (size_t)c * L.P;
-    const double* st = a.st;
-    for (int it = blockIdx.y * kGradWarps + warp; it < gi.total; it += gridDim.y * kGradWarps) {
-        if (it < gi.nW0 + gi.nCR) {
-            // rows r0, r0 + 1 of (A, B) times columns c0 .. c0 + 3 of (X, Y)
-            int sp, r0, c0, nr, nc, fA, fB, fX, fY, pbase, pstride;
-            if (it < gi.nW0) {
-                const int DB = (D + 3) / 4, HB = (H + 1) / 2;
-                c0 = 4 * (it % DB);
-                r0 = 2 * ((it / DB) % HB);
-                sp = it / (DB * HB);
-                nr = H; nc = D;
-                fA = gf.al; fB = gf.be; fX = gf.q; fY = gf.dq;
-                pbase = sp * L.mlp_stride;
-                pstride = D;
-            } else {
-                int x = it - gi.nW0;
-                const int KB = (KR + 3) / 4, NB = (NR + 1) / 2;
-                c0 = 4 * (x % KB);
-                x /= KB;
-                r0 = 2 * (x % NB);
-                x /= NB;
-                const int t2 = x % T;
-                sp = x / T;
-                nr = NR; nc = KR;
-                fA = gf.rho; fB = gf.p; fX = gf.F + t2 * KR; fY = gf.DF + t2 * KR;
-                pbase = L.off_cR + (sp * T + t2) * NR * KR;
-                pstride = KR;
-            }
-            // a row or column past the end repeats the last one; its sum is dropped
-            const double *pA[2], *pB[2], *pX[4], *pY[4];
-#pragma unroll
-            for (int r = 0; r < 2; ++r) {
-                pA[r] = st + (size_t)(fA + min(r0 + r, nr - 1)) * N;
-                pB[r] = st + (size_t)(fB + min(r0 + r, nr - 1)) * N;
-            }
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                pX[k] = st + (size_t)(fX + min(c0 + k, nc - 1)) * N;
-                pY[k] = st + (size_t)(fY + min(c0 + k, nc - 1)) * N;
-            }
-            double acc[2][4] = {};
-            for (int x = first[sp] + lane; x < first[sp + 1]; x += 32) {
-                const int i = order[x];
-                double vA[2], vB[2], vX[4], vY[4];
-#pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                    vA[r] = pA[r][i];
-                    vB[r] = pB[r][i];
-                }
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    vX[k] = pX[k][i];
-                    vY[k] = pY[k][i];
-                }
-#pragma unroll
-                for (int r = 0; r < 2; ++r)
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) acc[r][k] += vA[r] * vX[k] + vB[r] * vY[k];
-            }
-#pragma unroll
-            for (int r = 0; r < 2; ++r)
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const double v = group_sum<32>(acc[r][k]);
-                    if (lane == 0 && r0 + r < nr && c0 + k < nc) out[pbase + (r0 + r) * pstride + c0 + k] = v;
-                }
-            continue;
-        }
-        int x = it - gi.nW0 - gi.nCR, sp, r0, nr, f, pbase;
-        if (x < gi.nB) {
-            const int HB = (H + 3) / 4, which = x / (T * HB), y = x % (T * HB);
-            sp = y / HB;
-            r0 = 4 * (y % HB);
-            nr = H;
-            f = which ? gf.ga : gf.al;
-            pbase = sp * L.mlp_stride + H * D + which * H;
-        } else if ((x -= gi.nB) < gi.nCA) {
-            nr = T * a.NA * a.KA;
-            const int BB = (nr + 3) / 4;
-            sp = x / BB;
-            r0 = 4 * (x % BB);
-            f = gf.bins;
-            pbase = L.off_cA + sp * nr;
-        } else {
-            sp = x - gi.nCA;
-            double acc = 0.0;
-            for (int y = first[sp] + lane; y < first[sp + 1]; y += 32) acc += a.aE[a.cfg[order[y]]];
-            acc = group_sum<32>(acc);
-            if (lane == 0) out[sp * L.mlp_stride + H * D + 2 * H] = acc;
-            continue;
-        }
-        const double* pA[4];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) pA[r] = st + (size_t)(f + min(r0 + r, nr - 1)) * N;
-        double acc[4] = {};
-        for (int y = first[sp] + lane; y < first[sp + 1]; y += 32) {
-            const int i = order[y];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) acc[r] += pA[r][i];
-        }
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const double v = group_sum<32>(acc[r]);
-            if (lane == 0 && r0 + r < nr) out[pbase + r0 + r] = v;
-        }
-    }
-}
-
-__global__ void k64_grad_final(const F64Args a, int nchunk) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= a.L.P) return;
-    double acc = 0.0;
-    for (int c = 0; c < nchunk; ++c) acc += a.gpart[(size_t)c * a.L.P + p];
-    a.grad[p] = acc;
-}
-
 }  // namespace
-
-// lanes per atom: enough threads to fill the GPU (N G >= 2^17, about 1,024 per
-// SM), with G in {1, 8, 32}; a function of N alone
-int fp64_lanes_per_atom(int N) {
-    if (N >= (1 << 17)) return 1;
-    if (N >= (1 << 14)) return 8;
-    return 32;
-}
-
-int fp64_grad_fields(const F64Args& a) { return grad_fields(a).total; }
-
-int fp64_grad_chunks(int N) { return (N + kChunk - 1) / kChunk; }
 
 cudaError_t launch_promote(const float* src, double* dst, int n, cudaStream_t st) {
     if (n > 0) k_promote<<<(n + 255) / 256, 256, 0, st>>>(src, dst, n);
@@ -856,26 +603,36 @@ cudaError_t launch_promote(const float* src, double* dst, int n, cudaStream_t st
 }
 
 namespace {
+template <int G, class DM, class A>
+cudaError_t launch_efv_g(const A& a, cudaStream_t st) {
+    using R = ScalarT<A>;
+    constexpr int NG = Group64<G>::NG;
+    const int grid = (a.N + NG - 1) / NG;
+    const size_t s1 = sizeof(R) * (size_t)NG * Group64<G>(a.T, a.NA, a.KR, a.D).size;
+    const size_t s2 = sizeof(R) * (size_t)NG * a.T * a.KR +
+                      (kScatter<A> ? 0 : NG * (sizeof(R) * a.NA * kLM + sizeof(unsigned short) * kF64Slots));
+    cudaError_t e;
+    if (s1 > 48 * 1024 &&
+        (e = cudaFuncSetAttribute(k64_atom<G, DM, A>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024)))
+        return e;
+    if (s2 > 48 * 1024 &&
+        (e = cudaFuncSetAttribute(k64_force<G, DM, A>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024)))
+        return e;
+    k64_atom<G, DM, A><<<grid, kF64Threads, s1, st>>>(a);
+    k64_force<G, DM, A><<<grid, kF64Threads, s2, st>>>(a);
+    return cudaGetLastError();
+}
 template <class A>
 cudaError_t launch_efv_t(const A& a, int max_chunks, double* e_tot, double* virial, cudaStream_t st) {
-    if (a.N > 0) {
-        const int G = fp64_lanes_per_atom(a.N);
-        const int grid = (int)(((long long)a.N * G + kF64Block - 1) / kF64Block);
-        if (G == 1) {
-            k64_atom<1, A><<<grid, kF64Block, 0, st>>>(a);
-            k64_force<1, A><<<grid, kF64Block, 0, st>>>(a);
-        } else if (G == 8) {
-            k64_atom<8, A><<<grid, kF64Block, 0, st>>>(a);
-            k64_force<8, A><<<grid, kF64Block, 0, st>>>(a);
-        } else {
-            k64_atom<32, A><<<grid, kF64Block, 0, st>>>(a);
-            k64_force<32, A><<<grid, kF64Block, 0, st>>>(a);
-        }
-    }
-    if (max_chunks > 0) k64_chunk_reduce<A><<<max_chunks, kF64Red, 0, st>>>(a);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = cudaSuccess;
+    if (a.N > 0)
+        e = with_dims(a, [&](auto dm) {
+            using DM = decltype(dm);
+            return a.N <= kEvalLanes32 ? launch_efv_g<32, DM>(a, st) : launch_efv_g<8, DM>(a, st);
+        });
     if (e != cudaSuccess) return e;
-    return launch_final_reduce(a.B, a.chunk_start, a.partial, e_tot, virial, st);
+    if (max_chunks > 0) k64_totals<A><<<max_chunks, 320, 0, st>>>(a, e_tot, virial);
+    return cudaGetLastError();
 }
 }  // namespace
 
@@ -896,23 +653,6 @@ cudaError_t launch_loss_fp64(const F64Args& a, int max_chunks, const double* e_t
     if (max_chunks > 0) k64_loss_atoms<<<max_chunks, kF64Red, 0, st>>>(a, f_lbl, w[1], lam, a.partial);
     k64_loss_cfg<<<1, kF64Red, 0, st>>>(a, a.partial, e_tot, vir, e_lbl, v_lbl, w[0], w[1], w[2], mode, aE, mu,
                                         loss);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_grad_fp64(const F64Args& a, cudaStream_t st) {
-    if (a.N > 0) {
-        const int G = fp64_lanes_per_atom(a.N);
-        const int grid = (int)(((long long)a.N * G + kF64Block - 1) / kF64Block);
-        if (G == 1) k64_grad_atom<1><<<grid, kF64Block, 0, st>>>(a);
-        else if (G == 8) k64_grad_atom<8><<<grid, kF64Block, 0, st>>>(a);
-        else k64_grad_atom<32><<<grid, kF64Block, 0, st>>>(a);
-        // about 1,024 CTAs, each with at least one item per warp
-        const int nchunk = fp64_grad_chunks(a.N);
-        const int most = (grad_items64(a).total + kGradWarps - 1) / kGradWarps;
-        const int split = std::max(1, std::min(most, 1024 / nchunk));
-        k64_grad_partial<<<dim3(nchunk, split), 32 * kGradWarps, 0, st>>>(a);
-    }
-    k64_grad_final<<<(a.L.P + 255) / 256, 256, 0, st>>>(a, fp64_grad_chunks(a.N));
     return cudaGetLastError();
 }
 

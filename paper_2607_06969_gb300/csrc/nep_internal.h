@@ -156,11 +156,8 @@ cudaError_t launch_pack(const float* pos, const int* type, const int* atom_off, 
 // the same with the reduction chunks planned and the reduction tickets cleared
 cudaError_t launch_pack_plan(const float* pos, const int* type, const int* atom_off, int N, int B, int T,
                              float4* pos4, int* cfg, int* status, int* chunk_start, int* ticket, cudaStream_t st);
-cudaError_t launch_chunk_plan(const int* atom_off, int B, int* chunk_start, cudaStream_t st);
 // FP64 sums of E_i and the per-atom virials per configuration
 cudaError_t launch_totals(const EvalArgs& a, const FinishArgs& f, int max_chunks, cudaStream_t st);
-cudaError_t launch_final_reduce(int B, const int* chunk_start, const double* partial,
-                                double* e_tot, double* virial, cudaStream_t st);
 
 struct NbrWork {
     CellPlan* plan;        // [B]
@@ -205,13 +202,16 @@ struct F32Args {
     const int* shift;              // [cap][N] packed images, or null (minimum image)
     const float* prm;              // [P]
     float* e;                      // [N]     E_i
-    float* p;                      // [NR][N] dE_i/dq_n, radial n
-    float* R;                      // [NA*24][N] dE_i/dS_nlm
+    float* p;                      // [N][T][KR] dE_i/dq_n contracted with cR, per neighbour species
+    const int* cnt_ang;            // [N]
+    const int* rev;                // [cap_ang][N]
+    float4* fin;                   // [cap_ang][N] incoming angular pair forces
     float* w;                      // [9][N]  per-atom virial
     float* force;                  // [3][N]
     const int* atom_off;           // [B+1]
     const int* chunk_start;        // [B+1]
     double* partial;               // [chunks][10]
+    int* ticket;                   // [B] chunks summed so far
     int n_owned;                   // atoms [0, n_owned) enter the E and virial sums
 };
 cudaError_t launch_efv_generic(const F32Args& a, int max_chunks, double* e_tot, double* virial,
@@ -230,13 +230,14 @@ struct F64Args {
     const int* shift;              // [cap][N] packed images, or null (minimum image)
     const double* prm;             // [P]
     double* e;                     // [N]     E_i
-    double* p;                     // [NR][N] dE_i/dq_n, radial n
-    double* R;                     // [NA*24][N] dE_i/dS_nlm
+    double* p;                     // [N][T][KR] dE_i/dq_n contracted with cR, per neighbour species
+    double* R;                     // [N][NA][24] dE_i/dS_nlm
     double* w;                     // [9][N]  per-atom virial
     double* force;                 // [3][N]
     const int* atom_off;           // [B+1]
     const int* chunk_start;        // [B+1]
     double* partial;               // [chunks][10]
+    int* ticket;                   // [B] chunks summed so far
     int n_owned;                   // atoms [0, n_owned) enter the E and virial sums
     // training gradient
     const double* lam;             // [3][N] dL/dF
@@ -247,7 +248,6 @@ struct F64Args {
     double* grad;                  // [P]
 };
 cudaError_t launch_promote(const float* src, double* dst, int n, cudaStream_t st);
-int fp64_lanes_per_atom(int N);
 int fp64_grad_fields(const F64Args& a);
 int fp64_grad_chunks(int N);
 cudaError_t launch_efv_fp64(const F64Args& a, int max_chunks, double* e_tot, double* virial,

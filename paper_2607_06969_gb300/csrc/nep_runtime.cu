@@ -197,40 +197,6 @@ __global__ void __launch_bounds__(kTotalsThreads) k_totals(const EvalArgs a, Fin
     }
 }
 
-// FP64 path: one block per configuration: threads take chunk partials k = t, t+256, ...
-// and a fixed tree (warp shuffles, then the 8 warp sums in order) combines
-// them, so the sum order never changes
-__global__ void __launch_bounds__(kRedThreads) k_final_reduce(int B, const int* __restrict__ chunk_start,
-                                                              const double* __restrict__ partial,
-                                                              double* e_tot, double* virial) {
-    const int b = blockIdx.x;
-    if (b >= B) return;
-    double acc[10];
-#pragma unroll
-    for (int c = 0; c < 10; ++c) acc[c] = 0.0;
-    for (int k = chunk_start[b] + threadIdx.x; k < chunk_start[b + 1]; k += kRedThreads)
-#pragma unroll
-        for (int c = 0; c < 10; ++c) acc[c] += partial[(size_t)k * 10 + c];
-    __shared__ double red[10][kRedThreads / 32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int c = 0; c < 10; ++c) {
-        double v = acc[c];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) red[c][w] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < 10) {
-        double v = 0.0;
-        for (int q = 0; q < kRedThreads / 32; ++q) v += red[threadIdx.x][q];
-        if (threadIdx.x == 0) {
-            if (e_tot) e_tot[b] = v;
-        } else if (virial) {
-            virial[(size_t)b * 9 + threadIdx.x - 1] = v;
-        }
-    }
-}
-
 // ------------------------------------------------------- neighbour build
 // Cells per edge: floor(L / ((rc + 1e-3) / kCellDiv)) (at least 1), reduced
 // while the cell count of a configuration exceeds 2 N_b + 27.  The stencil
@@ -1157,19 +1123,8 @@ cudaError_t launch_pack_plan(const float* pos, const int* type, const int* atom_
     return cudaGetLastError();
 }
 
-cudaError_t launch_chunk_plan(const int* atom_off, int B, int* chunk_start, cudaStream_t st) {
-    k_chunk_plan<<<1, 1024, 0, st>>>(atom_off, B, chunk_start, nullptr);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_totals(const EvalArgs& a, const FinishArgs& f, int max_chunks, cudaStream_t st) {
     if (max_chunks > 0) k_totals<<<max_chunks, kTotalsThreads, 0, st>>>(a, f);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_final_reduce(int B, const int* chunk_start, const double* partial,
-                                double* e_tot, double* virial, cudaStream_t st) {
-    if (B > 0) k_final_reduce<<<B, kRedThreads, 0, st>>>(B, chunk_start, partial, e_tot, virial);
     return cudaGetLastError();
 }
 

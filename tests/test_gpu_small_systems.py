@@ -210,3 +210,77 @@ def test_lane_groups_training_agrees_with_one_thread_per_atom(nb, hname, counts,
         assert np.linalg.norm(np.asarray(x) - y) <= 1e-5 * np.linalg.norm(y)
     for x, y in zip(got, grads()):
         assert np.array_equal(x, y)
+
+
+SHAPES64 = dict(small=I.HYPER_SMALL, large=I.HYPER_LARGE,
+                narrow=I.Hyper(n_types=3, n_rad=5, n_ang=3, k_rad=6, k_ang=5, has_4body=1, n_hidden=7),
+                k12=I.Hyper(n_types=2, n_rad=11, n_ang=7, k_rad=10, k_ang=9, has_4body=0, n_hidden=35),
+                wide=I.Hyper(n_types=1, n_rad=16, n_ang=9, k_rad=13, k_ang=16, has_4body=1, n_hidden=33))
+
+
+def typed(s, h):
+    return I.System(pos=s.pos, types=(s.types % h.n_types).astype(np.int32), box=s.box, atom_off=s.atom_off)
+
+
+@pytest.mark.parametrize("name", list(SHAPES64))
+def test_fp64_and_generic_lane_group_sizes(nb, name):
+    """The FP64 evaluation and gradient, and the generic FP32 evaluation,
+    with 32 lanes per atom (up to 1,500 atoms) and with 8: a configuration
+    alone against the same one in a larger batch, for shapes on every set of
+    compiled loop bounds.  FP64 sums of some thousand terms: 1e-12; FP32: the
+    bars of the parity tests."""
+    import torch
+    h = SHAPES64[name]
+    one, two = I.packing_batch([43], tag=70), I.packing_batch([1470], tag=71)
+    both = I.System(pos=np.concatenate([one.pos, two.pos]), types=np.concatenate([one.types, two.types]),
+                    box=np.concatenate([one.box, two.box]), atom_off=np.array([0, 43, 1513]))
+    model = nb.Model(h, I.init_params(h, seed=6).astype(np.float32))
+    rng = np.random.default_rng(5)
+    a_e, lam, mu = rng.normal(size=2), rng.normal(size=(3, 1513)), rng.normal(size=(2, 9))
+    a_e[1] = 0.0
+    lam[:, 43:] = 0.0
+    mu[1] = 0.0
+    dev = lambda x: torch.tensor(np.ascontiguousarray(x), dtype=torch.float64, device="cuda")   # noqa: E731
+    res = []
+    for s, B in ((one, 1), (both, 2)):
+        s = typed(s, h)
+        dsys = nb.DeviceSystem.from_inputs(s)
+        nl = nb.NeighborList(s.n_atoms, 160, 80)
+        ws = nb.Workspace(model, s.n_atoms, B, 160, 80)
+        nb.neighbors(model, dsys, nl, 0.5, ws)
+        assert nb.check_list(nl) == nb.NEP_OK
+        e, f, et, v = nb.energy_forces_virial_fp64(model, dsys, nl, nb.Workspace64(model, s.n_atoms, B))
+        g = nb.param_grad_adjoint_fp64(model, dsys, nl, nb.Workspace64(model, s.n_atoms, B, train=True), dev(a_e[:B]),
+                                       dev(lam[:, :s.n_atoms]), dev(mu[:B]))
+        x = [e[:43], f[:, :43], et[:1], v[:1], g]
+        y = nb.energy_forces_virial(model, dsys, nl, ws)
+        res.append([t.cpu().numpy() for t in x] + [t.cpu().numpy() for t in (y[0][:43], y[1][:, :43], y[2][:1], y[3][:1])])
+    for a, b in zip(res[0][:5], res[1][:5]):
+        assert np.abs(a - b).max() <= 1e-12 * max(1.0, np.abs(a).max()) * 43
+    for got in res:                                   # the FP32 evaluation against FP64
+        assert np.abs(got[5] - got[0]).max() <= 1e-6 * max(1.0, np.abs(got[0]).max())
+        assert np.abs(got[6] - got[1]).max() <= 1e-4
+        assert np.abs(got[8] - got[3]).max() <= 1e-5 * 43 * max(1.0, np.abs(got[3]).max())
+
+
+@pytest.mark.parametrize("hname", ["small", "k12"])
+def test_fp64_and_generic_many_angular_pairs(nb, hname):
+    """More angular pairs than the FP64 force kernel keeps slots for (128),
+    against the FP32 evaluation of the same list (its own bars, scaled with
+    the forces)."""
+    h = SHAPES64[hname]
+    s = typed(I.packing_batch([400], density=0.32, dmin=1.0, tag=73), h)
+    model = nb.Model(h, I.init_params(h, seed=5).astype(np.float32))
+    dsys = nb.DeviceSystem.from_inputs(s)
+    nl = nb.NeighborList(s.n_atoms, 800, 320)
+    ws = nb.Workspace(model, s.n_atoms, 1, 800, 320)
+    nb.neighbors(model, dsys, nl, 0.0, ws)
+    assert nb.check_list(nl) == nb.NEP_OK, nb.last_error()
+    assert int(nl.cnt_ang.max()) > 128
+    e, f, et, v = [t.cpu().numpy() for t in nb.energy_forces_virial(model, dsys, nl, ws)]
+    e6, f6, et6, v6 = [t.cpu().numpy()
+                       for t in nb.energy_forces_virial_fp64(model, dsys, nl, nb.Workspace64(model, s.n_atoms, 1))]
+    scale = max(1.0, float(np.abs(f6).max()))
+    assert np.abs(e - e6).max() <= 1e-5 * max(1.0, np.abs(e6).max())
+    assert np.abs(f - f6).max() <= 1e-4 * scale
+    assert np.abs(v - v6).max() <= 1e-5 * 400 * max(1.0, np.abs(v6).max() / 400)
