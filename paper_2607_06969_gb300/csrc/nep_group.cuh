@@ -190,10 +190,12 @@ __device__ int group_sums(const EvalArgs& a, const float* sm, float* gb, float* 
     for (int t = 0; t < T; ++t)
 #pragma unroll
         for (int k = 0; k < KR; ++k) fb[t][k] = 0.0f;
+    constexpr int NA2 = (NA + 1) / 2;
+    float2 S2[NA2][MPL];                 // rows n two by two (paired FMAs)
 #pragma unroll
-    for (int n = 0; n < NA; ++n)
+    for (int n = 0; n < NA2; ++n)
 #pragma unroll
-        for (int x = 0; x < MPL; ++x) S[n][x] = 0.0f;
+        for (int x = 0; x < MPL; ++x) S2[n][x] = make_float2(0.0f, 0.0f);
     const int cmax = warp_max(cnt), amax = warp_max(cnt_ang);
     int total = 0;
     // a chunk's entries are read one chunk ahead, the indices two
@@ -249,11 +251,12 @@ __device__ int group_sums(const EvalArgs& a, const float* sm, float* gb, float* 
         }
         __syncwarp();
         for (int q = 0; q < np; ++q) {
-            float g[M::NAp];
+            float2 g[M::NAp / 2];
 #pragma unroll
             for (int n = 0; n < M::NAp; n += 4) {
                 const float4 v = ld4(gb + M::oG + q * M::NAp + n);
-                g[n] = v.x; g[n + 1] = v.y; g[n + 2] = v.z; g[n + 3] = v.w;
+                g[n / 2] = make_float2(v.x, v.y);
+                g[n / 2 + 1] = make_float2(v.z, v.w);
             }
 #pragma unroll
             for (int x = 0; x < MPL; ++x) {
@@ -261,7 +264,7 @@ __device__ int group_sums(const EvalArgs& a, const float* sm, float* gb, float* 
                 if (mm < kLM) {
                     const float Y = gb[M::oY + mm * M::GS + q];
 #pragma unroll
-                    for (int n = 0; n < NA; ++n) S[n][x] = fmaf(g[n], Y, S[n][x]);
+                    for (int n = 0; n < NA2; ++n) S2[n][x] = ffma2(g[n], make_float2(Y, Y), S2[n][x]);
                 }
             }
         }
@@ -286,8 +289,10 @@ __device__ int group_sums(const EvalArgs& a, const float* sm, float* gb, float* 
 #pragma unroll
     for (int n = 0; n < NA; ++n)
 #pragma unroll
-        for (int x = 0; x < MPL; ++x)
+        for (int x = 0; x < MPL; ++x) {
+            S[n][x] = n % 2 ? S2[n / 2][x].y : S2[n / 2][x].x;
             if (lane + x * G < kLM) gS[n * kLM + lane + x * G] = S[n][x];
+        }
     __syncwarp();
     return total;
 }

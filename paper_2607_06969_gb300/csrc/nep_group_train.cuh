@@ -15,16 +15,17 @@ namespace nep {
 
 #if defined(__CUDACC__)
 
+constexpr int kGradBlocks = 3;   // resident CTAs per SM the registers are held to; 4 spill (20,405 atoms 283 / 305 us)
+
 template <class C, int G>
 struct GroupGradSmem {
     static constexpr int NA = C::NA, T = C::T, KR = C::KR, KA = C::KA, D = C::D;
     static constexpr int NG = kGroupThreads / G, GS = G + 1;
-    static constexpr int NAp = round4(NA), NBINS = T * NA * KA;
-    // [G][2 NAp] g_n and g'_n (rhat . dr) of a chunk's pairs; then F and DF; then the bins
+    static constexpr int NAp = round4(NA);
+    // [G][2 NAp] g_n and g'_n (rhat . dr) of a chunk's pairs; then F and DF
     static constexpr int oG = 0;
-    static constexpr int szG0 = G * 2 * NAp > NBINS ? G * 2 * NAp : NBINS;
-    static constexpr int szG = round4(szG0 > 2 * T * KR ? szG0 : 2 * T * KR);
-    static constexpr int oF = oG, oDF = oF + T * KR, oB = oG;
+    static constexpr int szG = round4(G * 2 * NAp > 2 * T * KR ? G * 2 * NAp : 2 * T * KR);
+    static constexpr int oF = oG, oDF = oF + T * KR;
     // exchange buffer: Y_m, then dY_m; F partials, then DF's; the network's
     // vectors; then Q, Q', X, Z of a chunk's pairs
     static constexpr int oY = oG + szG;
@@ -83,7 +84,7 @@ __device__ __forceinline__ void lanes_rows_sum(float* buf, const float* v, float
 }
 
 template <class C, int G>
-__global__ void __launch_bounds__(kGroupThreads, 3) kg_grad(const TrainArgs t) {
+__global__ void __launch_bounds__(kGroupThreads, kGradBlocks) kg_grad(const TrainArgs t) {
     using M = GroupGradSmem<C, G>;
     using I = GroupSmem<C, G>;                       // the model image is kg_atom's
     constexpr int NR = C::NR, NA = C::NA, KR = C::KR, KA = C::KA, T = C::T, D = C::D;
@@ -117,12 +118,14 @@ __global__ void __launch_bounds__(kGroupThreads, 3) kg_grad(const TrainArgs t) {
         adjoint_frame(t, i, li, mu);
 
         // ---- sums F, S and their tangents DF, dS over the list
-        float S[NA][MPL], dS[NA][MPL];
+        constexpr int NA2 = (NA + 1) / 2;
+        float2 S[NA2][MPL], dS[NA2][MPL];            // rows n two by two (paired FMAs)
+        auto row = [](const float2 (&v)[NA2][MPL], int n, int x) { return n % 2 ? v[n / 2][x].y : v[n / 2][x].x; };
         float fb[T * KR], df[T * KR];
 #pragma unroll
-        for (int n = 0; n < NA; ++n)
+        for (int n = 0; n < NA2; ++n)
 #pragma unroll
-            for (int x = 0; x < MPL; ++x) S[n][x] = dS[n][x] = 0.0f;
+            for (int x = 0; x < MPL; ++x) S[n][x] = dS[n][x] = make_float2(0.0f, 0.0f);
 #pragma unroll
         for (int o = 0; o < T * KR; ++o) fb[o] = df[o] = 0.0f;
         const int cmax = warp_max(cnt), amax = warp_max(cnt_ang);
@@ -169,11 +172,11 @@ __global__ void __launch_bounds__(kGroupThreads, 3) kg_grad(const TrainArgs t) {
                     contract_pairs<NA, KA>(c2, f, g);
                     contract_pairs<NA, KA>(c2, fp, gp);
                 }
-                float* row = gb + M::oG + at * 2 * NAp;
+                float* gr = gb + M::oG + at * 2 * NAp;
 #pragma unroll
                 for (int n = 0; n < NAp; ++n) {
-                    row[n] = n < NA ? g[n] : 0.0f;
-                    row[NAp + n] = n < NA ? gp[n] * p.udr : 0.0f;
+                    gr[n] = n < NA ? g[n] : 0.0f;
+                    gr[NAp + n] = n < NA ? gp[n] * p.udr : 0.0f;
                 }
                 const Harm<float> ht = harm_of(p.dx * p.ir, p.dy * p.ir, p.dz * p.ir);
                 const HarmD<float> hd = unit_tangent(ht, p.drx, p.dry, p.drz, p.udr, p.ir);
@@ -195,27 +198,30 @@ __global__ void __launch_bounds__(kGroupThreads, 3) kg_grad(const TrainArgs t) {
                 }
                 __syncwarp();
                 for (int q = 0; q < np; ++q) {
-                    float g[NAp], A[NAp];
+                    float2 g[NAp / 2], A[NAp / 2];
 #pragma unroll
                     for (int n = 0; n < NAp; n += 4) {
                         const float4 v = ld4(gb + M::oG + q * 2 * NAp + n);
-                        g[n] = v.x; g[n + 1] = v.y; g[n + 2] = v.z; g[n + 3] = v.w;
+                        g[n / 2] = make_float2(v.x, v.y);
+                        g[n / 2 + 1] = make_float2(v.z, v.w);
                         if (!half) {
                             const float4 w = ld4(gb + M::oG + q * 2 * NAp + NAp + n);
-                            A[n] = w.x; A[n + 1] = w.y; A[n + 2] = w.z; A[n + 3] = w.w;
+                            A[n / 2] = make_float2(w.x, w.y);
+                            A[n / 2 + 1] = make_float2(w.z, w.w);
                         }
                     }
 #pragma unroll
                     for (int x = 0; x < MPL; ++x) {
                         if (lane + x * G >= kLM) continue;
                         const float Y = gb[M::oY + (lane + x * G) * GS + q];
+                        const float2 Y2 = make_float2(Y, Y);
 #pragma unroll
-                        for (int n = 0; n < NA; ++n) {
+                        for (int n = 0; n < NA2; ++n) {
                             if (half) {
-                                dS[n][x] = fmaf(g[n], Y, dS[n][x]);
+                                dS[n][x] = ffma2(g[n], Y2, dS[n][x]);
                             } else {
-                                S[n][x] = fmaf(g[n], Y, S[n][x]);
-                                dS[n][x] = fmaf(A[n], Y, dS[n][x]);
+                                S[n][x] = ffma2(g[n], Y2, S[n][x]);
+                                dS[n][x] = ffma2(A[n], Y2, dS[n][x]);
                             }
                         }
                     }
@@ -231,8 +237,8 @@ __global__ void __launch_bounds__(kGroupThreads, 3) kg_grad(const TrainArgs t) {
 #pragma unroll
             for (int x = 0; x < MPL; ++x)
                 if (lane + x * G < kLM) {
-                    gS[n * kLM + lane + x * G] = S[n][x];
-                    gD[n * kLM + lane + x * G] = dS[n][x];
+                    gS[n * kLM + lane + x * G] = row(S, n, x);
+                    gD[n * kLM + lane + x * G] = row(dS, n, x);
                 }
         __syncwarp();
         if (first) {
@@ -363,7 +369,8 @@ __global__ void __launch_bounds__(kGroupThreads, 3) kg_grad(const TrainArgs t) {
 #pragma unroll
             for (int n = 0; n < NA; ++n) {
                 const float pl = gb[M::oP + NR + n * 4 + l - 1], rl = gb[M::oRho + NR + n * 4 + l - 1];
-                float P = c2 * fmaf(rl, S[n][x], pl * dS[n][x]), R = c2 * pl * S[n][x];
+                const float Sv = row(S, n, x);
+                float P = c2 * fmaf(rl, Sv, pl * row(dS, n, x)), R = c2 * pl * Sv;
                 if (C::H4 && l == 2) {
                     const float p4 = gb[M::oP + NR + NA * 4 + n], r4 = gb[M::oRho + NR + NA * 4 + n];
                     const float J = gb[M::oJ + 5 * n + m - 3];
@@ -375,7 +382,13 @@ __global__ void __launch_bounds__(kGroupThreads, 3) kg_grad(const TrainArgs t) {
             }
         }
         __syncwarp();
-        for (int o = lane; o < M::NBINS; o += G) gb[M::oB + o] = 0.0f;
+        // lane's (n, k) sums for each species of the neighbour
+        constexpr int OPL = (NA * KA + G - 1) / G;
+        float bins[T][OPL];
+#pragma unroll
+        for (int u = 0; u < T; ++u)
+#pragma unroll
+            for (int x = 0; x < OPL; ++x) bins[u][x] = 0.0f;
 
         // ---- X_n, Z_n of the angular pairs and the c-gradient bins
         const bool kept = total <= kGroupSlots && cnt_ang <= 65536;
@@ -440,24 +453,34 @@ __global__ void __launch_bounds__(kGroupThreads, 3) kg_grad(const TrainArgs t) {
             for (int q = 0; q < nq; ++q) {
                 const int u = __shfl_sync(0xffffffffu, tq, gbase + q);
                 if (u < 0) continue;
-                for (int o = lane; o < NA * KA; o += G) {
+#pragma unroll
+                for (int x = 0; x < OPL; ++x) {
+                    const int o = lane + x * G;
+                    if (o >= NA * KA) continue;
                     const int n = o / KA, k = o % KA;
-                    float* b = gb + M::oB + u * NA * KA + o;
-                    *b = fmaf(gb[M::oY + k * GS + q], gb[M::oY + (2 * KA + n) * GS + q],
-                              fmaf(gb[M::oY + (KA + k) * GS + q], gb[M::oY + (2 * KA + NA + n) * GS + q], *b));
+                    const float f = gb[M::oY + k * GS + q], fp = gb[M::oY + (KA + k) * GS + q];
+                    const float X = gb[M::oY + (2 * KA + n) * GS + q], Z = gb[M::oY + (2 * KA + NA + n) * GS + q];
+#pragma unroll
+                    for (int v = 0; v < T; ++v)
+                        if (u == v) bins[v][x] = fmaf(f, X, fmaf(fp, Z, bins[v][x]));
                 }
             }
             __syncwarp();
         }
-        if (valid)
-            for (int o = lane; o < M::NBINS; o += G) t.bins[(size_t)o * N + i] = gb[M::oB + o];
+        if (valid) {
+#pragma unroll
+            for (int u = 0; u < T; ++u)
+#pragma unroll
+                for (int x = 0; x < OPL; ++x)
+                    if (lane + x * G < NA * KA) t.bins[(size_t)(u * NA * KA + lane + x * G) * N + i] = bins[u][x];
+        }
         __syncwarp();
     }
 }
 
 template <class C, int G>
 int group_grad_per_sm(int H) {
-    return std::max(1, std::min(3, kSmemPerSm / ((int)GroupGradSmem<C, G>::bytes(H) + 1024)));
+    return std::max(1, std::min(kGradBlocks, kSmemPerSm / ((int)GroupGradSmem<C, G>::bytes(H) + 1024)));
 }
 template <class C, int G>
 void launch_group_grad_g(const TrainArgs& t, cudaStream_t st) {
