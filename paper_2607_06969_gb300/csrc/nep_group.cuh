@@ -381,7 +381,9 @@ __global__ void __launch_bounds__(kGroupThreads, kGroupMinBlocks) kg_atom(const 
     constexpr int NR = C::NR, NA = C::NA, KR = C::KR, KA = C::KA, T = C::T, MPL = (kLM + G - 1) / G;
     extern __shared__ float sm[];
     const int N = a.N, H = a.H, kind = a.q16_kind;
-    group_load_model<C, G>(sm, a.params, H);
+    group_load_model<C, G>(sm, a.params, H);      // older than the kernel before this one
+    pdl_wait();
+    pdl_trigger();
     const int lane = threadIdx.x % G, group = threadIdx.x / G;
     float* gb = sm + M::groups(H) + group * M::group_size(H);
     float* gS = gb + M::S(H);
@@ -507,8 +509,6 @@ __global__ void __launch_bounds__(kGroupThreads) kg_finish(const EvalArgs a, con
     const AtomFrame fr = atom_frame(a, i);
     const int cnt = valid ? a.cnt[i] : 0, cnt_ang = a.cnt_ang[i];
     const float rcR2 = a.rc_rad * a.rc_rad, rcA2 = a.rc_ang * a.rc_ang, irR = 1.0f / a.rc_rad;
-    for (int o = lane; o < T * KR; o += G) Pi[group][o] = a.Pr[(size_t)i * T * KR + o];
-    __syncwarp();
     float acc[9];                                        // F, then xx yy zz xy xz yz
 #pragma unroll
     for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
@@ -516,6 +516,10 @@ __global__ void __launch_bounds__(kGroupThreads) kg_finish(const EvalArgs a, con
     int j0 = lane < cnt ? a.nbr[(size_t)lane * N + i] : i;
     int j1 = lane + G < cnt ? a.nbr[(size_t)(lane + G) * N + i] : i;
     float4 p0 = a.pos4[j0];
+    pdl_wait();                              // the list and the positions are older than kg_atom
+    pdl_trigger();
+    for (int o = lane; o < T * KR; o += G) Pi[group][o] = a.Pr[(size_t)i * T * KR + o];
+    __syncwarp();
     for (int s = lane; s < cnt; s += G) {
         GroupPair p;
         p.j = j0;
@@ -605,14 +609,13 @@ cudaError_t group_init_g() {
 template <class C, int G>
 cudaError_t launch_group_g(const EvalArgs& a, cudaStream_t st) {
     constexpr int NG = kGroupThreads / G;
-    kg_atom<C, G><<<persistent_grid((a.N + NG - 1) / NG, group_per_sm<C, G>(a.H)), kGroupThreads,
-                    GroupSmem<C, G>::bytes(a.H), st>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(kg_atom<C, G>, persistent_grid((a.N + NG - 1) / NG, group_per_sm<C, G>(a.H)), kGroupThreads,
+                      GroupSmem<C, G>::bytes(a.H), st, a);
 }
 template <class C, int G>
 void launch_group_finish_g(const EvalArgs& a, const FinishArgs& f, cudaStream_t st) {
     constexpr int NG = kGroupThreads / G;
-    kg_finish<C, G><<<(a.N + NG - 1) / NG, kGroupThreads, 0, st>>>(a, f);
+    launch_pdl(kg_finish<C, G>, (a.N + NG - 1) / NG, kGroupThreads, 0, st, a, f);
 }
 
 template <class C>

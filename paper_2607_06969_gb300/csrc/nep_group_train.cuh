@@ -92,7 +92,9 @@ __global__ void __launch_bounds__(kGroupThreads, kGradBlocks) kg_grad(const Trai
     extern __shared__ float sm[];
     const EvalArgs& a = t.e;
     const int N = a.N, H = a.H;
-    group_load_model<C, G>(sm, a.params, H);
+    group_load_model<C, G>(sm, a.params, H);      // older than the kernel before this one
+    pdl_wait();
+    pdl_trigger();
     const int lane = threadIdx.x % G, group = threadIdx.x / G;
     float* gb = sm + I::groups(H) + group * M::group_size(H);
     float* gS = gb + M::S(H);
@@ -485,8 +487,8 @@ int group_grad_per_sm(int H) {
 template <class C, int G>
 void launch_group_grad_g(const TrainArgs& t, cudaStream_t st) {
     constexpr int NG = kGroupThreads / G;
-    kg_grad<C, G><<<persistent_grid((t.e.N + NG - 1) / NG, group_grad_per_sm<C, G>(t.e.H)), kGroupThreads,
-                    GroupGradSmem<C, G>::bytes(t.e.H), st>>>(t);
+    launch_pdl(kg_grad<C, G>, persistent_grid((t.e.N + NG - 1) / NG, group_grad_per_sm<C, G>(t.e.H)), kGroupThreads,
+               GroupGradSmem<C, G>::bytes(t.e.H), st, t);
 }
 #endif
 

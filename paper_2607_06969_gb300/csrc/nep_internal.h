@@ -14,6 +14,35 @@
 
 namespace nep {
 
+#if defined(__CUDACC__)
+// Programmatic dependent launch between the kernels of a small system's call:
+// launch_pdl lets a kernel start while the one before it drains, which saves
+// about a microsecond of launch latency each and lets a kernel stage what it
+// can beforehand.  Every kernel launched so begins with
+//   (work that touches nothing the kernel before it writes or reads)
+//   pdl_wait()     the kernel before has completed and its writes are visible
+//   pdl_trigger()  the next kernel may start
+// in this order: since the trigger follows the wait, a kernel that runs ahead
+// of its wait knows everything before its predecessor complete.  After any
+// other kernel or operation the launch is an ordinary one.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <class... K, class... A>
+cudaError_t launch_pdl(void (*kernel)(K...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, K(args)...);
+}
+#endif
+
 // largest hidden width of the FP16/BF16 tensor-core network
 constexpr int kTcMaxHidden = 64;
 constexpr int kMaxTypes = 4;

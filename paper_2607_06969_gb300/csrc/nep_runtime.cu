@@ -107,6 +107,8 @@ __device__ __forceinline__ void pack_atom(const float* pos, const int* __restric
 __global__ void __launch_bounds__(256) k_pack(const float* __restrict__ pos, const int* __restrict__ type,
                                               const int* __restrict__ atom_off, int N, int B, int T, float4* pos4,
                                               int* cfg, int* status, int* chunk_start, int* ticket) {
+    pdl_wait();
+    pdl_trigger();
     if (chunk_start && blockIdx.x == gridDim.x - 1) {
         chunk_plan_block(atom_off, B, chunk_start, ticket);
         return;
@@ -145,6 +147,8 @@ __global__ void __launch_bounds__(kTotalsThreads) k_totals(const EvalArgs a, Fin
     const int total = f.chunk_start[B];
     const int lane = threadIdx.x & 31, c = threadIdx.x >> 5;
     if (k >= total) {
+        pdl_wait();
+        pdl_trigger();
         // the blocks past the last chunk (at least one per empty configuration)
         // write the zeros of configurations without atoms
         for (int b = k - total; b < B; b += gridDim.x - total)
@@ -161,10 +165,18 @@ __global__ void __launch_bounds__(kTotalsThreads) k_totals(const EvalArgs a, Fin
     const int k0 = f.chunk_start[b], nk = f.chunk_start[b + 1] - k0;
     const int a0 = f.atom_off[b] + (k - k0) * kChunk;
     const int a1 = min(min(f.atom_off[b + 1], a0 + kChunk), f.n_owned);
+    pdl_wait();                          // the plan is older than the kernel before this one
+    pdl_trigger();
     const float* src = c == 0 ? a.e_atom : a.wat + (size_t)(c - 1) * N;
     float h = 0.0f, l = 0.0f;
-#pragma unroll 4
-    for (int i = a0 + lane; i < a1; i += 32) two_sum_add(h, l, src[i]);
+    constexpr int kAhead = 16;           // loads in flight per lane
+    for (int i0 = a0 + lane; i0 < a1; i0 += 32 * kAhead) {
+        float x[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) x[u] = i0 + 32 * u < a1 ? src[i0 + 32 * u] : 0.0f;
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) two_sum_add(h, l, x[u]);
+    }
     for (int o = 16; o > 0; o >>= 1) {
         const float oh = __shfl_down_sync(0xffffffffu, h, o);
         const float ol = __shfl_down_sync(0xffffffffu, l, o);
@@ -409,6 +421,8 @@ __global__ void __launch_bounds__(1024) k_cells_small(
     const float* __restrict__ pos, const int* __restrict__ type, const int* __restrict__ atom_off,
     const float* __restrict__ box, int N, int B, int T, float rc, float4* pos4, int* cfg, int* status,
     CellPlan* plan, int* cell_of, int* cell_start, float4* cell_pos) {
+    pdl_wait();
+    pdl_trigger();
     extern __shared__ int cnt[];                    // [cells], then the cells' ends
     __shared__ int in_cell[kCellsSmallN];           // atoms in cell order, any order within a cell
     __shared__ int ws[32];
@@ -670,7 +684,7 @@ __global__ void __launch_bounds__(128) k_build(const float4* __restrict__ pos4,
 constexpr int kBuildWarps = 4;
 constexpr int kBuildSegs = 128;      // candidate ranges held at once
 constexpr int kBuildRows = 64;       // stencil rows per round, two per lane
-constexpr int kBuildWarpN = 40000;   // largest system: the whole list build, thread / warp per atom (the
+constexpr int kBuildWarpN = 48000;   // largest system: the whole list build, thread / warp per atom (the
                                      // reverse search alike): 7,200 atoms 150 / 56 us, 46,522 251 / 220
                                      // (packings, images), 57,600 203 / 238 (rock salt)
 constexpr float kBuildMinEdge = 16.0f;   // shortest box edge: the list cutoff over this (at most 34 ranges per row)
@@ -679,6 +693,8 @@ __global__ void __launch_bounds__(32 * kBuildWarps) k_build_warp(
     const CellPlan* __restrict__ plan, const int* __restrict__ cell_of, const int* __restrict__ cell_start,
     const float4* __restrict__ cell_pos, int N, float rc2_rad, float rc2_ang, float rc2_phys,
     unsigned char* __restrict__ row_start, unsigned char* __restrict__ slot_row, nep_nlist nl) {
+    pdl_wait();
+    pdl_trigger();
     __shared__ int s_q0[kBuildWarps][kBuildSegs], s_cum[kBuildWarps][kBuildSegs + 1];
     __shared__ int s_img[kBuildWarps][kBuildSegs];
     __shared__ unsigned short s_row[kBuildWarps][kBuildSegs];
@@ -901,6 +917,8 @@ template <int G>
 __global__ void __launch_bounds__(128) k_rev(int N, const int* __restrict__ cfg, const CellPlan* __restrict__ plan,
                                              const unsigned char* __restrict__ row_start,
                                              const unsigned char* __restrict__ slot_row, nep_nlist nl) {
+    pdl_wait();
+    pdl_trigger();
     const int i = (blockIdx.x * blockDim.x + threadIdx.x) / G;
     if (i >= N) return;
     const int na = nl.cnt_ang[i];
@@ -914,6 +932,8 @@ __global__ void __launch_bounds__(128) k_rev(int N, const int* __restrict__ cfg,
 // one Adam step per parameter; c1 = lr / (1 - beta1^t), c2 = 1 / sqrt(1 - beta2^t)
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
                        float* __restrict__ v, int n, float beta1, float beta2, float eps, float c1, float c2) {
+    pdl_wait();
+    pdl_trigger();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     const float gk = g[k];
@@ -961,6 +981,8 @@ __device__ __forceinline__ void kick_atom(float* __restrict__ vel, const float* 
 __global__ void k_kick(float* __restrict__ vel, const float* __restrict__ force,
                        const int* __restrict__ type, InvMass im, int N, float half_dt,
                        float* __restrict__ pos, float dt) {
+    pdl_wait();
+    pdl_trigger();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < N) kick_atom(vel, force, type[i], im, N, i, half_dt, pos, dt);
 }
@@ -971,6 +993,8 @@ __global__ void __launch_bounds__(256) k_kick_pack(float* __restrict__ vel, cons
                                                    float* __restrict__ pos, float dt,
                                                    const int* __restrict__ atom_off, int B, int T, float4* pos4,
                                                    int* cfg, int* status, int* chunk_start, int* ticket) {
+    pdl_wait();
+    pdl_trigger();
     if (chunk_start && blockIdx.x == gridDim.x - 1) {
         chunk_plan_block(atom_off, B, chunk_start, ticket);
         return;
@@ -992,6 +1016,8 @@ __device__ __forceinline__ float wrap_coord(float x, float L) {
 // each atom's configuration is found from the CSR offsets
 __global__ void k_wrap_seg(float* pos, const int* __restrict__ atom_off, int B, const float* __restrict__ box,
                            int N) {
+    pdl_wait();
+    pdl_trigger();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     const int b = find_segment(atom_off, B, i);
@@ -1005,6 +1031,8 @@ __global__ void __launch_bounds__(kRedThreads) k_loss_atoms(
     int N, int B, const int* __restrict__ atom_off, const int* __restrict__ chunk_start,
     const float* __restrict__ force, const float* __restrict__ f_lbl, float wF, float4* lam4,
     double* partial) {
+    pdl_wait();
+    pdl_trigger();
     const int k = blockIdx.x;
     const int total = chunk_start[B];
     if (k >= total) return;
@@ -1039,6 +1067,8 @@ __global__ void __launch_bounds__(kRedThreads) k_loss_cfg(
     const double* __restrict__ vir, const double* __restrict__ e_lbl,
     const double* __restrict__ v_lbl, float wE, float wF, float wV, int mode, float* aE, float* mu,
     double* loss) {
+    pdl_wait();
+    pdl_trigger();
     // FP64 division is slow on this GPU: each configuration divides once,
     // by its atom count, and the rest are products
     const double iB = 1.0 / (double)B;
@@ -1085,6 +1115,8 @@ __global__ void __launch_bounds__(kRedThreads) k_loss_cfg(
 __global__ void k_pack_adjoint(int N, int B, const float* __restrict__ lam,
                                const double* __restrict__ a_e, const double* __restrict__ mu_in,
                                float4* lam4, float* aE, float* mu) {
+    pdl_wait();
+    pdl_trigger();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < N) lam4[i] = make_float4(lam[i], lam[N + i], lam[2 * N + i], 0.0f);
     if (i < B) {
@@ -1101,7 +1133,7 @@ inline int blocks(int n, int t) { return (n + t - 1) / t; }
 cudaError_t launch_pack(const float* pos, const int* type, const int* atom_off, int N, int B,
                         int T, float4* pos4, int* cfg, int* status, cudaStream_t st) {
     if (N > 0)
-        k_pack<<<blocks(N, 256), 256, 0, st>>>(pos, type, atom_off, N, B, T, pos4, cfg, status, nullptr, nullptr);
+        launch_pdl(k_pack, blocks(N, 256), 256, 0, st, pos, type, atom_off, N, B, T, pos4, cfg, status, nullptr, nullptr);
     return cudaGetLastError();
 }
 
@@ -1112,11 +1144,11 @@ cudaError_t launch_pack_plan(const float* pos, const int* type, const int* atom_
                              float4* pos4, int* cfg, int* status, int* chunk_start, int* ticket, cudaStream_t st) {
     const bool fused = B <= kPlanFusedB;
     if (fused) {
-        k_pack<<<blocks(N, 256) + 1, 256, 0, st>>>(pos, type, atom_off, N, B, T, pos4, cfg, status, chunk_start,
+        launch_pdl(k_pack, blocks(N, 256) + 1, 256, 0, st, pos, type, atom_off, N, B, T, pos4, cfg, status, chunk_start,
                                                    ticket);
     } else {
         if (N > 0)
-            k_pack<<<blocks(N, 256), 256, 0, st>>>(pos, type, atom_off, N, B, T, pos4, cfg, status, nullptr,
+            launch_pdl(k_pack, blocks(N, 256), 256, 0, st, pos, type, atom_off, N, B, T, pos4, cfg, status, nullptr,
                                                    nullptr);
         k_chunk_plan<<<1, 1024, 0, st>>>(atom_off, B, chunk_start, ticket);
     }
@@ -1124,7 +1156,7 @@ cudaError_t launch_pack_plan(const float* pos, const int* type, const int* atom_
 }
 
 cudaError_t launch_totals(const EvalArgs& a, const FinishArgs& f, int max_chunks, cudaStream_t st) {
-    if (max_chunks > 0) k_totals<<<max_chunks, kTotalsThreads, 0, st>>>(a, f);
+    if (max_chunks > 0) launch_pdl(k_totals, max_chunks, kTotalsThreads, 0, st, a, f);
     return cudaGetLastError();
 }
 
@@ -1142,7 +1174,7 @@ cudaError_t launch_neighbors(const float* pos, const int* type, int T, float4* p
             (e = cudaFuncSetAttribute(k_cells_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sizeof(int) * (2 * kCellsSmallN + 27 * kCellsSmallB + 1))))
             return e;
-        k_cells_small<<<1, 1024, smem, st>>>(pos, type, atom_off, box, N, B, T, rc_list, pos4, cfg, nl->status,
+        launch_pdl(k_cells_small, 1, 1024, smem, st, pos, type, atom_off, box, N, B, T, rc_list, pos4, cfg, nl->status,
                                              w.plan, w.cell_of, w.cell_start, w.cell_pos);
     } else {
         if ((e = cudaMemsetAsync(nl->status, 0, 4 * sizeof(int), st))) return e;
@@ -1162,14 +1194,14 @@ cudaError_t launch_neighbors(const float* pos, const int* type, int T, float4* p
     }
     const float rr = rc_list * rc_list, ra = rc_list_ang * rc_list_ang, rp = rc_phys * rc_phys;
     if (N <= kBuildWarpN && min_edge * kBuildMinEdge >= rc_list)
-        k_build_warp<<<blocks(N, kBuildWarps), 32 * kBuildWarps, 0, st>>>(pos4, cfg, box, w.plan, w.cell_of,
+        launch_pdl(k_build_warp, blocks(N, kBuildWarps), 32 * kBuildWarps, 0, st, pos4, cfg, box, w.plan, w.cell_of,
                                                                           w.cell_start, w.cell_pos, N, rr, ra, rp,
                                                                           w.row_start, w.slot_row, *nl);
     else
         k_build<<<blocks(N, 128), 128, 0, st>>>(pos4, cfg, box, w.plan, w.cell_of, w.cell_start,
                                                 w.cell_pos, N, rr, ra, rp, w.shell, w.row_start, w.slot_row, *nl);
     if (N <= kRevWarpN)
-        k_rev<32><<<blocks(N, 4), 128, 0, st>>>(N, cfg, w.plan, w.row_start, w.slot_row, *nl);
+        launch_pdl(k_rev<32>, blocks(N, 4), 128, 0, st, N, cfg, w.plan, w.row_start, w.slot_row, *nl);
     else
         k_rev<1><<<blocks(N, 128), 128, 0, st>>>(N, cfg, w.plan, w.row_start, w.slot_row, *nl);
     return cudaGetLastError();
@@ -1177,7 +1209,7 @@ cudaError_t launch_neighbors(const float* pos, const int* type, int T, float4* p
 
 cudaError_t launch_adam(float* p, const float* g, float* m, float* v, int n, float beta1, float beta2,
                         float eps, float c1, float c2, cudaStream_t st) {
-    if (n > 0) k_adam<<<blocks(n, 256), 256, 0, st>>>(p, g, m, v, n, beta1, beta2, eps, c1, c2);
+    if (n > 0) launch_pdl(k_adam, blocks(n, 256), 256, 0, st, p, g, m, v, n, beta1, beta2, eps, c1, c2);
     return cudaGetLastError();
 }
 
@@ -1214,7 +1246,7 @@ cudaError_t launch_kick(float* vel, const float* force, const int* type, const f
                         int N, float half_dt, float* pos, float dt, cudaStream_t st) {
     InvMass im;
     for (int t = 0; t < kMaxTypes; ++t) im.v[t] = inv_mass[t];
-    if (N > 0) k_kick<<<blocks(N, 256), 256, 0, st>>>(vel, force, type, im, N, half_dt, pos, dt);
+    if (N > 0) launch_pdl(k_kick, blocks(N, 256), 256, 0, st, vel, force, type, im, N, half_dt, pos, dt);
     return cudaGetLastError();
 }
 
@@ -1225,7 +1257,7 @@ cudaError_t launch_kick_pack(float* vel, const float* force, const int* type, co
     for (int t = 0; t < kMaxTypes; ++t) im.v[t] = inv_mass[t];
     const bool fused = B <= kPlanFusedB;
     if (N > 0 || fused)
-        k_kick_pack<<<blocks(N, 256) + (fused ? 1 : 0), 256, 0, st>>>(vel, force, type, im, N, half_dt, pos, dt,
+        launch_pdl(k_kick_pack, blocks(N, 256) + (fused ? 1 : 0), 256, 0, st, vel, force, type, im, N, half_dt, pos, dt,
                                                                       atom_off, B, T, pos4, cfg, status,
                                                                       fused ? chunk_start : nullptr, ticket);
     if (!fused) k_chunk_plan<<<1, 1024, 0, st>>>(atom_off, B, chunk_start, ticket);
@@ -1238,9 +1270,9 @@ cudaError_t launch_loss(int N, int B, const int* atom_off, const int* chunk_star
                         const float* w, int mode, float4* lam4, float* aE, float* mu,
                         double* partial, double* loss, cudaStream_t st) {
     if (max_chunks > 0)
-        k_loss_atoms<<<max_chunks, kRedThreads, 0, st>>>(N, B, atom_off, chunk_start, force, f_lbl, w[1],
+        launch_pdl(k_loss_atoms, max_chunks, kRedThreads, 0, st, N, B, atom_off, chunk_start, force, f_lbl, w[1],
                                                          lam4, partial);
-    k_loss_cfg<<<1, kRedThreads, 0, st>>>(B, atom_off, chunk_start, partial, e_tot, vir, e_lbl, v_lbl,
+    launch_pdl(k_loss_cfg, 1, kRedThreads, 0, st, B, atom_off, chunk_start, partial, e_tot, vir, e_lbl, v_lbl,
                                           w[0], w[1], w[2], mode, aE, mu, loss);
     return cudaGetLastError();
 }
@@ -1248,12 +1280,12 @@ cudaError_t launch_loss(int N, int B, const int* atom_off, const int* chunk_star
 cudaError_t launch_pack_adjoint(int N, int B, const float* lam, const double* a_e, const double* mu_in,
                                 float4* lam4, float* aE, float* mu, cudaStream_t st) {
     const int n = N > B ? N : B;
-    if (n > 0) k_pack_adjoint<<<blocks(n, 256), 256, 0, st>>>(N, B, lam, a_e, mu_in, lam4, aE, mu);
+    if (n > 0) launch_pdl(k_pack_adjoint, blocks(n, 256), 256, 0, st, N, B, lam, a_e, mu_in, lam4, aE, mu);
     return cudaGetLastError();
 }
 
 cudaError_t launch_wrap_segments(float* pos, const int* atom_off, int B, const float* box, int N, cudaStream_t st) {
-    if (N > 0) k_wrap_seg<<<blocks(N, 256), 256, 0, st>>>(pos, atom_off, B, box, N);
+    if (N > 0) launch_pdl(k_wrap_seg, blocks(N, 256), 256, 0, st, pos, atom_off, B, box, N);
     return cudaGetLastError();
 }
 

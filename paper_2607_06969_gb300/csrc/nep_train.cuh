@@ -689,6 +689,8 @@ NEP_HD GradSmem<C> grad_smem(int H) {
 // accumulators, and the chunk's partials go out once
 template <class C>
 __global__ void __launch_bounds__(kGradThreads) k_grad_partial(const TrainArgs t) {
+    pdl_wait();
+    pdl_trigger();
     using G = GradStage<C>;
     constexpr int NR = C::NR, NA = C::NA, KR = C::KR, KA = C::KA, T = C::T;
     extern __shared__ float4 smem4[];
@@ -768,6 +770,8 @@ __global__ void __launch_bounds__(kGradThreads) k_grad_partial(const TrainArgs t
 constexpr int kFinalGroups = 8;
 template <class C>
 __global__ void __launch_bounds__(32 * kFinalGroups) k_grad_final(const TrainArgs t, int nchunk) {
+    pdl_wait();
+    pdl_trigger();
     __shared__ double part[kFinalGroups][32];
     const ParamLayout L = param_layout(C::T, C::NR, C::NA, C::KR, C::KA, C::H4, t.e.H);
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
@@ -818,10 +822,10 @@ cudaError_t train_t(const TrainArgs& t, cudaStream_t st, int G) {
         const int grid = (N + kBlock - 1) / kBlock;
         if (G) launch_group_grad_g<C, 32>(t, st);
         else k_tangent<C><<<grid, kBlock, smem, st>>>(t);
-        k_grad_partial<C><<<grad_chunks_t<C>(N), kGradThreads, grad_stage_bytes<C>(t.e.H), st>>>(t);
+        launch_pdl(k_grad_partial<C>, grad_chunks_t<C>(N), kGradThreads, grad_stage_bytes<C>(t.e.H), st, t);
     }
     const ParamLayout L = param_layout(C::T, C::NR, C::NA, C::KR, C::KA, C::H4, t.e.H);
-    k_grad_final<C><<<(L.P + 31) / 32, 32 * kFinalGroups, 0, st>>>(t, grad_chunks_t<C>(N));
+    launch_pdl(k_grad_final<C>, (L.P + 31) / 32, 32 * kFinalGroups, 0, st, t, grad_chunks_t<C>(N));
     return cudaGetLastError();
 }
 #endif
