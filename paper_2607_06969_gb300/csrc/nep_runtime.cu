@@ -415,8 +415,14 @@ __device__ __forceinline__ int floor_div(int a, int b) {
 // (as k_pack), the configurations' cell plans and their prefix, atoms counted
 // into cells in shared memory, the cells' scan, and the positions in cell
 // order, atoms of a cell by index.  One launch in place of twelve of about 2
-// us each: at 58 atoms those were half of the list build's time.
-constexpr int kCellsSmallN = 4096, kCellsSmallB = 256;
+// us each: at 58 atoms those were half of the list build's time.  The line
+// is what 32 KB of shared memory hold; near it the CTA alone is no faster on
+// the device (the whole build replayed from a graph: 7,200 atoms 54.1 us in
+// both forms; 7,653 atoms in 48 configurations 63.5 against 58.7), but called
+// in sequence the twelve launches wait for the host: a list and an evaluation
+// of 48 configurations with 5,800 atoms 121 us against 139, ten steps with a
+// rebuild at 7,200 atoms 566 against 586.
+constexpr int kCellsSmallN = 8192, kCellsSmallB = 256;
 __global__ void __launch_bounds__(1024) k_cells_small(
     const float* __restrict__ pos, const int* __restrict__ type, const int* __restrict__ atom_off,
     const float* __restrict__ box, int N, int B, int T, float rc, float4* pos4, int* cfg, int* status,
@@ -1169,8 +1175,8 @@ cudaError_t launch_neighbors(const float* pos, const int* type, int T, float4* p
     const int cmax = w.cmax;
     if (N > 0 && N <= kCellsSmallN && B <= kCellsSmallB) {
         const int smem = (int)sizeof(int) * (cmax + 1);
-        // 60 KB at most, which needs the attribute
-        if (smem > 30 * 1024 &&
+        // 93 KB at most (with 32 KB of static), which needs the attribute
+        if (smem > 8 * 1024 &&
             (e = cudaFuncSetAttribute(k_cells_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sizeof(int) * (2 * kCellsSmallN + 27 * kCellsSmallB + 1))))
             return e;

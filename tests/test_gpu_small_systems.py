@@ -142,9 +142,9 @@ def test_lane_groups_16bit_network(nb, hname, precision):
 
 
 @pytest.mark.parametrize("n,L,skin,copies", [(3, 5.0, 1.0, 30000), (58, 0.0, 0.0, 1500), (700, 0.0, 1.0, 120),
-                                             (4100, 0.0, 0.5, 22)])
+                                             (8190, 0.0, 0.5, 12), (8200, 0.0, 0.5, 12)])
 def test_list_build_small_and_large_forms_agree(nb, n, L, skin, copies):
-    """A configuration listed alone (binned by one CTA up to 4,096 atoms, a
+    """A configuration listed alone (binned by one CTA up to 8,192 atoms, a
     warp per atom in the build and the reverse search) gets, entry for entry,
     the list of each of its copies in a batch large enough for one thread per
     atom: a few atoms in a box shorter than the cutoff (stencils too large for
