@@ -230,42 +230,59 @@ int angular_variant(const nep_model* m, const nep_system* s) {
     const int b = size_bin(s);
     return m->tune_angular[b] >= 0 ? m->tune_angular[b] : nep::kDefaultAngularVariant;
 }
-int radial_block(const nep_model* m, const nep_system* s) { return m->tune_radial[size_bin(s)]; }
 int finish_block(const nep_model* m, const nep_system* s) { return m->tune_finish[size_bin(s)]; }
-// Lanes per atom of an evaluation: 0 for the one-thread-per-atom kernels.
-// A call whose launch choices the caller pinned (nep_set_variant,
-// nep_set_launch) runs those kernels.  The lines lie where the two forms
-// measured equal (one evaluation in a graph, rock salt at 0.033 atoms per A^3):
-//   32 against 8 lanes: 3,686 atoms 48.5 / 46.3 us (38-30-1), 57 / 56 (52-64-1)
-//   8 lanes against one thread: 19,757 atoms 97 / 123 us (38-30-1), 112 / 140
-//   (42-50-1), 147 / 154 (52-64-1); 35,374 atoms 144 / 124, 167 / 142, 221 / 157
-//   the same with the FP16 network: 100 / 135 and 152 / 193; 146 / 138, 226 / 199
-int group_lanes(const nep_model* m, const nep_system* s) {
-    if (m->pinned[size_bin(s)] || !m->ks->group_fits(m->hp.n_hidden)) return 0;
-    const bool wide = m->hp.n_hidden * m->lay.D > 2500;
-    const int most = (wide ? 20000 : 26000) + (m->hp.precision ? 6000 : 0);
-    return s->n_atoms <= 3000 ? 32 : (s->n_atoms <= most ? 8 : 0);
-}
-// Lanes per atom of the training operator's two parts, the forward of a loss
-// gradient and the per-atom backward; 0 for the one-thread-per-atom kernels,
-// which work together (their forward leaves records for their backward).
-// Measured with the reduction, uneven packings, graph (the group kernels,
-// forward 8 / backward 32 lanes, against one thread per atom):
-//   loss gradient: 10,204 atoms 177 / 253 us (38-30-1), 217 / 348 (42-50-1),
-//   289 / 398 (52-64-1); 20,405 atoms 292 / 329, 360 / 431, 496 / 501;
-//   31,888 atoms 440 / 386, 502 / 497, 722 / 599
-//   adjoint product (no forward): 20,405 atoms 201 / 289, 254 / 389, 348 / 459;
-//   31,888 atoms 317 / 342, 382 / 453, 567 / 554
-// The backward takes 32 lanes at every size: with 8 its 16 atoms per CTA need
-// more shared memory and spill (20,405 atoms 232 / 201 us).
-struct TrainLanes {
-    int forward, backward;
+// How an evaluation's work is split: lanes per atom of the atom kernel (radial
+// and angular sums, network, angular forces) and of the finish kernel, 0 for
+// one thread per atom, and the radial kernel's launch code where the atom
+// kernel does not replace it.  A call whose launch choices the caller pinned
+// (nep_set_variant, nep_set_launch) runs one thread per atom throughout.
+// The lines lie where the forms measured equal (one evaluation in a graph,
+// rock salt at 0.033 atoms per A^3; models 38-30-1, 42-50-1, 52-64-1):
+//   atom kernel, 32 against 8 lanes: 2,470 atoms 30.7 / 34.3, 33.0 / 36.3,
+//     34.3 / 40.0 us; 3,686: 35.5 / 34.4, 39.9 / 37.5, 42.5 / 44.1; 7,200:
+//     49.3 / 44.6, 54.6 / 48.4, 61.2 / 67.8, so the wide model keeps 32; its
+//     9,583 atoms 75.3 / 69.5
+//   atom kernel against the radial kernel by four lanes and the angular kernel:
+//     7,200 atoms 48.1 / 53.5, 48.1 / 66.2, 61.4 / 73.2 us; 12,442: 61.8 / 57.0,
+//     71.5 / 69.4, 86.6 / 76.3; FP16 network 12,442: 63.9 / 65.7, -, 91.4 / 102;
+//     15,818: 80.5 / 71.8, -, 115.9 / 110.7; 19,757: 93.2 / 90.1, -, 137.9 / 148.2;
+//     24,300: -, -, 148.8 / 154; 29,491: 119 / 102, -, 183 / 162 (the tensor-core
+//     kernel's tiles of 128 atoms fill whole waves up to 19,456 and 38,912 atoms)
+//   finish kernel, 8 lanes against one thread: 41,990 atoms 119 / 127, 149 / 156,
+//     170 / 179; 57,600: 146 / 145, 172 / 171, 192 / 193; 99,533: 260 / 231
+//   radial kernel, four lanes against one thread: 57,600 atoms 145 / 151, 171 /
+//     175, 193 / 200; 158,054: 368 / 379, 432 / 443, 489 / 500; 335,923: even;
+//     900,000: 1,654 / 1,576
+struct EvalSplit {
+    int atom, finish, radial;
 };
-TrainLanes train_lanes(const nep_model* m, const nep_system* s, bool loss) {
-    const int most = loss ? 22000 : 32000;
-    if (s->n_atoms == 0 || m->pinned[size_bin(s)] || !m->ks->group_train_fits(m->hp.n_hidden) || s->n_atoms > most)
-        return {0, 0};
-    return {s->n_atoms <= 3000 ? 32 : 8, 32};
+EvalSplit eval_split(const nep_model* m, const nep_system* s) {
+    const int N = s->n_atoms, bin = size_bin(s);
+    EvalSplit e{0, 0, m->tune_radial[bin]};
+    if (N == 0 || m->pinned[bin]) return e;
+    if (m->ks->group_fits(m->hp.n_hidden)) {
+        const bool wide = m->hp.n_hidden * m->lay.D > 2500;
+        const int most = !m->hp.precision ? 10000 : wide ? 25000 : 13500;
+        e.atom = N > most ? 0 : N <= (wide ? 8000 : 3000) ? 32 : 8;
+        e.finish = N > 50000 ? 0 : N <= 3000 ? 32 : 8;
+    }
+    if (N <= 200000) e.radial = nep::kRadialSplit;
+    return e;
+}
+// Lanes per atom of the training operator's per-atom backward, 0 for one thread
+// per atom, whose forward then leaves records for it.  A loss gradient's
+// forward is otherwise the plain evaluation; an adjoint product needs none.
+// Measured with the reduction, uneven packings, graph, against one thread per
+// atom (38-30-1, 42-50-1, 52-64-1):
+//   adjoint product: 20,405 atoms 181 / 289, 240 / 389, 332 / 459 us; 31,888
+//     267 / 342, 374 / 453, 533 / 554
+//   loss gradient: 31,888 atoms 365 / 376, 490 / 488, 660 / 570
+int train_lanes(const nep_model* m, const nep_system* s, bool loss) {
+    const int N = s->n_atoms;
+    const bool narrow = m->hp.n_ang <= 6;
+    const int most = loss ? (narrow ? 34000 : 25000) : (narrow ? 40000 : 32000);
+    if (N == 0 || m->pinned[size_bin(s)] || !m->ks->group_train_fits(m->hp.n_hidden) || N > most) return 0;
+    return 32;
 }
 bool block_choice(int b) {
     for (int c : nep::kBlockChoices)
@@ -488,13 +505,13 @@ nep_status efv_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, floa
     auto mark = [&](int k) -> cudaError_t {
         return nt ? cudaEventRecordWithFlags(m->timing[k], st, rec_flags) : cudaSuccess;
     };
-    const int G = N > 0 ? group_lanes(m, s) : 0;
+    const EvalSplit sp = eval_split(m, s);
     NEP_CUDA(mark(0), "timing event");
-    if (G) {
+    if (sp.atom) {
         NEP_CUDA(mark(1), "timing event");       // the radial sums are part of the next kernel
-        NEP_CUDA(m->ks->group_atom(a, st, G), "atom kernel");
+        NEP_CUDA(m->ks->group_atom(a, st, sp.atom), "atom kernel");
     } else {
-        if (N > 0) NEP_CUDA(m->ks->radial(a, st, radial_block(m, s)), "radial kernel");
+        if (N > 0) NEP_CUDA(m->ks->radial(a, st, sp.radial), "radial kernel");
         NEP_CUDA(mark(1), "timing event");
         if (N > 0) NEP_CUDA(m->ks->angular(a, st, vd), "angular kernel");
     }
@@ -510,13 +527,13 @@ nep_status efv_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, floa
     f.e_tot = e_tot;
     f.virial = virial;
     f.vel = nullptr;
-    if (G && kick) {
+    if (sp.finish && kick) {
         f.vel = kick->vel;
         f.half_dt = kick->half_dt;
         for (int t = 0; t < nep::kMaxTypes; ++t) f.inv_mass[t] = kick->inv_mass[t];
         kick->done = true;
     }
-    if (G) NEP_CUDA(m->ks->group_finish(a, f, w.max_chunks, st, G), "finish kernel");
+    if (sp.finish) NEP_CUDA(m->ks->group_finish(a, f, w.max_chunks, st, sp.finish), "finish kernel");
     else NEP_CUDA(m->ks->finish(a, f, w.max_chunks, st, finish_block(m, s)), "finish kernel");
     NEP_CUDA(mark(3), "timing event");
     return NEP_OK;
@@ -534,8 +551,8 @@ nep_status train_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, co
              "pack");
     nep::EvalArgs a = make_args(m, s, nl, work, w);
     a.q16_kind = 0;
-    const TrainLanes lanes = train_lanes(m, s, e_lbl != nullptr);
-    const int G = lanes.forward;
+    const int G = train_lanes(m, s, e_lbl != nullptr);
+    const EvalSplit sp = G ? eval_split(m, s) : EvalSplit{0, 0, 0};
     if (!G) {
         // the training variants of the forward kernels leave their records for the backward
         a.S = at<float>(work, w.S);
@@ -543,10 +560,14 @@ nep_status train_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, co
         a.cnt_compr = at<int>(work, tl.cnt_compr);
         a.q_out = at<float>(work, tl.q);
         a.p_out = at<float>(work, tl.p);
-        if (N > 0) NEP_CUDA(m->ks->radial(a, st, 0), "radial kernel");
-        if (N > 0) NEP_CUDA(m->ks->angular(a, st, angular_variant(m, s)), "angular kernel");
-    } else if (e_lbl) {
-        NEP_CUDA(m->ks->group_atom(a, st, G), "atom kernel");
+    }
+    if (N > 0 && (!G || e_lbl)) {
+        if (sp.atom) {
+            NEP_CUDA(m->ks->group_atom(a, st, sp.atom), "atom kernel");
+        } else {
+            NEP_CUDA(m->ks->radial(a, st, sp.radial), "radial kernel");
+            NEP_CUDA(m->ks->angular(a, st, angular_variant(m, s)), "angular kernel");
+        }
     }
     if (e_lbl) {
         // forward forces, energies and virials, then the loss and its adjoints
@@ -561,7 +582,7 @@ nep_status train_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, co
         f.e_tot = at<double>(work, tl.etot);
         f.virial = at<double>(work, tl.vir);
         f.vel = nullptr;
-        if (G) NEP_CUDA(m->ks->group_finish(a, f, w.max_chunks, st, G), "finish kernel");
+        if (sp.finish) NEP_CUDA(m->ks->group_finish(a, f, w.max_chunks, st, sp.finish), "finish kernel");
         else NEP_CUDA(m->ks->finish(a, f, w.max_chunks, st, 0), "finish kernel");
         NEP_CUDA(nep::launch_loss(N, B, s->atom_off, at<int>(work, w.chunk_start), w.max_chunks,
                                   at<float>(work, tl.force), f_lbl, at<double>(work, tl.etot),
@@ -592,7 +613,7 @@ nep_status train_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, co
     t.bins = at<float>(work, tl.bins);
     t.gpart = at<float>(work, tl.gpart);
     t.grad = grad;
-    NEP_CUDA(m->ks->train(t, st, lanes.backward), "gradient kernels");
+    NEP_CUDA(m->ks->train(t, st, G), "gradient kernels");
     return NEP_OK;
 }
 

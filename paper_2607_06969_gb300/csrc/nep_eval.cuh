@@ -915,9 +915,11 @@ NEP_HD void finish_atom(const EvalArgs& a, int i, float* force, float* e_out, fl
 // (nep_autotune).  Variant 0 (255 registers) keeps S and dE/dS on chip
 // without spills and is the default.
 NEP_HD constexpr int variant_minb(int v) { return v + 2; }
-// Default block sizes of the radial and finish kernels; the autotuner may
-// pick another of kBlockChoices per size class.  Each size keeps the
-// kernel at 64 registers (1,024 / block resident blocks).
+// Block sizes of the radial and finish kernels' training variants; the others
+// default to 64 (900,000 atoms: an evaluation 1,582 -> 1,573 us against 256
+// and 128), and the autotuner may pick another of kBlockChoices per size
+// class.  Each size keeps the kernel at 64 registers (1,024 / block resident
+// blocks).
 constexpr int kRadialBlock = 256;
 constexpr int kFinishThreads = 128;
 
@@ -934,6 +936,101 @@ template <class C, bool MINIMG, bool COMPR, int BLOCK = kRadialBlock>
 __global__ void __launch_bounds__(BLOCK, NEP_RADIAL_MINB * kRadialBlock / BLOCK) k_radial(const EvalArgs a) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < a.N) radial_atom<C, MINIMG, COMPR>(a, i);
+}
+
+// k_radial with kSplitLanes lanes per atom, for systems whose atoms alone are
+// too few threads: each lane takes every fourth list entry, the records go to
+// the same slots (lane order is list order), and the lanes' basis sums are
+// added at the end.  One thread per atom takes the time of one atom's walk, 26
+// us, up to about 40,000 atoms; four lanes take 12 us at 12,442 atoms and 15 at
+// 29,491.  Beyond the line of eval_split (nep_api.cu) the split's scattered
+// list reads cost more than it gains (900,000 atoms 362 -> 440 us).
+constexpr int kSplitLanes = 4;
+template <class C, bool MINIMG>
+__global__ void __launch_bounds__(128, 8) k_radial_split(const EvalArgs a) {
+    constexpr int KR = C::KR, T = C::T, G = kSplitLanes;
+    const int N = a.N, idx = blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = idx % G, ia = idx / G;
+    const bool valid = ia < N;
+    const int i = valid ? ia : N - 1;
+    const AtomFrame fr = atom_frame(a, i);
+    const float rcR2 = a.rc_rad * a.rc_rad, rcA2 = a.rc_ang * a.rc_ang, irR = 1.0f / a.rc_rad;
+    float fb[T][KR];
+#pragma unroll
+    for (int t = 0; t < T; ++t)
+#pragma unroll
+        for (int k = 0; k < KR; ++k) fb[t][k] = 0.0f;
+    const int cnt = valid ? a.cnt[i] : 0, cnt_ang = valid ? a.cnt_ang[i] : 0;
+    const int cmax = __reduce_max_sync(0xffffffffu, cnt), amax = __reduce_max_sync(0xffffffffu, cnt_ang);
+    const int gbase = (threadIdx.x & 31) & ~(G - 1);
+    const unsigned gmask = (1u << G) - 1u, below = (1u << lane) - 1u;
+    int nc = 0, nr = 0;
+    int j1 = lane < cnt ? a.nbr[lane * N + i] : i;
+    int j2 = lane + G < cnt ? a.nbr[(lane + G) * N + i] : i;
+    float4 p1 = a.pos4[j1];
+    for (int s0 = 0; s0 < cmax; s0 += G) {
+        const int s = s0 + lane, j = j1;
+        const bool act = s < cnt;
+        const float4 pj = p1;
+        const int sh = !MINIMG && act ? a.shift[s * N + i] : 0;
+        j1 = j2;
+        p1 = a.pos4[j1];
+        j2 = s + 2 * G < cnt ? a.nbr[(s + 2 * G) * N + i] : i;
+        float dx, dy, dz;
+        pair_vector(fr.pi, pj, fr.Lx, fr.Ly, fr.Lz, fr.iLx, fr.iLy, fr.iLz, MINIMG, sh, dx, dy, dz);
+        const float d2 = act ? norm2(dx, dy, dz) : rcR2;
+        const int tj = f2i(pj.w);
+        const bool in = d2 < rcR2;
+        if (in) {
+            float f[KR];
+            basis<KR>(dist_r(d2), irR, f);
+#pragma unroll
+            for (int t = 0; t < T; ++t) {
+                const float w = (tj == t) ? 1.0f : 0.0f;
+                const float2 w2 = make_float2(w, w);
+#pragma unroll
+                for (int k = 0; k + 1 < KR; k += 2) {
+                    const float2 v = ffma2(w2, make_float2(f[k], f[k + 1]), make_float2(fb[t][k], fb[t][k + 1]));
+                    fb[t][k] = v.x;
+                    fb[t][k + 1] = v.y;
+                }
+                if (KR % 2) fb[t][KR - 1] = fmaf(w, f[KR - 1], fb[t][KR - 1]);
+            }
+        }
+        if (a.rin) {
+            const bool rest = in && s >= cnt_ang;
+            const unsigned m = (__ballot_sync(0xffffffffu, rest) >> gbase) & gmask;
+            if (rest) {
+                const int at = (nr + __popc(m & below)) * N + i;
+                a.rin[at] = j;
+                if (!MINIMG) a.rin_sh[at] = sh;
+            }
+            nr += __popc(m);
+        }
+        if (s0 < amax) {
+            const bool ang = s < cnt_ang && d2 < rcA2;
+            const unsigned m = (__ballot_sync(0xffffffffu, ang) >> gbase) & gmask;
+            if (ang) {
+                const int addr = a.rev[s * N + i] * N + j;
+                a.comp[(nc + __popc(m & below)) * N + i] =
+                    make_float4(dx, dy, dz, i2f((int)(((unsigned)addr << 2) | (unsigned)tj)));
+            }
+            nc += __popc(m);
+        }
+    }
+#pragma unroll
+    for (int t = 0; t < T; ++t)
+#pragma unroll
+        for (int k = 0; k < KR; ++k) {
+            float v = fb[t][k];
+#pragma unroll
+            for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (valid && (t * KR + k) % G == lane) a.fb[(t * KR + k) * N + i] = v;
+        }
+    if (valid && lane == 0) {
+        a.cnt_comp[i] = nc;
+        if (a.rin) a.cnt_rin[i] = nr;
+    }
 }
 
 // Persistent: one CTA per resident slot, the model image staged once, then a
@@ -1052,8 +1149,9 @@ void launch_radial_b(const EvalArgs& a, cudaStream_t st) {
         k_radial<C, false, false, BLOCK><<<grid, BLOCK, 0, st>>>(a);
 }
 
-// block: one of kBlockChoices, 0 for the default; the training variant
-// (compacted records) always runs at the default block
+// block: one of kBlockChoices, 0 for the default (64), kRadialSplit for four
+// lanes per atom; the training variant (compacted records) always runs at
+// kRadialBlock
 template <class C>
 cudaError_t launch_radial_t(const EvalArgs& a, cudaStream_t st, int block) {
     if (a.N == 0) return cudaSuccess;
@@ -1063,7 +1161,13 @@ cudaError_t launch_radial_t(const EvalArgs& a, cudaStream_t st, int block) {
             k_radial<C, true, true><<<grid, kRadialBlock, 0, st>>>(a);
         else
             k_radial<C, false, true><<<grid, kRadialBlock, 0, st>>>(a);
-    } else if (block == 64) {
+    } else if (block == kRadialSplit) {
+        const int grid = (int)(((long long)a.N * kSplitLanes + 127) / 128);
+        if (a.min_image)
+            k_radial_split<C, true><<<grid, 128, 0, st>>>(a);
+        else
+            k_radial_split<C, false><<<grid, 128, 0, st>>>(a);
+    } else if (block == 64 || block == 0) {
         launch_radial_b<C, 64>(a, st);
     } else if (block == 128) {
         launch_radial_b<C, 128>(a, st);
@@ -1112,7 +1216,7 @@ cudaError_t launch_finish_t(const EvalArgs& a, const FinishArgs& f, int max_chun
                 k_finish<C, true, kFinishThreads, true><<<grid, kFinishThreads, 0, st>>>(a, f.force, f.e_out);
             else
                 k_finish<C, false, kFinishThreads, true><<<grid, kFinishThreads, 0, st>>>(a, f.force, f.e_out);
-        } else if (block == 64)
+        } else if (block == 64 || block == 0)
             launch_finish_b<C, 64>(a, f, st);
         else if (block == 256)
             launch_finish_b<C, 256>(a, f, st);

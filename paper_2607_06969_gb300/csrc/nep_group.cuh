@@ -15,11 +15,12 @@
 // Sums run in a fixed order, so results repeat bitwise.
 //
 // Measured (one evaluation in a graph, rock salt, 38-30-1 model, the reductions
-// included; one thread per atom -> the better of G = 8 and 32): 194 atoms 96 ->
-// 31 us, 3,686 atoms 106 -> 46, 7,200 atoms 106 -> 52, 19,757 atoms 123 -> 97;
-// at 35,374 atoms 124 -> 144, so larger systems keep one thread per atom.  What
-// bounds the group form: latency at a few hundred atoms; from about 10,000
-// atoms instruction issue (1,840 warp instructions per atom with G = 8, 2,900
+// included; three one-thread-per-atom kernels and two reductions -> the better
+// of G = 8 and 32): 3,686 atoms 106 -> 34 us, 7,200 atoms 106 -> 48.  From about
+// 10,000 atoms the radial sums by four lanes and the angular kernel take
+// kg_atom's place, and kg_finish alone stays to 50,000 (nep_api.cu has the
+// lines): 19,757 atoms 123 -> 77 us.  What bounds the group form: latency at a
+// few hundred atoms; from about 10,000 atoms instruction issue (1,840 warp instructions per atom with G = 8, 2,900
 // with G = 32) at 16 warps per SM.  G = 4 was slower than 8 at every size
 // (its 32 atoms per CTA leave 3 CTAs per SM).
 //

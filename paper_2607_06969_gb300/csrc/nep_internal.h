@@ -53,6 +53,7 @@ constexpr int kVariants = 3;              // angular kernel register budgets: 2,
 constexpr int kDefaultAngularVariant = 0; // 2 blocks per SM, S_nlm in tensor memory
 constexpr int kSizeBins = 32;             // tuning table: log2 of mean atoms per configuration
 constexpr int kBlockChoices[3] = {64, 128, 256};   // block sizes the tuner tries for radial / finish
+constexpr int kRadialSplit = 1;           // launch code of the radial kernel with four lanes per atom
 constexpr int kRowStride = 64;            // list build: bytes of per-atom stencil row starts
 
 // Stencil/cell plan of one configuration for the neighbour build.
@@ -161,7 +162,7 @@ struct KernelSet {
     size_t (*smem_bytes)(int H);
     cudaError_t (*init)(int H);   // set kernel attributes (dynamic shared memory)
     // block: threads per block of the radial / finish kernel, one of
-    // kBlockChoices, or 0 for the kernel's default
+    // kBlockChoices, or 0 for the kernel's default, or kRadialSplit (radial)
     cudaError_t (*radial)(const EvalArgs&, cudaStream_t, int block);
     cudaError_t (*angular)(const EvalArgs&, cudaStream_t, int variant);   // FP32 or tensor-core network
     cudaError_t (*finish)(const EvalArgs&, const FinishArgs&, int max_chunks, cudaStream_t, int block);
