@@ -277,12 +277,14 @@ EvalSplit eval_split(const nep_model* m, const nep_system* s) {
 //   adjoint product: 20,405 atoms 181 / 289, 240 / 389, 332 / 459 us; 31,888
 //     267 / 342, 374 / 453, 533 / 554
 //   loss gradient: 31,888 atoms 365 / 376, 490 / 488, 660 / 570
+// 16 lanes against 32: 2,548 atoms 80.5 / 83.2, 96.6 / 94.6, 115 / 107; 20,405
+//   281 / 300, 375 / 372, 496 / 489: for n_ang <= 6 (fewer sums per lane) only
 int train_lanes(const nep_model* m, const nep_system* s, bool loss) {
     const int N = s->n_atoms;
     const bool narrow = m->hp.n_ang <= 6;
     const int most = loss ? (narrow ? 34000 : 25000) : (narrow ? 40000 : 32000);
     if (N == 0 || m->pinned[size_bin(s)] || !m->ks->group_train_fits(m->hp.n_hidden) || N > most) return 0;
-    return 32;
+    return N > 2000 && narrow ? 16 : 32;
 }
 bool block_choice(int b) {
     for (int c : nep::kBlockChoices)

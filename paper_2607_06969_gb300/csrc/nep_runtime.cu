@@ -1031,6 +1031,19 @@ __global__ void k_wrap_seg(float* pos, const int* __restrict__ atom_off, int B, 
 }
 
 // ------------------------------------------------------------- loss adjoints
+// sum over the block in a fixed order (thread 0): warp shuffles, then the
+// warp sums in order, with one block-wide wait
+__device__ __forceinline__ double block_sum_fixed(double v) {
+    __shared__ double red[kRedThreads / 32];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double s = 0.0;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < kRedThreads / 32; ++w) s += red[w];
+    return s;
+}
+
 // Force residuals per chunk: lam_i = 2 wF (F_i - F_lbl,i) / (3 N_b B) and the
 // FP64 partial sum of |dF|^2 (Eq. 20).
 __global__ void __launch_bounds__(kRedThreads) k_loss_atoms(
@@ -1055,14 +1068,8 @@ __global__ void __launch_bounds__(kRedThreads) k_loss_atoms(
         lam4[i] = make_float4(cf * dx, cf * dy, cf * dz, 0.0f);
         acc += (double)dx * dx + (double)dy * dy + (double)dz * dz;
     }
-    __shared__ double red[kRedThreads];
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int o = kRedThreads / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) partial[k] = red[0];
+    acc = block_sum_fixed(acc);
+    if (threadIdx.x == 0) partial[k] = acc;
 }
 
 // Per-configuration loss terms and energy/virial adjoints (Eqs. 18-21), and
@@ -1107,14 +1114,8 @@ __global__ void __launch_bounds__(kRedThreads) k_loss_cfg(
         }
         if (nb > 0.0) acc += Lb;
     }
-    __shared__ double red[kRedThreads];
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int o = kRedThreads / 2; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0 && loss) *loss = red[0] * iB;
+    acc = block_sum_fixed(acc);
+    if (threadIdx.x == 0 && loss) *loss = acc * iB;
 }
 
 // External adjoints (vector-Jacobian product) into the kernels' layout.

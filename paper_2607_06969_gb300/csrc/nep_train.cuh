@@ -662,7 +662,11 @@ __global__ void __launch_bounds__(kBlock, NEP_MINB_TANGENT) k_tangent(const Trai
         cbins_atom<C>(t, nullptr, i);
     }
 }
-constexpr int kGradThreads = 256;
+// 512 threads share a staged tile's items, so that most models pass over them
+// in two rounds.  Loss gradient in a graph, 384 / 512 threads (38-30-1,
+// 42-50-1, 52-64-1): 2,548 atoms 80.4 / 77.2, 93.0 / 91.1, 105 / 104 us; 20,405
+// atoms 265 / 261, 358 / 345, 472 / 448
+constexpr int kGradThreads = 512;
 constexpr int kStageUnroll = 8;
 // shared memory of k_grad_partial: the staged tile, the field tables, the
 // chunk's accumulators
@@ -765,9 +769,10 @@ __global__ void __launch_bounds__(kGradThreads) k_grad_partial(const TrainArgs t
     }
     for (int p = threadIdx.x; p < L.P; p += blockDim.x) t.gpart[(size_t)blockIdx.x * L.P + p] = acc[p];
 }
-// FP64 sum over chunks: 32 parameters per CTA, 8 groups of chunks
-// (k = g mod 8) summed in order, then the 8 group sums in order
-constexpr int kFinalGroups = 8;
+// FP64 sum over chunks: 32 parameters per CTA, 32 groups of chunks
+// (k = g mod 32) summed in order, then the group sums in order (with 8 groups
+// each thread's 40 loads of a 319-chunk sum took 8.7 us)
+constexpr int kFinalGroups = 32;
 template <class C>
 __global__ void __launch_bounds__(32 * kFinalGroups) k_grad_final(const TrainArgs t, int nchunk) {
     pdl_wait();
@@ -797,6 +802,8 @@ cudaError_t train_init_t(int H) {
     const int smem = (int)smem_bytes_of<C>(H);
     cudaError_t e;
     if ((e = mlp_tc_init_t<C>(H))) return e;
+    if ((e = cudaFuncSetAttribute(kg_grad<C, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynSmem)))
+        return e;
     if ((e = cudaFuncSetAttribute(kg_grad<C, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxDynSmem)))
         return e;
     if ((e = cudaFuncSetAttribute(k_tangent<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem))) return e;
@@ -810,17 +817,19 @@ int grad_chunks_t(int N) { return grad_chunks_of(N); }
 // whether a model of H hidden units fits the group kernels' shared memory
 template <class C>
 bool group_train_fits_t(int H) {
-    return group_fits_t<C>(H) && GroupGradSmem<C, 32>::bytes(H) <= kMaxDynSmem;
+    return group_fits_t<C>(H) && GroupGradSmem<C, 16>::bytes(H) <= kMaxDynSmem &&
+           GroupGradSmem<C, 32>::bytes(H) <= kMaxDynSmem;
 }
 
-// G: lanes per atom of the per-atom backward (32), 0 for one thread per atom
+// G: lanes per atom of the per-atom backward (16 or 32), 0 for one thread per atom
 template <class C>
 cudaError_t train_t(const TrainArgs& t, cudaStream_t st, int G) {
     const int N = t.e.N;
     const size_t smem = smem_bytes_of<C>(t.e.H);
     if (N > 0) {
         const int grid = (N + kBlock - 1) / kBlock;
-        if (G) launch_group_grad_g<C, 32>(t, st);
+        if (G == 16) launch_group_grad_g<C, 16>(t, st);
+        else if (G) launch_group_grad_g<C, 32>(t, st);
         else k_tangent<C><<<grid, kBlock, smem, st>>>(t);
         launch_pdl(k_grad_partial<C>, grad_chunks_t<C>(N), kGradThreads, grad_stage_bytes<C>(t.e.H), st, t);
     }

@@ -182,11 +182,12 @@ def test_list_build_small_and_large_forms_agree(nb, n, L, skin, copies):
 
 
 @pytest.mark.parametrize("hname", list(MODELS))
-@pytest.mark.parametrize("counts,skin", [([1], 0.0), ([2, 0, 3], 0.0), ([24, 127, 130], 0.7), ([1500, 1501], 0.0)])
+@pytest.mark.parametrize("counts,skin", [([1], 0.0), ([2, 0, 3], 0.0), ([24, 127, 130], 0.7), ([900, 1101], 0.0),
+                                         ([1500, 1501], 0.0)])
 def test_lane_groups_training_agrees_with_one_thread_per_atom(nb, hname, counts, skin):
     """The loss gradient and the adjoint product by lane groups against the
     one-thread-per-atom kernels: remainders of a block, an empty
-    configuration, both forward group sizes, a list with a skin.  FP32 sums
+    configuration, each group size of forward and backward, a list with a skin.  FP32 sums
     of about 10^3 to 10^5 terms in another order: 1e-5 in relative L2 (the
     bar against the FP64 gradient is 1e-4)."""
     import torch
