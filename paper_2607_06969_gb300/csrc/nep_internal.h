@@ -199,7 +199,7 @@ struct NbrWork {
     float4* cell_pos;      // [N] positions in cell order, atom index bits in w
     int* scan_tmp;         // [ceil(Cmax/2048)+1]
     int2* shell;           // [cap][N] scratch for the list entries beyond rc_rad
-    unsigned char* row_start;   // [N][32] where each stencil row's angular entries start
+    unsigned char* row_start;   // [N][kRowStride] where each stencil row's angular entries start
     unsigned char* slot_row;    // [cap_ang][N] stencil row of each angular entry
     int cmax;
 };

@@ -416,12 +416,14 @@ __device__ __forceinline__ int floor_div(int a, int b) {
 // into cells in shared memory, the cells' scan, and the positions in cell
 // order, atoms of a cell by index.  One launch in place of twelve of about 2
 // us each: at 58 atoms those were half of the list build's time.  The line
-// is what 32 KB of shared memory hold; near it the CTA alone is no faster on
-// the device (the whole build replayed from a graph: 7,200 atoms 54.1 us in
-// both forms; 7,653 atoms in 48 configurations 63.5 against 58.7), but called
-// in sequence the twelve launches wait for the host: a list and an evaluation
-// of 48 configurations with 5,800 atoms 121 us against 139, ten steps with a
-// rebuild at 7,200 atoms 566 against 586.
+// is what 32 KB of shared memory hold; near it the CTA alone is little faster
+// on the device (the whole build replayed from a graph, twelve launches / one:
+// 7,200 atoms 54.1 / 49.7 us, 7,653 atoms in 48 configurations 58.7 / 56.5), but
+// called in sequence the twelve wait for the host: a list and an evaluation of
+// 48 configurations with 5,800 atoms 139 / 121 us, ten steps with a rebuild at
+// 7,200 atoms 586 / 566.  Bound by the latency of its phases: all atoms are
+// loaded before the first is used, and configurations' offsets, boxes and
+// plans are read from shared memory (7,200 atoms 19.8 -> 14.4 us).
 constexpr int kCellsSmallN = 8192, kCellsSmallB = 256;
 __global__ void __launch_bounds__(1024) k_cells_small(
     const float* __restrict__ pos, const int* __restrict__ type, const int* __restrict__ atom_off,
@@ -431,52 +433,61 @@ __global__ void __launch_bounds__(1024) k_cells_small(
     pdl_trigger();
     extern __shared__ int cnt[];                    // [cells], then the cells' ends
     __shared__ int in_cell[kCellsSmallN];           // atoms in cell order, any order within a cell
-    __shared__ int ws[32];
+    __shared__ CellPlan plan_s[kCellsSmallB];
+    __shared__ float box_s[3 * kCellsSmallB];
+    __shared__ int off_s[kCellsSmallB + 1], ws[32];
     const int tid = threadIdx.x;
+    constexpr int kPer = kCellsSmallN / 1024;
+    int id[kPer];
+    float4 q[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {                // every load in flight before the first is used
+        const int i = tid + u * 1024;
+        if (i < N) q[u] = make_float4(pos[i], pos[N + i], pos[2 * N + i], __int_as_float(type[i]));
+    }
     if (tid < 4) status[tid] = 0;
+    if (tid <= B) off_s[tid] = atom_off[tid];
+    if (tid < 3 * B) box_s[tid] = box[tid];
     __syncthreads();
     CellPlan p;
     p.base = 0;
-    if (tid < B) p = cell_plan_of(box, atom_off, tid, rc, status);
+    if (tid < B) p = cell_plan_of(box_s, off_s, tid, rc, status);
     int ncell;
     const int base = block_excl_scan_1024(p.base, ws, &ncell);
     if (tid < B) {
         p.base = base;
-        plan[tid] = p;
+        plan[tid] = plan_s[tid] = p;
     }
     for (int c = tid; c < ncell; c += 1024) cnt[c] = 0;
     __syncthreads();
-    constexpr int kPer = kCellsSmallN / 1024;
-    int id[kPer];
-    float4 q[kPer];
 #pragma unroll
     for (int u = 0; u < kPer; ++u) {
         const int i = tid + u * 1024;
         id[u] = -1;
         if (i >= N) continue;
-        int t = type[i];
+        int t = __float_as_int(q[u].w);
         if (t < 0 || t >= T) {
             set_flag(status, 3);
-            t = 0;
+            q[u].w = __int_as_float(0);
         }
-        const float x = pos[i], y = pos[N + i], z = pos[2 * N + i];
-        const int b = find_segment(atom_off, B, i);
-        const float L[3] = {box[3 * b], box[3 * b + 1], box[3 * b + 2]};
+        const int b = find_segment(off_s, B, i);
+        const float L[3] = {box_s[3 * b], box_s[3 * b + 1], box_s[3 * b + 2]};
+        const float x = q[u].x, y = q[u].y, z = q[u].z;
         if (!(x >= 0.0f && x < L[0] && y >= 0.0f && y < L[1] && z >= 0.0f && z < L[2]))
             set_flag(status, 3);                    // NaN and infinities fail the test too
-        pos4[i] = make_float4(x, y, z, __int_as_float(t));
+        pos4[i] = q[u];
         cfg[i] = b;
-        const CellPlan pb = plan[b];
+        const CellPlan& pb = plan_s[b];
         int c[3];
         cell_coords(pb, x, y, z, L, c);
         id[u] = pb.base + (c[0] * pb.nc[1] + c[1]) * pb.nc[2] + c[2];
-        q[u] = make_float4(x, y, z, __int_as_float(i));
         cell_of[i] = id[u];
         atomicAdd(cnt + id[u], 1);
     }
     __syncthreads();
-    // exclusive scan of the counts, each thread a contiguous run of cells
-    const int per = (ncell + 1023) / 1024, c0 = min(tid * per, ncell), c1 = min(c0 + per, ncell);
+    // exclusive scan of the counts, each thread a contiguous run of cells, an
+    // odd number so that the runs of a warp's threads start on distinct banks
+    const int per = ((ncell + 1023) / 1024) | 1, c0 = min(tid * per, ncell), c1 = min(c0 + per, ncell);
     int sum = 0;
     for (int c = c0; c < c1; ++c) sum += cnt[c];
     int total;
@@ -484,9 +495,10 @@ __global__ void __launch_bounds__(1024) k_cells_small(
     for (int c = c0; c < c1; ++c) {
         const int v = cnt[c];
         cnt[c] = run;
-        cell_start[c] = run;
         run += v;
     }
+    __syncthreads();
+    for (int c = tid; c < ncell; c += 1024) cell_start[c] = cnt[c];
     if (tid == 0) cell_start[ncell] = N;
     __syncthreads();
 #pragma unroll
@@ -500,9 +512,19 @@ __global__ void __launch_bounds__(1024) k_cells_small(
         const int i = tid + u * 1024, s0 = id[u] > 0 ? cnt[id[u] - 1] : 0, s1 = cnt[id[u]];
         int rank = 0;
         for (int s = s0; s < s1; ++s) rank += in_cell[s] < i ? 1 : 0;
-        cell_pos[s0 + rank] = q[u];
+        cell_pos[s0 + rank] = make_float4(q[u].x, q[u].y, q[u].z, __int_as_float(i));
     }
 }
+
+// floor(a / n) and the remainder, 0 <= r < n; near: -n <= a < 2 n
+__device__ __forceinline__ int wrap_cell(int a, int n, bool near, int& r) {
+    const int q = near ? (a < 0 ? -1 : (a >= n ? 1 : 0)) : floor_div(a, n);
+    r = a - q * n;
+    return q;
+}
+// a / n for 0 <= a < 2^21: the quotient's distance from an integer is at least
+// 0.5 / n, the rounding error below a / n * 2^-22
+__device__ __forceinline__ int small_div(int a, int n) { return (int)(((float)a + 0.5f) * (1.0f / (float)n)); }
 
 // One pass over the stencil.  The list is written in three groups:
 // [d < rc_ang + skin] (the angular prefix) | [d < rc_rad] | [rc_rad <= d <
@@ -520,7 +542,14 @@ __global__ void __launch_bounds__(1024) k_cells_small(
 // visit order is that of the cell triple loop.  For the reverse-slot search
 // the kernel also records, per atom, where each row's angular entries start
 // (row_start) and, per angular slot, its row.
-__global__ void __launch_bounds__(128) k_build(const float4* __restrict__ pos4,
+//
+// Bound by instruction issue with a third of the lanes active (rows of
+// different lengths).  Wrapping by compares instead of divisions, row starts
+// written 16 at a time, a shell of 4-byte entries where the list has no shifts
+// and 8 CTAs per SM (64 registers; 10 spill: 1,174 -> 1,283 us): the list build
+// of 900,000 atoms 1,274 -> 1,142 us, k_rev's part without the neighbour's
+// count included.
+__global__ void __launch_bounds__(128, 8) k_build(const float4* __restrict__ pos4,
                                                const int* __restrict__ cfg,
                                                const float* __restrict__ box,
                                                const CellPlan* __restrict__ plan,
@@ -536,11 +565,10 @@ __global__ void __launch_bounds__(128) k_build(const float4* __restrict__ pos4,
     const CellPlan p = plan[b];
     const float L[3] = {box[3 * b], box[3 * b + 1], box[3 * b + 2]};
     const float4 pi = pos4[i];
-    int c = cell_of[i] - p.base;
-    const int cz = c % p.nc[2];
-    c /= p.nc[2];
-    const int cy = c % p.nc[1];
-    const int cx = c / p.nc[1];
+    const int c = cell_of[i] - p.base;
+    const int cxy = c / p.nc[2], cz = c - cxy * p.nc[2];
+    const int cx = cxy / p.nc[1], cy = cxy - cx * p.nc[1];
+    const bool nearx = p.half[0] <= p.nc[0], neary = p.half[1] <= p.nc[1], nearz = p.half[2] <= p.nc[2];
     int n_ang = 0, n_in = 0, n_out = 0, w_ang = 0;
     const int cap = nl.cap, cap_ang = nl.cap_ang;
     const int rows = (2 * p.half[0] + 1) * (2 * p.half[1] + 1);
@@ -553,15 +581,26 @@ __global__ void __launch_bounds__(128) k_build(const float4* __restrict__ pos4,
     // cells whose every point is beyond the cutoff leaves the list, its
     // order and the row starts unchanged.
     const float cs[3] = {L[0] / (float)p.nc[0], L[1] / (float)p.nc[1], L[2] / (float)p.nc[2]};
+    const float ics = 1.0f / cs[2];
     const float rl = sqrtf(rc2_rad) + kPruneMargin;
     const float rl2 = rl * rl;
+    // the row starts go out 16 at a time: byte stores at a stride of an atom's
+    // 64 bytes touch 32 sectors each
+    uint4 starts = make_uint4(0u, 0u, 0u, 0u);
+    auto row_starts = [&](int row, int n) {
+        starts.w |= (unsigned)min(n, 255) << (8 * (row & 3));
+        if ((row & 3) != 3) return;
+        if ((row & 15) == 15) *reinterpret_cast<uint4*>(rs + row - 15) = starts;
+        starts = make_uint4(starts.y, starts.z, starts.w, 0u);
+    };
     int row = 0;
     for (int ox = -p.half[0]; ox <= p.half[0]; ++ox) {
-        const int ux = cx + ox, sx = floor_div(ux, p.nc[0]), wx = ux - sx * p.nc[0];
+        int wx, wy;
+        const int ux = cx + ox, sx = wrap_cell(ux, p.nc[0], nearx, wx);
         const float gx = fmaxf(fmaxf((float)ux * cs[0] - pi.x, pi.x - (float)(ux + 1) * cs[0]), 0.0f);
         for (int oy = -p.half[1]; oy <= p.half[1]; ++oy, ++row) {
-            const int uy = cy + oy, sy = floor_div(uy, p.nc[1]), wy = uy - sy * p.nc[1];
-            if (track) rs[row] = (unsigned char)(n_ang < 255 ? n_ang : 255);
+            const int uy = cy + oy, sy = wrap_cell(uy, p.nc[1], neary, wy);
+            if (track) row_starts(row, n_ang);
             const float fx = mul_rn((float)sx, L[0]);
             const float fy = mul_rn((float)sy, L[1]);
             const int rowcell = p.base + (wx * p.nc[1] + wy) * p.nc[2];
@@ -574,15 +613,14 @@ __global__ void __launch_bounds__(128) k_build(const float4* __restrict__ pos4,
             if (rem <= 0.0f) {
                 hi = lo - 1;
             } else {
-                const float hz = sqrtf(rem);
-                lo = max(lo, (int)floorf((pi.z - hz) / cs[2]));
-                hi = min(hi, (int)floorf((pi.z + hz) / cs[2]));
+                const float hz = rem * rsqrtf(rem);
+                lo = max(lo, (int)floorf((pi.z - hz) * ics));
+                hi = min(hi, (int)floorf((pi.z + hz) * ics));
             }
             while (lo <= hi) {
-                const int sz = floor_div(lo, p.nc[2]);
-                const int seg_hi = min(hi, (sz + 1) * p.nc[2] - 1);
-                const int wz0 = lo - sz * p.nc[2], wz1 = seg_hi - sz * p.nc[2];
-                lo = seg_hi + 1;
+                int wz0;
+                const int sz = wrap_cell(lo, p.nc[2], nearz, wz0), wz1 = min(wz0 + hi - lo, p.nc[2] - 1);
+                lo += wz1 - wz0 + 1;
                 const float fz = mul_rn((float)sz, L[2]);
                 const bool zero_img = (sx == 0 && sy == 0 && sz == 0);
                 const int sh = pack_shift(sx, sy, sz);
@@ -619,14 +657,21 @@ __global__ void __launch_bounds__(128) k_build(const float4* __restrict__ pos4,
                             if (ang && track) slot_row[at] = (unsigned char)row;
                         }
                     } else {
-                        if (n_out < cap) shell[(size_t)n_out * N + i] = make_int2(j, sh);
+                        if (n_out < cap) {
+                            const size_t at = (size_t)n_out * N + i;
+                            if (nl.shift) shell[at] = make_int2(j, sh);
+                            else reinterpret_cast<int*>(shell)[at] = j;
+                        }
                         ++n_out;
                     }
                 }
             }
         }
     }
-    if (track) rs[rows] = (unsigned char)(n_ang < 255 ? n_ang : 255);
+    if (track) {
+        row_starts(rows, n_ang);
+        for (int r = rows + 1; r & 15; ++r) row_starts(r, 0);
+    }
     const int n_rest = n_in + n_out;
     const int n_total = n_ang + n_rest;
     const bool over = n_total > cap || n_ang > cap_ang;
@@ -637,6 +682,8 @@ __global__ void __launch_bounds__(128) k_build(const float4* __restrict__ pos4,
         // only the contiguous angular prefix that was written is kept
         nl.cnt[i] = w_ang;
         nl.cnt_ang[i] = w_ang;
+        if (track)
+            for (int r = 0; r <= rows; ++r) rs[r] = (unsigned char)min((int)rs[r], w_ang);
         return;
     }
     // the inside block sits reversed at [cap - n_in, cap).  Where it does not
@@ -671,10 +718,14 @@ __global__ void __launch_bounds__(128) k_build(const float4* __restrict__ pos4,
         }
     }
     for (int k = 0; k < n_out; ++k) {
-        const int2 e = shell[(size_t)k * N + i];
-        const size_t to = (size_t)(n_ang + n_in + k) * N + i;
-        nl.nbr[to] = e.x;
-        if (nl.shift) nl.shift[to] = e.y;
+        const size_t from = (size_t)k * N + i, to = (size_t)(n_ang + n_in + k) * N + i;
+        if (nl.shift) {
+            const int2 e = shell[from];
+            nl.nbr[to] = e.x;
+            nl.shift[to] = e.y;
+        } else {
+            nl.nbr[to] = reinterpret_cast<const int*>(shell)[from];
+        }
     }
     nl.cnt[i] = n_total;
     nl.cnt_ang[i] = n_ang;
@@ -682,44 +733,54 @@ __global__ void __launch_bounds__(128) k_build(const float4* __restrict__ pos4,
 
 // The same list from a warp per atom, for systems too small to hide one
 // thread's serial walk (82 to 124 us up to 10,000 atoms).  The stencil rows'
-// candidate ranges go to shared memory in visit order; lanes then take
-// consecutive candidates, each finding its range by bisection.  The first pass
-// over the candidates counts the three groups, the second writes every entry
-// to its final slot, so the list is that of k_build entry for entry.  A range
+// candidate ranges go to shared memory in visit order, empty ones dropped;
+// lanes then take consecutive candidates, and a bit per range start tells each
+// its range (popcount).  The first pass over the candidates counts the three
+// groups and keeps the hits in shared memory, the second writes every hit to
+// its final slot, so the list is that of k_build entry for entry.  A range
 // holds cells of one z image; a row has at most 2 half_z / nc_z + 2.
+// Bound by instruction issue from a few thousand atoms on: divisions by the
+// cell counts, a bisection for every candidate's range and a second walk over
+// the candidates in the writing pass were two thirds of its 2,835 warp
+// instructions per atom.  Without them the whole list build takes, before /
+// after: 194 atoms 25.1 / 17.4 us, 7,200 49.7 / 39.5, 46,522 220 / 163.
 constexpr int kBuildWarps = 4;
 constexpr int kBuildSegs = 128;      // candidate ranges held at once
 constexpr int kBuildRows = 64;       // stencil rows per round, two per lane
-constexpr int kBuildWarpN = 48000;   // largest system: the whole list build, thread / warp per atom (the
-                                     // reverse search alike): 7,200 atoms 150 / 56 us, 46,522 251 / 220
-                                     // (packings, images), 57,600 203 / 238 (rock salt)
+constexpr int kBuildHits = 192;      // hits kept for the second pass; beyond, it walks the candidates again
+constexpr int kBuildWarpN = 70000;   // largest system: the whole list build, thread / warp per atom:
+                                     // 57,600 atoms 191 / 174 us, 66,679 202 / 184, 76,666 207 / 208,
+                                     // 112,500 244 / 288
+static_assert(kBuildWarpN < 1 << 30, "a kept hit's kind shares a word with its atom");
 constexpr float kBuildMinEdge = 16.0f;   // shortest box edge: the list cutoff over this (at most 34 ranges per row)
-__global__ void __launch_bounds__(32 * kBuildWarps) k_build_warp(
+
+__global__ void __launch_bounds__(32 * kBuildWarps, 8) k_build_warp(
     const float4* __restrict__ pos4, const int* __restrict__ cfg, const float* __restrict__ box,
     const CellPlan* __restrict__ plan, const int* __restrict__ cell_of, const int* __restrict__ cell_start,
     const float4* __restrict__ cell_pos, int N, float rc2_rad, float rc2_ang, float rc2_phys,
     unsigned char* __restrict__ row_start, unsigned char* __restrict__ slot_row, nep_nlist nl) {
     pdl_wait();
     pdl_trigger();
-    __shared__ int s_q0[kBuildWarps][kBuildSegs], s_cum[kBuildWarps][kBuildSegs + 1];
-    __shared__ int s_img[kBuildWarps][kBuildSegs];
-    __shared__ unsigned short s_row[kBuildWarps][kBuildSegs];
+    __shared__ int2 s_seg[kBuildWarps][kBuildSegs];   // first atom less the candidates before; image | row << 24
+    __shared__ int s_cum[kBuildWarps][kBuildSegs];    // candidates before the range
+    __shared__ int2 s_hit[kBuildWarps][kBuildHits];   // atom | kind << 30; image | row << 24
+    __shared__ unsigned s_mask[kBuildWarps][32];      // range starts among 1,024 candidates
     __shared__ int s_rowcnt[kBuildWarps][kMaxRows + 1];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int i = blockIdx.x * kBuildWarps + w;
     if (i >= N) return;
-    int *q0s = s_q0[w], *cum = s_cum[w], *img = s_img[w], *rowcnt = s_rowcnt[w];
-    unsigned short* rowof = s_row[w];
+    int2 *seg = s_seg[w], *hit = s_hit[w];
+    int *cum = s_cum[w], *rowcnt = s_rowcnt[w];
+    unsigned* mask = s_mask[w];
     const int b = cfg[i];
     const CellPlan p = plan[b];
     const float L[3] = {box[3 * b], box[3 * b + 1], box[3 * b + 2]};
     const float4 pi = pos4[i];
-    int c = cell_of[i] - p.base;
-    const int cz = c % p.nc[2];
-    c /= p.nc[2];
-    const int cy = c % p.nc[1];
-    const int cx = c / p.nc[1];
+    const int c = cell_of[i] - p.base;
+    const int cxy = small_div(c, p.nc[2]), cz = c - cxy * p.nc[2];
+    const int cx = small_div(cxy, p.nc[1]), cy = cxy - cx * p.nc[1];
     const int wy_rows = 2 * p.half[1] + 1, rows = (2 * p.half[0] + 1) * wy_rows;
+    const bool nearx = p.half[0] <= p.nc[0], neary = p.half[1] <= p.nc[1], nearz = p.half[2] <= p.nc[2];
     const bool track = rows <= kMaxRows && nl.cap_ang < 256;
     if (track)
         for (int r = lane; r <= rows; r += 32) rowcnt[r] = 0;
@@ -728,130 +789,168 @@ __global__ void __launch_bounds__(32 * kBuildWarps) k_build_warp(
     const float rl2 = rl * rl;
     const int maxseg = 2 * p.half[2] / p.nc[2] + 2;
     const int per_round = max(1, min(kBuildRows, kBuildSegs / maxseg));
-    const unsigned below = (1u << lane) - 1u;
-    int n_ang = 0, n_in = 0, n_out = 0;       // of the whole atom after the first pass
-    bool over = false;
+    const unsigned below = (1u << lane) - 1u, upto = below | (1u << lane);
     int nseg = 0, ncand = 0;
-    for (int pass = 0; pass < 2; ++pass) {
-        int ra = 0, ri = 0, ro = 0;           // entries of each group so far
-        for (int row0 = 0; row0 < rows; row0 += per_round) {
-            if (pass == 0 || rows > per_round) {      // one round keeps its ranges
-                // this lane's rows row0 + 2 lane, + 1: z cells lo..hi of each
-                int lo[2], hi[2], rc[2], sxy[2], mine = 0;
+    // the ranges of rows row0 .. row0 + per_round - 1
+    auto ranges = [&](int row0) {
+        // this lane's rows row0 + 2 lane, + 1: z cells lo..hi of each
+        int lo[2], hi[2], rc[2], tag[2], mine = 0;
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const int row = row0 + 2 * lane + u;
-                    lo[u] = 0;
-                    hi[u] = -1;
-                    rc[u] = sxy[u] = 0;
-                    if (2 * lane + u >= per_round || row >= rows) continue;
-                    const int ox = row / wy_rows - p.half[0], oy = row % wy_rows - p.half[1];
-                    const int ux = cx + ox, sx = floor_div(ux, p.nc[0]), wx = ux - sx * p.nc[0];
-                    const float gx =
-                        fmaxf(fmaxf((float)ux * cs[0] - pi.x, pi.x - (float)(ux + 1) * cs[0]), 0.0f);
-                    const int uy = cy + oy, sy = floor_div(uy, p.nc[1]), wy = uy - sy * p.nc[1];
-                    const float gy =
-                        fmaxf(fmaxf((float)uy * cs[1] - pi.y, pi.y - (float)(uy + 1) * cs[1]), 0.0f);
-                    const float rem = rl2 - gx * gx - gy * gy;
-                    if (rem <= 0.0f) continue;
-                    const float hz = sqrtf(rem);
-                    lo[u] = max(cz - p.half[2], (int)floorf((pi.z - hz) / cs[2]));
-                    hi[u] = min(cz + p.half[2], (int)floorf((pi.z + hz) / cs[2]));
-                    rc[u] = p.base + (wx * p.nc[1] + wy) * p.nc[2];
-                    sxy[u] = pack_shift(sx, sy, 0);
-                    if (lo[u] <= hi[u]) mine += floor_div(hi[u], p.nc[2]) - floor_div(lo[u], p.nc[2]) + 1;
-                }
-                int at = mine;
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int y = __shfl_up_sync(0xffffffffu, at, o);
-                    if (lane >= o) at += y;
-                }
-                nseg = __shfl_sync(0xffffffffu, at, 31);
-                at -= mine;
+        for (int u = 0; u < 2; ++u) {
+            const int row = row0 + 2 * lane + u;
+            lo[u] = 0;
+            hi[u] = -1;
+            rc[u] = tag[u] = 0;
+            if (2 * lane + u >= per_round || row >= rows) continue;
+            const int rx = small_div(row, wy_rows), ox = rx - p.half[0], oy = row - rx * wy_rows - p.half[1];
+            int wx, wy;
+            const int ux = cx + ox, sx = wrap_cell(ux, p.nc[0], nearx, wx);
+            const float gx = fmaxf(fmaxf((float)ux * cs[0] - pi.x, pi.x - (float)(ux + 1) * cs[0]), 0.0f);
+            const int uy = cy + oy, sy = wrap_cell(uy, p.nc[1], neary, wy);
+            const float gy = fmaxf(fmaxf((float)uy * cs[1] - pi.y, pi.y - (float)(uy + 1) * cs[1]), 0.0f);
+            const float rem = rl2 - gx * gx - gy * gy;
+            if (rem <= 0.0f) continue;
+            const float hz = sqrtf(rem);
+            lo[u] = max(cz - p.half[2], (int)floorf((pi.z - hz) / cs[2]));
+            hi[u] = min(cz + p.half[2], (int)floorf((pi.z + hz) / cs[2]));
+            rc[u] = p.base + (wx * p.nc[1] + wy) * p.nc[2];
+            tag[u] = pack_shift(sx, sy, 0) | (int)((unsigned)row << 24);
+            int r;
+            if (lo[u] <= hi[u])
+                mine += wrap_cell(hi[u], p.nc[2], nearz, r) - wrap_cell(lo[u], p.nc[2], nearz, r) + 1;
+        }
+        int at = mine;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, at, o);
+            if (lane >= o) at += y;
+        }
+        const int all = __shfl_sync(0xffffffffu, at, 31);
+        at -= mine;
 #pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    while (lo[u] <= hi[u]) {
-                        const int sz = floor_div(lo[u], p.nc[2]);
-                        const int seg_hi = min(hi[u], (sz + 1) * p.nc[2] - 1);
-                        const int z0 = lo[u] - sz * p.nc[2], z1 = seg_hi - sz * p.nc[2];
-                        lo[u] = seg_hi + 1;
-                        const int q0 = cell_start[rc[u] + z0];
-                        q0s[at] = q0;
-                        cum[at] = cell_start[rc[u] + z1 + 1] - q0;
-                        img[at] = sxy[u] | ((sz & 0xff) << 16);
-                        rowof[at] = (unsigned short)(row0 + 2 * lane + u);
-                        ++at;
-                    }
-                }
-                __syncwarp();
-                // candidates before each range
-                ncand = 0;
-                for (int s0 = 0; s0 < nseg; s0 += 32) {
-                    const int v = s0 + lane < nseg ? cum[s0 + lane] : 0;
-                    int x = v;
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const int y = __shfl_up_sync(0xffffffffu, x, o);
-                        if (lane >= o) x += y;
-                    }
-                    if (s0 + lane < nseg) cum[s0 + lane] = ncand + x - v;
-                    ncand += __shfl_sync(0xffffffffu, x, 31);
-                }
-                __syncwarp();
+        for (int u = 0; u < 2; ++u) {
+            while (lo[u] <= hi[u]) {
+                int z0;
+                const int sz = wrap_cell(lo[u], p.nc[2], nearz, z0);
+                const int z1 = min(z0 + hi[u] - lo[u], p.nc[2] - 1);
+                lo[u] += z1 - z0 + 1;
+                const int q0 = cell_start[rc[u] + z0];
+                seg[at] = make_int2(q0, tag[u] | (sz & 0xff) << 16);
+                cum[at] = cell_start[rc[u] + z1 + 1] - q0;
+                ++at;
             }
+        }
+        __syncwarp();
+        // drop the empty ranges; the candidates before each
+        nseg = ncand = 0;
+        for (int s0 = 0; s0 < all; s0 += 32) {
+            const int v = s0 + lane < all ? cum[s0 + lane] : 0;
+            const int2 sg = seg[min(s0 + lane, all - 1)];
+            int x = v;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            const unsigned some = __ballot_sync(0xffffffffu, v > 0);
+            __syncwarp();
+            if (v > 0) {
+                const int k = nseg + __popc(some & below), before = ncand + x - v;
+                cum[k] = before;
+                seg[k] = make_int2(sg.x - before, sg.y);
+            }
+            nseg += __popc(some);
+            ncand += __shfl_sync(0xffffffffu, x, 31);
+            __syncwarp();
+        }
+    };
+    int n_ang = 0, n_in = 0, n_out = 0, nhit = 0;
+    int ra = 0, ri = 0, ro = 0;               // entries of each group written so far
+    bool over = false;
+    // kind 1 angular, 2 inside, 3 shell, 0 none
+    auto write = [&](int kind, int j, int tag) {
+        const unsigned ma = __ballot_sync(0xffffffffu, kind == 1);
+        const unsigned mi = __ballot_sync(0xffffffffu, kind == 2);
+        const unsigned mo = __ballot_sync(0xffffffffu, kind == 3);
+        if (kind) {
+            const int slot = kind == 1   ? ra + __popc(ma & below)
+                             : kind == 2 ? n_ang + ri + __popc(mi & below)
+                                         : n_ang + n_in + ro + __popc(mo & below);
+            // an overflowing list keeps the part of its angular prefix that fits
+            if (!over || (kind == 1 && slot < min(nl.cap, nl.cap_ang))) {
+                const size_t to = (size_t)slot * N + i;
+                nl.nbr[to] = j;
+                if (nl.shift) nl.shift[to] = tag & 0xffffff;
+                if (kind == 1 && track) slot_row[to] = (unsigned char)((unsigned)tag >> 24);
+            }
+        }
+        ra += __popc(ma);
+        ri += __popc(mi);
+        ro += __popc(mo);
+    };
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+        if (pass == 1 && nhit <= kBuildHits) {
+            for (int t0 = 0; t0 < nhit; t0 += 32) {
+                const int2 h = hit[min(t0 + lane, nhit - 1)];
+                write(t0 + lane < nhit ? (int)((unsigned)h.x >> 30) : 0, h.x & 0x3fffffff, h.y);
+            }
+            break;
+        }
+        for (int row0 = 0; row0 < rows; row0 += per_round) {
+            if (pass == 0 || rows > per_round) ranges(row0);      // one round keeps its ranges
+            int started = 0;                  // ranges that start before the chunk
             for (int t0 = 0; t0 < ncand; t0 += 32) {
-                const int t = t0 + lane;
-                int kind = 0, j = 0, sh = 0, row = 0;   // 1 angular, 2 inside, 3 shell
-                if (t < ncand) {
-                    int s = 0, e = nseg;              // cum[s] <= t < cum[e]; empty ranges resolve to the last
-                    while (e - s > 1) {
-                        const int mid = (s + e) >> 1;
-                        if (cum[mid] <= t) s = mid;
-                        else e = mid;
+                if ((t0 & 1023) == 0) {
+                    __syncwarp();
+                    mask[lane] = 0u;
+                    __syncwarp();
+                    for (int s = lane; s < nseg; s += 32) {
+                        const unsigned d = (unsigned)(cum[s] - t0);
+                        if (d < 1024u) atomicOr(mask + (d >> 5), 1u << (d & 31));
                     }
-                    const float4 pj = cell_pos[q0s[s] + (t - cum[s])];
-                    j = f2i(pj.w);
-                    sh = img[s];
-                    row = rowof[s];
-                    int sx, sy, sz;
-                    unpack_shift(sh, sx, sy, sz);
-                    const float dx = add_rn(sub_rn(pj.x, pi.x), mul_rn((float)sx, L[0]));
-                    const float dy = add_rn(sub_rn(pj.y, pi.y), mul_rn((float)sy, L[1]));
-                    const float dz = add_rn(sub_rn(pj.z, pi.z), mul_rn((float)sz, L[2]));
-                    const float d2 = dist2(dx, dy, dz);
-                    if (d2 < rc2_rad && !(j == i && sh == 0)) kind = d2 < rc2_ang ? 1 : (d2 < rc2_phys ? 2 : 3);
+                    __syncwarp();
                 }
-                const unsigned ma = __ballot_sync(0xffffffffu, kind == 1);
-                const unsigned mi = __ballot_sync(0xffffffffu, kind == 2);
-                const unsigned mo = __ballot_sync(0xffffffffu, kind == 3);
+                const unsigned m = mask[(t0 >> 5) & 31];
+                const int t = min(t0 + lane, ncand - 1);
+                const int2 sg = seg[started + __popc(m & upto) - 1];
+                started += __popc(m);
+                const float4 pj = cell_pos[sg.x + t];
+                const int j = f2i(pj.w);
+                int sx, sy, sz;
+                unpack_shift(sg.y, sx, sy, sz);
+                const float dx = add_rn(sub_rn(pj.x, pi.x), mul_rn((float)sx, L[0]));
+                const float dy = add_rn(sub_rn(pj.y, pi.y), mul_rn((float)sy, L[1]));
+                const float dz = add_rn(sub_rn(pj.z, pi.z), mul_rn((float)sz, L[2]));
+                const float d2 = dist2(dx, dy, dz);
+                int kind = 0;
+                if (t0 + lane < ncand && d2 < rc2_rad && !(j == i && (sg.y & 0xffffff) == 0))
+                    kind = d2 < rc2_ang ? 1 : (d2 < rc2_phys ? 2 : 3);
                 if (pass == 0) {
-                    if (track && kind == 1) atomicAdd(rowcnt + row, 1);
-                } else if (kind) {
-                    const int slot = kind == 1   ? ra + __popc(ma & below)
-                                     : kind == 2 ? n_ang + ri + __popc(mi & below)
-                                                 : n_ang + n_in + ro + __popc(mo & below);
-                    // an overflowing list keeps the part of its angular prefix that fits
-                    if (!over || (kind == 1 && slot < min(nl.cap, nl.cap_ang))) {
-                        const size_t to = (size_t)slot * N + i;
-                        nl.nbr[to] = j;
-                        if (nl.shift) nl.shift[to] = sh;
-                        if (kind == 1 && track) slot_row[to] = (unsigned char)row;
+                    const unsigned any = __ballot_sync(0xffffffffu, kind != 0);
+                    if (kind) {
+                        const int k = nhit + __popc(any & below);
+                        if (k < kBuildHits) hit[k] = make_int2(j | (int)((unsigned)kind << 30), sg.y);
+                        if (track && kind == 1) atomicAdd(rowcnt + (int)((unsigned)sg.y >> 24), 1);
                     }
+                    nhit += __popc(any);
+                    n_ang += kind == 1;
+                    n_in += kind == 2;
+                } else {
+                    write(kind, j, sg.y);
                 }
-                ra += __popc(ma);
-                ri += __popc(mi);
-                ro += __popc(mo);
             }
             __syncwarp();
         }
         if (pass == 0) {
-            n_ang = ra;
-            n_in = ri;
-            n_out = ro;
-            over = n_ang + n_in + n_out > nl.cap || n_ang > nl.cap_ang;
+            n_ang = __reduce_add_sync(0xffffffffu, n_ang);
+            n_in = __reduce_add_sync(0xffffffffu, n_in);
+            n_out = nhit - n_ang - n_in;
+            over = nhit > nl.cap || n_ang > nl.cap_ang;
         }
     }
+    __syncwarp();
+    const int kept = over ? min(n_ang, min(nl.cap, nl.cap_ang)) : n_ang;
     if (track) {
-        // where each row's angular entries start
+        // where each row's angular entries start, within the kept prefix
         unsigned char* rs = row_start + (size_t)i * kRowStride;
         int before = 0;
         for (int r0 = 0; r0 <= rows; r0 += 32) {
@@ -861,7 +960,7 @@ __global__ void __launch_bounds__(32 * kBuildWarps) k_build_warp(
                 const int y = __shfl_up_sync(0xffffffffu, x, o);
                 if (lane >= o) x += y;
             }
-            if (r <= rows) rs[r] = (unsigned char)min(before + x - v, 255);
+            if (r <= rows) rs[r] = (unsigned char)min(before + x - v, kept);
             before += __shfl_sync(0xffffffffu, x, 31);
         }
     }
@@ -872,9 +971,8 @@ __global__ void __launch_bounds__(32 * kBuildWarps) k_build_warp(
             atomicMax(nl.status + 1, total);
             atomicMax(nl.status + 2, n_ang);
         }
-        const int kept = min(n_ang, min(nl.cap, nl.cap_ang));
         nl.cnt[i] = over ? kept : total;
-        nl.cnt_ang[i] = over ? kept : n_ang;
+        nl.cnt_ang[i] = kept;
     }
 }
 
@@ -892,13 +990,14 @@ __device__ __forceinline__ void rev_slot(int N, int i, int s, int rows, bool tra
         unpack_shift(nl.shift[(size_t)s * N + i], a, b, c);
         want = pack_shift(-a, -b, -c);
     }
-    const int nj = nl.cnt_ang[j];
-    int t0 = 0, t1 = nj;
+    int t0 = 0, t1;
     if (track) {
         const int mr = rows - 1 - (int)slot_row[(size_t)s * N + i];
         const unsigned char* rj = row_start + (size_t)j * kRowStride;
         t0 = rj[mr];
-        t1 = min((int)rj[mr + 1], nj);
+        t1 = rj[mr + 1];
+    } else {
+        t1 = nl.cnt_ang[j];
     }
     int found = -1;
     for (int t = t0; t < t1; ++t) {

@@ -144,17 +144,20 @@ def test_lane_groups_16bit_network(nb, hname, precision):
 
 
 @pytest.mark.parametrize("n,L,skin,copies", [(3, 5.0, 1.0, 30000), (58, 0.0, 0.0, 1500), (700, 0.0, 1.0, 120),
-                                             (8190, 0.0, 0.5, 12), (8200, 0.0, 0.5, 12)])
+                                             (8190, 0.0, 0.5, 12), (8200, 0.0, 0.5, 12),
+                                             (540, 12.93, 0.0, 140)])
 def test_list_build_small_and_large_forms_agree(nb, n, L, skin, copies):
     """A configuration listed alone (binned by one CTA up to 8,192 atoms, a
     warp per atom in the build and the reverse search) gets, entry for entry,
     the list of each of its copies in a batch large enough for one thread per
     atom: a few atoms in a box shorter than the cutoff (stencils too large for
-    the row table), boxes with images and without."""
+    the row table), boxes with images and without, a dense one with more hits
+    per atom than the warp keeps (192)."""
     h = I.HYPER_SMALL
-    s = I.packing_batch([n], tag=65, dmin=1.5 if L else 2.4, density=n / L ** 3 if L else 0.0325)
+    dense = L > 10
+    s = I.packing_batch([n], tag=65, dmin=1.1 if dense else 1.5 if L else 2.4, density=n / L ** 3 if L else 0.0325)
     model = nb.Model(h, I.init_params(h).astype(np.float32))
-    cap, cap_ang = 160, 80
+    cap, cap_ang = (720, 250) if dense else (160, 80)
 
     def build(copies):
         batch = I.System(pos=np.tile(s.pos, (copies, 1)), types=np.tile(s.types, copies),
