@@ -425,6 +425,8 @@ __device__ __forceinline__ int floor_div(int a, int b) {
 // loaded before the first is used, and configurations' offsets, boxes and
 // plans are read from shared memory (7,200 atoms 19.8 -> 14.4 us).
 constexpr int kCellsSmallN = 8192, kCellsSmallB = 256;
+constexpr int kCellsSmallStatic = (int)(sizeof(int) * kCellsSmallN + (sizeof(CellPlan) + 3 * sizeof(float)) * kCellsSmallB +
+                                        sizeof(int) * (kCellsSmallB + 1 + 32)) + 64;   // and padding
 __global__ void __launch_bounds__(1024) k_cells_small(
     const float* __restrict__ pos, const int* __restrict__ type, const int* __restrict__ atom_off,
     const float* __restrict__ box, int N, int B, int T, float rc, float4* pos4, int* cfg, int* status,
@@ -1275,8 +1277,8 @@ cudaError_t launch_neighbors(const float* pos, const int* type, int T, float4* p
     const int cmax = w.cmax;
     if (N > 0 && N <= kCellsSmallN && B <= kCellsSmallB) {
         const int smem = (int)sizeof(int) * (cmax + 1);
-        // 93 KB at most (with 32 KB of static), which needs the attribute
-        if (smem > 8 * 1024 &&
+        // with the static arrays past 48 KB (138 KB at most), which needs the attribute
+        if (smem + kCellsSmallStatic > 48 * 1024 &&
             (e = cudaFuncSetAttribute(k_cells_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sizeof(int) * (2 * kCellsSmallN + 27 * kCellsSmallB + 1))))
             return e;

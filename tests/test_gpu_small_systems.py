@@ -184,6 +184,21 @@ def test_list_build_small_and_large_forms_agree(nb, n, L, skin, copies):
             assert np.array_equal(one[4][used], many[4][:, cols][used])
 
 
+@pytest.mark.parametrize("n", [200, 480, 500, 900, 2100])
+def test_first_list_of_a_process(n):
+    """The one-block binning asks for its shared memory at every size that
+    needs it, also when no larger system came before: each in a new process."""
+    import subprocess
+    import sys
+    code = ("import numpy as np\nfrom paper_2607_06969_gb300 import binding as nb, inputs as I\n"
+            f"s = I.packing_batch([{n}], tag=67)\nh = I.HYPER_SMALL\n"
+            "m = nb.Model(h, I.init_params(h).astype(np.float32))\nd = nb.DeviceSystem.from_inputs(s)\n"
+            "nl = nb.NeighborList(s.n_atoms, 128, 64)\nws = nb.Workspace(m, s.n_atoms, 1, 128, 64)\n"
+            "nb.neighbors(m, d, nl, 0.0, ws)\nassert nb.check_list(nl) == nb.NEP_OK, nb.last_error()\n")
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
+
+
 @pytest.mark.parametrize("hname", list(MODELS))
 @pytest.mark.parametrize("counts,skin", [([1], 0.0), ([2, 0, 3], 0.0), ([24, 127, 130], 0.7), ([900, 1101], 0.0),
                                          ([1500, 1501], 0.0)])
