@@ -87,8 +87,9 @@ size_t nep_num_params(const nep_hparams* hp);
  * A shape with a compiled kernel set (nep_supported = 1) gets the fast path:
  * FP32, FP16 or BF16 network, every call.  Any other FP32 shape with n_rad,
  * n_ang <= 16 and k_rad, k_ang <= 16 (nep_supported = 2) gets the generic
- * path: runtime-shaped FP32 kernels that evaluate each pair term from both of
- * its atoms (about twice the fast path's pair work).  A generic model serves
+ * path: FP32 kernels with compiled bounds on the shape that evaluate each pair
+ * term from both of its atoms (about twice the fast path's pair work).  A
+ * generic model serves
  * nep_neighbors, the FP32 evaluations (nep_energy_forces_virial, _owned,
  * _noalloc), nep_md_step and the FP64 calls; nep_param_grad,
  * nep_param_grad_adjoint and nep_autotune return NEP_ERR_UNSUPPORTED (its
@@ -195,8 +196,8 @@ nep_status nep_energy_forces_virial(nep_model* m, const nep_system* sys, const n
  *   e_atom [N] double (may be NULL), force [3][N] double,
  *   e_tot [B] double, virial [B][9] double (row-major V_ab, Eq. 4)
  *   work   : >= nep_workspace_bytes_fp64(m, N, B) bytes, 256-byte aligned
- * One thread per atom; every pair term is evaluated by both of its atoms, so
- * the call is deterministic and allocation-free.  Needs n_rad, n_ang <= 16 and
+ * A group of lanes per atom; every pair term is evaluated by both of its atoms,
+ * so the call is deterministic and allocation-free.  Needs n_rad, n_ang <= 16 and
  * k_rad, k_ang <= 16 (else NEP_ERR_UNSUPPORTED); any precision setting. */
 size_t nep_workspace_bytes_fp64(const nep_model* m, int n_atoms, int n_cfg);
 nep_status nep_energy_forces_virial_fp64(nep_model* m, const nep_system* sys, const nep_nlist* nl,
@@ -409,34 +410,43 @@ nep_status nep_md_step(nep_model* m, const nep_system* sys, nep_nlist* nl, float
  *   the finish kernel at 64, 128 and 256 threads per block.
  * The fastest of each is stored in the model for the system's size class
  * (log2 of the mean atom count per configuration); later hot calls on
- * systems of that class use them.  Small systems gain from small blocks (more
- * blocks cover more SMs); large ones do not care.  Not a hot call: it
+ * systems of that class use them where these kernels run.  Smaller systems
+ * run kernels with several lanes per atom, whose choices are fixed, unless
+ * the class is pinned below: the radial kernel up to 200,000 atoms, the finish
+ * kernel up to 50,000, the angular kernel up to 10,000 (13,500 and 25,000 with
+ * the 16-bit network of narrow and wide models).  Not a hot call: it
  * synchronises `stream` and overwrites the workspace's scratch.
  * chosen[3] (may be NULL) receives the angular variant index (0, 1, 2 = 2, 3,
  * 4 blocks per SM), the radial and the finish block size.  Untuned classes
- * use variant 0, 256 (radial) and 128 (finish). */
+ * use variant 0 and 64 threads for both. */
 nep_status nep_autotune(nep_model* m, const nep_system* sys, const nep_nlist* nl, void* work,
                         size_t work_bytes, void* stream, int reps, int* chosen);
 
 /* Pin the angular kernel variant (0, 1, 2 = 2, 3, 4 resident blocks per SM;
  * -1 = back to the default) for one size class (0..31, as in nep_autotune)
- * or for all of them (size_class = -1).  Host only, no device work. */
+ * or for all of them (size_class = -1).  A pinned class runs one thread per
+ * atom at every size, the 16-bit networks on the tensor cores; otherwise small
+ * systems take the lane-group kernels, which round the same operands to 16
+ * bits and accumulate in FP32.  Host only, no device work. */
 nep_status nep_set_variant(nep_model* m, int size_class, int variant);
 
 /* Pin every launch choice of nep_autotune for one size class or all of them
  * (size_class = -1): the angular variant (-1 = default) and the radial and
- * finish block sizes (64, 128, 256, or 0 = default).  Host only.
- * NEP_ERR_ARG for any other value. */
+ * finish block sizes (64, 128, 256, or 0 = default).  A class with any choice
+ * but the defaults is pinned as by nep_set_variant.  Host only.  NEP_ERR_ARG
+ * for any other value. */
 nep_status nep_set_launch(nep_model* m, int size_class, int variant, int radial_block, int finish_block);
 
 /* Profiling hook: the next nep_energy_forces_virial / nep_md_step call of
  * this model records events[0] before the radial kernel (radial sums,
  * angular pair compaction), events[1] after it, events[2] after the angular
  * kernel (angular descriptors, network, angular pair forces) and events[3]
- * after the kernel that completes the forces, on the call's stream (events
- * are caller-created cudaEvent_t, n = 4; n = 0 clears).  One-shot: the
- * events are forgotten after that call.  The records are ordinary stream work
- * and can be captured into a CUDA graph. */
+ * after the kernels that complete the forces and the totals, on the call's
+ * stream.  Where one kernel does the radial and the angular work (small
+ * systems), events[1] comes before it.  (Events are caller-created
+ * cudaEvent_t, n = 4; n = 0 clears.)  One-shot: the events are forgotten after
+ * that call.  The records are ordinary stream work and can be captured into a
+ * CUDA graph. */
 nep_status nep_set_timing_events(nep_model* m, void* const* events, int n);
 
 /* Measurement helper, not part of the NEP path: the FP32 FMA throughput of

@@ -248,6 +248,12 @@ int finish_block(const nep_model* m, const nep_system* s) { return m->tune_finis
 //     15,818: 80.5 / 71.8, -, 115.9 / 110.7; 19,757: 93.2 / 90.1, -, 137.9 / 148.2;
 //     24,300: -, -, 148.8 / 154; 29,491: 119 / 102, -, 183 / 162 (the tensor-core
 //     kernel's tiles of 128 atoms fill whole waves up to 19,456 and 38,912 atoms)
+//   finish kernel, 32 / 16 / 8 lanes (the atom kernel at its best): 2,470 atoms
+//     30.8 / 31.4 / 32.7 us, 33.2 / 33.4 / 35.1, 34.6 / 35.0 / 36.2; 5,249: - /
+//     39.5 / 39.3, 44.9 / 44.5, 49.1 / 51.4; 7,200: - / 42.7 / 45.1, 46.5 / 48.6,
+//     59.1 / 61.7; 9,583: - / 54.1 / 49.0, 68.9 / 64.8, 72.9 / 68.9; ten MD steps of
+//     7,200 atoms 517 / 551, but with images a list and an evaluation of 48
+//     configurations with 5,800 atoms 100.8 / 97.0
 //   finish kernel, 8 lanes against one thread: 41,990 atoms 119 / 127, 149 / 156,
 //     170 / 179; 57,600: 146 / 145, 172 / 171, 192 / 193; 99,533: 260 / 231
 //   radial kernel, four lanes against one thread: 57,600 atoms 145 / 151, 171 /
@@ -256,7 +262,7 @@ int finish_block(const nep_model* m, const nep_system* s) { return m->tune_finis
 struct EvalSplit {
     int atom, finish, radial;
 };
-EvalSplit eval_split(const nep_model* m, const nep_system* s) {
+EvalSplit eval_split(const nep_model* m, const nep_system* s, bool images) {
     const int N = s->n_atoms, bin = size_bin(s);
     EvalSplit e{0, 0, m->tune_radial[bin]};
     if (N == 0 || m->pinned[bin]) return e;
@@ -264,7 +270,7 @@ EvalSplit eval_split(const nep_model* m, const nep_system* s) {
         const bool wide = m->hp.n_hidden * m->lay.D > 2500;
         const int most = !m->hp.precision ? 10000 : wide ? 25000 : 13500;
         e.atom = N > most ? 0 : N <= (wide ? 8000 : 3000) ? 32 : 8;
-        e.finish = N > 50000 ? 0 : N <= 3000 ? 32 : 8;
+        e.finish = N > 50000 ? 0 : N <= 3000 ? 32 : N <= 8000 && !images ? 16 : 8;
     }
     if (N <= 200000) e.radial = nep::kRadialSplit;
     return e;
@@ -507,7 +513,7 @@ nep_status efv_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, floa
     auto mark = [&](int k) -> cudaError_t {
         return nt ? cudaEventRecordWithFlags(m->timing[k], st, rec_flags) : cudaSuccess;
     };
-    const EvalSplit sp = eval_split(m, s);
+    const EvalSplit sp = eval_split(m, s, !nl->min_image);
     NEP_CUDA(mark(0), "timing event");
     if (sp.atom) {
         NEP_CUDA(mark(1), "timing event");       // the radial sums are part of the next kernel
@@ -554,7 +560,7 @@ nep_status train_impl(nep_model* m, const nep_system* s, const nep_nlist* nl, co
     nep::EvalArgs a = make_args(m, s, nl, work, w);
     a.q16_kind = 0;
     const int G = train_lanes(m, s, e_lbl != nullptr);
-    const EvalSplit sp = G ? eval_split(m, s) : EvalSplit{0, 0, 0};
+    const EvalSplit sp = G ? eval_split(m, s, !nl->min_image) : EvalSplit{0, 0, 0};
     if (!G) {
         // the training variants of the forward kernels leave their records for the backward
         a.S = at<float>(work, w.S);

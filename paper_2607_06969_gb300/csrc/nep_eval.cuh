@@ -965,17 +965,19 @@ __global__ void __launch_bounds__(128, 8) k_radial_split(const EvalArgs a) {
     const int gbase = (threadIdx.x & 31) & ~(G - 1);
     const unsigned gmask = (1u << G) - 1u, below = (1u << lane) - 1u;
     int nc = 0, nr = 0;
-    int j1 = lane < cnt ? a.nbr[lane * N + i] : i;
-    int j2 = lane + G < cnt ? a.nbr[(lane + G) * N + i] : i;
+    int j1 = lane < cnt ? a.nbr[lane * N + i] : i, j2 = lane + G < cnt ? a.nbr[(lane + G) * N + i] : i;
+    int h1 = !MINIMG && lane < cnt ? a.shift[lane * N + i] : 0;
+    int h2 = !MINIMG && lane + G < cnt ? a.shift[(lane + G) * N + i] : 0;
     float4 p1 = a.pos4[j1];
     for (int s0 = 0; s0 < cmax; s0 += G) {
-        const int s = s0 + lane, j = j1;
+        const int s = s0 + lane, j = j1, sh = h1;
         const bool act = s < cnt;
         const float4 pj = p1;
-        const int sh = !MINIMG && act ? a.shift[s * N + i] : 0;
         j1 = j2;
+        h1 = h2;
         p1 = a.pos4[j1];
         j2 = s + 2 * G < cnt ? a.nbr[(s + 2 * G) * N + i] : i;
+        if (!MINIMG) h2 = s + 2 * G < cnt ? a.shift[(s + 2 * G) * N + i] : 0;
         float dx, dy, dz;
         pair_vector(fr.pi, pj, fr.Lx, fr.Ly, fr.Lz, fr.iLx, fr.iLy, fr.iLz, MINIMG, sh, dx, dy, dz);
         const float d2 = act ? norm2(dx, dy, dz) : rcR2;

@@ -173,6 +173,13 @@ __device__ __forceinline__ GroupPair group_pair(const EvalArgs& a, const AtomFra
     return p;
 }
 
+// neighbour and image of list entry s, the atom itself past the end
+__device__ __forceinline__ void list_entry(const EvalArgs& a, int i, int s, int cnt, bool images, int& j, int& sh) {
+    const size_t at = (size_t)s * a.N + i;
+    j = s < cnt ? a.nbr[at] : i;
+    sh = images && s < cnt ? a.shift[at] : 0;
+}
+
 // Phases of one atom shared with the training kernels: radial sums F (shared
 // memory) and S_nlm (lane m, m + G, ... keeps S[.][m]) over the list.
 // Returns the number of angular pairs; their slots are in the group's list.
@@ -199,19 +206,22 @@ __device__ int group_sums(const EvalArgs& a, const float* sm, float* gb, float* 
         for (int x = 0; x < MPL; ++x) S2[n][x] = make_float2(0.0f, 0.0f);
     const int cmax = warp_max(cnt), amax = warp_max(cnt_ang);
     int total = 0;
-    // a chunk's entries are read one chunk ahead, the indices two
+    // a chunk's entries are read one chunk ahead, the indices and images two
     const int N = a.N;
-    int j1 = lane < cnt ? a.nbr[(size_t)lane * N + i] : i;
-    int j2 = lane + G < cnt ? a.nbr[(size_t)(lane + G) * N + i] : i;
+    const bool images = !a.min_image;
+    int j1 = i, j2 = i, h1 = 0, h2 = 0;
+    list_entry(a, i, lane, cnt, images, j1, h1);
+    list_entry(a, i, lane + G, cnt, images, j2, h2);
     float4 p1 = a.pos4[j1];
     for (int s0 = 0; s0 < cmax; s0 += G) {
         const int s = s0 + lane;
         const bool act = s < cnt;
         const float4 pj = p1;
-        const int sh = act && !a.min_image ? a.shift[(size_t)s * N + i] : 0;
+        const int sh = h1;
         j1 = j2;
+        h1 = h2;
         p1 = a.pos4[j1];
-        j2 = s + 2 * G < cnt ? a.nbr[(size_t)(s + 2 * G) * N + i] : i;
+        list_entry(a, i, s + 2 * G, cnt, images, j2, h2);
         GroupPair p;
         p.tj = f2i(pj.w);
         pair_vector(fr.pi, pj, fr.Lx, fr.Ly, fr.Lz, fr.iLx, fr.iLy, fr.iLz, a.min_image, sh, p.dx, p.dy, p.dz);
@@ -498,7 +508,11 @@ __global__ void __launch_bounds__(kGroupThreads, kGroupMinBlocks) kg_atom(const 
 // F_i and the per-atom virial: radial pair forces of both directions from the
 // projected adjoints of both atoms, the owner's angular part, and the incoming
 // angular slots (those whose pair lies inside rc_ang); in MD also the closing
-// half kick, which saves small systems its launch
+// half kick, which saves small systems its launch.  Bound by the latency of a
+// lane's entries: images are read with their indices, two entries ahead (48
+// replicas, ten FP16 MD steps 2,019 -> 1,965 us with k_radial_split's).  Rows
+// and slots also fetched an entry ahead measured slower (12,442 atoms 56.7 ->
+// 64.4 us an evaluation: more registers).
 template <class C, int G>
 __global__ void __launch_bounds__(kGroupThreads) kg_finish(const EvalArgs a, const FinishArgs fa) {
     constexpr int KR = C::KR, T = C::T, NG = kGroupThreads / G;
@@ -513,28 +527,32 @@ __global__ void __launch_bounds__(kGroupThreads) kg_finish(const EvalArgs a, con
     float acc[9];                                        // F, then xx yy zz xy xz yz
 #pragma unroll
     for (int k = 0; k < 9; ++k) acc[k] = 0.0f;
-    // positions are read one entry ahead, the indices two
-    int j0 = lane < cnt ? a.nbr[(size_t)lane * N + i] : i;
-    int j1 = lane + G < cnt ? a.nbr[(size_t)(lane + G) * N + i] : i;
+    // positions are read one entry ahead, the indices and images two
+    const bool images = !a.min_image;
+    int j0 = i, j1 = i, h0 = 0, h1 = 0;
+    list_entry(a, i, lane, cnt, images, j0, h0);
+    list_entry(a, i, lane + G, cnt, images, j1, h1);
     float4 p0 = a.pos4[j0];
     pdl_wait();                              // the list and the positions are older than kg_atom
     pdl_trigger();
-    for (int o = lane; o < T * KR; o += G) Pi[group][o] = a.Pr[(size_t)i * T * KR + o];
+    const float* Pr = after_wait(a.Pr);
+    for (int o = lane; o < T * KR; o += G) Pi[group][o] = Pr[(size_t)i * T * KR + o];
     __syncwarp();
     for (int s = lane; s < cnt; s += G) {
         GroupPair p;
         p.j = j0;
         const float4 pj = p0;
-        const int sh = a.min_image ? 0 : a.shift[(size_t)s * N + i];
+        const int sh = h0;
         j0 = j1;
+        h0 = h1;
         p0 = a.pos4[j0];
-        j1 = s + 2 * G < cnt ? a.nbr[(size_t)(s + 2 * G) * N + i] : i;
+        list_entry(a, i, s + 2 * G, cnt, images, j1, h1);
         p.tj = f2i(pj.w);
         pair_vector(fr.pi, pj, fr.Lx, fr.Ly, fr.Lz, fr.iLx, fr.iLy, fr.iLz, a.min_image, sh, p.dx, p.dy, p.dz);
         p.d2 = norm2(p.dx, p.dy, p.dz);
         if (!(p.d2 < rcR2)) continue;
         float Pj[KR];
-        const float* row = a.Pr + ((size_t)p.j * T + fr.ti) * KR;
+        const float* row = Pr + ((size_t)p.j * T + fr.ti) * KR;
         if (KR % 8 == 0) {
 #pragma unroll
             for (int k = 0; k < KR; k += 8) load8_ro(row + k, Pj + k);
@@ -634,6 +652,7 @@ cudaError_t launch_group_t(const EvalArgs& a, cudaStream_t st, int G) {
 template <class C>
 cudaError_t launch_group_finish_t(const EvalArgs& a, const FinishArgs& f, int max_chunks, cudaStream_t st, int G) {
     if (G == 32) launch_group_finish_g<C, 32>(a, f, st);
+    else if (G == 16) launch_group_finish_g<C, 16>(a, f, st);
     else launch_group_finish_g<C, 8>(a, f, st);
     return launch_totals(a, f, max_chunks, st);
 }

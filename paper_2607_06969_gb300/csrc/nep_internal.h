@@ -27,6 +27,14 @@ namespace nep {
 // other kernel or operation the launch is an ordinary one.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// A load through the read-only path carries no dependence on memory, so
+// nothing but its address keeps it behind the wait: such a kernel takes its
+// pointers without __restrict__, or through here after the wait.
+template <class T>
+__device__ __forceinline__ T* after_wait(T* p) {
+    asm volatile("" : "+l"(p)::"memory");
+    return p;
+}
 template <class... K, class... A>
 cudaError_t launch_pdl(void (*kernel)(K...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args) {
     cudaLaunchAttribute at[1];

@@ -88,15 +88,12 @@ __global__ void __launch_bounds__(1024) k_chunk_plan(const int* __restrict__ ato
     chunk_plan_block(atom_off, B, chunk_start, ticket);
 }
 
-__device__ __forceinline__ void pack_atom(const float* pos, const int* __restrict__ type,
-                                          const int* __restrict__ atom_off, int N, int B, int T, int i, float4* pos4,
-                                          int* cfg, int* status) {
-    int t = type[i];
+__device__ __forceinline__ void pack_atom(float x, float y, float z, int t, const int* atom_off, int B, int T, int i,
+                                          float4* pos4, int* cfg, int* status) {
     if (t < 0 || t >= T) {
         set_flag(status, 3);
         t = 0;
     }
-    const float x = pos[i], y = pos[N + i], z = pos[2 * (size_t)N + i];
     if (!(isfinite(x) && isfinite(y) && isfinite(z))) set_flag(status, 3);
     pos4[i] = make_float4(x, y, z, __int_as_float(t));
     cfg[i] = find_segment(atom_off, B, i);
@@ -104,8 +101,8 @@ __device__ __forceinline__ void pack_atom(const float* pos, const int* __restric
 
 // positions, species and configuration of each atom in the kernels' layout;
 // with chunk_start, one more block plans the reduction chunks meanwhile
-__global__ void __launch_bounds__(256) k_pack(const float* __restrict__ pos, const int* __restrict__ type,
-                                              const int* __restrict__ atom_off, int N, int B, int T, float4* pos4,
+__global__ void __launch_bounds__(256) k_pack(const float* pos, const int* type,
+                                              const int* atom_off, int N, int B, int T, float4* pos4,
                                               int* cfg, int* status, int* chunk_start, int* ticket) {
     pdl_wait();
     pdl_trigger();
@@ -114,7 +111,7 @@ __global__ void __launch_bounds__(256) k_pack(const float* __restrict__ pos, con
         return;
     }
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < N) pack_atom(pos, type, atom_off, N, B, T, i, pos4, cfg, status);
+    if (i < N) pack_atom(pos[i], pos[N + i], pos[2 * (size_t)N + i], type[i], atom_off, B, T, i, pos4, cfg, status);
 }
 
 constexpr int kRedThreads = 256;
@@ -428,8 +425,8 @@ constexpr int kCellsSmallN = 8192, kCellsSmallB = 256;
 constexpr int kCellsSmallStatic = (int)(sizeof(int) * kCellsSmallN + (sizeof(CellPlan) + 3 * sizeof(float)) * kCellsSmallB +
                                         sizeof(int) * (kCellsSmallB + 1 + 32)) + 64;   // and padding
 __global__ void __launch_bounds__(1024) k_cells_small(
-    const float* __restrict__ pos, const int* __restrict__ type, const int* __restrict__ atom_off,
-    const float* __restrict__ box, int N, int B, int T, float rc, float4* pos4, int* cfg, int* status,
+    const float* pos, const int* type, const int* atom_off,
+    const float* box, int N, int B, int T, float rc, float4* pos4, int* cfg, int* status,
     CellPlan* plan, int* cell_of, int* cell_start, float4* cell_pos) {
     pdl_wait();
     pdl_trigger();
@@ -757,9 +754,9 @@ static_assert(kBuildWarpN < 1 << 30, "a kept hit's kind shares a word with its a
 constexpr float kBuildMinEdge = 16.0f;   // shortest box edge: the list cutoff over this (at most 34 ranges per row)
 
 __global__ void __launch_bounds__(32 * kBuildWarps, 8) k_build_warp(
-    const float4* __restrict__ pos4, const int* __restrict__ cfg, const float* __restrict__ box,
-    const CellPlan* __restrict__ plan, const int* __restrict__ cell_of, const int* __restrict__ cell_start,
-    const float4* __restrict__ cell_pos, int N, float rc2_rad, float rc2_ang, float rc2_phys,
+    const float4* pos4, const int* cfg, const float* box,
+    const CellPlan* plan, const int* cell_of, const int* cell_start,
+    const float4* cell_pos, int N, float rc2_rad, float rc2_ang, float rc2_phys,
     unsigned char* __restrict__ row_start, unsigned char* __restrict__ slot_row, nep_nlist nl) {
     pdl_wait();
     pdl_trigger();
@@ -983,8 +980,8 @@ __global__ void __launch_bounds__(32 * kBuildWarps, 8) k_build_warp(
 // so only that row's stretch of j's prefix is searched; stencils too large
 // for the row table fall back to scanning j's whole prefix.
 __device__ __forceinline__ void rev_slot(int N, int i, int s, int rows, bool track,
-                                         const unsigned char* __restrict__ row_start,
-                                         const unsigned char* __restrict__ slot_row, const nep_nlist& nl) {
+                                         const unsigned char* row_start, const unsigned char* slot_row,
+                                         const nep_nlist& nl) {
     const int j = nl.nbr[(size_t)s * N + i];
     int want = 0;
     if (nl.shift) {
@@ -1021,9 +1018,9 @@ __device__ __forceinline__ void rev_slot(int N, int i, int s, int rows, bool tra
 // us, of 112,500 atoms 259 -> 262).
 constexpr int kRevWarpN = 80000;
 template <int G>
-__global__ void __launch_bounds__(128) k_rev(int N, const int* __restrict__ cfg, const CellPlan* __restrict__ plan,
-                                             const unsigned char* __restrict__ row_start,
-                                             const unsigned char* __restrict__ slot_row, nep_nlist nl) {
+__global__ void __launch_bounds__(128) k_rev(int N, const int* cfg, const CellPlan* plan,
+                                             const unsigned char* row_start,
+                                             const unsigned char* slot_row, nep_nlist nl) {
     pdl_wait();
     pdl_trigger();
     const int i = (blockIdx.x * blockDim.x + threadIdx.x) / G;
@@ -1037,7 +1034,7 @@ __global__ void __launch_bounds__(128) k_rev(int N, const int* __restrict__ cfg,
 
 // ------------------------------------------------------------ optimiser
 // one Adam step per parameter; c1 = lr / (1 - beta1^t), c2 = 1 / sqrt(1 - beta2^t)
-__global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
+__global__ void k_adam(float* __restrict__ p, const float* g, float* __restrict__ m,
                        float* __restrict__ v, int n, float beta1, float beta2, float eps, float c1, float c2) {
     pdl_wait();
     pdl_trigger();
@@ -1075,30 +1072,40 @@ struct InvMass {
     float v[kMaxTypes];
 };
 
-__device__ __forceinline__ void kick_atom(float* __restrict__ vel, const float* __restrict__ force, int type,
-                                          const InvMass& im, int N, int i, float half_dt, float* __restrict__ pos,
-                                          float dt) {
+// every load before the first store; x: the new position (if pos is given)
+__device__ __forceinline__ void kick_atom(float* vel, const float* force, int type, const InvMass& im, int N, int i,
+                                          float half_dt, float* pos, float dt, float (&x)[3]) {
     const float s = half_dt * im.v[type & (kMaxTypes - 1)];
+    float v[3];
+#pragma unroll
     for (int d = 0; d < 3; ++d) {
-        float v = vel[(size_t)d * N + i] + s * force[(size_t)d * N + i];
-        vel[(size_t)d * N + i] = v;
-        if (pos) pos[(size_t)d * N + i] += dt * v;
+        const size_t at = (size_t)d * N + i;
+        v[d] = vel[at] + s * force[at];
+        x[d] = pos ? pos[at] : 0.0f;
+    }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const size_t at = (size_t)d * N + i;
+        vel[at] = v[d];
+        x[d] += dt * v[d];
+        if (pos) pos[at] = x[d];
     }
 }
-__global__ void k_kick(float* __restrict__ vel, const float* __restrict__ force,
-                       const int* __restrict__ type, InvMass im, int N, float half_dt,
+__global__ void k_kick(float* __restrict__ vel, const float* force,
+                       const int* type, InvMass im, int N, float half_dt,
                        float* __restrict__ pos, float dt) {
     pdl_wait();
     pdl_trigger();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < N) kick_atom(vel, force, type[i], im, N, i, half_dt, pos, dt);
+    float x[3];
+    if (i < N) kick_atom(vel, force, type[i], im, N, i, half_dt, pos, dt, x);
 }
 // the opening half kick and the drift, then the atom packed at its new
 // position (as k_pack, whose launch and pass over the positions this saves)
-__global__ void __launch_bounds__(256) k_kick_pack(float* __restrict__ vel, const float* __restrict__ force,
-                                                   const int* __restrict__ type, InvMass im, int N, float half_dt,
+__global__ void __launch_bounds__(256) k_kick_pack(float* __restrict__ vel, const float* force,
+                                                   const int* type, InvMass im, int N, float half_dt,
                                                    float* __restrict__ pos, float dt,
-                                                   const int* __restrict__ atom_off, int B, int T, float4* pos4,
+                                                   const int* atom_off, int B, int T, float4* pos4,
                                                    int* cfg, int* status, int* chunk_start, int* ticket) {
     pdl_wait();
     pdl_trigger();
@@ -1108,8 +1115,10 @@ __global__ void __launch_bounds__(256) k_kick_pack(float* __restrict__ vel, cons
     }
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
-    kick_atom(vel, force, type[i], im, N, i, half_dt, pos, dt);
-    pack_atom(pos, type, atom_off, N, B, T, i, pos4, cfg, status);
+    const int t = type[i];
+    float x[3];
+    kick_atom(vel, force, t, im, N, i, half_dt, pos, dt, x);
+    pack_atom(x[0], x[1], x[2], t, atom_off, B, T, i, pos4, cfg, status);
 }
 
 // x wrapped into [0, L)
@@ -1121,7 +1130,7 @@ __device__ __forceinline__ float wrap_coord(float x, float L) {
     return x;
 }
 // each atom's configuration is found from the CSR offsets
-__global__ void k_wrap_seg(float* pos, const int* __restrict__ atom_off, int B, const float* __restrict__ box,
+__global__ void k_wrap_seg(float* pos, const int* atom_off, int B, const float* box,
                            int N) {
     pdl_wait();
     pdl_trigger();
@@ -1148,8 +1157,8 @@ __device__ __forceinline__ double block_sum_fixed(double v) {
 // Force residuals per chunk: lam_i = 2 wF (F_i - F_lbl,i) / (3 N_b B) and the
 // FP64 partial sum of |dF|^2 (Eq. 20).
 __global__ void __launch_bounds__(kRedThreads) k_loss_atoms(
-    int N, int B, const int* __restrict__ atom_off, const int* __restrict__ chunk_start,
-    const float* __restrict__ force, const float* __restrict__ f_lbl, float wF, float4* lam4,
+    int N, int B, const int* atom_off, const int* chunk_start,
+    const float* force, const float* f_lbl, float wF, float4* __restrict__ lam4,
     double* partial) {
     pdl_wait();
     pdl_trigger();
@@ -1176,10 +1185,10 @@ __global__ void __launch_bounds__(kRedThreads) k_loss_atoms(
 // Per-configuration loss terms and energy/virial adjoints (Eqs. 18-21), and
 // the batch loss summed in a fixed tree (one CTA).
 __global__ void __launch_bounds__(kRedThreads) k_loss_cfg(
-    int B, const int* __restrict__ atom_off, const int* __restrict__ chunk_start,
-    const double* __restrict__ partial, const double* __restrict__ e_tot,
-    const double* __restrict__ vir, const double* __restrict__ e_lbl,
-    const double* __restrict__ v_lbl, float wE, float wF, float wV, int mode, float* aE, float* mu,
+    int B, const int* atom_off, const int* chunk_start,
+    const double* partial, const double* e_tot,
+    const double* vir, const double* e_lbl,
+    const double* v_lbl, float wE, float wF, float wV, int mode, float* aE, float* mu,
     double* loss) {
     pdl_wait();
     pdl_trigger();
@@ -1220,8 +1229,8 @@ __global__ void __launch_bounds__(kRedThreads) k_loss_cfg(
 }
 
 // External adjoints (vector-Jacobian product) into the kernels' layout.
-__global__ void k_pack_adjoint(int N, int B, const float* __restrict__ lam,
-                               const double* __restrict__ a_e, const double* __restrict__ mu_in,
+__global__ void k_pack_adjoint(int N, int B, const float* lam,
+                               const double* a_e, const double* mu_in,
                                float4* lam4, float* aE, float* mu) {
     pdl_wait();
     pdl_trigger();
