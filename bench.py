@@ -150,15 +150,15 @@ def algorithmic_flops(h, nbar_rad: float, nbar_ang: float) -> dict:
 # capture (dram__bytes_read.sum + dram__bytes_write.sum) of the 460,800-atom
 # case of this workload (40^3 cells), divided by its atom count; traffic grows
 # in proportion to the atoms.  Valid only for the kernels as captured.
-TRAFFIC_PER_ATOM = {"radial": (239.36e6 + 195.71e6) / 460800,
-                    "angular": (279.96e6 + 208.61e6) / 460800,
-                    "finish": (384.11e6 + 19.88e6) / 460800}
+TRAFFIC_PER_ATOM = {"radial": (239.26e6 + 195.49e6) / 460800,
+                    "angular": (279.15e6 + 207.34e6) / 460800,
+                    "finish": (386.27e6 + 21.24e6) / 460800}
 
 
 def launches_per_step(rebuild: bool) -> int:
-    # kick, [pack, wrap, pack, cell plan, plan scan, bin, 3 scan, fill, sort, build, rev],
-    # pack, chunk plan, radial, angular, finish, chunk reduce, final reduce, kick
-    return 9 + (13 if rebuild else 0)
+    # kick with packing and chunk plan, radial, angular, finish, totals, kick; a rebuild step
+    # kicks and packs apart and adds wrap, pack, cell plan, plan scan, bin, 3 scan, fill, sort, build, rev
+    return 6 + (13 if rebuild else 0)
 
 
 # --------------------------------------------------------------- cpu legs

@@ -99,13 +99,14 @@ def assert_close(got, want, n, tol=1.0):
 @pytest.mark.parametrize("hname", list(MODELS))
 @pytest.mark.parametrize("counts,skin", [([1], 0.0), ([3], 0.0), ([2, 0, 33], 0.5), ([24, 127, 130], 1.0),
                                          ([1500, 1499], 0.0), ([1500, 1501], 0.0), ([3700, 17, 300], 1.0),
+                                         ([3701], 0.5), ([8000], 0.0), ([8001], 0.0),
                                          ([6000, 4000], 0.5), ([6000, 4001], 0.5), ([6000, 4001, 2], 0.0)])
 def test_lane_groups_agree_with_one_thread_per_atom(nb, hname, counts, skin):
-    """A group of lanes per atom (32 up to 3,000 atoms, then 8; above 10,000 for
-    the radial sums and the finish only): fewer atoms than one block holds,
-    remainders of a block, an empty configuration, both sides of the lines
-    between the forms, boxes shorter than the cutoff (images) and longer, with
-    a skin."""
+    """A group of lanes per atom (32 up to 3,000 atoms, then 8, the finish 16 up
+    to 8,000 without images; above 10,000 for the radial sums and the finish
+    only): fewer atoms than one block holds, remainders of a block, an empty
+    configuration, both sides of the lines between the forms, boxes shorter
+    than the cutoff (images) and longer, with a skin."""
     h = MODELS[hname]
     s, model, dsys, nl, ws = setup(nb, h, counts, 62, skin=skin, cap=160, cap_ang=80)
     assert_close(*both_forms(nb, model, dsys, nl, ws), np.diff(s.atom_off))
