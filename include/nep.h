@@ -87,9 +87,8 @@ size_t nep_num_params(const nep_hparams* hp);
  * A shape with a compiled kernel set (nep_supported = 1) gets the fast path:
  * FP32, FP16 or BF16 network, every call.  Any other FP32 shape with n_rad,
  * n_ang <= 16 and k_rad, k_ang <= 16 (nep_supported = 2) gets the generic
- * path: FP32 kernels with compiled bounds on the shape that evaluate each pair
- * term from both of its atoms (about twice the fast path's pair work).  A
- * generic model serves
+ * path: FP32 kernels with compiled bounds on the shape, two to three times the
+ * fast path's time.  A generic model serves
  * nep_neighbors, the FP32 evaluations (nep_energy_forces_virial, _owned,
  * _noalloc), nep_md_step and the FP64 calls; nep_param_grad,
  * nep_param_grad_adjoint and nep_autotune return NEP_ERR_UNSUPPORTED (its

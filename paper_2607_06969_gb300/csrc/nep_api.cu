@@ -430,8 +430,8 @@ bool fp64_supported(const nep_hparams& hp) {
 }
 
 // The generic FP32 evaluation (a model with no compiled kernel set): the
-// FP64 path's two kernels in float, every pair term evaluated from both of
-// its atoms, then the same FP64 sums.
+// FP64 path's two kernels in float, each angular pair force written to its
+// partner's reverse slot, then the same FP64 sums.
 nep_status efv_generic(nep_model* m, const nep_system* s, const nep_nlist* nl, float* e_atom, float* force,
                        double* e_tot, double* virial, void* work, const WsLayout& w, cudaStream_t st,
                        int n_owned) {

@@ -628,7 +628,7 @@ cudaError_t launch_efv_t(const A& a, int max_chunks, double* e_tot, double* viri
     if (a.N > 0)
         e = with_dims(a, [&](auto dm) {
             using DM = decltype(dm);
-            return a.N <= kEvalLanes32 ? launch_efv_g<32, DM>(a, st) : launch_efv_g<8, DM>(a, st);
+            return a.N <= (kScatter<A> ? kGenericLanes32 : kEvalLanes32) ? launch_efv_g<32, DM>(a, st) : launch_efv_g<8, DM>(a, st);
         });
     if (e != cudaSuccess) return e;
     if (max_chunks > 0) k64_totals<A><<<max_chunks, 320, 0, st>>>(a, e_tot, virial);

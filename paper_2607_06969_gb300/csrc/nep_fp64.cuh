@@ -8,7 +8,8 @@
 // compiled bounds (Dims64).  The same code in float is the generic FP32
 // evaluation of shapes without compiled kernels.
 //
-// A group of G lanes takes an atom (32 up to kEvalLanes32 atoms, then 8).
+// A group of G lanes takes an atom (32 up to kEvalLanes32 atoms, or
+// kGenericLanes32 in float, then 8).
 // Sums over the list run pair by pair in list order within a lane's share, the
 // few sums that cross lanes in an xor butterfly, whose fixed tree leaves the
 // same bits in every lane; for a given N, which fixes G, every result is
@@ -219,6 +220,10 @@ constexpr bool kScatter = std::is_same<A, F32Args>::value;
 
 // up to this many atoms the kernels take 32 lanes per atom, else 8
 constexpr int kEvalLanes32 = 1500;
+// the same for the generic path, whose pipe is not full at these sizes (32 / 8
+// lanes, models of 11/7 and 5/3 radial/angular functions): 2,566 atoms 57.4 /
+// 74.3 us, 60.1 / 70.2; 5,453 atoms 89.7 / 83.0, 89.1 / 74.7
+constexpr int kGenericLanes32 = 4000;
 
 // calls f with the loop bounds for the model's shape
 template <class A, class F>

@@ -247,13 +247,14 @@ def typed(s, h):
 @pytest.mark.parametrize("name", list(SHAPES64))
 def test_fp64_and_generic_lane_group_sizes(nb, name):
     """The FP64 evaluation and gradient, and the generic FP32 evaluation,
-    with 32 lanes per atom (up to 1,500 atoms) and with 8: a configuration
+    with 32 lanes per atom (up to 1,500 atoms; 4,000 generic) and with 8: a configuration
     alone against the same one in a larger batch, for shapes on every set of
     compiled loop bounds.  FP64 sums of some thousand terms: 1e-12; FP32: the
     bars of the parity tests."""
     import torch
     h = SHAPES64[name]
     one, two = I.packing_batch([43], tag=70), I.packing_batch([1470], tag=71)
+    rest = I.packing_batch([3960], tag=72)
     both = I.System(pos=np.concatenate([one.pos, two.pos]), types=np.concatenate([one.types, two.types]),
                     box=np.concatenate([one.box, two.box]), atom_off=np.array([0, 43, 1513]))
     model = nb.Model(h, I.init_params(h, seed=6).astype(np.float32))
@@ -279,6 +280,15 @@ def test_fp64_and_generic_lane_group_sizes(nb, name):
         res.append([t.cpu().numpy() for t in x] + [t.cpu().numpy() for t in (y[0][:43], y[1][:, :43], y[2][:1], y[3][:1])])
     for a, b in zip(res[0][:5], res[1][:5]):
         assert np.abs(a - b).max() <= 1e-12 * max(1.0, np.abs(a).max()) * 43
+    s = typed(I.System(pos=np.concatenate([one.pos, rest.pos]), types=np.concatenate([one.types, rest.types]),
+                       box=np.concatenate([one.box, rest.box]), atom_off=np.array([0, 43, 4003])), h)
+    dsys = nb.DeviceSystem.from_inputs(s)
+    nl = nb.NeighborList(s.n_atoms, 160, 80)
+    ws = nb.Workspace(model, s.n_atoms, 2, 160, 80)
+    nb.neighbors(model, dsys, nl, 0.5, ws)
+    assert nb.check_list(nl) == nb.NEP_OK
+    y = nb.energy_forces_virial(model, dsys, nl, ws)
+    res.append(res[0][:5] + [t.cpu().numpy() for t in (y[0][:43], y[1][:, :43], y[2][:1], y[3][:1])])
     for got in res:                                   # the FP32 evaluation against FP64
         assert np.abs(got[5] - got[0]).max() <= 1e-6 * max(1.0, np.abs(got[0]).max())
         assert np.abs(got[6] - got[1]).max() <= 1e-4
