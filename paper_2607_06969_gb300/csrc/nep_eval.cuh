@@ -941,10 +941,12 @@ __global__ void __launch_bounds__(BLOCK, NEP_RADIAL_MINB * kRadialBlock / BLOCK)
 // k_radial with kSplitLanes lanes per atom, for systems whose atoms alone are
 // too few threads: each lane takes every fourth list entry, the records go to
 // the same slots (lane order is list order), and the lanes' basis sums are
-// added at the end.  One thread per atom takes the time of one atom's walk, 26
-// us, up to about 40,000 atoms; four lanes take 12 us at 12,442 atoms and 15 at
-// 29,491.  Beyond the line of eval_split (nep_api.cu) the split's scattered
-// list reads cost more than it gains (900,000 atoms 362 -> 440 us).
+// added at the end.  One thread per atom takes the time of one atom's walk,
+// about 25 us, up to some 40,000 atoms; four lanes take 11.6 us for a training
+// batch of about 20,000 atoms.  One evaluation, one thread / four lanes: 57,600
+// atoms 151 / 145 us, 158,054 379 / 368; beyond the line of eval_split
+// (nep_api.cu) the split's scattered list reads cost more than it gains: 900,000
+// atoms 1,576 / 1,654.
 constexpr int kSplitLanes = 4;
 template <class C, bool MINIMG>
 __global__ void __launch_bounds__(128, 8) k_radial_split(const EvalArgs a) {
