@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kTotalsThreads) k_totals(const EvalArgs a, Fin
     const int k0 = f.chunk_start[b], nk = f.chunk_start[b + 1] - k0;
     const int a0 = f.atom_off[b] + (k - k0) * kChunk;
     const int a1 = min(min(f.atom_off[b + 1], a0 + kChunk), f.n_owned);
-    pdl_wait();                          // the plan is older than the kernel before this one
+    pdl_wait();                          // the plan is older than the kernel before this one (launch_totals)
     pdl_trigger();
     const float* src = c == 0 ? a.e_atom : a.wat + (size_t)(c - 1) * N;
     float h = 0.0f, l = 0.0f;
@@ -1272,8 +1272,16 @@ cudaError_t launch_pack_plan(const float* pos, const int* type, const int* atom_
     return cudaGetLastError();
 }
 
+// k_totals reads the chunk plan ahead of its wait, which needs a kernel between
+// the plan's writer and itself.  Without atoms there is none: it follows the
+// packing launch, which lets its successor start before the plan is written, so
+// there it is an ordinary launch.
 cudaError_t launch_totals(const EvalArgs& a, const FinishArgs& f, int max_chunks, cudaStream_t st) {
-    if (max_chunks > 0) launch_pdl(k_totals, max_chunks, kTotalsThreads, 0, st, a, f);
+    if (max_chunks <= 0) return cudaGetLastError();
+    if (a.N > 0)
+        launch_pdl(k_totals, max_chunks, kTotalsThreads, 0, st, a, f);
+    else
+        k_totals<<<max_chunks, kTotalsThreads, 0, st>>>(a, f);
     return cudaGetLastError();
 }
 

@@ -316,3 +316,54 @@ def test_fp64_and_generic_many_angular_pairs(nb, hname):
     assert np.abs(e - e6).max() <= 1e-5 * max(1.0, np.abs(e6).max())
     assert np.abs(f - f6).max() <= 1e-4 * scale
     assert np.abs(v - v6).max() <= 1e-5 * 400 * max(1.0, np.abs(v6).max() / 400)
+
+
+@pytest.mark.parametrize("n_cfg", [1, 3, 2049])
+def test_no_atoms_in_a_used_workspace(nb, n_cfg):
+    """Configurations without atoms in a workspace that other work left full
+    of words: the totals are zero, whatever stood where this call's chunk plan
+    goes (outputs preset, so that a total that is not written shows).  The
+    words, 2.0 in FP32, read as a plan whose chunks are all empty.  2,049
+    configurations: the plan has a launch of its own."""
+    import ctypes
+    import torch
+    h = I.HYPER_SMALL
+    s = I.System(pos=np.zeros((0, 3)), types=np.zeros(0, np.int32), box=np.full((n_cfg, 3), 20.0),
+                 atom_off=np.zeros(n_cfg + 1, np.int64))
+    model = nb.Model(h, I.init_params(h).astype(np.float32))
+    dsys = nb.DeviceSystem.from_inputs(s)
+    nl = nb.NeighborList(0, 64, 32)
+    ws = nb.Workspace(model, 0, n_cfg, 64, 32, train=True)
+    words = ws.buf[:ws.buf.numel() // 4 * 4].view(torch.float32)
+    out = (torch.empty(0, device="cuda"), torch.empty(3, 0, device="cuda"),
+           torch.empty(n_cfg, dtype=torch.float64, device="cuda"),
+           torch.empty(n_cfg, 9, dtype=torch.float64, device="cuda"))
+
+    def fresh():
+        words.fill_(2.0)
+        out[2].fill_(7.0)
+        out[3].fill_(7.0)
+
+    def zero():
+        assert torch.count_nonzero(out[2]).item() == 0 and torch.count_nonzero(out[3]).item() == 0
+
+    nb.neighbors(model, dsys, nl, 0.0, ws)
+    assert nb.check_list(nl) == nb.NEP_OK
+    fresh()
+    nb.energy_forces_virial(model, dsys, nl, ws, out=out)
+    zero()
+    fresh()
+    nb.check(nb.lib().nep_energy_forces_virial_owned(
+        model.handle, ctypes.byref(dsys.c), ctypes.byref(nl.c), 0, None, nb._ptr(out[1]), nb._ptr(out[2]),
+        nb._ptr(out[3]), ws.ptr, ws.bytes, nb._stream(None)), "nep_energy_forces_virial_owned")
+    zero()
+    vel = torch.zeros(3, 0, device="cuda")
+    for rebuild in (True, False):
+        fresh()
+        nb.md_step(model, dsys, nl, vel, out[1], out[2], out[3], I.MASSES.astype(np.float32), 2.0, 0.0, rebuild, ws)
+        zero()
+    fresh()
+    zeros = torch.zeros(n_cfg, dtype=torch.float64, device="cuda")
+    grad, loss = nb.param_grad(model, dsys, nl, ws, zeros, torch.zeros(3, 0, device="cuda"),
+                               torch.zeros(n_cfg, 9, dtype=torch.float64, device="cuda"))
+    assert torch.count_nonzero(grad).item() == 0 and loss.item() == 0.0
