@@ -96,6 +96,18 @@ NEP_HD void load8_ro(const float* p, float* v) {
 #endif
 }
 
+// the same by an ordinary (coherent) load, for data that the kernel in front may
+// still write when this one starts; the address must come from after_wait
+NEP_HD void load8(const float* p, float* v) {
+#if defined(__CUDA_ARCH__)
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "l"(p));
+#else
+    for (int k = 0; k < 8; ++k) v[k] = p[k];
+#endif
+}
+
 // Two independent FP32 FMAs in one paired instruction on the device
 // (a.x * b.x + c.x, a.y * b.y + c.y, each rounded once as fmaf rounds it):
 // pairing two accumulation chains leaves every result bit unchanged and

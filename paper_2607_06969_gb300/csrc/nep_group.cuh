@@ -555,7 +555,7 @@ __global__ void __launch_bounds__(kGroupThreads) kg_finish(const EvalArgs a, con
         const float* row = Pr + ((size_t)p.j * T + fr.ti) * KR;
         if (KR % 8 == 0) {
 #pragma unroll
-            for (int k = 0; k < KR; k += 8) load8_ro(row + k, Pj + k);
+            for (int k = 0; k < KR; k += 8) load8(row + k, Pj + k);
         } else {
 #pragma unroll
             for (int k = 0; k < KR; ++k) Pj[k] = row[k];

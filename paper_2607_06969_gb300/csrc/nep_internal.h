@@ -27,9 +27,12 @@ namespace nep {
 // other kernel or operation the launch is an ordinary one.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// A load through the read-only path carries no dependence on memory, so
-// nothing but its address keeps it behind the wait: such a kernel takes its
-// pointers without __restrict__, or through here after the wait.
+// Such a kernel loads nothing through the read-only path: that is defined only
+// for data that nobody writes while the kernel runs, and the kernel before is
+// still writing when this one starts; a load of that kind may also be moved
+// ahead of the wait.  So its pointers to const come without __restrict__, and
+// a pointer for a load that the compiler does not see goes through here after
+// the wait.
 template <class T>
 __device__ __forceinline__ T* after_wait(T* p) {
     asm volatile("" : "+l"(p)::"memory");

@@ -27,7 +27,7 @@ __device__ __forceinline__ int find_segment(const int* off, int B, int x) {
 // ------------------------------------------------------------------ packing
 // Exclusive scan of the configurations' chunk counts by one CTA (any multiple
 // of 32 threads up to 1,024), and the reduction tickets cleared.
-__device__ void chunk_plan_block(const int* __restrict__ atom_off, int B, int* chunk_start, int* ticket) {
+__device__ void chunk_plan_block(const int* atom_off, int B, int* chunk_start, int* ticket) {
     if (B <= 32) {                       // one warp, no block-wide waits
         const int b = threadIdx.x;
         if (b >= 32) return;
@@ -230,8 +230,7 @@ constexpr int kMaxRows = (2 * kCellDiv + 1) * (2 * kCellDiv + 1);
 static_assert(kMaxRows < kRowStride, "row starts must fit one atom's stride");
 
 // plan of one configuration; base holds its cell count until the prefix is taken
-__device__ CellPlan cell_plan_of(const float* __restrict__ box, const int* __restrict__ atom_off, int b, float rc,
-                                 int* status) {
+__device__ CellPlan cell_plan_of(const float* box, const int* atom_off, int b, float rc, int* status) {
     const int nb = atom_off[b + 1] - atom_off[b];
     float L[3] = {box[3 * b], box[3 * b + 1], box[3 * b + 2]};
     int nc[3];

@@ -753,7 +753,7 @@ __global__ void __launch_bounds__(kGradThreads) k_grad_partial(const TrainArgs t
                 const int fv = ok ? f : 2;
                 const int i = a0 + (ok ? rowatom[k] : 0);
                 const float* p = fv >= 2 ? src[fv] + i : (fv == 0 ? &a.pos4[i].w : t.aE + a.cfg[i]);
-                v[u] = __ldg(p);
+                v[u] = *p;
             }
 #pragma unroll
             for (int u = 0; u < kStageUnroll; ++u) {
