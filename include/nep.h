@@ -423,7 +423,8 @@ nep_status nep_autotune(nep_model* m, const nep_system* sys, const nep_nlist* nl
 
 /* Pin the angular kernel variant (0, 1, 2 = 2, 3, 4 resident blocks per SM;
  * -1 = back to the default) for one size class (0..31, as in nep_autotune)
- * or for all of them (size_class = -1).  A pinned class runs one thread per
+ * or for all of them (size_class = -1).  Block sizes that nep_set_launch
+ * pinned stay, and keep the class pinned.  A pinned class runs one thread per
  * atom at every size, the 16-bit networks on the tensor cores; otherwise small
  * systems take the lane-group kernels, which round the same operands to 16
  * bits and accumulate in FP32.  Host only, no device work. */

@@ -26,7 +26,11 @@ struct nep_model {
     int tune_angular[nep::kSizeBins];   // angular kernel variant per size class, -1 = default
     int tune_radial[nep::kSizeBins];    // radial kernel block size per size class, 0 = default
     int tune_finish[nep::kSizeBins];    // finish kernel block size per size class, 0 = default
-    bool pinned[nep::kSizeBins];        // the caller chose launch parameters of the one-thread-per-atom kernels
+    // which launch choices of the one-thread-per-atom kernels the caller made
+    // (the tuner's do not count); either pins the size class to those kernels
+    bool pin_variant[nep::kSizeBins];   // the angular variant
+    bool pin_blocks[nep::kSizeBins];    // the radial or the finish block size
+    bool pinned(int bin) const { return pin_variant[bin] || pin_blocks[bin]; }
 };
 
 namespace {
@@ -265,7 +269,7 @@ struct EvalSplit {
 EvalSplit eval_split(const nep_model* m, const nep_system* s, bool images) {
     const int N = s->n_atoms, bin = size_bin(s);
     EvalSplit e{0, 0, m->tune_radial[bin]};
-    if (N == 0 || m->pinned[bin]) return e;
+    if (N == 0 || m->pinned(bin)) return e;
     if (m->ks->group_fits(m->hp.n_hidden)) {
         const bool wide = m->hp.n_hidden * m->lay.D > 2500;
         const int most = !m->hp.precision ? 10000 : wide ? 25000 : 13500;
@@ -289,7 +293,7 @@ int train_lanes(const nep_model* m, const nep_system* s, bool loss) {
     const int N = s->n_atoms;
     const bool narrow = m->hp.n_ang <= 6;
     const int most = loss ? (narrow ? 34000 : 25000) : (narrow ? 40000 : 32000);
-    if (N == 0 || m->pinned[size_bin(s)] || !m->ks->group_train_fits(m->hp.n_hidden) || N > most) return 0;
+    if (N == 0 || m->pinned(size_bin(s)) || !m->ks->group_train_fits(m->hp.n_hidden) || N > most) return 0;
     return N > 2000 && narrow ? 16 : 32;
 }
 bool block_choice(int b) {
@@ -726,7 +730,7 @@ nep_status nep_create(const nep_hparams* hp, const float* params_host, size_t n_
         m->tune_angular[b] = -1;
         m->tune_radial[b] = 0;
         m->tune_finish[b] = 0;
-        m->pinned[b] = false;
+        m->pin_variant[b] = m->pin_blocks[b] = false;
     }
     cudaError_t e = ks ? ks->init(hp->n_hidden) : cudaSuccess;
     if (e == cudaSuccess && ks) e = ks->train_init(hp->n_hidden);
@@ -1260,7 +1264,7 @@ nep_status nep_set_variant(nep_model* m, int size_class, int variant) {
     for (int b = 0; b < nep::kSizeBins; ++b)
         if (size_class < 0 || b == size_class) {
             m->tune_angular[b] = variant;
-            m->pinned[b] = variant >= 0;
+            m->pin_variant[b] = variant >= 0;
         }
     return NEP_OK;
 }
@@ -1278,7 +1282,8 @@ nep_status nep_set_launch(nep_model* m, int size_class, int variant, int radial_
             m->tune_angular[b] = variant;
             m->tune_radial[b] = radial_block;
             m->tune_finish[b] = finish_block;
-            m->pinned[b] = variant >= 0 || radial_block || finish_block;
+            m->pin_variant[b] = variant >= 0;
+            m->pin_blocks[b] = radial_block || finish_block;
         }
     return NEP_OK;
 }

@@ -367,3 +367,28 @@ def test_no_atoms_in_a_used_workspace(nb, n_cfg):
     grad, loss = nb.param_grad(model, dsys, nl, ws, zeros, torch.zeros(3, 0, device="cuda"),
                                torch.zeros(n_cfg, 9, dtype=torch.float64, device="cuda"))
     assert torch.count_nonzero(grad).item() == 0 and loss.item() == 0.0
+
+
+def test_block_sizes_stay_pinned_without_a_variant(nb):
+    """A class with any launch choice but the defaults runs one thread per
+    atom: block sizes chosen by set_launch also do after set_variant(-1), which
+    gives up the variant only, and no longer do after set_launch()."""
+    h = I.HYPER_SMALL
+    s, model, dsys, nl, ws = setup(nb, h, [130, 300], 74)
+    run = lambda: nb.energy_forces_virial(model, dsys, nl, ws)[1].cpu().numpy()   # noqa: E731
+    default = run()
+    nb.set_variant(model, 0)
+    one_thread = run()
+    assert not np.array_equal(default, one_thread)    # the forms' sums differ in order
+    nb.set_launch(model, -1, 128, 256)
+    assert np.array_equal(run(), one_thread)
+    nb.set_variant(model, -1)
+    assert np.array_equal(run(), one_thread)
+    nb.set_launch(model, 0, 128, 0)
+    nb.set_variant(model, -1)
+    assert np.array_equal(run(), one_thread)
+    nb.set_launch(model)
+    assert np.array_equal(run(), default)
+    nb.set_variant(model, 0)
+    nb.set_variant(model, -1)
+    assert np.array_equal(run(), default)
