@@ -1,6 +1,8 @@
 // Model-independent kernels of libnep: input packing, the cell-list
 // neighbour build, the deterministic force gather with FP64 reductions, and
 // the velocity-Verlet updates.
+#include <limits>
+
 #include <cuda_runtime.h>
 
 #include "nep_device.cuh"
@@ -229,8 +231,12 @@ constexpr int kCellDiv = 3;
 constexpr int kMaxRows = (2 * kCellDiv + 1) * (2 * kCellDiv + 1);
 static_assert(kMaxRows < kRowStride, "row starts must fit one atom's stride");
 
-// plan of one configuration; base holds its cell count until the prefix is taken
-__device__ CellPlan cell_plan_of(const float* box, const int* atom_off, int b, float rc, int* status) {
+// plan of one configuration; base holds its cell count until the prefix is taken.
+// The build kernel is chosen by the host's copy of the boxes.  A box on the
+// device so much thinner that the cutoff reaches over more than max_images of
+// it is invalid input: its stencil has no rows (-1 of them; k_build_warp alone
+// sets a limit).
+__device__ CellPlan cell_plan_of(const float* box, const int* atom_off, int b, float rc, int max_images, int* status) {
     const int nb = atom_off[b + 1] - atom_off[b];
     float L[3] = {box[3 * b], box[3 * b + 1], box[3 * b + 2]};
     int nc[3];
@@ -256,15 +262,22 @@ __device__ CellPlan cell_plan_of(const float* box, const int* atom_off, int b, f
         p.half[d] = (int)ceilf((rc + kCellMargin) / cs);
         if (p.half[d] < 1) p.half[d] = 1;
     }
+    for (int d = 0; d < 3; ++d)
+        if (p.half[d] > (long long)max_images * p.nc[d]) {
+            set_flag(status, 3);
+            p.half[0] = -1;
+            p.half[1] = p.half[2] = 0;
+            break;
+        }
     p.base = nc[0] * nc[1] * nc[2];
     p.pad = 0;
     return p;
 }
 
 __global__ void k_cell_plan(const float* __restrict__ box, const int* __restrict__ atom_off, int B,
-                            float rc, CellPlan* plan, int* status) {
+                            float rc, int max_images, CellPlan* plan, int* status) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < B) plan[b] = cell_plan_of(box, atom_off, b, rc, status);
+    if (b < B) plan[b] = cell_plan_of(box, atom_off, b, rc, max_images, status);
 }
 
 __global__ void k_plan_scan(CellPlan* plan, int B) {
@@ -425,7 +438,7 @@ constexpr int kCellsSmallStatic = (int)(sizeof(int) * kCellsSmallN + (sizeof(Cel
                                         sizeof(int) * (kCellsSmallB + 1 + 32)) + 64;   // and padding
 __global__ void __launch_bounds__(1024) k_cells_small(
     const float* pos, const int* type, const int* atom_off,
-    const float* box, int N, int B, int T, float rc, float4* pos4, int* cfg, int* status,
+    const float* box, int N, int B, int T, float rc, int max_images, float4* pos4, int* cfg, int* status,
     CellPlan* plan, int* cell_of, int* cell_start, float4* cell_pos) {
     pdl_wait();
     pdl_trigger();
@@ -449,7 +462,7 @@ __global__ void __launch_bounds__(1024) k_cells_small(
     __syncthreads();
     CellPlan p;
     p.base = 0;
-    if (tid < B) p = cell_plan_of(box_s, off_s, tid, rc, status);
+    if (tid < B) p = cell_plan_of(box_s, off_s, tid, rc, max_images, status);
     int ncell;
     const int base = block_excl_scan_1024(p.base, ws, &ncell);
     if (tid < B) {
@@ -750,6 +763,8 @@ constexpr int kBuildWarpN = 70000;   // largest system: the whole list build, th
                                      // 57,600 atoms 191 / 174 us, 66,679 202 / 184, 76,666 207 / 208,
                                      // 112,500 244 / 288
 static_assert(kBuildWarpN < 1 << 30, "a kept hit's kind shares a word with its atom");
+constexpr int kBuildImages = 62;     // stencil half-width in boxes, at most, by the plan: 2 * 62 + 2 ranges per row
+static_assert(2 * kBuildImages + 2 <= kBuildSegs, "one row's ranges must fit");
 constexpr float kBuildMinEdge = 16.0f;   // shortest box edge: the list cutoff over this (at most 34 ranges per row)
 
 __global__ void __launch_bounds__(32 * kBuildWarps, 8) k_build_warp(
@@ -1291,6 +1306,8 @@ cudaError_t launch_neighbors(const float* pos, const int* type, int T, float4* p
                              float rc_phys, float min_edge, nep_nlist* nl, const NbrWork& w, cudaStream_t st) {
     cudaError_t e;
     const int cmax = w.cmax;
+    const bool warp_build = N <= kBuildWarpN && min_edge * kBuildMinEdge >= rc_list;
+    const int max_images = warp_build ? kBuildImages : std::numeric_limits<int>::max();
     if (N > 0 && N <= kCellsSmallN && B <= kCellsSmallB) {
         const int smem = (int)sizeof(int) * (cmax + 1);
         // with the static arrays past 48 KB (138 KB at most), which needs the attribute
@@ -1298,13 +1315,13 @@ cudaError_t launch_neighbors(const float* pos, const int* type, int T, float4* p
             (e = cudaFuncSetAttribute(k_cells_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sizeof(int) * (2 * kCellsSmallN + 27 * kCellsSmallB + 1))))
             return e;
-        launch_pdl(k_cells_small, 1, 1024, smem, st, pos, type, atom_off, box, N, B, T, rc_list, pos4, cfg, nl->status,
-                                             w.plan, w.cell_of, w.cell_start, w.cell_pos);
+        launch_pdl(k_cells_small, 1, 1024, smem, st, pos, type, atom_off, box, N, B, T, rc_list, max_images,
+                                             pos4, cfg, nl->status, w.plan, w.cell_of, w.cell_start, w.cell_pos);
     } else {
         if ((e = cudaMemsetAsync(nl->status, 0, 4 * sizeof(int), st))) return e;
         if (N == 0) return cudaSuccess;
         if ((e = launch_pack(pos, type, atom_off, N, B, T, pos4, cfg, nl->status, st))) return e;
-        k_cell_plan<<<blocks(B, 128), 128, 0, st>>>(box, atom_off, B, rc_list, w.plan, nl->status);
+        k_cell_plan<<<blocks(B, 128), 128, 0, st>>>(box, atom_off, B, rc_list, max_images, w.plan, nl->status);
         k_plan_scan<<<1, 32, 0, st>>>(w.plan, B);
         if ((e = cudaMemsetAsync(w.cell_cnt, 0, sizeof(int) * (size_t)(cmax + 1), st)) != cudaSuccess) return e;
         k_bin<<<blocks(N, 256), 256, 0, st>>>(pos, cfg, box, w.plan, N, w.cell_of, w.rank, w.cell_cnt, nl->status);
@@ -1317,7 +1334,7 @@ cudaError_t launch_neighbors(const float* pos, const int* type, int T, float4* p
         k_sort_cells<<<blocks(cmax, 128), 128, 0, st>>>(w.cell_start, cmax, w.cell_atoms, pos4, w.cell_pos);
     }
     const float rr = rc_list * rc_list, ra = rc_list_ang * rc_list_ang, rp = rc_phys * rc_phys;
-    if (N <= kBuildWarpN && min_edge * kBuildMinEdge >= rc_list)
+    if (warp_build)
         launch_pdl(k_build_warp, blocks(N, kBuildWarps), 32 * kBuildWarps, 0, st, pos4, cfg, box, w.plan, w.cell_of,
                                                                           w.cell_start, w.cell_pos, N, rr, ra, rp,
                                                                           w.row_start, w.slot_row, *nl);

@@ -392,3 +392,23 @@ def test_block_sizes_stay_pinned_without_a_variant(nb):
     nb.set_variant(model, 0)
     nb.set_variant(model, -1)
     assert np.array_equal(run(), default)
+
+
+def test_list_build_device_box_thinner_than_the_hosts(nb):
+    """The list build is chosen by the host's copy of the boxes.  Where the
+    device's box of a configuration is far thinner (its rows would have more
+    images than the warp build holds), the call ends with invalid input, that
+    configuration's lists are empty and the others' as before."""
+    h = I.HYPER_SMALL
+    s, model, dsys, nl, ws = setup(nb, h, [300, 40, 200], 75)
+    before = [t.cpu().numpy().reshape(-1, s.n_atoms) for t in (nl.cnt, nl.cnt_ang, nl.nbr)]
+    dsys.box[1] = 0.1
+    nb.neighbors(model, dsys, nl, 0.0, ws)
+    assert nb.check_list(nl) == nb.NEP_ERR_INPUT
+    after = [t.cpu().numpy().reshape(-1, s.n_atoms) for t in (nl.cnt, nl.cnt_ang, nl.nbr)]
+    assert not after[0][:, 300:340].any() and not after[1][:, 300:340].any()
+    for cols in (slice(0, 300), slice(340, 540)):
+        used = np.arange(len(before[2]))[:, None] < before[0][:, cols]
+        assert np.array_equal(before[0][:, cols], after[0][:, cols])
+        assert np.array_equal(before[1][:, cols], after[1][:, cols])
+        assert np.array_equal(before[2][:, cols][used], after[2][:, cols][used])
