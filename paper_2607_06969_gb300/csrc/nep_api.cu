@@ -282,18 +282,33 @@ EvalSplit eval_split(const nep_model* m, const nep_system* s, bool images) {
 // Lanes per atom of the training operator's per-atom backward, 0 for one thread
 // per atom, whose forward then leaves records for it.  A loss gradient's
 // forward is otherwise the plain evaluation; an adjoint product needs none.
-// Measured with the reduction, uneven packings, graph, against one thread per
-// atom (38-30-1, 42-50-1, 52-64-1):
-//   adjoint product: 20,405 atoms 181 / 289, 240 / 389, 332 / 459 us; 31,888
-//     267 / 342, 374 / 453, 533 / 554
-//   loss gradient: 31,888 atoms 365 / 376, 490 / 488, 660 / 570
-// 16 lanes against 32: 2,548 atoms 80.5 / 83.2, 96.6 / 94.6, 115 / 107; 20,405
+// The lines lie where the forms measured equal.  They follow the CTAs that fit
+// an SM beside the model's image (3, 2 or 1): with few of them kg_grad has too
+// few warps for its chains.  Lane groups / one thread per atom, equal packings:
+//   3 CTAs  38-30-1  loss 24,448 atoms 304 / 330 us, 30,976 375 / 362
+//                    adjoint 33,408 294 / 327
+//           42-50-1  loss 19,968 367 / 400, 24,448 416 / 421
+//                    adjoint 30,976 382 / 420
+//   2 CTAs  52-64-1  loss 13,952 341 / 387, 19,968 471 / 459, 24,448 535 / 481
+//                    adjoint 24,448 410 / 443, 30,976 523 / 503
+//           52-112-1 loss 13,952 434 / 452, 19,968 597 / 551; adjoint 24,448 525 / 545
+//   1 CTA   52-128-1 loss 9,000 391 / 426, 13,952 545 / 467, 24,448 882 / 609
+//                    adjoint 9,000 274 / 387, 13,952 430 / 428, 24,448 722 / 570
+//           38-200-1 loss 9,000 372 / 410, 13,952 528 / 455; adjoint 13,952 415 / 415
+// 16 lanes against 32: 2,548 atoms 80.5 / 83.2, 96.6 / 94.6, 115 / 107 us; 20,405
 //   281 / 300, 375 / 372, 496 / 489: for n_ang <= 6 (fewer sums per lane) only
 int train_lanes(const nep_model* m, const nep_system* s, bool loss) {
-    const int N = s->n_atoms;
-    const bool narrow = m->hp.n_ang <= 6;
-    const int most = loss ? (narrow ? 34000 : 25000) : (narrow ? 40000 : 32000);
-    if (N == 0 || m->pinned(size_bin(s)) || !m->ks->group_train_fits(m->hp.n_hidden) || N > most) return 0;
+    const int N = s->n_atoms, ctas = m->ks->group_train_ctas(m->hp.n_hidden);
+    if (N == 0 || m->pinned(size_bin(s)) || !ctas) return 0;
+    const bool narrow = m->hp.n_ang <= nep::kGradNarrowNA;
+    int most;
+    if (ctas >= 3)
+        most = loss ? (narrow ? 28000 : 25000) : (narrow ? 38000 : 32000);
+    else if (ctas == 2)
+        most = loss ? 18000 : 27000;
+    else
+        most = loss ? 10500 : 13000;
+    if (N > most) return 0;
     return N > 2000 && narrow ? 16 : 32;
 }
 bool block_choice(int b) {

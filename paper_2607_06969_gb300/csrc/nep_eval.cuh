@@ -1266,7 +1266,7 @@ cudaError_t init_t(int H) {
                                    &train_t<Cfg<NR, NA, KR, KA, H4, T>>,                         \
                                    &grad_chunks_t<Cfg<NR, NA, KR, KA, H4, T>>,                   \
                                    &group_fits_t<Cfg<NR, NA, KR, KA, H4, T>>,                    \
-                                   &group_train_fits_t<Cfg<NR, NA, KR, KA, H4, T>>,              \
+                                   &group_train_ctas_t<Cfg<NR, NA, KR, KA, H4, T>>,              \
                                    &group_init_t<Cfg<NR, NA, KR, KA, H4, T>>,                    \
                                    &launch_group_t<Cfg<NR, NA, KR, KA, H4, T>>,                  \
                                    &launch_group_finish_t<Cfg<NR, NA, KR, KA, H4, T>>};

@@ -65,6 +65,7 @@ constexpr int kDefaultAngularVariant = 0; // 2 blocks per SM, S_nlm in tensor me
 constexpr int kSizeBins = 32;             // tuning table: log2 of mean atoms per configuration
 constexpr int kBlockChoices[3] = {64, 128, 256};   // block sizes the tuner tries for radial / finish
 constexpr int kRadialSplit = 1;           // launch code of the radial kernel with four lanes per atom
+constexpr int kGradNarrowNA = 6;          // training backward: models up to this n_ang take 16 lanes per atom, others 32
 constexpr int kRowStride = 64;            // list build: bytes of per-atom stencil row starts
 
 // Stencil/cell plan of one configuration for the neighbour build.
@@ -182,7 +183,7 @@ struct KernelSet {
     int (*grad_chunks)(int N);
     // a group of G lanes per atom (nep_group.cuh), G = 8 or 32
     bool (*group_fits)(int H);
-    bool (*group_train_fits)(int H);
+    int (*group_train_ctas)(int H);   // CTAs of the backward that fit an SM, 0 if none
     cudaError_t (*group_init)(int H);
     cudaError_t (*group_atom)(const EvalArgs&, cudaStream_t, int G);
     cudaError_t (*group_finish)(const EvalArgs&, const FinishArgs&, int max_chunks, cudaStream_t, int G);

@@ -814,11 +814,14 @@ cudaError_t train_init_t(int H) {
 template <class C>
 int grad_chunks_t(int N) { return grad_chunks_of(N); }
 
-// whether a model of H hidden units fits the group kernels' shared memory
+// CTAs of kg_grad that fit an SM in the form that large batches take, 0 if a
+// model of H hidden units does not fit the group kernels' shared memory
 template <class C>
-bool group_train_fits_t(int H) {
-    return group_fits_t<C>(H) && GroupGradSmem<C, 16>::bytes(H) <= kMaxDynSmem &&
-           GroupGradSmem<C, 32>::bytes(H) <= kMaxDynSmem;
+int group_train_ctas_t(int H) {
+    if (!group_fits_t<C>(H) || GroupGradSmem<C, 16>::bytes(H) > kMaxDynSmem ||
+        GroupGradSmem<C, 32>::bytes(H) > kMaxDynSmem)
+        return 0;
+    return C::NA <= kGradNarrowNA ? group_grad_per_sm<C, 16>(H) : group_grad_per_sm<C, 32>(H);
 }
 
 // G: lanes per atom of the per-atom backward (16 or 32), 0 for one thread per atom

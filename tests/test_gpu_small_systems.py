@@ -412,3 +412,44 @@ def test_list_build_device_box_thinner_than_the_hosts(nb):
         assert np.array_equal(before[0][:, cols], after[0][:, cols])
         assert np.array_equal(before[1][:, cols], after[1][:, cols])
         assert np.array_equal(before[2][:, cols][used], after[2][:, cols][used])
+
+
+def wide_hidden(h, n):
+    return I.Hyper(**{**h.__dict__, "n_hidden": n})
+
+
+@pytest.mark.parametrize("h,total", [(I.HYPER_SMALL, 12000), (I.HYPER_SMALL, 28000), (I.HYPER_SMALL, 28001),
+                                     (I.HYPER_SMALL, 38000), (I.HYPER_SMALL, 38001),
+                                     (I.HYPER_TABLE2, 25000), (I.HYPER_TABLE2, 25001),
+                                     (I.HYPER_TABLE2, 32000), (I.HYPER_TABLE2, 32001),
+                                     (I.HYPER_LARGE, 18000), (I.HYPER_LARGE, 18001),
+                                     (I.HYPER_LARGE, 27000), (I.HYPER_LARGE, 27001),
+                                     (wide_hidden(I.HYPER_LARGE, 128), 10500), (wide_hidden(I.HYPER_LARGE, 128), 10501),
+                                     (wide_hidden(I.HYPER_SMALL, 200), 13000), (wide_hidden(I.HYPER_SMALL, 200), 13001)],
+                         ids=lambda x: str(x) if isinstance(x, int) else f"{x.dim}-{x.n_hidden}")
+def test_training_forms_agree_at_the_lines(nb, h, total):
+    """The loss gradient and the adjoint product on both sides of the lines
+    between lane groups and one thread per atom, for models of which three,
+    two and one block fit an SM, against one thread per atom; above 10,000
+    atoms the lane groups' forward is the four-lane radial kernel.  Bar as in
+    test_lane_groups_training_agrees_with_one_thread_per_atom."""
+    import torch
+    n = total // 40
+    s, model, dsys, nl, _ = setup(nb, h, [n] * 39 + [total - 39 * n], 76, cap=112, cap_ang=56)
+    ws = nb.Workspace(model, s.n_atoms, s.n_cfg, 112, 56, train=True)
+    rng = np.random.default_rng(4)
+    dev = lambda x, t: torch.tensor(np.ascontiguousarray(x), dtype=t, device="cuda")   # noqa: E731
+    e = dev(rng.normal(size=s.n_cfg), torch.float64)
+    f = dev(rng.normal(size=(3, s.n_atoms)), torch.float32)
+    v = dev(rng.normal(size=(s.n_cfg, 9)), torch.float64)
+
+    def grads():
+        g1, loss = nb.param_grad(model, dsys, nl, ws, e, f, v)
+        g2 = nb.param_grad_adjoint(model, dsys, nl, ws, e, f, v)
+        return g1.cpu().numpy(), loss.item(), g2.cpu().numpy()
+
+    got = grads()
+    nb.set_variant(model, 0)
+    want = grads()
+    for x, y in zip(got, want):
+        assert np.linalg.norm(np.asarray(x) - y) <= 1e-5 * np.linalg.norm(y)
