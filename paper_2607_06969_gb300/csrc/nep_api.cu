@@ -3,6 +3,7 @@
 // happens in the hot calls.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -683,10 +684,16 @@ nep_status neighbors_impl(nep_model* m, const nep_system* s, float skin, nep_nli
     nep_nlist copy = *nl;
     if (mi) copy.shift = nullptr;
     float min_edge = s->box_host[0];
-    for (int x = 1; x < 3 * B; ++x) min_edge = s->box_host[x] < min_edge ? s->box_host[x] : min_edge;
+    double density = 0.0;
+    for (int b = 0; b < B; ++b) {
+        const float* L = s->box_host + 3 * b;
+        for (int d = 0; d < 3; ++d) min_edge = L[d] < min_edge ? L[d] : min_edge;
+        const double n = s->atom_off_host[b + 1] - s->atom_off_host[b];
+        density += n * n / ((double)L[0] * L[1] * L[2] * std::max(N, 1));
+    }
     NEP_CUDA(nep::launch_neighbors(s->pos, s->type, m->hp.n_types, at<float4>(work, w.pos4), s->atom_off, s->box,
-                                   at<int>(work, w.cfg), N, B, rc_list, rc_list_ang, m->hp.rc_rad, min_edge, &copy,
-                                   nw, st),
+                                   at<int>(work, w.cfg), N, B, rc_list, rc_list_ang, m->hp.rc_rad, min_edge, density,
+                                   &copy, nw, st),
              "neighbour build");
     return NEP_OK;
 }

@@ -217,10 +217,12 @@ struct NbrWork {
 };
 size_t nbr_cell_capacity(int N, int B);
 // clears nl->status, packs the atoms and builds the list and its reverse index;
-// min_edge: the shortest box edge
+// min_edge: the shortest box edge; density: atoms per volume of an atom's own
+// configuration, averaged over the atoms
 cudaError_t launch_neighbors(const float* pos, const int* type, int T, float4* pos4, const int* atom_off,
                              const float* box, int* cfg, int N, int B, float rc_list, float rc_list_ang,
-                             float rc_phys, float min_edge, nep_nlist* nl, const NbrWork& w, cudaStream_t st);
+                             float rc_phys, float min_edge, double density, nep_nlist* nl, const NbrWork& w,
+                             cudaStream_t st);
 
 // FP64 evaluation and training gradient (nep_fp64.cu): runtime
 // hyper-parameters, every quantity in double.  Bounds of the per-thread

@@ -1,6 +1,7 @@
 // Model-independent kernels of libnep: input packing, the cell-list
 // neighbour build, the deterministic force gather with FP64 reductions, and
 // the velocity-Verlet updates.
+#include <algorithm>
 #include <limits>
 
 #include <cuda_runtime.h>
@@ -762,6 +763,17 @@ constexpr int kBuildHits = 192;      // hits kept for the second pass; beyond, i
 constexpr int kBuildWarpN = 70000;   // largest system: the whole list build, thread / warp per atom:
                                      // 57,600 atoms 191 / 174 us, 66,679 202 / 184, 76,666 207 / 208,
                                      // 112,500 244 / 288
+// With few entries per atom a thread's walk is short and the warp's rows and
+// scans are what counts, so the line falls with the mean list length that the
+// boxes' volumes give (uniform gases, rc 8 A, thread / warp per atom):
+//   entries  21: 50,000 atoms 131 / 129 us, 60,000 138 / 146
+//             7: 30,000 103 / 97, 40,000 111 / 115, 69,000 121 / 156
+//           3.5: 20,000 91 / 86, 30,000 93 / 99
+//             2: 14,000 82 / 78, 20,000 86 / 88, 60,000 108 / 152
+//           0.1: 10,000 107 / 106, 14,000 115 / 117, 30,000 134 / 152
+inline int build_warp_most(double entries) {
+    return (int)std::min({14000.0 + 3100.0 * entries, 28000.0 + 1100.0 * entries, (double)kBuildWarpN});
+}
 static_assert(kBuildWarpN < 1 << 30, "a kept hit's kind shares a word with its atom");
 constexpr int kBuildImages = 62;     // stencil half-width in boxes, at most, by the plan: 2 * 62 + 2 ranges per row
 static_assert(2 * kBuildImages + 2 <= kBuildSegs, "one row's ranges must fit");
@@ -1029,8 +1041,11 @@ __device__ __forceinline__ void rev_slot(int N, int i, int s, int rows, bool tra
 // G = 1: one thread per atom; G = 32: a warp per atom, a lane per slot.  The
 // warps lose the coalescing of the slot-major list, but up to kRevWarpN atoms
 // the shorter walk is worth more (the list build of 57,600 atoms 214 -> 203
-// us, of 112,500 atoms 259 -> 262).
-constexpr int kRevWarpN = 80000;
+// us, of 112,500 atoms 259 -> 262).  With few entries per atom most lanes have
+// none (gases, thread / warp per atom: 7 entries, 50,000 atoms 113 / 112 us,
+// 69,000 114 / 121; 0.7, 30,000 97 / 97, 40,000 102 / 107, 69,000 108 / 119).
+constexpr int kRevWarpN = 80000, kRevWarpSparseN = 40000;
+constexpr double kRevSparse = 7.5;
 template <int G>
 __global__ void __launch_bounds__(128) k_rev(int N, const int* cfg, const CellPlan* plan,
                                              const unsigned char* row_start,
@@ -1303,10 +1318,12 @@ size_t nbr_cell_capacity(int N, int B) { return 2 * (size_t)N + 27 * (size_t)B; 
 
 cudaError_t launch_neighbors(const float* pos, const int* type, int T, float4* pos4, const int* atom_off,
                              const float* box, int* cfg, int N, int B, float rc_list, float rc_list_ang,
-                             float rc_phys, float min_edge, nep_nlist* nl, const NbrWork& w, cudaStream_t st) {
+                             float rc_phys, float min_edge, double density, nep_nlist* nl, const NbrWork& w,
+                             cudaStream_t st) {
     cudaError_t e;
     const int cmax = w.cmax;
-    const bool warp_build = N <= kBuildWarpN && min_edge * kBuildMinEdge >= rc_list;
+    const double entries = density * 4.18879 * rc_list * rc_list * rc_list;   // 4 pi / 3
+    const bool warp_build = N <= build_warp_most(entries) && min_edge * kBuildMinEdge >= rc_list;
     const int max_images = warp_build ? kBuildImages : std::numeric_limits<int>::max();
     if (N > 0 && N <= kCellsSmallN && B <= kCellsSmallB) {
         const int smem = (int)sizeof(int) * (cmax + 1);
@@ -1341,7 +1358,7 @@ cudaError_t launch_neighbors(const float* pos, const int* type, int T, float4* p
     else
         k_build<<<blocks(N, 128), 128, 0, st>>>(pos4, cfg, box, w.plan, w.cell_of, w.cell_start,
                                                 w.cell_pos, N, rr, ra, rp, w.shell, w.row_start, w.slot_row, *nl);
-    if (N <= kRevWarpN)
+    if (N <= (entries < kRevSparse ? kRevWarpSparseN : kRevWarpN))
         launch_pdl(k_rev<32>, blocks(N, 4), 128, 0, st, N, cfg, w.plan, w.row_start, w.slot_row, *nl);
     else
         k_rev<1><<<blocks(N, 128), 128, 0, st>>>(N, cfg, w.plan, w.row_start, w.slot_row, *nl);

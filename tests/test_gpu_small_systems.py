@@ -453,3 +453,45 @@ def test_training_forms_agree_at_the_lines(nb, h, total):
     want = grads()
     for x, y in zip(got, want):
         assert np.linalg.norm(np.asarray(x) - y) <= 1e-5 * np.linalg.norm(y)
+
+
+@pytest.mark.parametrize("n,entries", [(9000, 0.5), (12000, 3.0), (20500, 5.0)])
+def test_list_build_forms_agree_on_sparse_systems(nb, n, entries):
+    """Gases: the line between a warp and a thread per atom falls with the
+    mean list length, and with it that of the reverse search.  A configuration
+    alone (below the lines) gets, entry for entry, the list of each of its two
+    copies (above them); and the pairs are those of a k-d tree."""
+    from scipy.spatial import cKDTree
+    h = I.HYPER_SMALL
+    rc = h.rc_rad
+    L = np.float32((n * 4.0 / 3.0 * np.pi * rc ** 3 / entries) ** (1.0 / 3.0))
+    pos = (np.random.default_rng(7).random((n, 3)) * L * 0.9999).astype(np.float32)
+    types = (np.arange(n) % 3).astype(np.int32)
+    model = nb.Model(h, I.init_params(h).astype(np.float32))
+
+    def build(copies):
+        s = I.System(pos=np.tile(pos, (copies, 1)), types=np.tile(types, copies),
+                     box=np.full((copies, 3), L), atom_off=n * np.arange(copies + 1))
+        dsys = nb.DeviceSystem.from_inputs(s)
+        nl = nb.NeighborList(s.n_atoms, 64, 48)
+        nb.neighbors(model, dsys, nl, 0.0, nb.Workspace(model, s.n_atoms, copies, 64, 48))
+        assert nb.check_list(nl) == nb.NEP_OK, nb.last_error()
+        return [t.cpu().numpy().reshape(-1, s.n_atoms) for t in (nl.cnt, nl.cnt_ang, nl.nbr, nl.rev)]
+
+    one, two = build(1), build(2)
+    used = np.arange(64)[:, None] < one[0]
+    ang = np.arange(48)[:, None] < one[1]
+    for c in (0, 1):
+        cols = slice(c * n, (c + 1) * n)
+        assert np.array_equal(one[0], two[0][:, cols]) and np.array_equal(one[1], two[1][:, cols])
+        assert np.array_equal(one[2][used], two[2][:, cols][used] - c * n)
+        assert np.array_equal(one[3][ang], two[3][:, cols][ang])
+    # pairs nearer to the cutoff than FP32 rounds a distance in this box may go either way
+    eps = 4.0 * float(L) * 2.0 ** -24
+    tree = cKDTree(pos.astype(np.float64), boxsize=float(L))
+    sure, maybe = (tree.query_pairs(rc + d, output_type="ndarray") for d in (-eps, eps))
+    code = lambda i, j: set((np.minimum(i, j).astype(np.int64) * n + np.maximum(i, j)).tolist())   # noqa: E731
+    slot, i = np.nonzero(used)
+    got = code(i, one[2][slot, i])
+    assert len(slot) == 2 * len(got)
+    assert code(*sure.T) <= got <= code(*maybe.T)
