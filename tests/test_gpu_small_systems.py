@@ -495,3 +495,33 @@ def test_list_build_forms_agree_on_sparse_systems(nb, n, entries):
     got = code(i, one[2][slot, i])
     assert len(slot) == 2 * len(got)
     assert code(*sure.T) <= got <= code(*maybe.T)
+
+
+@pytest.mark.parametrize("n,box", [(58, (3000.0, 3000.0, 3000.0)), (700, (2900.0, 500.0, 40.0)),
+                                   (700, (30.0, 900.0, 3100.0)), (9000, (3050.0, 2000.0, 300.0))])
+def test_list_of_atoms_in_a_nearly_empty_box(nb, n, box):
+    """Boxes with far more cutoff-sized cells than twice the atoms, where the
+    plan merges cells, edge by edge: the pairs are those of a k-d tree."""
+    from scipy.spatial import cKDTree
+    h = I.HYPER_SMALL
+    box = np.array(box, np.float32)
+    rng = np.random.default_rng(8)
+    centre = rng.random((n // 4 + 1, 3)) * box       # small clusters, so that there are pairs
+    pos = centre[rng.integers(0, len(centre), n)] + rng.normal(0.0, 3.0, (n, 3))
+    pos = np.minimum((pos % box).astype(np.float32), np.nextafter(box, np.float32(0.0)))
+    s = I.System(pos=pos, types=(np.arange(n) % 3).astype(np.int32), box=box[None], atom_off=np.array([0, n]))
+    model = nb.Model(h, I.init_params(h).astype(np.float32))
+    dsys = nb.DeviceSystem.from_inputs(s)
+    nl = nb.NeighborList(n, 64, 48)
+    nb.neighbors(model, dsys, nl, 0.0, nb.Workspace(model, n, 1, 64, 48))
+    assert nb.check_list(nl) == nb.NEP_OK, nb.last_error()
+    cnt, nbr = nl.cnt.cpu().numpy(), nl.nbr.cpu().numpy().reshape(-1, n)
+    slot, i = np.nonzero(np.arange(64)[:, None] < cnt)
+    code = lambda i, j: set((np.minimum(i, j).astype(np.int64) * n + np.maximum(i, j)).tolist())   # noqa: E731
+    got = code(i, nbr[slot, i])
+    # pairs nearer to the cutoff than FP32 rounds a distance in this box may go either way
+    eps = 4.0 * float(box.max()) * 2.0 ** -24
+    tree = cKDTree(pos.astype(np.float64), boxsize=box.astype(np.float64))
+    sure, maybe = (tree.query_pairs(h.rc_rad + d, output_type="ndarray") for d in (-eps, eps))
+    assert len(sure) > n // 2 and len(slot) == 2 * len(got)
+    assert code(*sure.T) <= got <= code(*maybe.T)
