@@ -779,14 +779,16 @@ constexpr int kBuildWarpN = 70000;   // largest system: the whole list build, th
                                      // 112,500 244 / 288
 // With few entries per atom a thread's walk is short and the warp's rows and
 // scans are what counts, so the line falls with the mean list length that the
-// boxes' volumes give (uniform gases, rc 8 A, thread / warp per atom):
-//   entries  21: 50,000 atoms 131 / 129 us, 60,000 138 / 146
-//             7: 30,000 103 / 97, 40,000 111 / 115, 69,000 121 / 156
-//           3.5: 20,000 91 / 86, 30,000 93 / 99
-//             2: 14,000 82 / 78, 20,000 86 / 88, 60,000 108 / 152
-//           0.1: 10,000 107 / 106, 14,000 115 / 117, 30,000 134 / 152
+// boxes' volumes give (uniform gases, thread / warp per atom):
+//   entries  28: 60,000 atoms 177 / 154 us, 69,000 180 / 169
+//            14: 46,000 129 / 119, 60,000 133 / 140
+//           9.3: 46,000 119 / 117, 50,000 120 / 121, 69,000 126 / 150
+//           4.7: 30,000 95 / 89, 36,000 95 / 97, 69,000 110 / 145
+//           2.3: 20,000 79 / 75, 25,000 79 / 81, 60,000 92 / 129
+//           0.5: 14,000 68 / 64, 16,000 67 / 68, 30,000 70 / 85
+//          0.05: 10,000 62 / 60, 12,000 61 / 62, 30,000 65 / 83
 inline int build_warp_most(double entries) {
-    return (int)std::min({14000.0 + 3100.0 * entries, 28000.0 + 1100.0 * entries, (double)kBuildWarpN});
+    return (int)std::min({12000.0 + 5000.0 * entries, 29000.0 + 1650.0 * entries, (double)kBuildWarpN});
 }
 static_assert(kBuildWarpN < 1 << 30, "a kept hit's kind shares a word with its atom");
 constexpr int kBuildImages = 62;     // stencil half-width in boxes, at most, by the plan: 2 * 62 + 2 ranges per row
@@ -1056,10 +1058,11 @@ __device__ __forceinline__ void rev_slot(int N, int i, int s, int rows, bool tra
 // warps lose the coalescing of the slot-major list, but up to kRevWarpN atoms
 // the shorter walk is worth more (the list build of 57,600 atoms 214 -> 203
 // us, of 112,500 atoms 259 -> 262).  With few entries per atom most lanes have
-// none (gases, thread / warp per atom: 7 entries, 50,000 atoms 113 / 112 us,
-// 69,000 114 / 121; 0.7, 30,000 97 / 97, 40,000 102 / 107, 69,000 108 / 119).
-constexpr int kRevWarpN = 80000, kRevWarpSparseN = 40000;
-constexpr double kRevSparse = 7.5;
+// none (gases, thread / warp per atom: 4.7 entries, 50,000 atoms 106 / 104 us,
+// 69,000 107 / 110; 2.3, 40,000 88 / 87, 46,000 89 / 90, 69,000 91 / 95; 0.5,
+// 36,000 75 / 74, 40,000 71 / 75, 69,000 74 / 83).
+constexpr int kRevWarpN = 80000, kRevWarpSparseN = 42000;
+constexpr double kRevSparse = 4.0;
 template <int G>
 __global__ void __launch_bounds__(128) k_rev(int N, const int* cfg, const CellPlan* plan,
                                              const unsigned char* row_start,

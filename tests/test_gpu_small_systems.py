@@ -455,7 +455,7 @@ def test_training_forms_agree_at_the_lines(nb, h, total):
         assert np.linalg.norm(np.asarray(x) - y) <= 1e-5 * np.linalg.norm(y)
 
 
-@pytest.mark.parametrize("n,entries", [(9000, 0.5), (12000, 3.0), (20500, 5.0)])
+@pytest.mark.parametrize("n,entries", [(9000, 0.5), (14000, 3.0), (21500, 3.5)])
 def test_list_build_forms_agree_on_sparse_systems(nb, n, entries):
     """Gases: the line between a warp and a thread per atom falls with the
     mean list length, and with it that of the reverse search.  A configuration
