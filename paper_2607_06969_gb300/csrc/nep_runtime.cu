@@ -2,7 +2,6 @@
 // neighbour build, the deterministic force gather with FP64 reductions, and
 // the velocity-Verlet updates.
 #include <algorithm>
-#include <limits>
 
 #include <cuda_runtime.h>
 
@@ -235,8 +234,8 @@ static_assert(kMaxRows < kRowStride, "row starts must fit one atom's stride");
 // plan of one configuration; base holds its cell count until the prefix is taken.
 // The build kernel is chosen by the host's copy of the boxes.  A box on the
 // device so much thinner that the cutoff reaches over more than max_images of
-// it is invalid input: its stencil has no rows (-1 of them; k_build_warp alone
-// sets a limit).
+// it (0: any number) is invalid input: its stencil has no rows (-1 of them;
+// k_build_warp alone sets a limit).
 __device__ CellPlan cell_plan_of(const float* box, const int* atom_off, int b, float rc, int max_images, int* status) {
     const int nb = atom_off[b + 1] - atom_off[b];
     float L[3] = {box[3 * b], box[3 * b + 1], box[3 * b + 2]};
@@ -265,10 +264,10 @@ __device__ CellPlan cell_plan_of(const float* box, const int* atom_off, int b, f
         for (int d = 0; d < 3; ++d) nc[d] = min(nc[d], t);
     }
     while ((long long)nc[0] * nc[1] * nc[2] > cap) {
-        int m = 0;
-        if (nc[1] > nc[m]) m = 1;
-        if (nc[2] > nc[m]) m = 2;
-        nc[m] -= 1;
+        const bool y = nc[1] > nc[0], z = nc[2] > max(nc[0], nc[1]);
+        nc[2] -= z;
+        nc[1] -= y && !z;
+        nc[0] -= !y && !z;
     }
     CellPlan p;
     for (int d = 0; d < 3; ++d) {
@@ -277,13 +276,12 @@ __device__ CellPlan cell_plan_of(const float* box, const int* atom_off, int b, f
         p.half[d] = (int)ceilf((rc + kCellMargin) / cs);
         if (p.half[d] < 1) p.half[d] = 1;
     }
-    for (int d = 0; d < 3; ++d)
-        if (p.half[d] > (long long)max_images * p.nc[d]) {
-            set_flag(status, 3);
-            p.half[0] = -1;
-            p.half[1] = p.half[2] = 0;
-            break;
-        }
+    if (max_images && (p.half[0] > max_images * p.nc[0] || p.half[1] > max_images * p.nc[1] ||
+                       p.half[2] > max_images * p.nc[2])) {
+        set_flag(status, 3);
+        p.half[0] = -1;
+        p.half[1] = p.half[2] = 0;
+    }
     p.base = nc[0] * nc[1] * nc[2];
     p.pad = 0;
     return p;
@@ -1341,7 +1339,7 @@ cudaError_t launch_neighbors(const float* pos, const int* type, int T, float4* p
     const int cmax = w.cmax;
     const double entries = density * 4.18879 * rc_list * rc_list * rc_list;   // 4 pi / 3
     const bool warp_build = N <= build_warp_most(entries) && min_edge * kBuildMinEdge >= rc_list;
-    const int max_images = warp_build ? kBuildImages : std::numeric_limits<int>::max();
+    const int max_images = warp_build ? kBuildImages : 0;
     if (N > 0 && N <= kCellsSmallN && B <= kCellsSmallB) {
         const int smem = (int)sizeof(int) * (cmax + 1);
         // with the static arrays past 48 KB (138 KB at most), which needs the attribute
