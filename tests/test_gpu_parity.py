@@ -241,7 +241,9 @@ def test_every_angular_variant(nb, variant):
 
 def test_autotune_variants_agree(nb):
     """Every compiled register-budget variant and block size computes the
-    same E, F, V; the autotuner picks valid choices and later calls use them."""
+    same E, F, V.  The autotuner picks valid choices; a call after it agrees
+    (at this size the lane groups run, whose choices are fixed), and the kernels
+    that it chooses for run where the choices are pinned."""
     h = I.HYPER_SMALL
     s = I.packing_batch([57, 100, 250], tag=67)
     th = I.init_params(h).astype(np.float32)

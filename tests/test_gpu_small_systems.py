@@ -525,3 +525,83 @@ def test_list_of_atoms_in_a_nearly_empty_box(nb, n, box):
     sure, maybe = (tree.query_pairs(h.rc_rad + d, output_type="ndarray") for d in (-eps, eps))
     assert len(sure) > n // 2 and len(slot) == 2 * len(got)
     assert code(*sure.T) <= got <= code(*maybe.T)
+
+
+def exactly(n, seed=1):
+    """Rock salt with vacancies, n atoms (the last ones left out)."""
+    ncell = int(np.ceil((n / 7.0) ** (1.0 / 3.0)))
+    s = I.rocksalt(ncell, vacancy=0.1, seed=seed)
+    assert s.n_atoms >= n
+    return I.System(pos=((s.pos + 1.5) % s.box[0])[:n], types=s.types[:n], box=s.box, atom_off=np.array([0, n]))
+
+
+def listed(nb, h, s, skin, precision=0):
+    model = nb.Model(h, I.init_params(h, seed=5).astype(np.float32), precision=precision)
+    dsys = nb.DeviceSystem.from_inputs(s)
+    nl = nb.NeighborList(s.n_atoms, 160, 80)
+    ws = nb.Workspace(model, s.n_atoms, s.n_cfg, 160, 80)
+    nb.neighbors(model, dsys, nl, skin, ws)
+    assert nb.check_list(nl) == nb.NEP_OK, nb.last_error()
+    return model, dsys, nl, ws
+
+
+@pytest.mark.parametrize("hname,n", [("small", 50000), ("small", 50001), ("large", 50000), ("large", 50001),
+                                     ("table2", 200000), ("table2", 200001)])
+def test_large_split_lines_agree_with_one_thread_per_atom(nb, hname, n):
+    """The finish kernel's last lane-group size and the four-lane radial
+    kernel's, and the sizes after them, on one large box."""
+    s = exactly(n)
+    model, dsys, nl, ws = listed(nb, MODELS[hname], s, 1.0)
+    assert_close(*both_forms(nb, model, dsys, nl, ws), np.diff(s.atom_off))
+
+
+@pytest.mark.parametrize("hname,precision,n", [("small", 1, 3000), ("small", 2, 3001), ("small", 1, 13500),
+                                               ("small", 2, 13501), ("large", 1, 8000), ("large", 2, 8001),
+                                               ("large", 1, 25000), ("large", 2, 25001)])
+def test_lane_groups_16bit_network_at_the_lines(nb, hname, precision, n):
+    """As test_lane_groups_16bit_network (its bars), with 32 and with 8 lanes
+    per atom and with the tensor-core kernel after the four-lane radial one:
+    both sides of the lines of a narrow and of a wide network."""
+    s = exactly(n)
+    model, dsys, nl, ws = listed(nb, MODELS[hname], s, 0.5, precision=precision)
+    got, want = both_forms(nb, model, dsys, nl, ws)
+    step = 2.0 ** -11 if precision == 1 else 2.0 ** -8
+    assert np.abs(got[0] - want[0]).max() <= 0.5 * step
+    assert np.sqrt(np.mean((got[1] - want[1]) ** 2)) <= 0.1 * step
+
+
+def test_list_build_of_one_large_box(nb):
+    """One box of 45,000 atoms (a warp per atom in the build and the reverse
+    search) and two copies of it (a thread per atom in both): the same lists,
+    entry for entry."""
+    n = 45000
+    s = exactly(n)
+    lists = []
+    for copies in (1, 2):
+        batch = I.System(pos=np.tile(s.pos, (copies, 1)), types=np.tile(s.types, copies),
+                         box=np.repeat(s.box, copies, 0), atom_off=n * np.arange(copies + 1))
+        _, _, nl, _ = listed(nb, I.HYPER_SMALL, batch, 1.0)
+        lists.append([t.cpu().numpy().reshape(-1, batch.n_atoms) for t in (nl.cnt, nl.cnt_ang, nl.nbr, nl.rev)])
+    one, two = lists
+    used, ang = np.arange(160)[:, None] < one[0], np.arange(80)[:, None] < one[1]
+    for c in (0, 1):
+        cols = slice(c * n, (c + 1) * n)
+        assert np.array_equal(one[0], two[0][:, cols]) and np.array_equal(one[1], two[1][:, cols])
+        assert np.array_equal(one[2][used], two[2][:, cols][used] - c * n)
+        assert np.array_equal(one[3][ang], two[3][:, cols][ang])
+
+
+def test_many_configurations(nb):
+    """The chunk plan rides in the packing launch up to 2,048 configurations
+    and has a launch of its own from there on: the totals of the same 2,048
+    are the same bits, and those of E the sums of E_i."""
+    h = I.HYPER_SMALL
+    counts = [3, 1, 4, 2] * 512
+    res = []
+    for extra in ([], [5]):
+        s, model, dsys, nl, ws = setup(nb, h, counts + extra, 77)
+        res.append([t.cpu().numpy() for t in nb.energy_forces_virial(model, dsys, nl, ws)])
+        sums = np.add.reduceat(res[-1][0].astype(np.float64), s.atom_off[:-1])
+        assert np.abs(res[-1][2] - sums).max() <= 1e-12 * np.abs(sums).max()
+    same = [np.array_equal(a[..., :k], b[..., :k]) for a, b, k in zip(res[0][:3], res[1][:3], (5120, 5120, 2048))]
+    assert all(same) and np.array_equal(res[0][3], res[1][3][:2048])
