@@ -253,11 +253,16 @@ int finish_block(const nep_model* m, const nep_system* s) { return m->tune_finis
 //     15,818: 80.5 / 71.8, -, 115.9 / 110.7; 19,757: 93.2 / 90.1, -, 137.9 / 148.2;
 //     24,300: -, -, 148.8 / 154; 29,491: 119 / 102, -, 183 / 162 (the tensor-core
 //     kernel's tiles of 128 atoms fill whole waves up to 19,456 and 38,912 atoms)
-//   finish kernel, 32 / 16 / 8 lanes (the atom kernel at its best): 2,470 atoms
-//     30.8 / 31.4 / 32.7 us, 33.2 / 33.4 / 35.1, 34.6 / 35.0 / 36.2; 5,249: - /
-//     39.5 / 39.3, 44.9 / 44.5, 49.1 / 51.4; 7,200: - / 42.7 / 45.1, 46.5 / 48.6,
-//     59.1 / 61.7; 9,583: - / 54.1 / 49.0, 68.9 / 64.8, 72.9 / 68.9; ten MD steps of
-//     7,200 atoms 517 / 551, but with images a list and an evaluation of 48
+//   finish kernel, 32 / 16 / 8 lanes (the atom kernel at its best; packings):
+//     2,500 atoms 29.7 / 30.4 / 31.4 us, 33.5 / 33.8 / 36.0, 34.9 / 35.1 / 36.8;
+//     3,500: 33.4 / 32.8 / 33.9, 35.6 / 36.4 / 36.9, 37.7 / 39.5 / 45.1; 4,500:
+//     41.8 / 37.6 / 36.8, 44.2 / 42.0 / 43.1, 49.3 / 46.2 / 47.2; 6,000: 44.1 /
+//     39.5 / 44.0, 49.4 / 44.6 / 49.3, 58.4 / 53.8 / 54.9; 7,200: 49.7 / 44.7 /
+//     47.3, 50.5 / 45.6 / 49.5, 62.9 / 57.9 / 61.5; 7,900: 53.2 / 48.3 / 48.8,
+//     65.6 / 62.2 / 57.1, 72.2 / 68.2 / 67.2; 8,500: 54.2 / 50.3 / 48.5, 66.5 /
+//     63.0 / 58.1, 74.6 / 70.9 / 66.7.  The lead between the lines moves with
+//     how full the last wave of each form is.  Ten MD steps of 7,200 atoms 517 /
+//     551 by 16 / 8 lanes, but with images a list and an evaluation of 48
 //     configurations with 5,800 atoms 100.8 / 97.0
 //   finish kernel, 8 lanes against one thread: 41,990 atoms 119 / 127, 149 / 156,
 //     170 / 179; 57,600: 146 / 145, 172 / 171, 192 / 193; 99,533: 260 / 231

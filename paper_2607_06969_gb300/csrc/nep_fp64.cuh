@@ -53,14 +53,10 @@ __device__ __forceinline__ float sqrt_r(float x) { return sqrtf(x); }
 __device__ __forceinline__ double rint_r(double x) { return rint(x); }
 __device__ __forceinline__ float rint_r(float x) { return rintf(x); }
 
-// sum over the G aligned lanes of an atom; every lane receives the same bits.
-// The shuffles name only the group's lanes: a group whose atom index is past
-// N leaves as a whole, while the other groups of its warp go on.
-template <int G, class R>
-__device__ __forceinline__ R group_sum(R v) {
-    const unsigned mask = G == 32 ? 0xffffffffu : (((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1)));
+// sum over the warp; every lane receives the same bits
+__device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
-    for (int o = G / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 
@@ -218,7 +214,17 @@ __device__ __forceinline__ void basis_derivs(R r, R irc, int K, Out out) {
 template <class A>
 constexpr bool kScatter = std::is_same<A, F32Args>::value;
 
-// up to this many atoms the kernels take 32 lanes per atom, else 8
+// Up to this many atoms the kernels take 32 lanes per atom, else 8.  Packings in
+// a graph, 32 / 8 lanes, evaluation and loss gradient:
+//   38-30-1: 1,300 atoms 232 / 280 us, 516 / 652; 1,600 241 / 287, 562 / 664;
+//     2,000 311 / 289, 779 / 672
+//   52-64-1: 1,600 290 / 382, 757 / 900; 2,000 369 / 383, 952 / 908; 2,600
+//     465 / 438, 1,139 / 1,052
+//   11/7 radial/angular functions, 2 species: 1,300 370 / 430, 873 / 962; 1,600
+//     433 / 333, 1,031 / 770
+//   5/3 functions: 1,000 154 / 259, 388 / 572; 1,300 258 / 259, 593 / 574; 1,600
+//     294 / 266, 714 / 582
+// so the line lies in the middle of where the shapes cross, 1,300 to 2,000.
 constexpr int kEvalLanes32 = 1500;
 // the same for the generic path, whose pipe is not full at these sizes (32 / 8
 // lanes, models of 11/7 and 5/3 radial/angular functions): 2,566 atoms 57.4 /

@@ -545,7 +545,7 @@ __global__ void __launch_bounds__(32 * kGradWarps) k64_grad_partial(const F64Arg
             for (int r = 0; r < 2; ++r)
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const double v = group_sum<32>(acc[r][k]);
+                    const double v = warp_sum(acc[r][k]);
                     if (lane == 0 && r0 + r < nr && c0 + k < nc) out[pbase + (r0 + r) * pstride + c0 + k] = v;
                 }
             continue;
@@ -569,7 +569,7 @@ __global__ void __launch_bounds__(32 * kGradWarps) k64_grad_partial(const F64Arg
             sp = x - gi.nCA;
             double acc = 0.0;
             for (int y = first[sp] + lane; y < first[sp + 1]; y += 32) acc += a.aE[a.cfg[order[y]]];
-            acc = group_sum<32>(acc);
+            acc = warp_sum(acc);
             if (lane == 0) out[sp * L.mlp_stride + H * D + 2 * H] = acc;
             continue;
         }
@@ -584,7 +584,7 @@ __global__ void __launch_bounds__(32 * kGradWarps) k64_grad_partial(const F64Arg
         }
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            const double v = group_sum<32>(acc[r]);
+            const double v = warp_sum(acc[r]);
             if (lane == 0 && r0 + r < nr) out[pbase + r0 + r] = v;
         }
     }
