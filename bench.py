@@ -723,6 +723,16 @@ def mixed_leg(nb, torch, I, ncell: int = 80) -> dict:
     return out
 
 
+def launch_in_effect(h, chosen, n_atoms: int, precision: int = 0) -> dict:
+    """The tuner's choices that a system of n_atoms runs with; None where its
+    kernels are the lane-group ones, whose launch is fixed (the lines stand at
+    nep_autotune in include/nep.h)."""
+    atom = 10000 if not precision else 25000 if h.n_hidden * h.dim > 2500 else 13500
+    return {"angular_variant": chosen[0] if n_atoms > atom else None,
+            "radial_block": chosen[1] if n_atoms > 200000 else None,
+            "finish_block": chosen[2] if n_atoms > 50000 else None}
+
+
 def replicas_leg(nb, torch, I, K: int = 20, dist=None, world: int = 1, rank: int = 0) -> dict:
     """Secondary leg: 1,024 independent periodic packings, N log-uniform in
     [64, 4096] (~975k atoms), config-0 NEP with the FP16 tensor-core network,
@@ -818,7 +828,7 @@ def replicas_leg(nb, torch, I, K: int = 20, dist=None, world: int = 1, rank: int
             "per_replica_loop": {"ms_per_step": ms_loop, "replica_steps_per_s": B_all / (ms_loop * 1e-3),
                                  "steps": KL},
             "speedup_vs_loop": ms_loop / ms,
-            "autotuned": {"angular_variant": chosen[0], "radial_block": chosen[1], "finish_block": chosen[2]},
+            "autotuned": launch_in_effect(h, chosen, N, 1),
             "bins": replica_bins(nb, torch, I, s, h, th, K) if world == 1 else None}
 
 
@@ -838,8 +848,9 @@ def subset(I, s, idx):
 def replica_bins(nb, torch, I, s, h, th, K: int) -> list:
     """The replica batch split by size class (log2 of the atom count): per
     class, its replicas as one batch at the default launch choices and at
-    the autotuned ones (radial and finish block sizes, angular variant),
-    against a loop that steps each replica with its own launches."""
+    the autotuned ones (radial and finish block sizes, angular variant, as far
+    as they are in effect at the batch's size), against a loop that steps each
+    replica with its own launches."""
     masses = I.MASSES.astype(np.float32)
     counts = np.diff(s.atom_off)
     cls = np.floor(np.log2(counts)).astype(int)
@@ -882,8 +893,7 @@ def replica_bins(nb, torch, I, s, h, th, K: int) -> list:
                      "default": {"ms_per_step": ms_default, "replica_steps_per_s": B / (ms_default * 1e-3)},
                      "tuned": {"ms_per_step": ms_tuned, "replica_steps_per_s": B / (ms_tuned * 1e-3),
                                "atom_steps_per_s": sb.n_atoms / (ms_tuned * 1e-3),
-                               "angular_variant": chosen[0], "radial_block": chosen[1],
-                               "finish_block": chosen[2]},
+                               **launch_in_effect(h, chosen, sb.n_atoms, 1)},
                      "loop": {"ms_per_replica_step": ms_loop_per_replica,
                               "replica_steps_per_s": 1e3 / ms_loop_per_replica, "sampled_replicas": len(loop)},
                      "speedup_vs_loop": (ms_loop_per_replica * B) / ms_tuned})
@@ -1205,8 +1215,8 @@ def main():
                 "config": {"workload": WORKLOAD, "n_atoms": N, "parallelism": f"replicas x{world}",
                            "l2": "inputs larger than L2 (neighbour list 0.40 GB, pair scratch 1.4 GB)",
                            "graph": "K steps captured in one CUDA graph",
-                           "launch": ({"autotuned": True, "angular_variant": tuned[0], "radial_block": tuned[1],
-                                       "finish_block": tuned[2]} if tuned else {"autotuned": False})},
+                           "launch": ({"autotuned": True, **launch_in_effect(h, tuned, N)} if tuned
+                                      else {"autotuned": False})},
                 "roofline": roofline, "cpu_baseline": cpu,
                 "e2e": {"value": e2e_val, "unit": "atom-steps/s", "steps": KE,
                         "h2d_bytes_per_step": 24 * N, "d2h_bytes_per_step": 36 * N + 8 + 72},
