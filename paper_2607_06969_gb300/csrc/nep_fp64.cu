@@ -31,7 +31,7 @@ __device__ void group64_sums(const A& a, const Group64<G>& o, R* gb, const Frame
     constexpr int GS = Group64<G>::GS, MPL = Group64<G>::MPL, KW = Group64<G>::KW, KX = Group64<G>::KX;
     constexpr int PARTS = Group64<G>::PARTS;
     const int NA = DM::NA(a), KR = DM::KR(a), KA = DM::KA(a);
-    const R irR = R(1.0) / (R)a.rc_rad, irA = R(1.0) / (R)a.rc_ang;
+    const Cutoff<R> cutR((R)a.rc_rad), cutA((R)a.rc_ang);
     int* tj = reinterpret_cast<int*>(gb + o.oT);
     const int gbase = (threadIdx.x & 31) & ~(G - 1);
     const unsigned gmask = G == 32 ? 0xffffffffu : ((1u << (G & 31)) - 1u), below = (1u << lane) - 1u;
@@ -54,7 +54,7 @@ __device__ void group64_sums(const A& a, const Group64<G>& o, R* gb, const Frame
         const int ni = __popc(mi), ati = __popc(mi & below);
         if (in) {
             tj[ati] = p.tj;
-            basis_values<DM::KX>(p.r, irR, KR, [&](int k, R f) { gb[o.oY + k * GS + ati] = f; });
+            basis_values<DM::KX>(p.r, cutR, KR, [&](int k, R f) { gb[o.oY + k * GS + ati] = f; });
         }
         __syncwarp();
         for (int q = part; q < ni; q += PARTS) {
@@ -77,7 +77,7 @@ __device__ void group64_sums(const A& a, const Group64<G>& o, R* gb, const Frame
         const int na = __popc(ma), at = __popc(ma & below);
         if (ang) {
             R f[DM::KX];
-            basis_values<DM::KX>(p.r, irA, KA, [&](int k, R v) { f[k] = v; });
+            basis_values<DM::KX>(p.r, cutA, KA, [&](int k, R v) { f[k] = v; });
             const R* c = a.prm + a.L.off_cA + (size_t)(fr.ti * a.T + p.tj) * NA * KA;
 #pragma unroll
             for (int n = 0; n < NAX; ++n) {
@@ -188,9 +188,9 @@ __device__ R group64_network(const A& a, const Group64<G>& o, R* gb, int ti, int
 
 // g_n = sum_k c[n][k] Q_k and g'_n with Q'_k, c = cA[ti][tj]
 template <class DM, class A, class R>
-__device__ __forceinline__ void angular_g(const A& a, int ti, int tj, R r, R irA, int NA, int KA, R* g, R* gp) {
+__device__ __forceinline__ void angular_g(const A& a, int ti, int tj, R r, const Cutoff<R>& cutA, int NA, int KA, R* g, R* gp) {
     R f[DM::KX], fp[DM::KX];
-    basis_derivs<DM::KX>(r, irA, KA, [&](int k, R v, R d) {
+    basis_derivs<DM::KX>(r, cutA, KA, [&](int k, R v, R d) {
         f[k] = v;
         fp[k] = d;
     });
@@ -210,10 +210,10 @@ __device__ __forceinline__ void angular_g(const A& a, int ti, int tj, R r, R irA
 
 // the same for both orders of the pair: (g, g') from cA[ti][tj], (h, h') from cA[tj][ti]
 template <class DM, class A, class R>
-__device__ __forceinline__ void angular_g2(const A& a, int ti, int tj, R r, R irA, int NA, int KA, R* g, R* gp, R* h,
+__device__ __forceinline__ void angular_g2(const A& a, int ti, int tj, R r, const Cutoff<R>& cutA, int NA, int KA, R* g, R* gp, R* h,
                                            R* hp) {
     R f[DM::KX], fp[DM::KX];
-    basis_derivs<DM::KX>(r, irA, KA, [&](int k, R v, R d) {
+    basis_derivs<DM::KX>(r, cutA, KA, [&](int k, R v, R d) {
         f[k] = v;
         fp[k] = d;
     });
@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(kF64Threads) k64_atom(const A a) {
         // the owner's angular pair forces, and each pair's to its reverse slot
         __syncwarp();
         const R* Ri = gb + o.oS;
-        const R irA = R(1.0) / (R)a.rc_ang;
+        const Cutoff<R> cutA((R)a.rc_ang);
         const int KA = DM::KA(a);
         R acc[12];
 #pragma unroll
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(kF64Threads) k64_atom(const A a) {
             PairT<R> p;
             if (!pair_at(a, fr, s, p) || !(p.r < (R)a.rc_ang)) continue;
             R g[NAX], gp[NAX];
-            angular_g<DM>(a, fr.ti, p.tj, p.r, irA, NA, KA, g, gp);
+            angular_g<DM>(a, fr.ti, p.tj, p.r, cutA, NA, KA, g, gp);
             const Harm<R> ht = harm_of(p.u[0], p.u[1], p.u[2]);
             HarmSums<R> hs(ht);
 #pragma unroll
@@ -367,7 +367,7 @@ __global__ void __launch_bounds__(kF64Threads) k64_force(const A a) {
         for (int x = lane; x < own; x += G) Ri[x] = a.R[(size_t)i * own + x];
     for (int x = lane; x < T * KR; x += G) Pi[x] = a.p[(size_t)i * T * KR + x];
     __syncwarp();
-    const R irR = R(1.0) / (R)a.rc_rad;
+    const Cutoff<R> cutR((R)a.rc_rad);
     R acc[12];
 #pragma unroll
     for (int c = 0; c < 12; ++c) acc[c] = R(0.0);
@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(kF64Threads) k64_force(const A a) {
             const R* pi = Pi + p.tj * KR;
             const R* pj = a.p + ((size_t)p.j * T + fr.ti) * KR;
             R di = R(0.0), dj = R(0.0);
-            basis_derivs<DM::KX>(p.r, irR, KR, [&](int k, R, R fp) {
+            basis_derivs<DM::KX>(p.r, cutR, KR, [&](int k, R, R fp) {
                 di += pi[k] * fp;
                 dj += pj[k] * fp;
             });
@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(kF64Threads) k64_force(const A a) {
     }
     __syncwarp();
     if constexpr (!kScatter<A>) {
-        const R irA = R(1.0) / (R)a.rc_ang;
+        const Cutoff<R> cutA((R)a.rc_ang);
         const int KA = DM::KA(a);
         const bool kept = na <= kF64Slots && nc <= 65536;
         const int n2 = kept ? na : nc;
@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(kF64Threads) k64_force(const A a) {
             PairT<R> p;
             if (!pair_at(a, fr, kept ? (int)slots[c2] : c2, p) || !(p.r < (R)a.rc_ang)) continue;
             R g[NAX], gp[NAX], h[NAX], hp[NAX];
-            angular_g2<DM>(a, fr.ti, p.tj, p.r, irA, NA, KA, g, gp, h, hp);
+            angular_g2<DM>(a, fr.ti, p.tj, p.r, cutA, NA, KA, g, gp, h, hp);
             const Harm<R> ht = harm_of(p.u[0], p.u[1], p.u[2]);
             const R* Rj = a.R + (size_t)p.j * NA * kLM;
             HarmSums<R> hs(ht);

@@ -170,10 +170,26 @@ __device__ __forceinline__ int warp_max_i(int v) { return __reduce_max_sync(0xff
 __device__ __forceinline__ double cospi_r(double z) { return cospi(z); }
 __device__ __forceinline__ float cospi_r(float z) { return cospif(z); }
 
+// A cutoff, and x / rc.  In float the product with the rounded 1 / rc is off by
+// the same fraction for every pair, up to 6e-8, which energies and virials add
+// up instead of averaging out; one correction by the residual takes that away.
+// Virial against 64 bits, 9,956 atoms: 11/7 functions and two species 1.5e-6
+// without and 2.7e-7 with it, 5/3 functions 5.9e-7 and 6.7e-8 (134.1 / 134.9 us).
+template <class R>
+struct Cutoff {
+    R rc, inv;
+    __device__ explicit Cutoff(R c) : rc(c), inv(R(1.0) / c) {}
+    __device__ __forceinline__ R over(R x) const {
+        const R q = x * inv;
+        if constexpr (std::is_same<R, float>::value) return fmaf(fmaf(-q, rc, x), inv, q);
+        return q;
+    }
+};
+
 // out(k, Q_k(r)) for k < K (Eqs. 12-15)
 template <int KX, class R, class Out>
-__device__ __forceinline__ void basis_values(R r, R irc, int K, Out out) {
-    const R z = r * irc, fc2 = R(0.25) * (R(1.0) + cospi_r(z)), t = z - R(1.0), x = R(2.0) * t * t - R(1.0);
+__device__ __forceinline__ void basis_values(R r, const Cutoff<R>& cut, int K, Out out) {
+    const R z = cut.over(r), fc2 = R(0.25) * (R(1.0) + cospi_r(z)), t = z - R(1.0), x = R(2.0) * t * t - R(1.0);
     R Tm = R(1.0), Tk = x;
     out(0, R(2.0) * fc2);
     if (K > 1) out(1, (x + R(1.0)) * fc2);
@@ -188,12 +204,12 @@ __device__ __forceinline__ void basis_values(R r, R irc, int K, Out out) {
 }
 // out(k, Q_k(r), dQ_k/dr) for k < K
 template <int KX, class R, class Out>
-__device__ __forceinline__ void basis_derivs(R r, R irc, int K, Out out) {
-    const R z = r * irc;
+__device__ __forceinline__ void basis_derivs(R r, const Cutoff<R>& cut, int K, Out out) {
+    const R z = cut.over(r);
     R sp, cp;
     sincospi_r(z, &sp, &cp);
-    const R fc2 = R(0.25) * (R(1.0) + cp), dfc2 = R(-0.25 * kPi) * irc * sp;
-    const R t = z - R(1.0), x = R(2.0) * t * t - R(1.0), a = R(4.0) * t * irc * fc2;
+    const R fc2 = R(0.25) * (R(1.0) + cp), dfc2 = cut.over(R(-0.25 * kPi)) * sp;
+    const R t = z - R(1.0), x = R(2.0) * t * t - R(1.0), a = cut.over(R(4.0) * t) * fc2;
     R Tm = R(1.0), Tk = x, dTm = R(0.0), dTk = R(1.0);
     out(0, R(2.0) * fc2, R(2.0) * dfc2);
     if (K > 1) out(1, (x + R(1.0)) * fc2, a + (x + R(1.0)) * dfc2);

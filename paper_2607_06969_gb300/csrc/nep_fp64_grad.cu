@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(kGrad64Threads) k64_grad_atom(const F64Args a)
     const double li[3] = {a.lam[i], a.lam[N + i], a.lam[2 * N + i]};
     const double* mu = a.mu + 9 * fr.b;
     const double aE = a.aE[fr.b];
-    const double irR = 1.0 / a.rc_rad, irA = 1.0 / a.rc_ang;
+    const Cutoff<double> cutR(a.rc_rad), cutA(a.rc_ang);
     const int nc = valid ? a.cnt[i] : 0, cmax = warp_max_i(nc);
 
     // ---- F[t][k] = sum Q_k, DF[t][k] = sum Q'_k (rhat . dr); S_nlm and
@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(kGrad64Threads) k64_grad_atom(const F64Args a)
             tangent64(a, li, mu, p, dr);
             udr = p.u[0] * dr[0] + p.u[1] * dr[1] + p.u[2] * dr[2];
             tj[ati] = p.tj;
-            basis_derivs<DM::KX>(p.r, irR, KR, [&](int k, double f, double fp) {
+            basis_derivs<DM::KX>(p.r, cutR, KR, [&](int k, double f, double fp) {
                 gb[o.oY + k * GS + ati] = f;
                 gb[o.oY + (KR + k) * GS + ati] = fp * udr;
             });
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(kGrad64Threads) k64_grad_atom(const F64Args a)
         const int na = __popc(ma), at = __popc(ma & below);
         if (ang) {
             double f[DM::KX], fp[DM::KX];
-            basis_derivs<DM::KX>(p.r, irA, KA, [&](int k, double v, double d) {
+            basis_derivs<DM::KX>(p.r, cutA, KA, [&](int k, double v, double d) {
                 f[k] = v;
                 fp[k] = d;
             });
@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(kGrad64Threads) k64_grad_atom(const F64Args a)
             tangent64(a, li, mu, p, dr);
             const double udr = p.u[0] * dr[0] + p.u[1] * dr[1] + p.u[2] * dr[2];
             tj[at] = p.tj;
-            basis_derivs<DM::KX>(p.r, irA, KA, [&](int k, double f, double fp) {
+            basis_derivs<DM::KX>(p.r, cutA, KA, [&](int k, double f, double fp) {
                 gb[o.oY + k * GS + at] = f;
                 gb[o.oY + (KA + k) * GS + at] = fp;
             });

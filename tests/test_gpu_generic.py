@@ -154,3 +154,37 @@ def test_generic_training_calls(nb):
                                                      pairs, lab["Etot"], lab["F"], lab["V"]), th, idx)
     got = g.cpu().numpy()[idx]
     assert np.linalg.norm(got - ref) <= 1e-9 * max(np.linalg.norm(ref), 1e-30)
+
+
+@pytest.mark.parametrize("name", list(SHAPES))
+def test_generic_virial_has_no_common_error(nb, name):
+    """Roundings that differ from pair to pair average out in the virial of
+    some thousand atoms; one that all pairs share, such as a rounded 1/rc (up
+    to 2^-24 of it), does not.  What scaling r does to the virial is taken from
+    the FP64 evaluation with cutoffs changed by 0.1%; the FP32 virial, over four
+    systems, has to lie within 2^-26 of that."""
+    h = SHAPES[name]
+    got, bar = [], []
+    for seed in range(4):
+        s = I.rocksalt(9, vacancy=0.13, seed=seed)
+        s.pos = (s.pos + 1.5) % s.box[0]
+        if h.n_types < 3:
+            s.types = (s.types % h.n_types).astype(np.int32)
+        th = I.init_params(h, seed=seed + 1).astype(np.float32)
+        dsys = nb.DeviceSystem.from_inputs(s)
+        nl = nb.NeighborList(s.n_atoms, 160, 80)
+
+        def virial64(scale):
+            m = nb.Model(I.Hyper(**{**h.__dict__, "rc_rad": h.rc_rad * scale, "rc_ang": h.rc_ang * scale}), th)
+            return nb.energy_forces_virial_fp64(m, dsys, nl, nb.Workspace64(m, s.n_atoms, 1))[3].cpu().numpy()
+
+        model = nb.Model(h, th)
+        ws = nb.Workspace(model, s.n_atoms, 1, 160, 80)
+        nb.neighbors(model, dsys, nl, 0.5, ws)
+        assert nb.check_list(nl) == nb.NEP_OK
+        v = nb.energy_forces_virial(model, dsys, nl, ws)[3].cpu().numpy()
+        want, other = virial64(1.0), virial64(1.001)
+        got.append(np.linalg.norm(v - want) / np.linalg.norm(want))
+        bar.append(np.linalg.norm(other - want) / np.linalg.norm(want) / 1e-3)
+    rms = lambda x: float(np.sqrt(np.mean(np.square(x))))   # noqa: E731
+    assert rms(got) <= rms(bar) * 2.0 ** -26, (rms(got), rms(bar) * 2.0 ** -26)
