@@ -135,7 +135,9 @@ typedef struct {
  * by the FP32 predicate dx = (x_j - x_i) + s_x L_x (and y, z),
  * d2 = (dx*dx + dy*dy) + dz*dz, d2 < fl32(rc*rc) (the sum over j of Eq. 3).
  * Its first cnt_ang[i] entries are exactly those with d < rc_ang + skin; the
- * remaining ones are ordered with d < rc_rad before d >= rc_rad.
+ * remaining ones are ordered with d < rc_rad before d >= rc_rad.  The FP32
+ * calls take angular pairs from that prefix, so a list serves the model that
+ * built it and others whose cutoffs are no longer than that model's.
  *   nbr   [cap][N] int   slot-major: nbr[s*N + i] = j
  *   shift [cap][N] int   packed image (int8 sx | sy << 8 | sz << 16); may be
  *                        NULL when every box edge >= 2*(rc_rad+skin)+1e-3,
